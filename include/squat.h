@@ -110,7 +110,7 @@ int squat_build_subspace_from_gram(squat_subspace *s, const double *gram, int ra
  * Orthonormalisation is Cholesky QR (twice for the last basis).  A direction whose pivot falls below 1e-13 of its
  * diagonal entry (start block or Gram matrix of rank < rank_r within the block, or cond(M) on the block beyond
  * ~1e6) is dropped and contributes nothing; squat_subspace_eig_sweeps then reports, per head, the number of basis
- * columns kept (= rank_r when nothing was dropped) instead of a sweep count.  The eigenvalue / eigenvector arrays
+ * columns kept (= rank_r when nothing was dropped) instead of an iteration count.  The eigenvalue / eigenvector arrays
  * of squat_subspace_export are scratch after this call.  Enqueues on `stream`.
  */
 int squat_build_subspace_power(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
@@ -134,8 +134,8 @@ int squat_build_subspace_power_from_gram(squat_subspace *s, const double *gram, 
 int squat_subspace_export(const squat_subspace *s, void *stream, float *W_host, double *gram_host,
                           double *eigval_host, double *eigvec_host);
 int squat_subspace_import(squat_subspace *s, const float *W_host, void *stream);
-/* Diagnostics of the last build: Jacobi sweeps the eigensolver ran for each head.  Synchronises
- * `stream`.  sweeps_host is a host array of n_kv_heads ints. */
+/* Diagnostics of the last build: iterations of the slowest secular equation of the eigensolver for
+ * each head (power build: basis columns kept).  Synchronises `stream`.  sweeps_host is a host array of n_kv_heads ints. */
 int squat_subspace_eig_sweeps(const squat_subspace *s, void *stream, int *sweeps_host);
 
 /*

@@ -182,7 +182,7 @@ def squat_subspace_import(s: Subspace, W, stream=None):
 
 
 def squat_subspace_eig_sweeps(s: Subspace, stream=None):
-    """Jacobi sweeps the eigensolver ran for each head in the last build (diagnostic)."""
+    """Iterations of the eigensolver's slowest secular equation for each head in the last build (diagnostic)."""
     import numpy as np
     out = np.zeros(s.n_kv_heads, dtype=np.int32)
     _check(_load().squat_subspace_eig_sweeps(s.handle, _stream(stream), out.ctypes.data_as(ctypes.c_void_p)),

@@ -127,6 +127,8 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     const size_t o_val = carve((size_t)n_kv_heads * D * sizeof(double));
     const size_t o_vec = carve(hdd * sizeof(double));
     const size_t o_swp = carve((size_t)n_kv_heads * sizeof(int));
+    const size_t o_tri = carve((size_t)n_kv_heads * 3 * D * sizeof(double));
+    const size_t o_scl = carve((size_t)n_kv_heads * sizeof(double));
     const size_t o_exact = carve(sizeof(int));
     const size_t o_lr = carve((size_t)n_kv_heads * D * 2 * SQUAT_LOWRANK_MAX_R * sizeof(float));
     char *base = nullptr;
@@ -139,6 +141,8 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     s->eigval = reinterpret_cast<double *>(base + o_val);
     s->eigvec = reinterpret_cast<double *>(base + o_vec);
     s->eig_sweeps = reinterpret_cast<int *>(base + o_swp);
+    s->tri = reinterpret_cast<double *>(base + o_tri);
+    s->eig_scale = reinterpret_cast<double *>(base + o_scl);
     s->exact_blocks = reinterpret_cast<int *>(base + o_exact);
     s->lr_table = reinterpret_cast<float *>(base + o_lr);
     const int all_exact = D / 32;        // W starts as zero: every channel is uncorrected

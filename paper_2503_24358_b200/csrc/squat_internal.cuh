@@ -26,7 +26,9 @@ struct squat_subspace {
     double *gram_partial;  // [chunks, H, d, d] per-chunk partial Gram matrices (deterministic reduction)
     double *eigval;        // [H, d] descending
     double *eigvec;        // [H, d, d], row i = eigenvector i
-    int *eig_sweeps;       // [H] sweeps of the last eigen-decomposition
+    int *eig_sweeps;       // [H] iterations of the last eigen-decomposition's slowest secular equation (power build: columns kept)
+    double *tri;           // [H, 3, d] tridiagonal form: diagonal, subdiagonal, 1 / h of the reflectors (eig.cu)
+    double *eig_scale;     // [H] power of two that was taken out of the Gram matrix before its tridiagonalisation
     unsigned *status;      // device status word of this device
     // host path only (created on its first call): two side streams and the events that order them
     cudaStream_t side[2];

@@ -3,10 +3,7 @@
 //   gram_kernel      M_h = Qc^T Qc for the stacked prompt queries of KV head h (Section 3.2;
 //                    Algorithm 1 line 5 needs only the right singular vectors and singular values
 //                    of Qc, i.e. the eigen-pairs of M_h; GQA stacking rule of Appendix C).
-//   eig_cluster_kernel  eigen-decomposition of M_h: Cholesky M_h + shift I = L L^T, then one-sided (Hestenes)
-//                    Jacobi on the columns of L: rotations make the columns orthogonal, L V = U Sigma;
-//                    the normalised columns U are the eigenvectors v_i of M_h and the squared column
-//                    norms, minus the shift, its eigenvalues sigma_i^2.
+//   (eig.cu)         eigen-decomposition of M_h: eigenvectors v_i and eigenvalues sigma_i^2.
 //   assemble_kernel  P_inv = (I + lambda Qhat^T Qhat)^{-1} = I - sum_i s_i/(1+s_i) v_i v_i^T with
 //                    s_i = lambda sigma_i^2 (Woodbury with orthonormal v_i; footnote of Prop. 4),
 //                    then the update matrices B_t H_t of Lemma 3 read off the LDL^T factorisation
@@ -19,7 +16,6 @@
 // weight lambda sigma^2, so single precision anywhere in this step changes quantized codes
 // downstream; products of bf16 inputs are exact in fp64 and everything stays fp64 until W is
 // rounded to float32 at the very end.
-#include <cooperative_groups.h>
 #include <type_traits>
 #include <utility>
 #include "squat_internal.cuh"
@@ -211,68 +207,7 @@ __global__ void __launch_bounds__(GRED_THREADS) gram_reduce_kernel(const double 
     }
 }
 
-// ------------------------------------------------------------------------------------- eigen
-constexpr int EIG_MAX_SWEEPS = 40;
-
-// Eigen-decomposition of M: Cholesky M + shift I = L L^T, then one-sided (Hestenes) Jacobi on the columns of L.
-// L has the square root of M's condition number and L^T L is much closer to diagonal than M^2, which cuts the
-// sweeps (14 -> 10 on the 4096-token workload).  The shift (1e-12 of the trace) keeps the factorisation defined
-// for rank-deficient M and is subtracted from the eigenvalues at the end; eigenvectors are unaffected by it.
-// Rotations are skipped below 1e-14 relative; a sweep that applied none above that level is the last.
-//
-// One head is worked on by a cluster of 4 CTAs (4 SMs per head instead of 1; a 32-head layer then occupies 128
-// of the 148 SMs).  The 128 columns form 8 blocks of 16, and every CTA holds two blocks with ALL their rows, so a
-// rotation of two columns held by the same CTA needs no communication at all: a team of 16 lanes owns the pair
-// (8 rows per lane), the dot product is a 4-step shuffle reduction, and rounds inside a CTA are separated by a
-// barrier among the 8 working warps only.
-// A sweep is
-//   one intra phase   15 rounds that pair the columns inside each held block (8 + 8 pairs per round), then
-//   7 block rounds    of 16 rounds each that pair every column of one held block with every column of the other;
-//                     after each block round one block of every CTA moves to another CTA (schedule below), so
-//                     that over the 7 block rounds every block has met every other one.
-// So the CTAs talk 7 times per sweep instead of once per round.  After a block round every column sits in some
-// team's registers and is written straight into the spare buffer of its next holder (through distributed shared
-// memory if that is a peer); one cluster barrier per move publishes the data and guarantees that nobody is a block
-// round behind, which is what makes the spare buffers free.  The squared column norms ride along with the block:
-// they are refreshed from the data at the start of a sweep and updated by each rotation in between
-// (alpha' = alpha - t gamma, beta' = beta + t gamma), so a round reduces one dot product, not three.
-// The Cholesky factorisation is done redundantly by each CTA on a full copy (it is a small part of the time).
-namespace cg = cooperative_groups;
-constexpr int ECL = 4;                       // CTAs per cluster
-constexpr int ECT = 512;                     // threads per CTA: 16 warps = 16 column pairs per round
-constexpr int BW = 16;                       // columns per block
-constexpr int BLD = D + 2;                   // column stride inside a block buffer (doubles)
-constexpr int BLK_DOUBLES = BW * BLD + BW;   // 16 columns and their 16 squared norms
-// Block schedule of a sweep: 7 block rounds, each pairing the two blocks a CTA holds, such that every two of the 8
-// blocks meet exactly once (a 1-factorisation of K8 found by a randomised search; of the candidates tried, the one
-// that needed the fewest sweeps on the benchmark's Gram matrices) while only ONE block per CTA changes
-// hands between consecutive rounds -- the minimum, since two blocks that have met must part.  Move m (after
-// block round m): bit c of MOVE_KEEP1[m] says that CTA c keeps its slot-1 block (else its slot-0 block); the other
-// one goes to CTA (MOVE_TO[m] >> 2c) & 3, where it becomes slot 1.  The schedule is positional, so it covers all
-// pairs from whatever arrangement the previous sweep left.
-__constant__ unsigned char MOVE_KEEP1[7] = {0x5, 0xb, 0x9, 0xd, 0xe, 0x5, 0x5};
-__constant__ unsigned char MOVE_TO[7] = {0x1e, 0x4b, 0xb1, 0x4e, 0x39, 0x8d, 0x1e};
-constexpr unsigned BLK_BYTES = BLK_DOUBLES * (unsigned)sizeof(double);
 static_assert(GRAM_TILES_PER_WARP * (GRAM_THREADS / 32) == 136, "the warps share the upper triangle evenly");
-static_assert(D / BW == 2 * ECL, "two blocks per CTA");
-static_assert(BLK_BYTES % 16 == 0, "bulk copies move 16-byte units");
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-    return v;
-}
-
-// 1/sqrt(x) for a normal positive double: hardware seed y (relative error 2^-22), residual r = 1 - x y^2, and one
-// third-order correction y (1 + r/2 + 3 r^2/8); what is left, about r^3/3, is far below a double's rounding.
-__device__ __forceinline__ double rsqrt_nr(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double r = fma(-(x * y), y, 1.0);
-    return fma(y * r, fma(0.375, r, 0.5), y);
-}
 
 // 1/x for a normal double: hardware seed (about 20 bits), two Newton steps y <- y + y (1 - x y)
 __device__ __forceinline__ double rcp_nr(double x)
@@ -281,274 +216,6 @@ __device__ __forceinline__ double rcp_nr(double x)
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     y = fma(y, fma(-x, y, 1.0), y);
     return fma(y, fma(-x, y, 1.0), y);
-}
-
-__device__ __forceinline__ void named_bar_sync(int id, int count) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
-
-// One Jacobi rotation of a column pair (P, Q) held in registers by a team of 16 lanes (both halves of a warp work
-// on different pairs): lane l owns rows l, l + 16, ..., l + 112.  alpha, beta are the (cached) squared norms, kept by
-// every lane; gamma = P . Q is reduced here.  New P = c P - s Q, new Q = s P + c Q with the angle that makes them
-// orthogonal (tan 2theta = 2 gamma / (beta - alpha), |theta| <= pi/4), from two reciprocal square roots.  A pair
-// already orthogonal to 1e-14 relative, or numerically null twice over, is left alone (returns 0); otherwise
-// returns 1, or 3 when the pair started above the convergence level.
-constexpr int TLN = 16;                      // lanes per team
-constexpr int TROWS = D / TLN;               // rows per lane of a team: 2 tl + 32 i and 2 tl + 1 + 32 i, i < TROWS / 2
-__device__ __forceinline__ void load_col(double (&x)[TROWS], const double *col, int tl)
-{
-#pragma unroll
-    for (int i = 0; i < TROWS / 2; ++i) {
-        const double2 v = *reinterpret_cast<const double2 *>(col + 2 * tl + 2 * TLN * i);
-        x[2 * i] = v.x;
-        x[2 * i + 1] = v.y;
-    }
-}
-__device__ __forceinline__ void store_col(double *col, const double (&x)[TROWS], int tl)
-{
-#pragma unroll
-    for (int i = 0; i < TROWS / 2; ++i) *reinterpret_cast<double2 *>(col + 2 * tl + 2 * TLN * i) = make_double2(x[2 * i], x[2 * i + 1]);
-}
-__device__ __forceinline__ int rotate_regs(double (&xp)[TROWS], double (&xq)[TROWS], double &alpha, double &beta, double null_thr)
-{
-    double g0 = 0.0, g1 = 0.0;
-#pragma unroll
-    for (int i = 0; i < TROWS; i += 2) { g0 = fma(xp[i], xq[i], g0); g1 = fma(xp[i + 1], xq[i + 1], g1); }
-    double gam = g0 + g1;
-#pragma unroll
-    for (int m = TLN / 2; m >= 1; m >>= 1) gam += __shfl_xor_sync(0xffffffffu, gam, m);
-    const double g2 = gam * gam, ab = alpha * beta;
-    if (!((alpha > null_thr || beta > null_thr) && g2 > 1e-28 * ab)) return 0;      // uniform over the team
-    const double diff = beta - alpha;
-    const double inv_r = rsqrt_nr(fma(diff, diff, 4.0 * g2));
-    const double hc = fma(0.5 * fabs(diff), inv_r, 0.5);              // (1 + cos 2theta)/2 = c^2, in [1/2, 1]
-    const double inv_c = rsqrt_nr(hc);
-    const double c = hc * inv_c;
-    const double sm = gam * inv_r * inv_c;
-    const double s = diff < 0.0 ? -sm : sm;
-    const double t = s * inv_c;                                       // tan(theta)
-#pragma unroll
-    for (int i = 0; i < TROWS; ++i) {
-        const double p = xp[i], q = xq[i];
-        xp[i] = c * p - s * q;
-        xq[i] = s * p + c * q;
-    }
-    alpha -= t * gam;
-    beta += t * gam;
-    return g2 > 1e-14 * ab ? 3 : 1;
-}
-
-__global__ void __cluster_dims__(ECL, 1, 1) __launch_bounds__(ECT, 1) eig_cluster_kernel(
-    const double *__restrict__ gram, double *__restrict__ eigval, double *__restrict__ eigvec,
-    int *__restrict__ sweeps_out, unsigned *__restrict__ status)
-{
-    cg::cluster_group cluster = cg::this_cluster();
-    const int crank = (int)cluster.block_rank();
-    extern __shared__ __align__(16) double sm[];
-    double *blk = sm;                                  // [2 buffers][2 slots][BLK_DOUBLES]: the held blocks and the spare
-    double *nall = blk + 4 * BLK_DOUBLES;              // [ECL][32] final column norms of the whole cluster
-    double *lcol = nall + ECL * 32;                    // [2][D] column of L being eliminated (double-buffered)
-    double *red = lcol + 2 * D;                        // [16] per-warp partial sums
-    int *flags = reinterpret_cast<int *>(red + 16);    // [ECL] "rotated above the convergence level" per CTA
-    const int h = blockIdx.x / ECL, tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    const double *M = gram + (long long)h * D * D;
-
-    // Cholesky factorisation M + shift I = L L^T with the matrix in REGISTERS: thread (lane, warp) owns the
-    // elements (row lane + 32 i, column warp + 16 k), i < 4, k < 8; only those on or below the diagonal are used.
-    // Step j: the warp that owns column j gets the pivot by a shuffle, scales its column and publishes it in shared
-    // memory; after ONE barrier (the column buffer alternates) every thread subtracts the rank-1 term from its
-    // elements.  Columns of the two blocks this CTA starts with go straight into the block buffers:
-    // positions crank (slot 0) and 7 - crank (slot 1).
-    double a[4][8];
-    double tr = 0.0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = lane + 32 * i, c = warp + 16 * k;
-            a[i][k] = M[c * D + r];                    // M is symmetric: read along the contiguous direction
-            if (r == c) tr += a[i][k];
-        }
-    tr = warp_sum(tr);
-    if (lane == 0) red[warp] = tr;
-    __syncthreads();
-    double trace = 0.0;
-#pragma unroll
-    for (int w = 0; w < 16; ++w) trace += red[w];
-    const double shift = trace > 0.0 ? 1e-12 * trace : 1e-300;       // M + shift I = L L^T
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (lane + 32 * i == warp + 16 * k) a[i][k] += shift;
-#pragma unroll
-    for (int kj = 0; kj < 8; ++kj) {
-        const int slot = kj == crank ? 0 : (kj == 2 * ECL - 1 - crank ? 1 : -1);
-#pragma unroll 1
-        for (int wj = 0; wj < 16; ++wj) {
-            const int j = 16 * kj + wj;
-            double *lc = lcol + (j & 1) * D;
-            if (warp == wj) {
-                double piv = __shfl_sync(0xffffffffu, a[kj >> 1][kj], j & 31);
-                piv = piv > 0.0 ? piv : shift;
-                const double inv = rsqrt_nr(piv);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = lane + 32 * i;
-                    const double l = r > j ? a[i][kj] * inv : (r == j ? piv * inv : 0.0);
-                    lc[r] = l;
-                    if (slot >= 0) blk[slot * BLK_DOUBLES + wj * BLD + r] = l;
-                }
-            }
-            __syncthreads();
-            double lr[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) lr[i] = lc[lane + 32 * i];
-#pragma unroll
-            for (int k = kj; k < 8; ++k) {
-                const int c = warp + 16 * k;
-                if (c > j) {                           // warp-uniform
-                    const double lcc = lc[c];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (32 * i + 31 >= 16 * k) a[i][k] = fma(-lr[i], lcc, a[i][k]);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    const double null_thr = 4.0 * shift;
-    cluster.sync();                                    // every CTA of the cluster is running before anybody writes into it
-
-    // squared norms of the 32 held columns, from the data: warp w takes columns w and w + 16
-    auto refresh_norms = [&](double *cur) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            double *col = cur + k * BLK_DOUBLES + warp * BLD;
-            double s = 0.0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { const double v = col[lane + 32 * i]; s = fma(v, v, s); }
-            s = warp_sum(s);
-            if (lane == 0) cur[k * BLK_DOUBLES + BW * BLD + warp] = s;
-        }
-        __syncthreads();
-    };
-
-    int cur_buf = 0;                                   // which buffer holds the blocks
-    bool converged = false;
-    int sweep = 0;
-    for (; sweep < EIG_MAX_SWEEPS && !converged; ++sweep) {
-        int big = 0;
-        double *cur = blk + cur_buf * 2 * BLK_DOUBLES;
-        refresh_norms(cur);
-        // Pairs are worked on by 16 teams of 16 lanes (warps 0-7); they keep in step through a barrier of their own.
-        const int team = tid / TLN, tl = tid % TLN;
-        constexpr int TEAM_THREADS = 16 * TLN;
-        // intra phase: round-robin of the 16 columns of a block; teams 0-7 on slot 0, teams 8-15 on slot 1
-        if (tid < TEAM_THREADS) {
-            double *b = cur + (team >> 3) * BLK_DOUBLES, *nb = b + BW * BLD;
-            const int t = team & 7;
-            for (int round = 0; round < BW - 1; ++round) {
-                int p, q;
-                if (t == 0) { p = BW - 1; q = round; }
-                else { p = (round + t) % (BW - 1); q = (round - t + (BW - 1)) % (BW - 1); }
-                double xp[TROWS], xq[TROWS];
-                load_col(xp, b + p * BLD, tl);
-                load_col(xq, b + q * BLD, tl);
-                double alpha = nb[p], beta = nb[q];
-                const int did = rotate_regs(xp, xq, alpha, beta, null_thr);
-                if (did) {
-                    store_col(b + p * BLD, xp, tl);
-                    store_col(b + q * BLD, xq, tl);
-                    if (tl == 0) { nb[p] = alpha; nb[q] = beta; }
-                }
-                big |= did >> 1;
-                named_bar_sync(1, TEAM_THREADS);
-            }
-        }
-        __syncthreads();
-        for (int br = 0; br < 2 * ECL - 1; ++br) {
-            cur = blk + cur_buf * 2 * BLK_DOUBLES;
-            // block round: team t keeps column t of slot 0 in registers and meets column (t + round) mod 16 of slot 1
-            if (tid < TEAM_THREADS) {
-                double *b0 = cur, *b1 = cur + BLK_DOUBLES, *n0 = b0 + BW * BLD, *n1 = b1 + BW * BLD;
-                double xa[TROWS], xb[TROWS];
-                load_col(xa, b0 + team * BLD, tl);
-                double alpha = n0[team], beta = 0.0;
-                for (int round = 0; round < BW; ++round) {
-                    const int q = (team + round) & (BW - 1);
-                    load_col(xb, b1 + q * BLD, tl);
-                    beta = n1[q];
-                    const int did = rotate_regs(xa, xb, alpha, beta, null_thr);
-                    if (did && round < BW - 1) {
-                        store_col(b1 + q * BLD, xb, tl);
-                        if (tl == 0) n1[q] = beta;
-                    }
-                    big |= did >> 1;
-                    named_bar_sync(1, TEAM_THREADS);
-                }
-                // Move the blocks on.  After the last round every column sits in some team's registers (column `team`
-                // of slot 0 and column team + 15 mod 16 of slot 1).  Each CTA keeps one of its two blocks (it becomes
-                // slot 0 of the other buffer: plain stores) and sends the other to a peer (slot 1 of the peer's other
-                // buffer: stores through distributed shared memory), as the schedule says.  That buffer is free: its
-                // owner left it when it began this block round.
-                const bool keep1 = (MOVE_KEEP1[br] >> crank) & 1;
-                double *kept_home = blk + ((cur_buf ^ 1) * 2 + 0) * BLK_DOUBLES;
-                double *sent_home = cluster.map_shared_rank(blk + ((cur_buf ^ 1) * 2 + 1) * BLK_DOUBLES, (MOVE_TO[br] >> (2 * crank)) & 3);
-                double *d0 = keep1 ? sent_home : kept_home, *d1 = keep1 ? kept_home : sent_home;
-                const int ql = (team + BW - 1) & (BW - 1);
-                store_col(d0 + team * BLD, xa, tl);
-                store_col(d1 + ql * BLD, xb, tl);
-                if (tl == 0) { d0[BW * BLD + team] = alpha; d1[BW * BLD + ql] = beta; }
-            }
-            if (br == 2 * ECL - 2) {
-                // the sweep is the last one if no CTA of the cluster rotated a pair from above the convergence level
-                big = __syncthreads_or(big);
-                if (tid < ECL) *cluster.map_shared_rank(&flags[crank], tid) = big ? 1 : 0;
-            }
-            cluster.sync();                            // blocks (and flags) have arrived; nobody is behind by a block round
-            cur_buf ^= 1;
-        }
-        int any = 0;
-#pragma unroll
-        for (int r = 0; r < ECL; ++r) any |= flags[r];  // rewritten only after seven more cluster barriers
-        converged = any == 0;
-    }
-    if (tid == 0 && crank == 0) {
-        sweeps_out[h] = sweep;
-        if (!converged) atomicOr(status, SQUAT_FLAG_NO_CONVERGE);
-    }
-
-    // singular values of L = sqrt(mu + shift) are the column norms; rank them over the whole cluster
-    double *cur = blk + cur_buf * 2 * BLK_DOUBLES;
-    refresh_norms(cur);
-    if (tid < 32) {
-        const double n2 = cur[(tid >> 4) * BLK_DOUBLES + BW * BLD + (tid & 15)];
-        const double nv = sqrt(n2);
-#pragma unroll
-        for (int r = 0; r < ECL; ++r) *cluster.map_shared_rank(&nall[crank * 32 + tid], r) = nv;
-    }
-    cluster.sync();
-    for (int k = 0; k < 2; ++k) {                      // warp w writes held columns w (slot 0) and w (slot 1)
-        const int id = crank * 32 + k * BW + warp;
-        const double mine = nall[id];
-        int rk = 0;
-        for (int j = lane; j < D; j += 32) {
-            const double o = nall[j];
-            rk += (o > mine) || (o == mine && j < id);
-        }
-#pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) rk += __shfl_xor_sync(0xffffffffu, rk, m);
-        const double *col = cur + k * BLK_DOUBLES + warp * BLD;
-        const double inv = mine > 0.0 ? 1.0 / mine : 0.0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            eigvec[(long long)h * D * D + (long long)rk * D + lane + 32 * i] = col[lane + 32 * i] * inv;
-        if (lane == 0) {
-            const double mu_out = mine * mine - shift;
-            eigval[(long long)h * D + rk] = mu_out > 0.0 ? mu_out : 0.0;
-        }
-    }
-    cluster.sync();                                    // no CTA exits while a peer may still write into it
 }
 
 // ------------------------------------------------------------------------------------- assemble
@@ -714,16 +381,6 @@ int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
     gram_reduce_kernel<<<dim3(GRED_UNITS / GRED_THREADS, H), GRED_THREADS, 0, st>>>(s->gram_partial, chunks, H, s->gram);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
-}
-
-int squat_launch_eig(squat_subspace *s, cudaStream_t st)
-{
-    const size_t smem = sizeof(double) * (4 * BLK_DOUBLES + ECL * 32 + 2 * D + 16) + sizeof(int) * ECL;
-    SQUAT_CUDA(cudaFuncSetAttribute(eig_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    eig_cluster_kernel<<<s->n_kv_heads * ECL, ECT, smem, st>>>(s->gram, s->eigval, s->eigvec, s->eig_sweeps, s->status);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
     return SQUAT_OK;

@@ -1,0 +1,57 @@
+"""GPU: the eigen-decomposition of step 1 (tridiagonal reduction, divide and conquer) on spectra where it can go wrong --
+multiple and clustered eigenvalues, rank deficiency, a matrix that is diagonal or tridiagonal already, decades of grading,
+extreme scales -- against numpy's symmetric eigensolver, through squat_build_subspace_from_gram."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2503_24358_b200 as sq
+
+pytestmark = pytest.mark.gpu
+D = 128
+
+
+def _matrix(kind):
+    rng = np.random.default_rng(11)
+    Q = np.linalg.qr(rng.standard_normal((D, D)))[0]
+    spectrum = lambda mu: (Q * mu) @ Q.T
+    if kind == "identity":
+        return 3.0 * np.eye(D)
+    if kind == "diagonal":
+        return np.diag(rng.uniform(0.0, 1.0, D))
+    if kind == "tridiagonal":
+        return np.diag(np.full(D, 2.0)) - np.diag(np.ones(D - 1), 1) - np.diag(np.ones(D - 1), -1)
+    if kind == "four-fold":
+        return spectrum(np.repeat([1.0, 2.0, 3.0, 4.0], D // 4))
+    if kind == "rank-1":
+        return np.outer(Q[0], Q[0])
+    if kind == "rank-33":
+        return spectrum(np.where(np.arange(D) < 33, rng.uniform(1.0, 2.0, D), 0.0))
+    if kind == "graded":
+        return spectrum(np.logspace(0, -20, D))
+    if kind == "clusters":
+        return spectrum(np.repeat([1.0, 1e-3, 1e-6, 1e-9], D // 4) * (1 + 1e-13 * rng.standard_normal(D)))
+    if kind == "blocks":
+        return np.kron(np.eye(8), np.ones((16, 16))) + 0.01 * np.eye(D)
+    return float(kind) * spectrum(rng.uniform(0.1, 1.0, D))           # scale
+
+
+@pytest.mark.parametrize("kind", ["identity", "diagonal", "tridiagonal", "four-fold", "rank-1", "rank-33", "graded", "clusters",
+                                  "blocks", "1e-70", "1e80"])
+def test_eigen_pairs(kind):
+    M = _matrix(kind)
+    M = 0.5 * (M + M.T)
+    s = sq.Subspace(2, D)
+    # head 1 holds another matrix: the heads' clusters must not mix
+    both = np.stack([M, np.roll(np.roll(M, 5, 0), 5, 1)])
+    sq.squat_build_subspace_from_gram(s, torch.from_numpy(both).cuda(), 8, 1e-3)
+    out = sq.squat_subspace_export(s, ("eigval", "eigvec"))
+    for h in range(2):
+        mu, V = out["eigval"][h], out["eigvec"][h]                    # rows of V
+        ref = np.linalg.eigvalsh(both[h])[::-1]
+        top = ref[0]
+        assert np.all(np.diff(mu) <= 0.0) and np.abs(mu - np.maximum(ref, 0.0)).max() <= 2e-12 * top
+        assert np.abs(V @ V.T - np.eye(D)).max() <= 1e-13
+        assert np.abs((both[h] / top) @ V.T - V.T * (mu / top)).max() <= 2e-12
+    assert sq.squat_get_device_status(clear=True) & sq.FLAG_NO_CONVERGE == 0
+    s.close()
