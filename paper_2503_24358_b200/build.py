@@ -15,7 +15,7 @@ OBJ_DIR = os.path.join(_HERE, "build")
 LIB = os.path.join(_HERE, "libsquat.so")
 OBJ_DIR_CHECKED = os.path.join(_HERE, "build_checked")
 LIB_CHECKED = os.path.join(_HERE, "libsquat_checked.so")
-SOURCES = ["api.cu", "values.cu", "keys.cu", "subspace.cu", "eig.cu", "power.cu", "attention.cu", "peak.cu", "keys_lowrank.cu"]
+SOURCES = ["api.cu", "values.cu", "keys.cu", "subspace.cu", "eig.cu", "power.cu", "attention.cu", "attention_mma.cu", "peak.cu", "keys_lowrank.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
@@ -34,8 +34,8 @@ def _deps_mtime():
 
 def _compile(src, verbose, obj_dir=OBJ_DIR, extra=()):
     obj = os.path.join(obj_dir, src.replace(".cu", ".o"))
-    hdr_time = max(os.path.getmtime(os.path.join(CSRC, "squat_internal.cuh")),
-                   os.path.getmtime(os.path.join(INCLUDE, "squat.h")))
+    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")] + [os.path.join(INCLUDE, "squat.h")]
+    hdr_time = max(os.path.getmtime(p) for p in headers)
     src_path = os.path.join(CSRC, src)
     if os.path.exists(obj) and os.path.getmtime(obj) >= max(os.path.getmtime(src_path), hdr_time):
         return obj

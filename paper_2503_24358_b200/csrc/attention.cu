@@ -4,18 +4,18 @@
 //
 //   out_hq = softmax_i( s <q_hq, k_i> ) . v_i ,   k_i, v_i = dequantized cache rows, then the residual rows
 //
-// The cache is never dequantized to memory.  Per-channel key metadata folds into the query: for the G tokens
-// that share (scale_c, zero_c),  <q, deq(k_t)> = sum_c (q_c scale_c) code_tc + sum_c q_c zero_c, so a group
-// costs one scaled copy of the query and each token one dot product with its 128 codes.  Per-token value
-// metadata folds into the weight: p_t deq(v_t)_c = (p_t scale_tg) code_tc + p_t zero_tg.  Codes become floats
-// without a conversion: the code bits are shifted under the top of a float's mantissa, giving 1 + code / 2^bits
-// exactly (two integer instructions); the "1 +" is taken out again through one constant per group.
+// The cache is never dequantized to memory.  Keys stored after the rotary embedding: attn_mma_kernel (attention_mma.cu), both
+// phases on the integer tensor cores.  Here:
 //
-// attn_partial_kernel   grid (token chunks of 256..1024 x query-head passes, KV heads, batch).  Key phase: a warp takes
+// attn_partial_kernel   keys stored before the rotary embedding.  Grid (token chunks of 256..1024 x query-head passes, KV
+//                       heads, batch).  Key phase: a warp takes
 //                       32 tokens (lane = token, its codes are 2 or 4 128-bit loads), scores go to shared
 //                       memory.  Then the chunk's maximum and exp().  Value phase: a warp reads 128 bytes of
 //                       codes per step (lane = one 32-bit word of one of 4 or 2 tokens) and accumulates
-//                       weight x code for its channels.  Writes (unnormalised sum, max, denominator) per chunk.
+//                       weight x code for its channels; per-token value metadata folds into the weight: p_t deq(v_t)_c =
+//                       (p_t scale_tg) code_tc + p_t zero_tg.  Codes become floats without a conversion: the code bits are
+//                       shifted under the top of a float's mantissa, giving 1 + code / 2^bits exactly; the "1 +" is taken
+//                       out again through one constant per group.  Writes (unnormalised sum, max, denominator) per chunk.
 // attn_combine_kernel   grid (query heads, batch): adds the residual buffer's tokens (plain fp32 dot products)
 //                       and merges the chunks with the usual max / denominator rescaling.
 //
@@ -29,9 +29,8 @@
 // sines come from two tables the host fills in float64 (squat_rope_table_fill); the kernel only multiplies.  The
 // key metadata cannot be folded into the query on this path: each pair is dequantized (one FMA per element),
 // turned (4) and multiplied with the block-turned query of every head (2 per head).
-#include "squat_internal.cuh"
 #include <type_traits>
-#include <cuda_fp16.h>
+#include "attention.cuh"
 
 namespace {
 
@@ -39,27 +38,6 @@ constexpr int D = SQUAT_D;
 constexpr int AT_THREADS = 256;
 constexpr int AT_WARPS = AT_THREADS / 32;
 constexpr int AT_CHUNK = 1024;            // most tokens per CTA (the launcher takes 256, 512 or 1024: enough CTAs to fill the GPU)
-
-struct AttnParams {
-    const void *q;             // [B, Hq, D]
-    int q_bf16;
-    int B, Hq, H, T;           // T: quantized tokens per (batch, head)
-    const unsigned char *kc, *vc;
-    const void *ks, *kz, *vs, *vz;   // float32, or binary16 in the M16 instances
-    long long csb, csh;        // cache strides in tokens
-    int G;
-    const void *k_res, *v_res; // [B, H, R, D]
-    int res_bf16, R;
-    float scale;
-    float *part;               // [B, Hq, nchunk, D]
-    float *ml;                 // [B, Hq, nchunk, 2]
-    int nchunk, chunk;         // chunk: tokens per CTA, a multiple of 256
-    float *out;                // [B, Hq, D]
-    // rotary tables (pre-embedding key storage only): cos/sin of (32 a theta_i) [blocks][64] and of (l theta_i) [32][64]
-    const float2 *rope_a, *rope_b;
-    long long first_pos;       // position of cached token 0; a multiple of 32
-    int meta16;                // the cache's scales and zero-points are binary16
-};
 
 // 1 + code / 2^BITS as a float, for the code at position i of a 32-bit word (low bits first)
 // A constant the compiler has to keep in a register: `(x & mask) | constant` is then ONE three-input logic instruction
@@ -123,12 +101,6 @@ __device__ __forceinline__ float sum2f(u64 v)
     return lo + hi;
 }
 
-__device__ __forceinline__ float warp_sum_f(float v)
-{
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-    return v;
-}
 __device__ __forceinline__ float warp_max_f(float v)
 {
 #pragma unroll
@@ -136,34 +108,8 @@ __device__ __forceinline__ float warp_max_f(float v)
     return v;
 }
 
-__device__ __forceinline__ float load_elem(const void *p, long long idx, int bf16)
-{
-    if (bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p)[idx]);
-    return reinterpret_cast<const float *>(p)[idx];
-}
-
-// scale / zero-point element i of a metadata array stored as float32 or binary16
-template <bool M16>
-__device__ __forceinline__ float meta_at(const void *p, long long i)
-{
-    if (M16) return __half2float(__ldg(reinterpret_cast<const __half *>(p) + i));
-    return __ldg(reinterpret_cast<const float *>(p) + i);
-}
-// four consecutive elements starting at i (a multiple of 4)
-template <bool M16>
-__device__ __forceinline__ float4 meta4_at(const void *p, long long i)
-{
-    if (M16) {
-        const uint2 r = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p) + i));
-        const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&r.x));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&r.y));
-        return make_float4(a.x, a.y, b.x, b.y);
-    }
-    return __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(p) + i));
-}
-
-template <int BITS, int NQ, bool ROPE, bool M16>
-__global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? (ROPE ? 2 : 3) : (ROPE ? 3 : 4)) attn_partial_kernel(const AttnParams p)
+template <int BITS, int NQ, bool M16>
+__global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? 2 : 3) attn_partial_kernel(const AttnParams p)
 {
     constexpr int WPT = D * BITS / 32;                          // 32-bit words per token: 8 or 16
     constexpr int CPW = 32 / BITS;                              // codes per word: 16 or 8
@@ -175,8 +121,8 @@ __global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? (ROPE ? 2 : 3) : (ROPE ?
     float *qs = qsm + NQ * D;                                   // [warps][NQ][D] query x key scale x 2^BITS of the warp's group
     float *sc = qs + AT_WARPS * NQ * D;                         // [NQ][AT_CHUNK] scores, then weights
     float *red = sc + NQ * AT_CHUNK;                            // [NQ][warps] and [NQ] scratch of the reductions
-    float2 *lane_turn = reinterpret_cast<float2 *>(red + NQ * AT_WARPS + 8);   // ROPE: [64][32] cos/sin of (lane theta_i)
-    float4 *sz_all = reinterpret_cast<float4 *>(lane_turn + 64 * 32);           // ROPE: [warps][64] (S_i, Z_i, S_{i+64}, Z_{i+64})
+    float2 *lane_turn = reinterpret_cast<float2 *>(red + NQ * AT_WARPS + 8);   // [64][32] cos/sin of (lane theta_i)
+    float4 *sz_all = reinterpret_cast<float4 *>(lane_turn + 64 * 32);           // [warps][64] (S_i, Z_i, S_{i+64}, Z_{i+64})
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int chunk = blockIdx.x % p.nchunk, qpass = blockIdx.x / p.nchunk;
     const int h = blockIdx.y, b = blockIdx.z;
@@ -188,145 +134,61 @@ __global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? (ROPE ? 2 : 3) : (ROPE ?
 
     for (int i = tid; i < NQ * D; i += AT_THREADS) {
         const int qi = i / D, c = i % D;
-        qsm[i] = qi < nq_here ? p.scale * load_elem(p.q, ((long long)b * p.Hq + hq0 + qi) * D + c, p.q_bf16) : 0.0f;
+        qsm[i] = qi < nq_here ? p.scale * attn_load_elem(p.q, ((long long)b * p.Hq + hq0 + qi) * D + c, p.q_bf16) : 0.0f;
     }
-    if (ROPE) {
-        for (int i = tid; i < 64 * 32; i += AT_THREADS) lane_turn[i] = __ldg(p.rope_b + (i & 31) * 64 + (i >> 5));   // [pair][lane]
-    }
+    for (int i = tid; i < 64 * 32; i += AT_THREADS) lane_turn[i] = __ldg(p.rope_b + (i & 31) * 64 + (i >> 5));   // [pair][lane]
     __syncthreads();
 
     // ---------------------------------------------------------------- key phase: scores
     float *qsw = qs + warp * NQ * D;
     for (int blk = t0 + 32 * warp; blk < t1; blk += 32 * AT_WARPS) {
         const long long mrow = (ctok0 / p.G + blk / p.G) * D;
-        if (ROPE) {
-            // ---- keys stored before the rotary embedding
-            const long long a_blk = (p.first_pos + blk) >> 5;          // block turn: the same for the warp's 32 tokens
-            float2 *qb = reinterpret_cast<float2 *>(qsw);              // [NQ][64]: the heads' queries turned back by the block turn
-            float4 *sz = sz_all + warp * 64;
-            // this lane's token's codes first: their latency overlaps the tables' and the metadata's
-            const uint4 *cp = reinterpret_cast<const uint4 *>(p.kc + (ctok0 + blk + lane) * (long long)(D * BITS / 8));
-            uint32_t wd[WPT];
-#pragma unroll
-            for (int v4 = 0; v4 < WPT / 4; ++v4) {
-                const uint4 cw = __ldg(cp + v4);
-                wd[4 * v4] = cw.x; wd[4 * v4 + 1] = cw.y; wd[4 * v4 + 2] = cw.z; wd[4 * v4 + 3] = cw.w;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int i = lane + 32 * hh;
-                const float2 cs = __ldg(p.rope_a + a_blk * 64 + i);
-#pragma unroll
-                for (int qi = 0; qi < NQ; ++qi) {
-                    const float q0 = qsm[qi * D + i], q1 = qsm[qi * D + i + 64];
-                    qb[qi * 64 + i] = make_float2(fmaf(q0, cs.x, q1 * cs.y), fmaf(q1, cs.x, -q0 * cs.y));
-                }
-                const float s0 = meta_at<M16>(p.ks, mrow + i) * LV, s1 = meta_at<M16>(p.ks, mrow + i + 64) * LV;
-                sz[i] = make_float4(s0, meta_at<M16>(p.kz, mrow + i) - s0, s1, meta_at<M16>(p.kz, mrow + i + 64) - s1);
-            }
-            __syncwarp();
-            float acc[NQ][2];
-#pragma unroll
-            for (int qi = 0; qi < NQ; ++qi) acc[qi][0] = acc[qi][1] = 0.0f;
-#pragma unroll
-            for (int wi = 0; wi < WPT / 2; ++wi)
-#pragma unroll
-                for (int pos = 0; pos < CPW; ++pos) {
-                    const int i = wi * CPW + pos;                       // pair (i, i + 64): same code position, WPT / 2 words apart
-                    const float4 m4 = sz[i];
-                    const float k0 = fmaf(code_as_float<BITS>(wd[wi], pos, one_bits), m4.x, m4.y);
-                    const float k1 = fmaf(code_as_float<BITS>(wd[wi + WPT / 2], pos, one_bits), m4.z, m4.w);
-                    const float2 cs = lane_turn[i * 32 + lane];
-                    const float r0 = fmaf(k0, cs.x, -k1 * cs.y), r1 = fmaf(k0, cs.y, k1 * cs.x);
-#pragma unroll
-                    for (int qi = 0; qi < NQ; ++qi) {
-                        const float2 qq = qb[qi * 64 + i];
-                        acc[qi][pos & 1] = fmaf(r1, qq.y, fmaf(r0, qq.x, acc[qi][pos & 1]));
-                    }
-                }
-#pragma unroll
-            for (int qi = 0; qi < NQ; ++qi) sc[qi * AT_CHUNK + blk - t0 + lane] = acc[qi][0] + acc[qi][1];
-            continue;
-        }
-        const float4 s4 = meta4_at<M16>(p.ks, mrow + 4 * lane);
-        const float4 z4 = meta4_at<M16>(p.kz, mrow + 4 * lane);
-        // this lane's token's codes: asked for before the metadata are worked on, so that the two loads' latencies overlap
+        const long long a_blk = (p.first_pos + blk) >> 5;          // block turn: the same for the warp's 32 tokens
+        float2 *qb = reinterpret_cast<float2 *>(qsw);              // [NQ][64]: the heads' queries turned back by the block turn
+        float4 *sz = sz_all + warp * 64;
+        // this lane's token's codes first: their latency overlaps the tables' and the metadata's
         const uint4 *cp = reinterpret_cast<const uint4 *>(p.kc + (ctok0 + blk + lane) * (long long)(D * BITS / 8));
-        uint4 cwv[WPT / 4];
-#pragma unroll
-        for (int v4 = 0; v4 < WPT / 4; ++v4) cwv[v4] = __ldg(cp + v4);
-        float k0[NQ];
-        __syncwarp();
-#pragma unroll
-        for (int qi = 0; qi < NQ; ++qi) {
-            const float4 qv = *reinterpret_cast<const float4 *>(qsm + qi * D + 4 * lane);
-            const float4 v = make_float4(qv.x * s4.x * LV, qv.y * s4.y * LV, qv.z * s4.z * LV, qv.w * s4.w * LV);
-            *reinterpret_cast<float4 *>(qsw + qi * D + 4 * lane) = v;
-            const float zs = qv.x * z4.x + qv.y * z4.y + qv.z * z4.z + qv.w * z4.w;
-            // sum_c q_c zero_c - sum_c qs'_c bias_c takes the codes' constants out again: "1 +", or for 2-bit codes
-            // "4 +" on even and "1 +" on odd channels (code_pair_as_floats)
-            k0[qi] = PAIRS ? warp_sum_f(zs - (4.0f * v.x + v.y + 4.0f * v.z + v.w)) : warp_sum_f(zs - (v.x + v.y + v.z + v.w));
-        }
-        __syncwarp();
-        if (PAIRS) {
-            // two channels per instruction: (f_even, f_odd) x (q'_even, q'_odd) into two packed accumulators per head
-            u64 acc2[NQ][2];
-#pragma unroll
-            for (int qi = 0; qi < NQ; ++qi) acc2[qi][0] = acc2[qi][1] = 0ull;
-#pragma unroll
-            for (int v4 = 0; v4 < WPT / 4; ++v4) {
-                const uint4 cw = cwv[v4];
-                const uint32_t w4[4] = {cw.x, cw.y, cw.z, cw.w};
-#pragma unroll
-                for (int wi = 0; wi < 4; ++wi)
-#pragma unroll
-                    for (int i4 = 0; i4 < CPW / 4; ++i4) {
-                        const int ch = (v4 * 4 + wi) * CPW + 4 * i4;
-                        float f0, f1, f2, f3;
-                        code_pair_as_floats(w4[wi], 2 * i4, f0, f1, one_bits, four_bits);
-                        code_pair_as_floats(w4[wi], 2 * i4 + 1, f2, f3, one_bits, four_bits);
-                        const u64 fa = pack2f(f0, f1), fb = pack2f(f2, f3);
-#pragma unroll
-                        for (int qi = 0; qi < NQ; ++qi) {
-                            const ulonglong2 qq = *reinterpret_cast<const ulonglong2 *>(qsw + qi * D + ch);
-                            acc2[qi][0] = ffma2(fa, qq.x, acc2[qi][0]);
-                            acc2[qi][1] = ffma2(fb, qq.y, acc2[qi][1]);
-                        }
-                    }
-            }
-#pragma unroll
-            for (int qi = 0; qi < NQ; ++qi)
-                sc[qi * AT_CHUNK + blk - t0 + lane] = (sum2f(acc2[qi][0]) + sum2f(acc2[qi][1])) + k0[qi];
-        } else {
-        float acc[NQ][4];                                      // four partial sums per query head: independent FMA chains
-#pragma unroll
-        for (int qi = 0; qi < NQ; ++qi) acc[qi][0] = acc[qi][1] = acc[qi][2] = acc[qi][3] = 0.0f;
+        uint32_t wd[WPT];
 #pragma unroll
         for (int v4 = 0; v4 < WPT / 4; ++v4) {
-            const uint4 cw = cwv[v4];
-            const uint32_t w4[4] = {cw.x, cw.y, cw.z, cw.w};
+            const uint4 cw = __ldg(cp + v4);
+            wd[4 * v4] = cw.x; wd[4 * v4 + 1] = cw.y; wd[4 * v4 + 2] = cw.z; wd[4 * v4 + 3] = cw.w;
+        }
+        __syncwarp();
 #pragma unroll
-            for (int wi = 0; wi < 4; ++wi)
+        for (int hh = 0; hh < 2; ++hh) {
+            const int i = lane + 32 * hh;
+            const float2 cs = __ldg(p.rope_a + a_blk * 64 + i);
 #pragma unroll
-                for (int i4 = 0; i4 < CPW / 4; ++i4) {
-                    const int ch = (v4 * 4 + wi) * CPW + 4 * i4;
-                    const float f0 = code_as_float<BITS>(w4[wi], 4 * i4, one_bits), f1 = code_as_float<BITS>(w4[wi], 4 * i4 + 1, one_bits),
-                                f2 = code_as_float<BITS>(w4[wi], 4 * i4 + 2, one_bits), f3 = code_as_float<BITS>(w4[wi], 4 * i4 + 3, one_bits);
+            for (int qi = 0; qi < NQ; ++qi) {
+                const float q0 = qsm[qi * D + i], q1 = qsm[qi * D + i + 64];
+                qb[qi * 64 + i] = make_float2(fmaf(q0, cs.x, q1 * cs.y), fmaf(q1, cs.x, -q0 * cs.y));
+            }
+            const float s0 = attn_meta<M16>(p.ks, mrow + i) * LV, s1 = attn_meta<M16>(p.ks, mrow + i + 64) * LV;
+            sz[i] = make_float4(s0, attn_meta<M16>(p.kz, mrow + i) - s0, s1, attn_meta<M16>(p.kz, mrow + i + 64) - s1);
+        }
+        __syncwarp();
+        float acc[NQ][2];
 #pragma unroll
-                    for (int qi = 0; qi < NQ; ++qi) {
-                        const float4 qq = *reinterpret_cast<const float4 *>(qsw + qi * D + ch);
-                        acc[qi][0] = fmaf(f0, qq.x, acc[qi][0]);
-                        acc[qi][1] = fmaf(f1, qq.y, acc[qi][1]);
-                        acc[qi][2] = fmaf(f2, qq.z, acc[qi][2]);
-                        acc[qi][3] = fmaf(f3, qq.w, acc[qi][3]);
-                    }
+        for (int qi = 0; qi < NQ; ++qi) acc[qi][0] = acc[qi][1] = 0.0f;
+#pragma unroll
+        for (int wi = 0; wi < WPT / 2; ++wi)
+#pragma unroll
+            for (int pos = 0; pos < CPW; ++pos) {
+                const int i = wi * CPW + pos;                       // pair (i, i + 64): same code position, WPT / 2 words apart
+                const float4 m4 = sz[i];
+                const float k0 = fmaf(code_as_float<BITS>(wd[wi], pos, one_bits), m4.x, m4.y);
+                const float k1 = fmaf(code_as_float<BITS>(wd[wi + WPT / 2], pos, one_bits), m4.z, m4.w);
+                const float2 cs = lane_turn[i * 32 + lane];
+                const float r0 = fmaf(k0, cs.x, -k1 * cs.y), r1 = fmaf(k0, cs.y, k1 * cs.x);
+#pragma unroll
+                for (int qi = 0; qi < NQ; ++qi) {
+                    const float2 qq = qb[qi * 64 + i];
+                    acc[qi][pos & 1] = fmaf(r1, qq.y, fmaf(r0, qq.x, acc[qi][pos & 1]));
                 }
-        }
+            }
 #pragma unroll
-        for (int qi = 0; qi < NQ; ++qi)
-            sc[qi * AT_CHUNK + blk - t0 + lane] = ((acc[qi][0] + acc[qi][1]) + (acc[qi][2] + acc[qi][3])) + k0[qi];
-        }
+        for (int qi = 0; qi < NQ; ++qi) sc[qi * AT_CHUNK + blk - t0 + lane] = acc[qi][0] + acc[qi][1];
     }
     __syncthreads();
 
@@ -357,7 +219,7 @@ __global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? (ROPE ? 2 : 3) : (ROPE ?
             sc[qi * AT_CHUNK + i] = e;
             s += e;
         }
-        s = warp_sum_f(s);
+        s = attn_warp_sum(s);
         if (lane == 0) red[qi * AT_WARPS + warp] = s;
     }
     __syncthreads();
@@ -430,14 +292,14 @@ __global__ void __launch_bounds__(AT_THREADS, NQ >= 4 ? (ROPE ? 2 : 3) : (ROPE ?
     for (; tk + TPI < vend; tk += 2 * TPI) {                    // two steps' loads in flight before either is used
         const long long c0 = ctok0 + tk, c1 = c0 + TPI;
         const uint32_t w0 = __ldg(vcw + c0 * WPT + j), w1 = __ldg(vcw + c1 * WPT + j);
-        const float s0 = meta_at<M16>(p.vs, c0 * ng + gidx), z0 = meta_at<M16>(p.vz, c0 * ng + gidx);
-        const float s1 = meta_at<M16>(p.vs, c1 * ng + gidx), z1 = meta_at<M16>(p.vz, c1 * ng + gidx);
+        const float s0 = attn_meta<M16>(p.vs, c0 * ng + gidx), z0 = attn_meta<M16>(p.vz, c0 * ng + gidx);
+        const float s1 = attn_meta<M16>(p.vs, c1 * ng + gidx), z1 = attn_meta<M16>(p.vz, c1 * ng + gidx);
         vstep(tk, w0, s0, z0);
         vstep(tk + TPI, w1, s1, z1);
     }
     if (tk < vend) {
         const long long c0 = ctok0 + tk;
-        vstep(tk, __ldg(vcw + c0 * WPT + j), meta_at<M16>(p.vs, c0 * ng + gidx), meta_at<M16>(p.vz, c0 * ng + gidx));
+        vstep(tk, __ldg(vcw + c0 * WPT + j), attn_meta<M16>(p.vs, c0 * ng + gidx), attn_meta<M16>(p.vz, c0 * ng + gidx));
     }
     // add the group constant, fold the token classes of the warp, then the warps
     __syncthreads();                                            // everybody is done reading sc: reuse it as [warps][NQ][D]
@@ -501,7 +363,7 @@ __global__ void __launch_bounds__(CB_THREADS, RES_BF16 ? 2 : 1) attn_combine_ker
     const int c = tid % D, grp = tid / D;
     const int warp = tid >> 5, lane = tid & 31;
     const int h = hq / (p.Hq / p.H);
-    if (tid < D) qv[tid] = p.scale * load_elem(p.q, ((long long)b * p.Hq + hq) * D + tid, p.q_bf16);
+    if (tid < D) qv[tid] = p.scale * attn_load_elem(p.q, ((long long)b * p.Hq + hq) * D + tid, p.q_bf16);
     __syncthreads();
     const long long rbase = ((long long)b * p.H + h) * p.R * D;
     const float *ml = p.ml + ((long long)b * p.Hq + hq) * p.nchunk * 2;
@@ -563,7 +425,7 @@ __global__ void __launch_bounds__(CB_THREADS, RES_BF16 ? 2 : 1) attn_combine_ker
                 }
                 k4 = make_float4(rot[0], rot[1], rot[2], rot[3]);
             }
-            const float sdot = warp_sum_f(fmaf(q4.x, k4.x, fmaf(q4.y, k4.y, fmaf(q4.z, k4.z, q4.w * k4.w))));
+            const float sdot = attn_warp_sum(fmaf(q4.x, k4.x, fmaf(q4.y, k4.y, fmaf(q4.z, k4.z, q4.w * k4.w))));
             if (lane == 0) w[t] = sdot;
         }
     }
@@ -627,13 +489,13 @@ __global__ void __launch_bounds__(CB_THREADS, RES_BF16 ? 2 : 1) attn_combine_ker
     }
 }
 
-template <int BITS, int NQ, bool ROPE, bool M16>
-int launch_partial_r(const AttnParams &p, int qpasses, cudaStream_t st)
+template <int BITS, int NQ, bool M16>
+int launch_partial_m(const AttnParams &p, int qpasses, cudaStream_t st)
 {
-    const size_t smem = sizeof(float) * (NQ * D + AT_WARPS * NQ * D + NQ * AT_CHUNK + NQ * AT_WARPS + 8) +
-                        (ROPE ? sizeof(float2) * 64 * 32 + sizeof(float4) * AT_WARPS * 64 : 0);
-    SQUAT_CUDA(cudaFuncSetAttribute(attn_partial_kernel<BITS, NQ, ROPE, M16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attn_partial_kernel<BITS, NQ, ROPE, M16><<<dim3(p.nchunk * qpasses, p.H, p.B), AT_THREADS, smem, st>>>(p);
+    const size_t smem = sizeof(float) * (NQ * D + AT_WARPS * NQ * D + NQ * AT_CHUNK + NQ * AT_WARPS + 8) + sizeof(float2) * 64 * 32 +
+                        sizeof(float4) * AT_WARPS * 64;
+    SQUAT_CUDA(cudaFuncSetAttribute(attn_partial_kernel<BITS, NQ, M16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    attn_partial_kernel<BITS, NQ, M16><<<dim3(p.nchunk * qpasses, p.H, p.B), AT_THREADS, smem, st>>>(p);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
     return SQUAT_OK;
@@ -641,8 +503,7 @@ int launch_partial_r(const AttnParams &p, int qpasses, cudaStream_t st)
 template <int BITS, int NQ>
 int launch_partial(const AttnParams &p, int qpasses, cudaStream_t st)
 {
-    if (p.meta16) return p.rope_a ? launch_partial_r<BITS, NQ, true, true>(p, qpasses, st) : launch_partial_r<BITS, NQ, false, true>(p, qpasses, st);
-    return p.rope_a ? launch_partial_r<BITS, NQ, true, false>(p, qpasses, st) : launch_partial_r<BITS, NQ, false, false>(p, qpasses, st);
+    return p.meta16 ? launch_partial_m<BITS, NQ, true>(p, qpasses, st) : launch_partial_m<BITS, NQ, false>(p, qpasses, st);
 }
 
 }  // namespace
@@ -673,7 +534,9 @@ int squat_launch_decode_attention(const void *q, int q_dtype, int batch, int Hq,
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    p.chunk = AT_CHUNK;                                          // smaller chunks while that leaves fewer than ~4 CTAs per SM
+    p.status = squat_status_word();
+    if (!p.status) return SQUAT_ERR_CUDA;
+    p.chunk = p.rope_a ? AT_CHUNK : ATTN_MMA_TILE * ATTN_MMA_MAX_TILES;                                          // smaller chunks while that leaves fewer than ~4 CTAs per SM
     while (p.chunk > 256 && (long long)batch * H * ((T + p.chunk - 1) / p.chunk) < 4LL * sms) p.chunk /= 2;
     p.nchunk = (T + p.chunk - 1) / p.chunk;
     p.part = workspace;
@@ -681,7 +544,8 @@ int squat_launch_decode_attention(const void *q, int q_dtype, int batch, int Hq,
     const int qpk = Hq / H;
     if (p.nchunk > 0) {
         int rc;
-        if (qpk == 1) rc = bits == 2 ? launch_partial<2, 1>(p, 1, st) : launch_partial<4, 1>(p, 1, st);
+        if (!p.rope_a) rc = squat_launch_attn_mma(p, bits, st);
+        else if (qpk == 1) rc = bits == 2 ? launch_partial<2, 1>(p, 1, st) : launch_partial<4, 1>(p, 1, st);
         else if (qpk == 2) rc = bits == 2 ? launch_partial<2, 2>(p, 1, st) : launch_partial<4, 2>(p, 1, st);
         else rc = bits == 2 ? launch_partial<2, 4>(p, (qpk + 3) / 4, st) : launch_partial<4, 4>(p, (qpk + 3) / 4, st);
         if (rc != SQUAT_OK) return rc;

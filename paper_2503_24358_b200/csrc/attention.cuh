@@ -1,0 +1,65 @@
+// What the two partial kernels of the reader (attention.cu, attention_mma.cu) and its combine kernel share.
+#pragma once
+#include <cuda_fp16.h>
+#include "squat_internal.cuh"
+
+struct AttnParams {
+    const void *q;             // [B, Hq, D]
+    int q_bf16;
+    int B, Hq, H, T;           // T: quantized tokens per (batch, head)
+    const unsigned char *kc, *vc;
+    const void *ks, *kz, *vs, *vz;   // float32, or binary16 in the M16 instances
+    long long csb, csh;        // cache strides in tokens
+    int G;
+    const void *k_res, *v_res; // [B, H, R, D]
+    int res_bf16, R;
+    float scale;
+    float *part;               // [B, Hq, nchunk, D]
+    float *ml;                 // [B, Hq, nchunk, 2]
+    int nchunk, chunk;         // chunk: tokens per CTA, a multiple of 256
+    float *out;                // [B, Hq, D]
+    // rotary tables (pre-embedding key storage only): cos/sin of (32 a theta_i) [blocks][64] and of (l theta_i) [32][64]
+    const float2 *rope_a, *rope_b;
+    long long first_pos;       // position of cached token 0; a multiple of 32
+    int meta16;                // the cache's scales and zero-points are binary16
+    unsigned *status;          // device status word
+};
+
+__device__ __forceinline__ float attn_warp_sum(float v)
+{
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+    return v;
+}
+
+__device__ __forceinline__ float attn_load_elem(const void *p, long long idx, int bf16)
+{
+    if (bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p)[idx]);
+    return reinterpret_cast<const float *>(p)[idx];
+}
+
+// scale / zero-point element i of a metadata array stored as float32 or binary16
+template <bool M16>
+__device__ __forceinline__ float attn_meta(const void *p, long long i)
+{
+    if (M16) return __half2float(__ldg(reinterpret_cast<const __half *>(p) + i));
+    return __ldg(reinterpret_cast<const float *>(p) + i);
+}
+
+// four consecutive elements starting at i (a multiple of 4)
+template <bool M16>
+__device__ __forceinline__ float4 attn_meta4(const void *p, long long i)
+{
+    if (M16) {
+        const uint2 r = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p) + i));
+        const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&r.x));
+        const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&r.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    return __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(p) + i));
+}
+
+// scores and values of a cache whose keys are stored after the rotary embedding, on the integer tensor cores
+constexpr int ATTN_MMA_TILE = 128;            // tokens per product
+constexpr int ATTN_MMA_MAX_TILES = 8;         // tiles per CTA: chunks of at most 1024 tokens
+int squat_launch_attn_mma(const AttnParams &p, int bits, cudaStream_t st);
