@@ -1,4 +1,4 @@
-// What the two partial kernels of the reader (attention.cu, attention_mma.cu) and its combine kernel share.
+// What the reader's kernels share (attention.cu, attention_mma.cuh).
 #pragma once
 #include <cuda_fp16.h>
 #include "squat_internal.cuh"
@@ -14,9 +14,9 @@ struct AttnParams {
     const void *k_res, *v_res; // [B, H, R, D]
     int res_bf16, R;
     float scale;
-    float *part;               // [B, Hq, nchunk, D]
-    float *ml;                 // [B, Hq, nchunk, 2]
-    int nchunk, chunk;         // chunk: tokens per CTA, a multiple of 256
+    float *part;               // [B, Hq, parts, D], parts = nchunk and, if R > 0, the residual buffer
+    float *ml;                 // [B, Hq, parts, 2]
+    int nchunk, chunk;         // chunk: tokens per CTA, a power of two, 256 .. 1024
     float *out;                // [B, Hq, D]
     // rotary tables (pre-embedding key storage only): cos/sin of (32 a theta_i) [blocks][64] and of (l theta_i) [32][64]
     const float2 *rope_a, *rope_b;
@@ -59,7 +59,7 @@ __device__ __forceinline__ float4 attn_meta4(const void *p, long long i)
     return __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(p) + i));
 }
 
-// scores and values of a cache whose keys are stored after the rotary embedding, on the integer tensor cores
 constexpr int ATTN_MMA_TILE = 128;            // tokens per product
 constexpr int ATTN_MMA_MAX_TILES = 8;         // tiles per CTA: chunks of at most 1024 tokens
-int squat_launch_attn_mma(const AttnParams &p, int bits, cudaStream_t st);
+int squat_launch_attn_mma(const AttnParams &p, int bits, cudaStream_t st);     // keys stored after the rotary embedding
+int squat_launch_attn_rope(const AttnParams &p, int bits, cudaStream_t st);    // before it

@@ -1,493 +1,7 @@
-// Reader of the packed cache, keys stored after the rotary embedding: scores and weighted values of a chunk of tokens on
-// the integer tensor cores (tcgen05.mma.kind::i8, 32-bit integer accumulators in tensor memory).
-//
-// A 2- or 4-bit code is an exact byte after one shift and one mask per FOUR (two) codes, and sums of byte products are
-// exact, so the only rounding left is the one that puts the other operand in fixed point:
-//   scores   <q, k_t> = sum_c (q_c scale_c) code_tc + sum_c q_c zero_c.  q_c scale_c, scaled by a power of two to 31 bits of
-//            the group's largest one, is four signed base-256 digits; the product of the codes of 128 tokens (A: 128 x 128
-//            bytes) with the digits (B: one column per token group, head and digit) gives four integers per token and
-//            head, which are put together in float32.  31 bits of the largest term are more than a float32 sum keeps.
-//   values   sum_t (w_t scale_tg) code_tc + sum_t w_t zero_tg.  The same with the roles turned: A = the codes transposed (the
-//            same bytes in shared memory, described as M-major), B = the digits of w_t scale_tg, one column per channel
-//            group, head and digit.  Accumulated over the chunk's tiles in tensor memory.
-// A lane owns a token (its row of key codes, its weight, its value metadata); a warp makes the digits of the query for one
-// token group.  Key codes are A in tensor memory (row = lane), so they never cross shared memory, whose wavefronts were the
-// tightest pipe with both operands there (78 % busy); value codes, which must be read transposed, go through it.  The digits
-// of four heads are one 16-byte store: an int's bytes ARE its base-256 digits, and B is described as N-major, so nothing is
-// transposed.  Within a 32-bit word of codes the unpacking leaves the channels interleaved (byte i of piece j is channel
-// (8 / BITS) i + j of the word); the same order is used for the other operand.
-//
-// Bound: HBM (bits / 8 + metadata bytes per cached element) for long caches.  The CUDA-core form that this replaces spent
-// two instructions per code and head and was bound by them.  64 x 32 heads x 4096 tokens (1.07 GB): 341 -> 216 us, 63 % of
-// DRAM throughput; 16 x 8 KV heads x 8160 tokens with four query heads each: 142 -> 61 us.
-#include "attention.cuh"
-
-namespace {
-
-constexpr int D = SQUAT_D;
-constexpr int THREADS = 128, WARPS = 4;
-constexpr int TILE = ATTN_MMA_TILE, MAX_TILES = ATTN_MMA_MAX_TILES;
-typedef unsigned long long u64;
-
-__device__ __forceinline__ unsigned smem_u32(const void *ptr) { return (unsigned)__cvta_generic_to_shared(ptr); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptors.  Codes: 128-byte rows (token), 128-byte swizzle, groups of 8 rows 1024 bytes apart;
-// K-major for the scores (K = channel), M-major for the values (K = token).  Digits: no swizzle, N-major: 16 bytes of
-// columns x 8 rows of K are one 128-byte piece, the next 8 rows follow 160 bytes on (leading offset; 160, so that the
-// lanes' 16-byte stores fall on distinct banks), the next 16 columns come after all 128 rows (stride offset).
-constexpr unsigned DIG_PIECE = 160, DIG_CHUNK = DIG_PIECE * (D / 8);
-__device__ __forceinline__ u64 codes_desc(unsigned addr)
-{
-    return (u64)((addr & 0x3FFFF) >> 4) | ((u64)1 << 16) | ((u64)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-__device__ __forceinline__ u64 digits_desc(unsigned addr)
-{
-    return (u64)((addr & 0x3FFFF) >> 4) | ((u64)(DIG_PIECE >> 4) << 16) | ((u64)(DIG_CHUNK >> 4) << 32) | (1ull << 46);
-}
-// instruction descriptor: int32 accumulator, A unsigned bytes, B signed bytes, M = 128, N = n, B N-major, A K-major (scores) or M-major (values)
-__host__ __device__ constexpr unsigned idesc_i8(int n, bool a_m_major)
-{
-    return (2u << 4) | (1u << 10) | ((a_m_major ? 1u : 0u) << 15) | (1u << 16) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-__device__ __forceinline__ void mma_i8(unsigned d_taddr, u64 a_desc, u64 b_desc, unsigned idesc, unsigned accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_taddr), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// the same with A in tensor memory (row = lane, four bytes a column)
-__device__ __forceinline__ void mma_i8_ta(unsigned d_taddr, unsigned a_taddr, u64 b_desc, unsigned idesc, unsigned accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n}"
-                 ::"r"(d_taddr), "r"(a_taddr), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void tmem_st16(unsigned taddr, const uint32_t (&r)[16])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-                   "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-__device__ __forceinline__ void tc_commit(unsigned mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-// Bounded wait for a phase of an mbarrier: false when the limit ran out (the caller records it and moves on).
-__device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
-{
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-__device__ __forceinline__ void tmem_ld4(unsigned taddr, int (&r)[4])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ float warp_max(float x)
-{
-    float r;
-    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-// the NG value scales (or zero-points) of a token, zeros for a token past the end
-template <int NG, bool M16>
-__device__ __forceinline__ void load_vmeta(const void *p, long long token, bool in, float (&out)[NG])
-{
-    if constexpr (NG == 4) {
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (in) v = attn_meta4<M16>(p, token * 4);
-        out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-    } else {
-#pragma unroll
-        for (int g = 0; g < NG; ++g) out[g] = in ? attn_meta<M16>(p, token * NG + g) : 0.0f;
-    }
-}
-
-// Power of two that takes values up to mx (>= 0) to at most 2^30, and its inverse (NaN for a non-finite mx)
-__device__ __forceinline__ float fixed_scale(float mx, float &inv)
-{
-    const int e = max((int)(__float_as_uint(mx) >> 23) & 0xff, 30);
-    inv = e == 255 ? __uint_as_float(0x7fc00000u) : __uint_as_float((unsigned)(e - 29) << 23);
-    return __uint_as_float((unsigned)(283 - e) << 23);
-}
-// round(x) as four signed base-256 digits, lowest in the lowest byte
-__device__ __forceinline__ unsigned digits_of(float x)
-{
-    return ((unsigned)__float2int_rn(x) + 0x00808080u) ^ 0x00808080u;
-}
-// the number whose digits were multiplied, times inv
-__device__ __forceinline__ float from_digits(const int (&d)[4], float inv)
-{
-    return fmaf((float)(d[3] * 256 + d[2]), 65536.0f, (float)(d[1] * 256 + d[0])) * inv;
-}
-
-// Unpacking leaves every code where it is in its byte: piece j of a word is (x >> 0) & (mask << BITS j), four bytes that
-// hold 2^(BITS j) times a code.  The factor is a power of two: the query's digits take it out before they are rounded (31
-// bits of the largest term, at least 25 for the last piece), the values' sums afterwards.
-// the same for sums over a whole chunk, whose digits may not be joined in 32 bits
-__device__ __forceinline__ float from_long_digits(const int (&d)[4], float inv)
-{
-    return fmaf(fmaf((float)d[3], 256.0f, (float)d[2]), 65536.0f, fmaf((float)d[1], 256.0f, (float)d[0])) * inv;
-}
-
-// byte k of an unpacked row holds this channel, 2^(BITS piece_at(k)) times its code
-template <int BITS>
-__device__ __forceinline__ int channel_at(int k)
-{
-    constexpr int PIECES = 8 / BITS, PER_WORD = 32 / BITS;     // pieces of four bytes per word of codes
-    return k / PER_WORD * PER_WORD + (k & 3) * PIECES + (k % PER_WORD >> 2);
-}
-template <int BITS>
-__device__ __forceinline__ int piece_at(int k) { return k % (32 / BITS) >> 2; }
-
-template <int BITS, int NQ, int NG>
-struct Shape {
-    static constexpr int N = NG * NQ * 4 < 16 ? 16 : NG * NQ * 4;
-    static constexpr int TMEM_COLS = 32 + N > 64 ? 128 : 64;    // the keys' bytes, the accumulator of the scores, then of the values
-    static constexpr int DIG_BYTES = N / 16 * (int)DIG_CHUNK;
-    static constexpr size_t SMEM = 1024 + TILE * D + 2 * DIG_BYTES + sizeof(float) * MAX_TILES * TILE * NQ;
-};
-
-template <int BITS, int NQ, int NG, bool M16>
-__global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : 6) attn_mma_kernel(const AttnParams p)
-{
-    using S = Shape<BITS, NQ, NG>;
-    constexpr int G = D / NG, WPT = D * BITS / 32;              // tokens (or channels) per group; 32-bit words per token
-    constexpr uint32_t MASK = BITS == 2 ? 0x03030303u : 0x0F0F0F0Fu;
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *codes_sm = smem_raw + (1024 - (smem_u32(smem_raw) & 1023)) % 1024;      // [128 rows][128 bytes] of value codes, swizzled
-    unsigned char *digits_sm = codes_sm + TILE * D;                                        // [2][N / 16][16][8][16 bytes]
-    float *sc_sm = reinterpret_cast<float *>(digits_sm + 2 * S::DIG_BYTES) + threadIdx.x;  // [tiles][NQ][128]: this lane's scores
-    __shared__ __align__(8) u64 mbar;
-    __shared__ unsigned tmem_sm;
-    __shared__ float2 qz_sm[MAX_TILES][NG][NQ];                 // inverse of the fixed point, sum of query x zero-point
-    __shared__ float red_sm[WARPS][NG * NQ + NQ + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunk = blockIdx.x % p.nchunk, qpass = blockIdx.x / p.nchunk;
-    const int h = blockIdx.y, b = blockIdx.z;
-    const int qpk = p.Hq / p.H, hq0 = h * qpk + qpass * NQ, nq_here = min(NQ, qpk - qpass * NQ);
-    const int t0 = chunk * p.chunk, n_tok = min(p.T - t0, p.chunk), tiles = (n_tok + TILE - 1) / TILE;
-    const long long ctok0 = (long long)b * p.csb + (long long)h * p.csh + t0;               // first token of the chunk
-
-    // Codes of a tile, zeros past the end of the chunk.  Keys: lane = token, its whole row.  Values: a warp's 32 rows as
-    // contiguous 512-byte pieces, LPT lanes a row (half the cache lines of the other form per load).
-    constexpr int LPT = WPT / 4, TPL = 32 / LPT;
-    const unsigned char *k_row = p.kc + (ctok0 + tid) * (long long)(D * BITS / 8);
-    const int v_tok = 32 * warp + lane / LPT;
-    const unsigned char *v_row = p.vc + (ctok0 + v_tok) * (long long)(D * BITS / 8) + lane % LPT * 16;
-    uint4 cw[LPT];
-    auto load_keys = [&](int tile) {
-        const bool in = tile * TILE + tid < n_tok;
-        const uint4 *src = reinterpret_cast<const uint4 *>(k_row + tile * (TILE * D * BITS / 8));
-#pragma unroll
-        for (int i = 0; i < LPT; ++i) cw[i] = in ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
-    };
-    auto load_values = [&](int tile) {
-        const unsigned char *src = v_row + tile * (TILE * D * BITS / 8);
-#pragma unroll
-        for (int i = 0; i < LPT; ++i)
-            cw[i] = tile * TILE + v_tok + TPL * i < n_tok ? ldg128(src + i * TPL * (D * BITS / 8)) : make_uint4(0, 0, 0, 0);
-    };
-    load_keys(0);
-    // Which (token group, head) digits a warp makes: 4 / NG warps share a group and deal its heads among them.  A lane makes
-    // those of channels 4 lane .. 4 lane + 3.
-    constexpr int WPG = WARPS / NG, HPW = (NQ + WPG - 1) / WPG;
-    const int my_group = warp / WPG, my_head0 = warp % WPG * HPW;
-    const bool makes = my_head0 < NQ;
-    float4 ks, kz;                                              // scales and zero-points of those channels in the warp's group
-    const long long mrow0 = (ctok0 / G + my_group) * D + 4 * lane;
-    auto load_kmeta = [&](int tile) {
-        const bool in = makes && tile * TILE + my_group * G < n_tok;
-        ks = in ? attn_meta4<M16>(p.ks, mrow0 + tile * (NG * D)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        kz = in ? attn_meta4<M16>(p.kz, mrow0 + tile * (NG * D)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    };
-    load_kmeta(0);
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sm)), "r"((unsigned)S::TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    float q[HPW][4];
-    int dig_at[4];                                              // where the lane's digits go
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-        for (int j = 0; j < HPW; ++j) {
-            const int qi = my_head0 + j;
-            q[j][i] = qi < nq_here ? p.scale * attn_load_elem(p.q, ((long long)b * p.Hq + hq0 + qi) * D + 4 * lane + i, p.q_bf16) : 0.0f;
-        }
-        const int k = BITS == 2 ? 16 * (lane >> 2) + 4 * i + (lane & 3) : 8 * (lane >> 1) + 4 * (i & 1) + 2 * (lane & 1) + (i >> 1);
-        const int n = (my_group * NQ + my_head0) * 4;
-        dig_at[i] = n / 16 * DIG_CHUNK + k / 8 * DIG_PIECE + k % 8 * 16 + n % 16;
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const unsigned tmem = tmem_sm, t_lanes = tmem + ((unsigned)(warp * 32) << 16), t_mine = t_lanes + 32 + my_group * NQ * 4;
-    bool ok = true;
-
-    // a row of key codes as 128 bytes in tensor memory, this lane's
-    auto unpack_keys = [&]() {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            uint32_t r[16];
-#pragma unroll
-            for (int w = 0; w < WPT / 2; ++w) {
-                const uint4 &v = cw[(half * WPT / 2 + w) / 4];
-                const uint32_t x = w % 4 == 0 ? v.x : w % 4 == 1 ? v.y : w % 4 == 2 ? v.z : v.w;
-#pragma unroll
-                for (int j = 0; j < 8 / BITS; ++j) r[w * (8 / BITS) + j] = x & (MASK << (BITS * j));
-            }
-            tmem_st16(t_lanes + 16 * half, r);
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    };
-    // rows of value codes as 128 bytes in shared memory: 16-byte piece c of row r sits at piece c ^ (r mod 8)
-    auto unpack_values = [&]() {
-#pragma unroll
-        for (int i = 0; i < LPT; ++i) {
-            const int r = v_tok + TPL * i, swz = r & 7, c0 = lane % LPT * (8 / LPT);
-            unsigned char *row = codes_sm + r * D;
-            const uint32_t x[4] = {cw[i].x, cw[i].y, cw[i].z, cw[i].w};
-            if (BITS == 2) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    *reinterpret_cast<uint4 *>(row + (((c0 + e) ^ swz) << 4)) = make_uint4(x[e] & MASK, x[e] & (MASK << 2), x[e] & (MASK << 4), x[e] & (MASK << 6));
-            } else {
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    *reinterpret_cast<uint4 *>(row + (((c0 + e) ^ swz) << 4)) =
-                        make_uint4(x[2 * e] & MASK, x[2 * e] & (MASK << 4), x[2 * e + 1] & MASK, x[2 * e + 1] & (MASK << 4));
-            }
-        }
-    };
-    // The four 32-deep steps of a tile's product: the codes advance by 32 channels (keys) or 32 tokens (values), the digits by
-    // 32 rows.  One product is in flight at a time; the digits of the next one are made meanwhile in the other buffer.
-    unsigned issued = 0;
-    auto issue = [&](int buf, bool values, bool accumulate) {
-        if (tid == 0) {
-            tc_fence_after();
-            const u64 a = codes_desc(smem_u32(codes_sm)), dg = digits_desc(smem_u32(digits_sm + buf * S::DIG_BYTES));
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                if (values) mma_i8(tmem + 32, a + s * 32 * D / 16, dg + s * 4 * DIG_PIECE / 16, idesc_i8(S::N, true), s > 0 || accumulate);
-                else mma_i8_ta(tmem + 32, tmem + 8 * s, dg + s * 4 * DIG_PIECE / 16, idesc_i8(S::N, false), s > 0);
-            }
-            tc_commit(smem_u32(&mbar));
-        }
-        ++issued;
-    };
-    auto wait_product = [&]() {
-        ok = mbar_wait(smem_u32(&mbar), (issued - 1) & 1) && ok;
-        tc_fence_after();
-    };
-
-    // ---------------------------------------------------------------- scores
-    float mx[NQ], vmax = 0.0f;
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) mx[j] = -INFINITY;
-    auto read_scores = [&](int tile) {
-        wait_product();
-        int d[NQ][4];
-#pragma unroll
-        for (int j = 0; j < NQ; ++j) tmem_ld4(t_mine + j * 4, d[j]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const bool in = tile * TILE + tid < n_tok;
-#pragma unroll
-        for (int j = 0; j < NQ; ++j) {
-            const float2 iz = qz_sm[tile][my_group][j];
-            const float s = in ? from_digits(d[j], iz.x) + iz.y : -INFINITY;
-            sc_sm[(tile * NQ + j) * TILE] = s;
-            mx[j] = max_nan(mx[j], s);
-        }
-    };
-#pragma unroll 1
-    for (int tile = 0; tile < tiles; ++tile) {
-        const int buf = tile & 1;
-        float vs[NG];
-        load_vmeta<NG, M16>(p.vs, ctok0 + tile * TILE + tid, tile * TILE + tid < n_tok, vs);
-        uint32_t dig[4][HPW];
-#pragma unroll
-        for (int j = 0; j < HPW; ++j) {
-            const float zs = attn_warp_sum(fmaf(q[j][0], kz.x, q[j][1] * kz.y) + fmaf(q[j][2], kz.z, q[j][3] * kz.w));
-            constexpr float P1 = BITS == 2 ? 0.25f : 0.0625f, P2 = BITS == 2 ? 0.0625f : 1.0f, P3 = BITS == 2 ? 0.015625f : 0.0625f;
-            const float f[4] = {q[j][0] * ks.x, q[j][1] * ks.y, q[j][2] * ks.z, q[j][3] * ks.w};
-            float inv;
-            const float up = fixed_scale(warp_max(max_nan(max_nan(fabsf(f[0]), fabsf(f[1])), max_nan(fabsf(f[2]), fabsf(f[3])))), inv);
-            if (lane == 0 && my_head0 + j < NQ) qz_sm[tile][my_group][my_head0 + j] = make_float2(inv, zs);
-            dig[0][j] = digits_of(f[0] * up);
-            dig[1][j] = digits_of(f[1] * (up * P1));
-            dig[2][j] = digits_of(f[2] * (up * P2));
-            dig[3][j] = digits_of(f[3] * (up * P3));
-        }
-        if (tile + 1 < tiles) load_kmeta(tile + 1);
-        if (makes) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                unsigned char *dst = digits_sm + buf * S::DIG_BYTES + dig_at[i];
-                if constexpr (HPW == 4) *reinterpret_cast<uint4 *>(dst) = make_uint4(dig[i][0], dig[i][1], dig[i][2], dig[i][3]);
-                else if constexpr (HPW == 2) *reinterpret_cast<uint2 *>(dst) = make_uint2(dig[i][0], dig[i][1]);
-                else *reinterpret_cast<uint32_t *>(dst) = dig[i][0];
-            }
-        }
-        if (tile > 0) read_scores(tile - 1);                    // also frees the keys' columns and the accumulator
-        unpack_keys();
-        if (tile + 1 < tiles) load_keys(tile + 1);
-        else load_values(0);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        issue(buf, false, false);
-#pragma unroll
-        for (int g = 0; g < NG; ++g) vmax = max_nan(vmax, fabsf(vs[g]));
-    }
-    float vs[NG], vz[NG];
-    load_vmeta<NG, M16>(p.vs, ctok0 + tid, tid < n_tok, vs);
-    load_vmeta<NG, M16>(p.vz, ctok0 + tid, tid < n_tok, vz);
-    read_scores(tiles - 1);
-
-    // ---------------------------------------------------------------- maxima over the chunk
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        mx[j] = warp_max(mx[j]);
-        if (lane == 0) red_sm[warp][j] = mx[j];
-    }
-    vmax = warp_max(vmax);
-    if (lane == 0) red_sm[warp][NQ] = vmax;
-    tc_fence_before();                                          // the score columns have been read; the values' product reuses them
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) mx[j] = max_nan(max_nan(red_sm[0][j], red_sm[1][j]), max_nan(red_sm[2][j], red_sm[3][j]));
-    vmax = max_nan(max_nan(red_sm[0][NQ], red_sm[1][NQ]), max_nan(red_sm[2][NQ], red_sm[3][NQ]));
-    float inv_v;
-    const float up_v = fixed_scale(vmax, inv_v);
-
-    // ---------------------------------------------------------------- weights, weighted values
-    float zacc[NG][NQ], den[NQ];
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        den[j] = 0.0f;
-#pragma unroll
-        for (int g = 0; g < NG; ++g) zacc[g][j] = 0.0f;
-    }
-    unsigned char *const my_dig = digits_sm + tid / 8 * DIG_PIECE + tid % 8 * 16;
-#pragma unroll 1
-    for (int tile = 0; tile < tiles; ++tile) {
-        const int buf = tile & 1;
-        float w[NQ];
-#pragma unroll
-        for (int j = 0; j < NQ; ++j) {
-            w[j] = expf(sc_sm[(tile * NQ + j) * TILE] - mx[j]);
-            den[j] += w[j];
-        }
-        uint32_t dig[S::N / 4];
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            const float vu = vs[g] * up_v;
-#pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                zacc[g][j] = fmaf(w[j], vz[g], zacc[g][j]);
-                dig[g * NQ + j] = digits_of(w[j] * vu);
-            }
-        }
-#pragma unroll
-        for (int i = NG * NQ; i < S::N / 4; ++i) dig[i] = 0;
-        if (tile + 1 < tiles) {
-            load_vmeta<NG, M16>(p.vs, ctok0 + (tile + 1) * TILE + tid, (tile + 1) * TILE + tid < n_tok, vs);
-            load_vmeta<NG, M16>(p.vz, ctok0 + (tile + 1) * TILE + tid, (tile + 1) * TILE + tid < n_tok, vz);
-        }
-#pragma unroll
-        for (int c = 0; c < S::N / 16; ++c)
-            *reinterpret_cast<uint4 *>(my_dig + buf * S::DIG_BYTES + c * DIG_CHUNK) = make_uint4(dig[4 * c], dig[4 * c + 1], dig[4 * c + 2], dig[4 * c + 3]);
-        if (tile > 0) wait_product();
-        unpack_values();
-        if (tile + 1 < tiles) load_values(tile + 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        issue(buf, true, tile > 0);
-    }
-    // sums of the weights and of weight x zero-point over the chunk
-    __syncthreads();                                            // the maxima in red_sm have been read
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        den[j] = attn_warp_sum(den[j]);
-        if (lane == 0) red_sm[warp][NG * NQ + j] = den[j];
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            zacc[g][j] = attn_warp_sum(zacc[g][j]);
-            if (lane == 0) red_sm[warp][g * NQ + j] = zacc[g][j];
-        }
-    }
-    wait_product();
-    int d[NQ][4];
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) tmem_ld4(t_mine + j * 4, d[j]);       // lane = channel: a warp's 32 channels share a group
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    if (!ok) atomicOr(p.status, SQUAT_FLAG_DEVICE_TIMEOUT);
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((unsigned)S::TMEM_COLS) : "memory");
-    const int c = channel_at<BITS>(tid);
-    inv_v *= 1.0f / (float)(1 << BITS * piece_at<BITS>(tid));
-#pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        if (j >= nq_here) break;
-        const int zi = my_group * NQ + j;
-        const float z = (red_sm[0][zi] + red_sm[1][zi]) + (red_sm[2][zi] + red_sm[3][zi]);
-        const long long row = ((long long)b * p.Hq + hq0 + j) * p.nchunk + chunk;
-        p.part[row * D + c] = from_long_digits(d[j], inv_v) + z;
-        if (tid == 0) {
-            const int di = NG * NQ + j;
-            *reinterpret_cast<float2 *>(p.ml + row * 2) = make_float2(mx[j], (red_sm[0][di] + red_sm[1][di]) + (red_sm[2][di] + red_sm[3][di]));
-        }
-    }
-}
-
-template <int BITS, int NQ, int NG, bool M16>
-int launch(const AttnParams &p, int qpasses, cudaStream_t st)
-{
-    constexpr size_t smem = Shape<BITS, NQ, NG>::SMEM;
-    SQUAT_CUDA(cudaFuncSetAttribute(attn_mma_kernel<BITS, NQ, NG, M16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attn_mma_kernel<BITS, NQ, NG, M16><<<dim3(p.nchunk * qpasses, p.H, p.B), THREADS, smem, st>>>(p);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
-}
-template <int BITS, int NQ>
-int launch_g(const AttnParams &p, int qpasses, cudaStream_t st)
-{
-    if (p.meta16) return p.G == 32 ? launch<BITS, NQ, 4, true>(p, qpasses, st) : p.G == 64 ? launch<BITS, NQ, 2, true>(p, qpasses, st) : launch<BITS, NQ, 1, true>(p, qpasses, st);
-    return p.G == 32 ? launch<BITS, NQ, 4, false>(p, qpasses, st) : p.G == 64 ? launch<BITS, NQ, 2, false>(p, qpasses, st) : launch<BITS, NQ, 1, false>(p, qpasses, st);
-}
-template <int BITS>
-int launch_q(const AttnParams &p, cudaStream_t st)
-{
-    const int qpk = p.Hq / p.H;
-    return qpk == 1 ? launch_g<BITS, 1>(p, 1, st) : qpk == 2 ? launch_g<BITS, 2>(p, 1, st) : launch_g<BITS, 4>(p, (qpk + 3) / 4, st);
-}
-
-}  // namespace
+// Instances of the reader's kernel (attention_mma.cuh) for keys stored after the rotary embedding.
+#include "attention_mma.cuh"
 
 int squat_launch_attn_mma(const AttnParams &p, int bits, cudaStream_t st)
 {
-    return bits == 2 ? launch_q<2>(p, st) : launch_q<4>(p, st);
+    return bits == 2 ? launch_q<false, 2>(p, st) : launch_q<false, 4>(p, st);
 }
