@@ -110,16 +110,23 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+# Addresses and streams go to the library as plain integers (the argument types are declared in _load), and the current
+# stream's handle is asked for without the Stream object around it (3 us), where this torch has that call.
+_raw_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_current_stream is not None:
+        return _raw_current_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dev(t: torch.Tensor, name: str):
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Subspace:
@@ -261,7 +268,7 @@ def squat_write_path_host(s: Subspace, q, k, v, rank_r, lam, block_g, bits, grou
         if t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous host tensor")
     B, H, T, d = k.shape
-    hp = lambda t: ctypes.c_void_p(t.data_ptr())
+    hp = torch.Tensor.data_ptr
     meta = (k_scales, k_zeros, v_scales, v_zeros)
     m16 = all(t.dtype == torch.float16 for t in meta)
     if not m16 and not all(t.dtype == torch.float32 for t in meta):
@@ -297,7 +304,7 @@ def squat_append_window_host(s: Subspace, k, v, bits, group_size, k_codes, k_sca
         if t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous host tensor")
     B, H, T, d = k.shape
-    hp = lambda t: ctypes.c_void_p(t.data_ptr())
+    hp = torch.Tensor.data_ptr
     meta = (k_scales, k_zeros, v_scales, v_zeros)
     m16 = all(t.dtype == torch.float16 for t in meta)
     if not m16 and not all(t.dtype == torch.float32 for t in meta):

@@ -68,6 +68,30 @@ int squat_cuda_fail(cudaError_t e)
 
 void squat_count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+int squat_sm_count()
+{
+    static std::atomic<int> sms[MAX_DEVICES];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return 148;
+    int n = sms[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
+        sms[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+int squat_allow_smem(const void *kernel, size_t bytes, std::atomic<unsigned long long> &done)
+{
+    int dev = 0;
+    SQUAT_CUDA(cudaGetDevice(&dev));
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (bit && (done.load(std::memory_order_acquire) & bit)) return SQUAT_OK;
+    SQUAT_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return SQUAT_OK;
+}
+
 unsigned *squat_status_word()
 {
     int dev = 0;
@@ -111,9 +135,8 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     memset(s, 0, sizeof(*s));
     s->n_kv_heads = n_kv_heads;
     s->head_dim = head_dim;
-    int sms = 148;
     if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return SQUAT_ERR_CUDA; }
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
+    const int sms = squat_sm_count();
     s->gram_chunks_cap = (2 * sms) / n_kv_heads;        // 2 resident CTAs per SM: one wave
     if (s->gram_chunks_cap < 1) s->gram_chunks_cap = 1;
     const size_t hdd = (size_t)n_kv_heads * D * D;

@@ -82,9 +82,7 @@ int squat_launch_decode_attention(const void *q, int q_dtype, int batch, int Hq,
     p.kc = kc; p.vc = vc; p.ks = ks; p.kz = kz; p.vs = vs; p.vz = vz; p.csb = csb; p.csh = csh; p.G = G;
     p.k_res = k_res; p.v_res = v_res; p.res_bf16 = res_dtype == SQUAT_BF16; p.R = R;
     p.scale = scale; p.out = out;
-    int sms = 148, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = squat_sm_count();
     p.status = squat_status_word();
     if (!p.status) return SQUAT_ERR_CUDA;
     p.chunk = ATTN_MMA_TILE * ATTN_MMA_MAX_TILES;                // smaller chunks while that leaves fewer than ~4 CTAs per SM

@@ -709,7 +709,8 @@ template <bool ROPE, int BITS, int NQ, int NG, bool M16>
 int launch(const AttnParams &p, int qpasses, cudaStream_t st)
 {
     constexpr size_t smem = Shape<BITS, NQ, NG, ROPE>::SMEM;
-    SQUAT_CUDA(cudaFuncSetAttribute(attn_mma_kernel<BITS, NQ, NG, M16, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static std::atomic<unsigned long long> allowed{0};
+    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(attn_mma_kernel<BITS, NQ, NG, M16, ROPE>), smem, allowed)) return rc;
     attn_mma_kernel<BITS, NQ, NG, M16, ROPE><<<dim3((p.nchunk + (p.R > 0)) * qpasses, p.H, p.B), THREADS, smem, st>>>(p);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();

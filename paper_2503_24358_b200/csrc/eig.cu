@@ -886,7 +886,8 @@ int squat_launch_eig(squat_subspace *s, cudaStream_t st)
     tridiag_kernel<<<H, TRI_THREADS, 0, st>>>(s->gram, s->tri, s->gram_partial, s->eig_scale);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
-    SQUAT_CUDA(cudaFuncSetAttribute(dc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DcShared)));
+    static std::atomic<unsigned long long> allowed{0};
+    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(dc_kernel), sizeof(DcShared), allowed)) return rc;
     dc_kernel<<<H * DC_CTAS, DC_THREADS, sizeof(DcShared), st>>>(s->tri, s->gram_partial, s->eig_scale, s->eigval, s->eigvec,
                                                                  s->eig_sweeps, s->status);
     squat_count_launch();

@@ -722,7 +722,8 @@ __global__ void __launch_bounds__(256) pack_w_kernel(const float *__restrict__ W
 template <int BITS, int NW, bool BF16, bool M16>
 int launch_keys_inst(const KeyParams &p, int grid, size_t smem, cudaStream_t st)
 {
-    SQUAT_CUDA(cudaFuncSetAttribute(quant_keys_kernel<BITS, NW, BF16, M16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static std::atomic<unsigned long long> allowed{0};
+    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(quant_keys_kernel<BITS, NW, BF16, M16>), smem, allowed)) return rc;
     quant_keys_kernel<BITS, NW, BF16, M16><<<grid, TC_THREADS, smem, st>>>(p);
     return SQUAT_OK;
 }
@@ -737,9 +738,7 @@ int launch_keys(KeyParams p, int dtype, int meta16, cudaStream_t st)
     p.tiles_per_head = (int)tiles_per_head;
     p.total_tiles = (int)(tiles_per_head * p.H);
 
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = squat_sm_count();
     constexpr int GPT = 4 / NW;
     constexpr int NTEAMS = TC_SLOTS * GPT;
     // 193 KB: well over half an SM's shared memory, so two CTAs (each asking for all 512 tensor-memory columns)

@@ -381,9 +381,7 @@ __global__ void __launch_bounds__(LR_THREADS, LR_CTAS_PER_SM) quant_keys_lowrank
 template <int BITS, int G>
 int launch_lowrank(const LrParams &p, int H, int dtype, int meta16, cudaStream_t st)
 {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = squat_sm_count();
     constexpr int TEAMS = LR_WARPS / (G == 128 ? 2 : 1);
     const int ctas_needed = (p.team_tasks + TEAMS - 1) / TEAMS;
     int per_head = (2 * LR_CTAS_PER_SM * sms + H - 1) / H;   // two waves of the resident CTAs, over all heads

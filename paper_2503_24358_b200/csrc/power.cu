@@ -332,12 +332,14 @@ int squat_launch_power(squat_subspace *s, const double *start, long long start_s
 {
     if (rank_r <= 32) {
         const size_t smem = PowerLayout<32>::doubles * sizeof(double);
-        SQUAT_CUDA(cudaFuncSetAttribute(power_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        static std::atomic<unsigned long long> allowed{0};
+        if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(power_kernel<32>), smem, allowed)) return rc;
         power_kernel<32><<<s->n_kv_heads, PW_THREADS, smem, st>>>(s->gram, start, start_stride_h, rank_r, iters, lambda,
                                                                s->eigvec, s->eig_sweeps);
     } else {
         const size_t smem = PowerLayout<64>::doubles * sizeof(double);
-        SQUAT_CUDA(cudaFuncSetAttribute(power_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        static std::atomic<unsigned long long> allowed{0};
+        if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(power_kernel<64>), smem, allowed)) return rc;
         power_kernel<64><<<s->n_kv_heads, PW_THREADS, smem, st>>>(s->gram, start, start_stride_h, rank_r, iters, lambda,
                                                                s->eigvec, s->eig_sweeps);
     }

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
 #include "../../include/squat.h"
 
 #define SQUAT_D 128   // the only head dimension the key path and the subspace build are built for
@@ -40,6 +41,10 @@ struct squat_subspace {
 int squat_cuda_fail(cudaError_t e);          // records the error text, returns SQUAT_ERR_CUDA
 unsigned *squat_status_word();               // device address of the status word of the current device
 void squat_count_launch(unsigned n = 1);
+int squat_sm_count();                        // SMs of the current device (asked for once per device)
+// Dynamic shared memory above 48 KB has to be allowed once per kernel and device; `done` is a bit per device that the
+// launcher keeps for its kernel, so that a launch does not pay for the call again (it costs as much as a tenth of one).
+int squat_allow_smem(const void *kernel, size_t bytes, std::atomic<unsigned long long> &done);
 #define SQUAT_CUDA(call) do { cudaError_t e__ = (call); if (e__ != cudaSuccess) return squat_cuda_fail(e__); } while (0)
 #define SQUAT_LAUNCH_CHECK() do { cudaError_t e__ = cudaGetLastError(); if (e__ != cudaSuccess) return squat_cuda_fail(e__); } while (0)
 

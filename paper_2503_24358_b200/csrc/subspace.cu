@@ -389,7 +389,8 @@ int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads
 int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_blocks, cudaStream_t st)
 {
     const size_t smem = sizeof(double) * (D * ASM_LD + 5 * D + 64 * D);
-    SQUAT_CUDA(cudaFuncSetAttribute(assemble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static std::atomic<unsigned long long> allowed{0};
+    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(assemble_kernel), smem, allowed)) return rc;
     assemble_kernel<<<s->n_kv_heads, ASM_THREADS, smem, st>>>(s->eigval, s->eigvec, rank_r, lambda, block_g, s->Wt, left_rows);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();

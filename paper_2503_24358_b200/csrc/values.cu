@@ -494,9 +494,7 @@ int squat_launch_dequant(int kind, const unsigned char *codes, const void *scale
                          int batch, int H, int T, int d, int bits, int G, long long isb, long long ish,
                          void *out, int out_dtype, int meta16, cudaStream_t st)
 {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = squat_sm_count();
     const long long rows = (long long)batch * H;
     if (rows == 0 || T == 0) return SQUAT_OK;
     const int per_tok = d / 8;
