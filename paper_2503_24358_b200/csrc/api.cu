@@ -150,6 +150,9 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     const size_t o_val = carve((size_t)n_kv_heads * D * sizeof(double));
     const size_t o_vec = carve(hdd * sizeof(double));
     const size_t o_swp = carve((size_t)n_kv_heads * sizeof(int));
+    const size_t o_gmax = carve((size_t)n_kv_heads * s->gram_chunks_cap * D / 2 * sizeof(unsigned));
+    const size_t o_rcnt = carve((size_t)n_kv_heads * sizeof(int));
+    const size_t o_rem = carve((size_t)n_kv_heads * SQUAT_GRAM_REM_CAP * sizeof(SquatGramRem));
     const size_t o_tri = carve((size_t)n_kv_heads * 3 * D * sizeof(double));
     const size_t o_scl = carve((size_t)n_kv_heads * sizeof(double));
     const size_t o_exact = carve(sizeof(int));
@@ -164,6 +167,9 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     s->eigval = reinterpret_cast<double *>(base + o_val);
     s->eigvec = reinterpret_cast<double *>(base + o_vec);
     s->eig_sweeps = reinterpret_cast<int *>(base + o_swp);
+    s->gram_max = reinterpret_cast<unsigned *>(base + o_gmax);
+    s->gram_rem_count = reinterpret_cast<int *>(base + o_rcnt);
+    s->gram_rem = reinterpret_cast<SquatGramRem *>(base + o_rem);
     s->tri = reinterpret_cast<double *>(base + o_tri);
     s->eig_scale = reinterpret_cast<double *>(base + o_scl);
     s->exact_blocks = reinterpret_cast<int *>(base + o_exact);

@@ -9,6 +9,12 @@
 #define SQUAT_D 128   // the only head dimension the key path and the subspace build are built for
 #define SQUAT_LOWRANK_MAX_R 8   // largest subspace rank the rank-r form of the key quantizer is built for (keys_lowrank.cu)
 
+#define SQUAT_GRAM_REM_CAP 256   // remainders listed per head by the integer Gram kernel (gram_i8.cu)
+struct SquatGramRem {
+    int row, channel;
+    double r;
+};
+
 struct squat_subspace {
     int n_kv_heads;
     int head_dim;
@@ -25,6 +31,9 @@ struct squat_subspace {
     int prefer_dense;      // 1: squat_quantize_keys uses the dense kernel even when lr_table is valid
     double *gram;          // [H, d, d] Gram matrices
     double *gram_partial;  // [chunks, H, d, d] per-chunk partial Gram matrices (deterministic reduction)
+    unsigned *gram_max;    // [H, gram_chunks_cap, d / 2], rem_count [H], rem [H, SQUAT_GRAM_REM_CAP]: see gram_i8.cu
+    int *gram_rem_count;
+    SquatGramRem *gram_rem;
     double *eigval;        // [H, d] descending
     double *eigvec;        // [H, d, d], row i = eigenvector i
     int *eig_sweeps;       // [H] iterations of the last eigen-decomposition's slowest secular equation (power build: columns kept)
@@ -51,6 +60,8 @@ int squat_allow_smem(const void *kernel, size_t bytes, std::atomic<unsigned long
 // ---- kernel launchers (one per .cu) ---------------------------------------------------
 int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
                       long long stride_h, long long stride_t, cudaStream_t st);
+int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st);
+bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens);
 int squat_launch_eig(squat_subspace *s, cudaStream_t st);
 int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_blocks, cudaStream_t st);
 int squat_launch_power(squat_subspace *s, const double *start, long long start_stride_h, int rank_r, int iters,

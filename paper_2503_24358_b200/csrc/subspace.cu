@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
 int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
                       long long stride_h, long long stride_t, cudaStream_t st)
 {
+    if (squat_gram_i8_fits(s, dtype, n_q_heads, n_tokens)) return squat_launch_gram_i8(s, q, n_q_heads, n_tokens, stride_h, stride_t, st);
     const int H = s->n_kv_heads, qpk = n_q_heads / H;
     const long long N = (long long)n_tokens * qpk;
     int chunks = s->gram_chunks_cap;
