@@ -82,11 +82,23 @@ int squat_launch_decode_attention(const void *q, int q_dtype, int batch, int Hq,
     p.kc = kc; p.vc = vc; p.ks = ks; p.kz = kz; p.vs = vs; p.vz = vz; p.csb = csb; p.csh = csh; p.G = G;
     p.k_res = k_res; p.v_res = v_res; p.res_bf16 = res_dtype == SQUAT_BF16; p.R = R;
     p.scale = scale; p.out = out;
-    const int sms = squat_sm_count();
     p.status = squat_status_word();
     if (!p.status) return SQUAT_ERR_CUDA;
-    p.chunk = ATTN_MMA_TILE * ATTN_MMA_MAX_TILES;                // smaller chunks while that leaves fewer than ~4 CTAs per SM
-    while (p.chunk > 256 && (long long)batch * H * ((T + p.chunk - 1) / p.chunk) < 4LL * sms) p.chunk /= 2;
+    // Tokens per CTA.  A CTA costs its tiles (2.2 times as much where the scores stay on the CUDA cores) and about 1.5 tiles (4,
+    // with the rotary table) more to begin and end; once there are more CTAs than places, the last of them leave half a CTA's time idle.  Long chunks
+    // win where there are many waves (64 x 32 heads x 4096 tokens: 1024 tokens 267 us, 512 288), short ones where there are
+    // about two (5 x 32 x 3520, pre-rotary: 81, 74) or less than one.
+    const int qpk = Hq / H, nq = qpk >= 3 ? 4 : qpk, passes = (qpk + nq - 1) / nq;
+    const double slots = (double)squat_sm_count() * ATTN_CTAS_PER_SM(nq, p.rope_a != nullptr), units = (double)batch * H * passes, tile = p.rope_a ? 2.2 : 1.0, begin = p.rope_a ? 4.0 : 1.5;
+    double best = 0.0;
+    p.chunk = 256;
+    for (int chunk = 256; chunk <= ATTN_MMA_TILE * ATTN_MMA_MAX_TILES; chunk *= 2) {
+        const int n = (T + chunk - 1) / chunk;
+        const double cta = (T < chunk ? T : chunk) / (double)ATTN_MMA_TILE * tile + begin;
+        const double all = units * (T / (double)ATTN_MMA_TILE * tile + begin * n + (R > 0 ? 2.0 : 0.0)) / slots;
+        const double cost = units * (n + (R > 0)) <= slots ? cta : all + 0.5 * cta;
+        if (chunk == 256 || cost < best) { best = cost; p.chunk = chunk; }
+    }
     p.nchunk = (T + p.chunk - 1) / p.chunk;
     p.part = workspace;
     p.ml = workspace + (size_t)batch * Hq * (p.nchunk + (R > 0)) * D;

@@ -61,5 +61,7 @@ __device__ __forceinline__ float4 attn_meta4(const void *p, long long i)
 
 constexpr int ATTN_MMA_TILE = 128;            // tokens per product
 constexpr int ATTN_MMA_MAX_TILES = 8;         // tiles per CTA: chunks of at most 1024 tokens
+// resident CTAs per SM the kernel is built for, by query heads per pass (96 or 128 registers: six CTAs of 80 were slower)
+constexpr int ATTN_CTAS_PER_SM(int nq, bool rope) { return nq >= 4 || rope ? 4 : 5; }
 int squat_launch_attn_mma(const AttnParams &p, int bits, cudaStream_t st);     // keys stored after the rotary embedding
 int squat_launch_attn_rope(const AttnParams &p, int bits, cudaStream_t st);    // before it

@@ -106,19 +106,31 @@ __device__ __forceinline__ float max_nan(float a, float b)
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
 }
-// the NG value scales (or zero-points) of a token, zeros for a token past the end
-template <int NG, bool M16>
-__device__ __forceinline__ void load_vmeta(const void *p, long long token, bool in, float (&out)[NG])
-{
-    if constexpr (NG == 4) {
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (in) v = attn_meta4<M16>(p, token * 4);
-        out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-    } else {
+// N scales or zero-points as they were loaded (float32 or binary16); they become floats where they are used, so that nothing
+// waits for a load where it is issued
+template <int N, bool M16>
+struct Meta {
+    using raw_t = typename std::conditional<M16, typename std::conditional<N == 4, uint2, typename std::conditional<N == 2, uint32_t, unsigned short>::type>::type,
+                                            typename std::conditional<N == 4, float4, typename std::conditional<N == 2, float2, float>::type>::type>::type;
+    raw_t raw;
+    __device__ __forceinline__ void load(const void *p, long long i) { raw = __ldg(reinterpret_cast<const raw_t *>(p) + i); }   // i: in units of N
+    __device__ __forceinline__ void get(float (&out)[N]) const
+    {
+        if constexpr (M16) {
+            uint32_t w[2] = {0, 0};
+            if constexpr (N == 4) { w[0] = raw.x; w[1] = raw.y; }
+            else w[0] = raw;
 #pragma unroll
-        for (int g = 0; g < NG; ++g) out[g] = in ? attn_meta<M16>(p, token * NG + g) : 0.0f;
+            for (int g = 0; g < N; ++g) out[g] = __half2float(__ushort_as_half((unsigned short)(w[g / 2] >> (16 * (g & 1)))));
+        } else if constexpr (N == 4) {
+            out[0] = raw.x; out[1] = raw.y; out[2] = raw.z; out[3] = raw.w;
+        } else if constexpr (N == 2) {
+            out[0] = raw.x; out[1] = raw.y;
+        } else {
+            out[0] = raw;
+        }
     }
-}
+};
 
 // Power of two that takes values up to mx (>= 0) to at most 2^30, and its inverse (NaN for a non-finite mx)
 __device__ __forceinline__ float fixed_scale(float mx, float &inv)
@@ -220,12 +232,15 @@ __device__ __forceinline__ void residual_part(const AttnParams &p, float *sm, in
                 const float4 o = make_float4(__shfl_xor_sync(0xffffffffu, x.x, 16), __shfl_xor_sync(0xffffffffu, x.y, 16),
                                              __shfl_xor_sync(0xffffffffu, x.z, 16), __shfl_xor_sync(0xffffffffu, x.w, 16));
                 const float oth[4] = {o.x, o.y, o.z, o.w};
+                const float4 *ta = reinterpret_cast<const float4 *>(p.rope_a + (pos >> 5) * 64 + 4 * (lane & 15));
+                const float4 *tb = reinterpret_cast<const float4 *>(p.rope_b + (pos & 31) * 64 + 4 * (lane & 15));
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int at = 4 * (lane & 15) + c;
-                    const float2 ca = __ldg(p.rope_a + (pos >> 5) * 64 + at), cb = __ldg(p.rope_b + (pos & 31) * 64 + at);
-                    const float cc = fmaf(ca.x, cb.x, -ca.y * cb.y), ss = fmaf(ca.y, cb.x, ca.x * cb.y);
-                    e[c] = fmaf(e[c], cc, sign * oth[c] * ss);
+                for (int c = 0; c < 4; c += 2) {
+                    const float4 ca = __ldg(ta + c / 2), cb = __ldg(tb + c / 2);
+                    const float c0 = fmaf(ca.x, cb.x, -ca.y * cb.y), s0 = fmaf(ca.y, cb.x, ca.x * cb.y);
+                    const float c1 = fmaf(ca.z, cb.z, -ca.w * cb.w), s1 = fmaf(ca.w, cb.z, ca.z * cb.w);
+                    e[c] = fmaf(e[c], c0, sign * oth[c] * s0);
+                    e[c + 1] = fmaf(e[c + 1], c1, sign * oth[c + 1] * s1);
                 }
             }
 #pragma unroll
@@ -329,7 +344,7 @@ __device__ __forceinline__ float code_as_float(uint32_t w, int i, uint32_t one_b
 }
 
 template <int BITS, int NQ, int NG, bool M16, bool ROPE>
-__global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 : 6) attn_mma_kernel(const AttnParams p)
+__global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_kernel(const AttnParams p)
 {
     using S = Shape<BITS, NQ, NG, ROPE>;
     constexpr int G = D / NG, WPT = D * BITS / 32;              // tokens (or channels) per group; 32-bit words per token
@@ -354,24 +369,21 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
     const int t0 = chunk * p.chunk, n_tok = min(p.T - t0, p.chunk), tiles = (n_tok + TILE - 1) / TILE;
     const long long ctok0 = (long long)b * p.csb + (long long)h * p.csh + t0;               // first token of the chunk
 
-    // Codes of a tile, zeros past the end of the chunk.  Keys: lane = token, its whole row.  Values: a warp's 32 rows as
-    // contiguous 512-byte pieces, LPT lanes a row (half the cache lines of the other form per load).
+    // Codes of a tile.  Keys: lane = token, its whole row.  Values: a warp's 32 rows as contiguous 512-byte pieces, LPT lanes a
+    // row (half the cache lines of the other form per load).  Past the end of the chunk its last token stands in (its score
+    // is -inf, its weight 0), so that no load hangs on a condition.
     constexpr int LPT = WPT / 4, TPL = 32 / LPT;
-    const unsigned char *k_row = p.kc + (ctok0 + tid) * (long long)(D * BITS / 8);
-    const int v_tok = 32 * warp + lane / LPT;
-    const unsigned char *v_row = p.vc + (ctok0 + v_tok) * (long long)(D * BITS / 8) + lane % LPT * 16;
+    const unsigned char *k_base = p.kc + ctok0 * (D * BITS / 8), *v_base = p.vc + ctok0 * (D * BITS / 8) + lane % LPT * 16;
+    const int v_tok = 32 * warp + lane / LPT, last_tok = n_tok - 1;
     uint4 cw[LPT];
     auto load_keys = [&](int tile) {
-        const bool in = tile * TILE + tid < n_tok;
-        const uint4 *src = reinterpret_cast<const uint4 *>(k_row + tile * (TILE * D * BITS / 8));
+        const uint4 *src = reinterpret_cast<const uint4 *>(k_base + min(tile * TILE + tid, last_tok) * (D * BITS / 8));
 #pragma unroll
-        for (int i = 0; i < LPT; ++i) cw[i] = in ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
+        for (int i = 0; i < LPT; ++i) cw[i] = __ldg(src + i);
     };
     auto load_values = [&](int tile) {
-        const unsigned char *src = v_row + tile * (TILE * D * BITS / 8);
 #pragma unroll
-        for (int i = 0; i < LPT; ++i)
-            cw[i] = tile * TILE + v_tok + TPL * i < n_tok ? ldg128(src + i * TPL * (D * BITS / 8)) : make_uint4(0, 0, 0, 0);
+        for (int i = 0; i < LPT; ++i) cw[i] = ldg128(v_base + min(tile * TILE + v_tok + TPL * i, last_tok) * (D * BITS / 8));
     };
     load_keys(0);
     // Which (token group, head) digits a warp makes: 4 / NG warps share a group and deal its heads among them.  A lane makes
@@ -379,13 +391,15 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
     constexpr int WPG = WARPS / NG, HPW = (NQ + WPG - 1) / WPG;
     const int my_group = warp / WPG, my_head0 = warp % WPG * HPW;
     const bool makes = my_head0 < NQ;
-    float4 ks, kz;                                              // scales and zero-points of those channels in the warp's group
-    const long long mrow0 = (ctok0 / G + my_group) * D + 4 * lane;
+    Meta<4, M16> ks_next, kz_next;                              // scales and zero-points of those channels in the warp's group
     auto load_kmeta = [&](int tile) {
-        const bool in = makes && tile * TILE + my_group * G < n_tok;
-        ks = in ? attn_meta4<M16>(p.ks, mrow0 + tile * (NG * D)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        kz = in ? attn_meta4<M16>(p.kz, mrow0 + tile * (NG * D)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const long long at = (ctok0 + min(tile * TILE + my_group * G, n_tok - G)) / G * (D / 4) + lane;
+        ks_next.load(p.ks, at);
+        kz_next.load(p.kz, at);
     };
+    Meta<NG, M16> vs_next, vz_next;                             // this lane's token's value scales and zero-points
+    auto load_vs = [&](int tile) { vs_next.load(p.vs, ctok0 + min(tile * TILE + tid, last_tok)); };
+    auto load_vz = [&](int tile) { vz_next.load(p.vz, ctok0 + min(tile * TILE + tid, last_tok)); };
     if (!ROPE) load_kmeta(0);
 
     if (warp == 0) {
@@ -502,23 +516,38 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
         float2 *qb = reinterpret_cast<float2 *>(reinterpret_cast<float4 *>(sc_sm - tid + MAX_TILES * TILE * NQ) + WARPS * 64) + warp * 64 * NQ;
         const uint32_t one_bits = in_register(0x3F800000u);
         constexpr float LV = float(1 << BITS);
+        // the next tile's block turn and key metadata, asked for a tile ahead like the codes
+        float2 turn[2];
+        Meta<1, M16> ms[4], mz[4];
+        auto load_block = [&](int tile) {
+            const int tok = min(tile * TILE + 32 * warp, n_tok - 32);
+            const long long mrow = (ctok0 + tok) / G * D, a_blk = (p.first_pos + t0 + tok) >> 5;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) turn[i] = __ldg(p.rope_a + a_blk * 64 + lane + 32 * i);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                ms[i].load(p.ks, mrow + lane + 32 * i);
+                mz[i].load(p.kz, mrow + lane + 32 * i);
+            }
+        };
+        load_block(0);
 #pragma unroll 1
         for (int tile = 0; tile < tiles; ++tile) {
             const int tok = tile * TILE + 32 * warp;                   // the warp's first token; n_tok is a multiple of 32
-            float vs[NG];
-            load_vmeta<NG, M16>(p.vs, ctok0 + tile * TILE + tid, tile * TILE + tid < n_tok, vs);
+            load_vs(tile);
             if (tok < n_tok) {
-                const long long mrow = (ctok0 + tok) / G * D, a_blk = (p.first_pos + t0 + tok) >> 5;
                 __syncwarp();
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     const int i = lane + 32 * hh;
-                    const float2 cs = __ldg(p.rope_a + a_blk * 64 + i);
+                    const float2 cs = turn[hh];
 #pragma unroll
                     for (int j = 0; j < NQ; ++j)
                         qb[j * 64 + i] = make_float2(fmaf(q[j][hh], cs.x, q[j][hh + 2] * cs.y), fmaf(q[j][hh + 2], cs.x, -q[j][hh] * cs.y));
-                    const float s0 = attn_meta<M16>(p.ks, mrow + i) * LV, s1 = attn_meta<M16>(p.ks, mrow + i + 64) * LV;
-                    sz[i] = make_float4(s0, attn_meta<M16>(p.kz, mrow + i) - s0, s1, attn_meta<M16>(p.kz, mrow + i + 64) - s1);
+                    float s0[1], s1[1], z0[1], z1[1];
+                    ms[hh].get(s0); ms[hh + 2].get(s1);
+                    mz[hh].get(z0); mz[hh + 2].get(z1);
+                    sz[i] = make_float4(s0[0] * LV, z0[0] - s0[0] * LV, s1[0] * LV, z1[0] - s1[0] * LV);
                 }
                 __syncwarp();
             }
@@ -547,14 +576,20 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
                         }
                     }
             }
-            if (tile + 1 < tiles) load_keys(tile + 1);
-            else load_values(0);
+            if (tile + 1 < tiles) {
+                load_keys(tile + 1);
+                load_block(tile + 1);
+            } else {
+                load_values(0);
+            }
 #pragma unroll
             for (int j = 0; j < NQ; ++j) {
                 const float s = tok < n_tok ? acc[j][0] + acc[j][1] : -INFINITY;
                 sc_sm[(tile * NQ + j) * TILE] = s;
                 mx[j] = max_nan(mx[j], s);
             }
+            float vs[NG];
+            vs_next.get(vs);
 #pragma unroll
             for (int g = 0; g < NG; ++g) vmax = max_nan(vmax, fabsf(vs[g]));
         }
@@ -562,14 +597,16 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
 #pragma unroll 1
         for (int tile = 0; tile < tiles; ++tile) {
             const int buf = tile & 1;
-            float vs[NG];
-            load_vmeta<NG, M16>(p.vs, ctok0 + tile * TILE + tid, tile * TILE + tid < n_tok, vs);
+            load_vs(tile);
+            float ks[4], kz[4];
+            ks_next.get(ks);
+            kz_next.get(kz);
             uint32_t dig[4][HPW];
 #pragma unroll
             for (int j = 0; j < HPW; ++j) {
-                const float zs = attn_warp_sum(fmaf(q[j][0], kz.x, q[j][1] * kz.y) + fmaf(q[j][2], kz.z, q[j][3] * kz.w));
+                const float zs = attn_warp_sum(fmaf(q[j][0], kz[0], q[j][1] * kz[1]) + fmaf(q[j][2], kz[2], q[j][3] * kz[3]));
                 constexpr float P1 = BITS == 2 ? 0.25f : 0.0625f, P2 = BITS == 2 ? 0.0625f : 1.0f, P3 = BITS == 2 ? 0.015625f : 0.0625f;
-                const float f[4] = {q[j][0] * ks.x, q[j][1] * ks.y, q[j][2] * ks.z, q[j][3] * ks.w};
+                const float f[4] = {q[j][0] * ks[0], q[j][1] * ks[1], q[j][2] * ks[2], q[j][3] * ks[3]};
                 float inv;
                 const float up = fixed_scale(warp_max(max_nan(max_nan(fabsf(f[0]), fabsf(f[1])), max_nan(fabsf(f[2]), fabsf(f[3])))), inv);
                 if (lane == 0 && my_head0 + j < NQ) qz_sm[tile][my_group][my_head0 + j] = make_float2(inv, zs);
@@ -596,14 +633,15 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
             tc_fence_before();
             __syncthreads();
             issue(buf, false, false);
+            float vs[NG];
+            vs_next.get(vs);
 #pragma unroll
             for (int g = 0; g < NG; ++g) vmax = max_nan(vmax, fabsf(vs[g]));
         }
         read_scores(tiles - 1);
     }
-    float vs[NG], vz[NG];
-    load_vmeta<NG, M16>(p.vs, ctok0 + tid, tid < n_tok, vs);
-    load_vmeta<NG, M16>(p.vz, ctok0 + tid, tid < n_tok, vz);
+    load_vs(0);
+    load_vz(0);
 
     // ---------------------------------------------------------------- maxima over the chunk
 #pragma unroll
@@ -639,6 +677,13 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
             w[j] = expf(sc_sm[(tile * NQ + j) * TILE] - mx[j]);
             den[j] += w[j];
         }
+        float vs[NG], vz[NG];
+        vs_next.get(vs);
+        vz_next.get(vz);
+        if (tile + 1 < tiles) {
+            load_vs(tile + 1);
+            load_vz(tile + 1);
+        }
         uint32_t dig[S::N / 4];
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
@@ -651,10 +696,6 @@ __global__ void __launch_bounds__(THREADS, NQ >= 4 ? 4 : ROPE ? 5 : NQ == 1 ? 7 
         }
 #pragma unroll
         for (int i = NG * NQ; i < S::N / 4; ++i) dig[i] = 0;
-        if (tile + 1 < tiles) {
-            load_vmeta<NG, M16>(p.vs, ctok0 + (tile + 1) * TILE + tid, (tile + 1) * TILE + tid < n_tok, vs);
-            load_vmeta<NG, M16>(p.vz, ctok0 + (tile + 1) * TILE + tid, (tile + 1) * TILE + tid < n_tok, vz);
-        }
 #pragma unroll
         for (int c = 0; c < S::N / 16; ++c)
             *reinterpret_cast<uint4 *>(my_dig + buf * S::DIG_BYTES + c * DIG_CHUNK) = make_uint4(dig[4 * c], dig[4 * c + 1], dig[4 * c + 2], dig[4 * c + 3]);
