@@ -219,8 +219,62 @@ __device__ __forceinline__ double rcp_nr(double x)
 }
 
 // ------------------------------------------------------------------------------------- assemble
-constexpr int ASM_THREADS = 512;
-constexpr int ASM_LD = D + 1;
+// P_inv and its LDL^T factorisation, one CTA per head.  The 136 tiles of 8 x 8 on or below the diagonal live in registers
+// as accumulators of the fp64 tensor path, dealt column by column to the 16 warps; the factorisation goes by panels of 8
+// columns: the owners of a column of tiles publish it, four warps (a thread per row, the 8 x 8 diagonal block factored by
+// each of them for itself, so that nothing is handed over in between) solve for the panel's rows, and every warp subtracts
+// the panel's product from its later tiles.  Two barriers per panel, 32 in all; one column at a time took 128 steps of a
+// barrier and a pass through shared memory each (36 us on 32 heads, of which the dependent divisions are 5).
+constexpr int ASM_THREADS = 512, ASM_WARPS = 16;
+constexpr int ASM_LD = D + 1;                  // row stride of L in shared memory (block updates)
+constexpr int ASM_LDU = D + 4;                 // of the staged vectors: 4 mod 16, fragments without bank conflicts
+constexpr int ASM_LDP = 12;                    // of a panel's rows: fragments without bank conflicts
+constexpr int ASM_TILES = 9;                   // tiles per warp, at most
+constexpr int ASM_STAGE = 32;                  // vectors staged at a time
+constexpr size_t ASM_SMEM = sizeof(double) * (D * ASM_LD + 3 * D * ASM_LDP + D);
+static_assert(2 * ASM_STAGE * ASM_LDU <= D * ASM_LD && ASM_SMEM <= 227 * 1024, "shared memory of assemble_kernel");
+
+// row and column of the u-th tile of the lower triangle, column by column
+__device__ __forceinline__ void asm_tile(int u, int &ti, int &tj)
+{
+    int c = 0, len = 16;
+    while (u >= len) { u -= len; --len; ++c; }
+    tj = c;
+    ti = c + u;
+}
+
+// X <- X inverse(Lb) for the rows below a diagonal block Lb (unit lower, GB x GB, at A[c0][c0]): four lanes a row, columns
+// dealt cyclically, from the last column down.
+template <int GB>
+__device__ __forceinline__ void block_solve(double *A, int tid)
+{
+    constexpr int PER = GB / 4, BLOCKS = D / GB - 1;
+    const int sub = tid & 3;
+    int item = tid >> 2;                       // (block, row below it)
+    for (;; item += ASM_THREADS / 4) {
+        int t = 0, row = item;
+        while (t < BLOCKS && row >= D - (t + 1) * GB) { row -= D - (t + 1) * GB; ++t; }
+        const bool live = t < BLOCKS;
+        if (!__any_sync(0xffffffffu, live)) break;
+        const int c0 = live ? t * GB : 0;
+        double *x_sm = A + (live ? (t + 1) * GB + row : 0) * ASM_LD + c0;
+        const double *lb = A + c0 * ASM_LD + c0;
+        double x[PER];
+#pragma unroll
+        for (int m = 0; m < PER; ++m) x[m] = x_sm[4 * m + sub];
+#pragma unroll
+        for (int c = GB - 1; c >= 1; --c) {
+            const double xc = __shfl_sync(0xffffffffu, x[c / 4], c % 4, 4);
+#pragma unroll
+            for (int m = 0; m <= (c - 1) / 4; ++m)
+                if (4 * m + 3 < c || 4 * m + sub < c) x[m] = fma(-xc, lb[c * ASM_LD + 4 * m + sub], x[m]);
+        }
+        if (live) {
+#pragma unroll
+            for (int m = 0; m < PER; ++m) x_sm[4 * m + sub] = x[m];
+        }
+    }
+}
 
 __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
     const double *__restrict__ eigval, const double *__restrict__ eigvec, int rank_r, double lambda, int g,
@@ -229,129 +283,128 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
     // left_rows = 0: P_inv = I - sum_i s_i/(1+s_i) v_i v_i^T from eigen-pairs (rows i of eigvec, eigval).
     // left_rows > 0: P_inv = I - sum_i z_i x_i^T with x_i = row i and z_i = row left_rows + i of eigvec (block power build).
     extern __shared__ __align__(16) double sm[];
-    double *A = sm;                         // A[row * ASM_LD + col]
-    double *colv = sm + D * ASM_LD;         // [2 parities][l, v][D]: column j of L and of the matrix, as published
-    double *coef = colv + 4 * D;            // s_i / (1 + s_i)
-    const int h = blockIdx.x, tid = threadIdx.x;
+    double *A = sm;                             // [D][ASM_LD] L, for block updates only
+    double *U = A;                              // [ASM_STAGE][ASM_LDU] right vectors, before there is an L
+    double *UL = U + ASM_STAGE * ASM_LDU;       // the same, left vectors times -coefficient
+    double *P = A + D * ASM_LD;                 // [D][ASM_LDP] the panel's columns of the matrix
+    double *Lp = P + D * ASM_LDP, *Vp = Lp + D * ASM_LDP;     // the panel's rows of L and of L D
+    double *coef = Vp + D * ASM_LDP;            // -s_i / (1 + s_i)
+    const int h = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int fr = lane >> 2, fk = lane & 3;
     const double *V = eigvec + (long long)h * D * D;
+    float *out = Wt + (long long)h * D * D;
 
     if (tid < D) {
         double mu = eigval[(long long)h * D + tid];
         if (!(mu > 0.0)) mu = 0.0;
         const double s = lambda * mu;
-        coef[tid] = (tid < rank_r) ? (left_rows > 0 ? 1.0 : s / (1.0 + s)) : 0.0;
+        coef[tid] = (tid < rank_r) ? (left_rows > 0 ? -1.0 : -s / (1.0 + s)) : 0.0;
     }
+    int ti[ASM_TILES], tj[ASM_TILES];
+    double c[ASM_TILES][2];
+#pragma unroll
+    for (int n = 0; n < ASM_TILES; ++n) {
+        const int u = warp + ASM_WARPS * n;
+        ti[n] = tj[n] = 16;                     // no tile
+        if (u < 136) asm_tile(u, ti[n], tj[n]);
+        c[n][0] = ti[n] == tj[n] && fr == 2 * fk ? 1.0 : 0.0;
+        c[n][1] = ti[n] == tj[n] && fr == 2 * fk + 1 ? 1.0 : 0.0;
+    }
+    for (int i0 = 0; i0 < rank_r; i0 += ASM_STAGE) {
+        const int ni = rank_r - i0 < ASM_STAGE ? rank_r - i0 : ASM_STAGE, nk = (ni + 3) / 4 * 4;
+        __syncthreads();
+        for (int idx = tid; idx < nk * D; idx += ASM_THREADS) {
+            const int e = idx / D, i = idx % D;
+            U[e * ASM_LDU + i] = e < ni ? V[(long long)(i0 + e) * D + i] : 0.0;
+            UL[e * ASM_LDU + i] = e < ni ? coef[i0 + e] * V[(long long)(left_rows + i0 + e) * D + i] : 0.0;
+        }
+        __syncthreads();
+        for (int e = 0; e < nk; e += 4) {
+#pragma unroll
+            for (int n = 0; n < ASM_TILES; ++n) {
+                if (ti[n] == 16) continue;      // warp-uniform
+                dmma_m8n8k4(c[n][0], c[n][1], UL[(e + fk) * ASM_LDU + 8 * ti[n] + fr], U[(e + fk) * ASM_LDU + 8 * tj[n] + fr]);
+            }
+        }
+    }
+    auto publish = [&](int p) {                 // the tiles of column p, as rows of 8
+#pragma unroll
+        for (int n = 0; n < ASM_TILES; ++n)
+            if (tj[n] == p) *reinterpret_cast<double2 *>(&P[(8 * ti[n] + fr) * ASM_LDP + 2 * fk]) = make_double2(c[n][0], c[n][1]);
+    };
+    publish(0);
     __syncthreads();
-    // The matrix lives in REGISTERS from here to the end of the factorisation: thread (lane, warp) owns the elements
-    // (row lane + 32 i, column warp + 16 k), i < 4, k < 8; only those on or below the diagonal are used.
-    const int warp = tid >> 5, lane = tid & 31;
-    double a[4][8];
-    // P_inv = I - sum_{i<r} coef_i v_i v_i^T; the eigenvectors are staged 32 at a time in shared memory
-    {
-        double *U = coef + D;                           // [32][D] staged eigenvectors (right vectors)
-        double *UL = left_rows > 0 ? U + 32 * D : U;    // [32][D] staged left vectors
+#pragma unroll 1
+    for (int p = 0; p < 16; ++p) {
+        if (tid < D) {
+            double d[8][8], v[8], l[8];         // the diagonal block (lower half) and this thread's row
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int k = 0; k < 8; ++k) a[i][k] = (lane + 32 * i == warp + 16 * k) ? 1.0 : 0.0;
-        for (int i0 = 0; i0 < rank_r; i0 += 32) {
-            const int ni = rank_r - i0 < 32 ? rank_r - i0 : 32;
-            __syncthreads();
-            for (int idx = tid; idx < ni * D; idx += ASM_THREADS) U[idx] = V[(long long)i0 * D + idx];
-            if (left_rows > 0)
-                for (int idx = tid; idx < ni * D; idx += ASM_THREADS) UL[idx] = V[(long long)(left_rows + i0) * D + idx];
-            __syncthreads();
-            for (int e = 0; e < ni; ++e) {
-                const double cf = -coef[i0 + e];
-                double vr[4], vc[8];
+                for (int k = 0; k <= i; ++k) d[i][k] = P[(8 * p + i) * ASM_LDP + k];
+            const bool below = tid >= 8 * p;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) vr[i] = cf * UL[e * D + lane + 32 * i];
+            for (int k = 0; k < 8; ++k) v[k] = below ? P[tid * ASM_LDP + k] : 0.0;
+            // column k: v_k = L_rk d_k is final, l_k = v_k / d_k; later columns lose v_k times row element L_ck
 #pragma unroll
-                for (int k = 0; k < 8; ++k) vc[k] = U[e * D + warp + 16 * k];
+            for (int k = 0; k < 8; ++k) {
+                const double inv = rcp_nr(d[k][k]);
+                l[k] = v[k] * inv;
+#pragma unroll
+                for (int i = k + 1; i < 8; ++i) {
+                    const double li = d[i][k] * inv;                  // L_ik of the diagonal block
+#pragma unroll
+                    for (int z = i; z < 8; ++z) d[z][i] = fma(-li, d[z][k], d[z][i]);
+                    v[i] = fma(-li, v[k], v[i]);
+                }
+            }
+            if (below) {
+#pragma unroll
+                for (int k = 0; k < 8; k += 2) {
+                    *reinterpret_cast<double2 *>(&Lp[tid * ASM_LDP + k]) = make_double2(-l[k], -l[k + 1]);
+                    *reinterpret_cast<double2 *>(&Vp[tid * ASM_LDP + k]) = make_double2(v[k], v[k + 1]);
+                }
+            }
+            if (g == 1) {
+                // Wt[j][j'] = W[j'][j] = L[j'][j] below the diagonal, zero on and above it
+#pragma unroll
+                for (int k = 0; k < 8; ++k) out[(8 * p + k) * D + tid] = tid > 8 * p + k ? (float)l[k] : 0.0f;
+            } else if (below) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (32 * i + 31 >= 16 * k) a[i][k] = fma(vr[i], vc[k], a[i][k]);
+                    if (tid > 8 * p + k) A[tid * ASM_LD + 8 * p + k] = l[k];
             }
         }
-    }
-    __syncthreads();
-    // LDL^T (right-looking), afterwards the strict lower triangle holds L.  Step j: the warp that owns column j gets
-    // the pivot d_j by a shuffle and publishes v = column j and l = v / d_j in shared memory; after ONE barrier (the
-    // buffers alternate) every thread subtracts l_r v_c from its elements.
-    {
-        double *pub = colv;                             // [2 parities][l, v][D], overlays colv, lcol and more
+        __syncthreads();
 #pragma unroll
-        for (int kj = 0; kj < 8; ++kj) {
-#pragma unroll 1
-            for (int wj = 0; wj < 16; ++wj) {
-                const int j = 16 * kj + wj;
-                double *lp = pub + (j & 1) * 2 * D, *vp = lp + D;
-                if (warp == wj) {
-                    const double d = __shfl_sync(0xffffffffu, a[kj >> 1][kj], j & 31);
-                    const double inv = rcp_nr(d);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int r = lane + 32 * i;
-                        const double v = a[i][kj], l = v * inv;
-                        if (r > j) { lp[r] = l; vp[r] = v; a[i][kj] = l; }
-                    }
-                }
-                __syncthreads();
-                double lr[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) lr[i] = lp[lane + 32 * i];     // rows <= j hold stale values: only feed unused elements
-#pragma unroll
-                for (int k = kj; k < 8; ++k) {
-                    const int c = warp + 16 * k;
-                    if (c > j) {                        // warp-uniform
-                        const double vc = vp[c];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (32 * i + 31 >= 16 * k) a[i][k] = fma(-lr[i], vc, a[i][k]);
-                    }
-                }
-            }
+        for (int n = 0; n < ASM_TILES; ++n) {
+            if (tj[n] == 16 || tj[n] <= p) continue;
+            const double *lp = Lp + (8 * ti[n] + fr) * ASM_LDP + fk, *vp = Vp + (8 * tj[n] + fr) * ASM_LDP + fk;
+            dmma_m8n8k4(c[n][0], c[n][1], lp[0], vp[0]);
+            dmma_m8n8k4(c[n][0], c[n][1], lp[4], vp[4]);
         }
+        if (p < 15) publish(p + 1);
+        __syncthreads();
     }
-    float *out = Wt + (long long)h * D * D;
-    if (g == 1) {
-        // Wt[j][j'] = W[j'][j] = L[j'][j] below the diagonal, zero on and above it: straight from the registers
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = lane + 32 * i, c = warp + 16 * k;
-                out[c * D + r] = (r > c) ? (float)a[i][k] : 0.0f;
-            }
-        return;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = lane + 32 * i, c = warp + 16 * k;
-            if (r > c) A[r * ASM_LD + c] = a[i][k];
-        }
-    __syncthreads();
+    if (g == 1) return;
     // g > 1: block column t becomes L[rest, blk] * inverse(unit-lower diagonal block)
-    if (g > 1) {
+    if (g == 64) block_solve<64>(A, tid);
+    else if (g == 32) block_solve<32>(A, tid);
+    else {
         const int T = D / g;
         for (int idx = tid; idx < D * (T - 1); idx += ASM_THREADS) {
             const int row = idx % D, t = idx / D;          // block t: columns [t*g, (t+1)*g)
             const int c0 = t * g;
             if (row < c0 + g) continue;
             double *x = A + row * ASM_LD + c0;
-            for (int c = g - 2; c >= 0; --c) {
-                double s = x[c];
-                for (int cp = c + 1; cp < g; ++cp) s = fma(-x[cp], A[(c0 + cp) * ASM_LD + c0 + c], s);
-                x[c] = s;
+            for (int cc = g - 2; cc >= 0; --cc) {
+                double s = x[cc];
+                for (int cp = cc + 1; cp < g; ++cp) s = fma(-x[cp], A[(c0 + cp) * ASM_LD + c0 + cc], s);
+                x[cc] = s;
             }
         }
-        __syncthreads();
     }
+    __syncthreads();
     // Wt[j][j'] = W[j'][j]: zero on and above the block diagonal
     for (int idx = tid; idx < D * D; idx += ASM_THREADS) {
         const int j = idx / D, jp = idx % D;
@@ -389,7 +442,7 @@ int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads
 
 int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_blocks, cudaStream_t st)
 {
-    const size_t smem = sizeof(double) * (D * ASM_LD + 5 * D + 64 * D);
+    constexpr size_t smem = ASM_SMEM;
     static std::atomic<unsigned long long> allowed{0};
     if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(assemble_kernel), smem, allowed)) return rc;
     assemble_kernel<<<s->n_kv_heads, ASM_THREADS, smem, st>>>(s->eigval, s->eigvec, rank_r, lambda, block_g, s->Wt, left_rows);
