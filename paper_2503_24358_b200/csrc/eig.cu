@@ -9,6 +9,7 @@
 // tenth of the time.  Measured on the 32 heads of a 4096-token prompt: 98 + 83 us.  What was here before, one-sided Jacobi
 // on a Cholesky factor, needed 10 sweeps of 127 dependent rounds: 677 us.
 #include <cooperative_groups.h>
+#include <type_traits>
 #include "squat_internal.cuh"
 
 namespace {
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(TRI_THREADS, 1) tridiag_kernel(
 // kept above DC_ZMIN instead.  Both are backward errors of the size that any eigensolver commits, and the work does not
 // depend on the data.
 //
-// Four CTAs work on a head.  Each solves a 32 x 32 diagonal block alone (merges to 2, 4, .. 32), two share a merge to 64
+// Four CTAs work on a head.  Each solves a 32 x 32 diagonal block alone (rotations to 2, merges to 4, 8, .. 32), two share a merge to 64
 // and four the one to 128; a CTA always owns 32 roots, eight lanes each, and the 32 eigenvectors that belong to them.
 // What the next merge needs (eigenvalues, eigenvectors, roots) is written straight into the peers' shared memory.
 // Warps 8-15 meanwhile make the triangular factors of the blocked reflectors and then help to apply them.
@@ -403,7 +404,7 @@ __device__ __forceinline__ void secular_root(const double *ds, const double *zs,
     {
         const double rmid = rcp_nr(mid);
         const double c = f + zi2 * rmid - zr * rmid;                  // the poles' terms at the middle taken out
-        if (last) mu = zi2 / c;
+        if (last) mu = zi2 * rcp_nr(c);
         else {
             const double sg = right ? -1.0 : 1.0;
             const double a = fma(c, gap, sg * (zi2 + zr)), b = (right ? zr : zi2) * gap;
@@ -411,7 +412,7 @@ __device__ __forceinline__ void secular_root(const double *ds, const double *zs,
             // left: a > 0 ? 2b / (a + r) : (a - r) / 2c;   right: a < 0 ? 2b / (a - r) : -(a + r) / 2c
             const bool first = right ? a < 0.0 : a > 0.0;
             const double num = first ? 2.0 * b : sg * (a - sg * r), den = first ? a + sg * r : 2.0 * c;
-            mu = num / den;
+            mu = num * rcp_nr(den);
         }
         if (!(mu > lo && mu < hi)) mu = 0.5 * (lo + hi);
     }
@@ -449,7 +450,7 @@ __device__ __forceinline__ void secular_root(const double *ds, const double *zs,
                 num = a <= 0.0 ? a - disc : 2.0 * b;
                 den = a <= 0.0 ? 2.0 * c : a + disc;
             }
-            double nw = mu + (last ? di : 0.0) + num / den;
+            double nw = mu + (last ? di : 0.0) + num * rcp_nr(den);     // a zero den: not a number, bisected
             if (!(nw > lo && nw < hi) || (it % 5 == 4 && fabs(w) > 0.1 * pw)) {
                 const double g = sqrt_nr(fmax(alo, 1e-34 * ahi) * ahi);
                 nw = ahi > 8.0 * alo ? (right ? -g : g) : 0.5 * (lo + hi);
@@ -596,7 +597,21 @@ __device__ __forceinline__ void dc_merge_local(DcShared &sm, int &buf, int blk, 
     work_sync();
     dc_vectors<N>(sm, sm.mu32, sm.k32, 0, tid);
     work_sync();
-    {
+    if constexpr (N >= 16) {                   // 8 x 8 tiles on the problems' diagonal blocks, two a warp at most
+        const int warp = tid >> 5, lane = tid & 31;
+        constexpr int PER_ROW = N / 8, TILES = 4 * PER_ROW;
+#pragma unroll
+        for (int u = warp; u < TILES; u += DC_WORK / 32) {
+            const int ti = u / PER_ROW, tj = ti / PER_ROW * PER_ROW + u % PER_ROW;       // tile row and column in the 32 x 32 block
+            const int k0 = 8 * ti / M * M;     // the columns of the child that the row belongs to
+            double acc[2] = {0.0, 0.0};
+#pragma unroll
+            for (int kx = 0; kx < M; kx += 4)
+                dmma(acc[0], acc[1], q[(8 * ti + (lane >> 2)) * DC_LD + k0 + kx + (lane & 3)], sm.s[(k0 + kx + (lane & 3)) * DC_LD + 8 * tj + (lane >> 2)]);
+            const int r = 8 * ti + (lane >> 2), c = 8 * tj + 2 * (lane & 3);
+            *reinterpret_cast<double2 *>(&qn[r * DC_LD + c]) = make_double2(acc[0] * sm.norm[c], acc[1] * sm.norm[c + 1]);
+        }
+    } else {
         const int c = tid & 31, p = c / N * N;
         const double nv = sm.norm[c];
 #pragma unroll
@@ -731,13 +746,31 @@ __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS, 1)
         if (tid < D - 1) v -= fmax(fabs(sm.e[tid]), DC_RHOMIN);
         sm.d32[0][tid & 31] = v;
     }
-    for (int i = tid; i < 32 * DC_LD; i += DC_THREADS) sm.q32[0][i] = i / DC_LD == i % DC_LD ? 1.0 : 0.0;
+    for (int i = tid; i < 32 * DC_LD; i += DC_THREADS) sm.q32[0][i] = 0.0;
+    __syncthreads();
+    if (tid < 16) {                            // the 2 x 2 diagonal blocks by one rotation each
+        const int i = 2 * tid;
+        const double a = sm.d32[0][i], c = sm.d32[0][i + 1], e = sm.e[32 * rank + i];
+        // the corners between the two were not torn: a and c have lost |e| in vain
+        const double add = fmax(fabs(e), DC_RHOMIN), a1 = a + add, c1 = c + add;
+        const double half = 0.5 * (c1 - a1), r = sqrt_nr(fma(half, half, e * e));
+        const double den = fabs(half) + r, tn = den > 1e-290 ? (half >= 0.0 ? e : -e) * rcp_nr(den) : 0.0;   // tan of the angle, at most 1
+        const double cs = rsqrt_nr(fma(tn, tn, 1.0)), sn = tn * cs;
+        const double lo = fma(-tn, e, a1), hi = fma(tn, e, c1);       // of (cs, -sn) and (sn, cs)
+        const bool swap = lo > hi;
+        sm.d32[0][i] = swap ? hi : lo;
+        sm.d32[0][i + 1] = swap ? lo : hi;
+        const double v0[2] = {cs, sn}, v1[2] = {-sn, cs};             // rows of the matrix whose columns are the vectors
+        sm.q32[0][i * DC_LD + i] = v0[swap];
+        sm.q32[0][i * DC_LD + i + 1] = v0[!swap];
+        sm.q32[0][(i + 1) * DC_LD + i] = v1[swap];
+        sm.q32[0][(i + 1) * DC_LD + i + 1] = v1[!swap];
+    }
     __syncthreads();
 
     int most = 0;
     if (warp < DC_WORK / 32) {
         int buf = 0;
-        dc_merge_local<2>(sm, buf, rank, tid, most);
         dc_merge_local<4>(sm, buf, rank, tid, most);
         dc_merge_local<8>(sm, buf, rank, tid, most);
         dc_merge_local<16>(sm, buf, rank, tid, most);
@@ -830,12 +863,18 @@ __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS, 1)
             double acc[4][2] = {};
             const double *ua = u + (8 * ti + (lane >> 2)) * DC_LDU + (lane & 3);
             const double *xb = sm.x + (lane & 3) * DC_LD + 8 * tj + (lane >> 2);
-            for (int i = 16 * b + 8 * half; i < D; i += 16) {
-                dmma(acc[0][0], acc[0][1], ua[i], xb[i * DC_LD]);
-                dmma(acc[1][0], acc[1][1], ua[i + 4], xb[(i + 4) * DC_LD]);
+            for (int i = 16 * b + 8 * half; i < D; i += 32) {          // four products in flight
+                const bool two = i + 16 < D;
+                const double a0 = ua[i], b0 = xb[i * DC_LD], a1 = ua[i + 4], b1 = xb[(i + 4) * DC_LD];
+                const double a2 = two ? ua[i + 16] : 0.0, b2 = two ? xb[(i + 16) * DC_LD] : 0.0;
+                const double a3 = two ? ua[i + 20] : 0.0, b3 = two ? xb[(i + 20) * DC_LD] : 0.0;
+                dmma(acc[0][0], acc[0][1], a0, b0);
+                dmma(acc[1][0], acc[1][1], a1, b1);
+                dmma(acc[2][0], acc[2][1], a2, b2);
+                dmma(acc[3][0], acc[3][1], a3, b3);
             }
             const int r = 8 * ti + (lane >> 2), c = 8 * tj + 2 * (lane & 3);
-            *reinterpret_cast<double2 *>(&sm.y[half][r * DC_LD + c]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+            *reinterpret_cast<double2 *>(&sm.y[half][r * DC_LD + c]) = make_double2((acc[0][0] + acc[1][0]) + (acc[2][0] + acc[3][0]), (acc[0][1] + acc[1][1]) + (acc[2][1] + acc[3][1]));
         }
         __syncthreads();
         if (warp < 8) {                        // Z = T Y
@@ -849,14 +888,31 @@ __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS, 1)
             *reinterpret_cast<double2 *>(&sm.z[r * DC_LD + c]) = make_double2(-(acc[0][0] + acc[1][0]), -(acc[0][1] + acc[1][1]));
         }
         __syncthreads();
-        for (int rt = 2 * b + (warp >> 2); rt < 16; rt += 4) {        // X += U^T (-Z): tile row rt, tile column warp % 4
-            const int tj = warp & 3, r = 8 * rt + (lane >> 2), c = 8 * tj + 2 * (lane & 3);
-            double2 acc = *reinterpret_cast<const double2 *>(&sm.x[r * DC_LD + c]);
-            const double *ua = u + (lane & 3) * DC_LDU + r;
+        {   // X += U^T (-Z): tile column warp % 4, tile rows 2 b + warp / 4, + 4, .. (four at most, in flight together)
+            const int tj = warp & 3, c = 8 * tj + 2 * (lane & 3), rt0 = 2 * b + (warp >> 2);
             const double *zb = sm.z + (lane & 3) * DC_LD + 8 * tj + (lane >> 2);
+            double z[4];
 #pragma unroll
-            for (int kx = 0; kx < 16; kx += 4) dmma(acc.x, acc.y, ua[kx * DC_LDU], zb[kx * DC_LD]);
-            *reinterpret_cast<double2 *>(&sm.x[r * DC_LD + c]) = acc;
+            for (int kx = 0; kx < 4; ++kx) z[kx] = zb[4 * kx * DC_LD];
+            auto update = [&](auto count) {
+                constexpr int NT = decltype(count)::value;
+                double2 acc[NT];
+#pragma unroll
+                for (int n = 0; n < NT; ++n) acc[n] = *reinterpret_cast<const double2 *>(&sm.x[(8 * (rt0 + 4 * n) + (lane >> 2)) * DC_LD + c]);
+#pragma unroll
+                for (int kx = 0; kx < 4; ++kx)
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) dmma(acc[n].x, acc[n].y, u[(4 * kx + (lane & 3)) * DC_LDU + 8 * (rt0 + 4 * n) + (lane >> 2)], z[kx]);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) *reinterpret_cast<double2 *>(&sm.x[(8 * (rt0 + 4 * n) + (lane >> 2)) * DC_LD + c]) = acc[n];
+            };
+            switch ((19 - rt0) / 4) {          // warp-uniform
+            case 4: update(std::integral_constant<int, 4>{}); break;
+            case 3: update(std::integral_constant<int, 3>{}); break;
+            case 2: update(std::integral_constant<int, 2>{}); break;
+            case 1: update(std::integral_constant<int, 1>{}); break;
+            default: break;
+            }
         }
     }
     __syncthreads();
