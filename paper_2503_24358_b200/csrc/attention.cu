@@ -21,10 +21,10 @@ namespace {
 constexpr int D = SQUAT_D;
 
 // One CTA per (batch, query head), thread = channel: parts rescaled to the common maximum and added.
-__global__ void __launch_bounds__(D) attn_combine_kernel(const AttnParams p)
+__global__ void __launch_bounds__(D) attn_combine_kernel(AttnParams p)
 {
     const int hq = blockIdx.x, b = blockIdx.y, c = threadIdx.x, parts = p.nchunk + (p.R > 0);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_wait(p.part, p.ml);
     const long long row = ((long long)b * p.Hq + hq) * parts;
     const float2 *ml = reinterpret_cast<const float2 *>(p.ml) + row;
     const float *part = p.part + row * D + c;
@@ -104,16 +104,5 @@ int squat_launch_decode_attention(const void *q, int q_dtype, int batch, int Hq,
     p.ml = workspace + (size_t)batch * Hq * (p.nchunk + (R > 0)) * D;
     const int rc = p.rope_a ? squat_launch_attn_rope(p, bits, st) : squat_launch_attn_mma(p, bits, st);
     if (rc != SQUAT_OK) return rc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(Hq, batch);
-    cfg.blockDim = dim3(D);
-    cfg.stream = st;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    SQUAT_CUDA(cudaLaunchKernelEx(&cfg, attn_combine_kernel, p));
-    squat_count_launch();
-    return SQUAT_OK;
+    return squat_launch(attn_combine_kernel, dim3(Hq, batch), D, 0, st, p);
 }

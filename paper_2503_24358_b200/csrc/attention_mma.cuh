@@ -344,7 +344,7 @@ __device__ __forceinline__ float code_as_float(uint32_t w, int i, uint32_t one_b
 }
 
 template <int BITS, int NQ, int NG, bool M16, bool ROPE>
-__global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_kernel(const AttnParams p)
+__global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_kernel(AttnParams p)
 {
     using S = Shape<BITS, NQ, NG, ROPE>;
     constexpr int G = D / NG, WPT = D * BITS / 32;              // tokens (or channels) per group; 32-bit words per token
@@ -361,6 +361,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     const int parts = p.nchunk + (p.R > 0), chunk = blockIdx.x % parts, qpass = blockIdx.x / parts;
     const int h = blockIdx.y, b = blockIdx.z;
     const int qpk = p.Hq / p.H, hq0 = h * qpk + qpass * NQ, nq_here = min(NQ, qpk - qpass * NQ);
+    grid_wait(p.q, p.kc, p.vc, p.ks, p.kz, p.vs, p.vz, p.k_res, p.v_res, p.rope_a, p.rope_b);
     if (chunk == p.nchunk) {
         if (p.res_bf16) residual_part<NQ, ROPE, true>(p, reinterpret_cast<float *>(smem_raw), h, b, hq0, nq_here, parts);
         else residual_part<NQ, ROPE, false>(p, reinterpret_cast<float *>(smem_raw), h, b, hq0, nq_here, parts);
@@ -752,10 +753,7 @@ int launch(const AttnParams &p, int qpasses, cudaStream_t st)
     constexpr size_t smem = Shape<BITS, NQ, NG, ROPE>::SMEM;
     static std::atomic<unsigned long long> allowed{0};
     if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(attn_mma_kernel<BITS, NQ, NG, M16, ROPE>), smem, allowed)) return rc;
-    attn_mma_kernel<BITS, NQ, NG, M16, ROPE><<<dim3((p.nchunk + (p.R > 0)) * qpasses, p.H, p.B), THREADS, smem, st>>>(p);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
+    return squat_launch(attn_mma_kernel<BITS, NQ, NG, M16, ROPE>, dim3((p.nchunk + (p.R > 0)) * qpasses, p.H, p.B), THREADS, smem, st, p);
 }
 template <bool ROPE, int BITS, int NQ>
 int launch_g(const AttnParams &p, int qpasses, cudaStream_t st)

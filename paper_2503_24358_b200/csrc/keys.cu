@@ -243,11 +243,11 @@ __device__ __forceinline__ void load_row(RawRow<BF16> &r, const void *row, int c
     if (BF16) {
         const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(row) + chan);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) r.v[i] = __ldg(q + i);
+        for (int i = 0; i < 4; ++i) r.v[i] = *(q + i);
     } else {
         const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(row) + chan);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) r.v[i] = __ldg(q + i);
+        for (int i = 0; i < 8; ++i) r.v[i] = *(q + i);
     }
 }
 // channel pair q (channels 2q, 2q + 1) of the row as two floats
@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_kernel(const KeyPara
         if (n > two_heads_end - start) n = two_heads_end - start;
         return n;
     };
+    grid_wait();          // (its global loads are plain ones; laundering p here would cost registers the sweeps need)
     const unsigned img_mbar = smem_u32(mbar + TC_SLOTS);
     unsigned img_phase = 0;
 
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_kernel(const KeyPara
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(img_mbar), "r"(1) : "memory");
         shared_words[1] = 0;
-        shared_words[2 + TC_SLOTS] = (unsigned)__ldg(p.exact_blocks);
+        shared_words[2 + TC_SLOTS] = (unsigned)*(p.exact_blocks);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // the first head's image is on its way while the rest of the set-up runs
         if (t_lo < t_hi) {
@@ -724,8 +725,7 @@ int launch_keys_inst(const KeyParams &p, int grid, size_t smem, cudaStream_t st)
 {
     static std::atomic<unsigned long long> allowed{0};
     if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(quant_keys_kernel<BITS, NW, BF16, M16>), smem, allowed)) return rc;
-    quant_keys_kernel<BITS, NW, BF16, M16><<<grid, TC_THREADS, smem, st>>>(p);
-    return SQUAT_OK;
+    return squat_launch(quant_keys_kernel<BITS, NW, BF16, M16>, grid, TC_THREADS, smem, st, p);
 }
 
 template <int BITS, int NW>
@@ -749,10 +749,7 @@ int launch_keys(KeyParams p, int dtype, int meta16, cudaStream_t st)
     int rc;
     if (dtype == SQUAT_BF16) rc = meta16 ? launch_keys_inst<BITS, NW, true, true>(p, grid, smem, st) : launch_keys_inst<BITS, NW, true, false>(p, grid, smem, st);
     else rc = meta16 ? launch_keys_inst<BITS, NW, false, true>(p, grid, smem, st) : launch_keys_inst<BITS, NW, false, false>(p, grid, smem, st);
-    if (rc != SQUAT_OK) return rc;
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
+    return rc;
 }
 
 }  // namespace

@@ -179,11 +179,11 @@ __device__ __forceinline__ void load16(Raw16<BF16> &r, const void *row, int chan
     if (BF16) {
         const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(row) + chan);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) r.v[i] = __ldg(q + i);
+        for (int i = 0; i < 2; ++i) r.v[i] = *(q + i);
     } else {
         const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(row) + chan);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) r.v[i] = __ldg(q + i);
+        for (int i = 0; i < 4; ++i) r.v[i] = *(q + i);
     }
 }
 template <bool BF16>
@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(LR_THREADS, LR_CTAS_PER_SM) quant_keys_lowrank
     __shared__ __align__(16) float table[D * ROW];
     __shared__ float2 meta_all[LR_WARPS][2][BLK];   // (scale, zero) of the block just swept, per warp and span
     __shared__ float2 red_all[LR_WARPS / 2][2][2];  // G = 128: [team][parity][warp of the team] (min, max)
+    grid_wait();          // (its global loads are plain ones)
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int team = warp / NW, wteam = warp % NW;
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(LR_THREADS, LR_CTAS_PER_SM) quant_keys_lowrank
     {
         const float4 *src = reinterpret_cast<const float4 *>(p.table + (long long)head * D * ROW);
         for (int i = threadIdx.x; i < D * ROW / 4; i += LR_THREADS)
-            if (SQ_CHK_G(p.status, src + i, 16, p.x_table)) reinterpret_cast<float4 *>(table)[i] = __ldg(src + i);
+            if (SQ_CHK_G(p.status, src + i, 16, p.x_table)) reinterpret_cast<float4 *>(table)[i] = *(src + i);
     }
     __syncthreads();
     float2(*meta)[BLK] = meta_all[warp];
@@ -388,13 +389,10 @@ int launch_lowrank(const LrParams &p, int H, int dtype, int meta16, cudaStream_t
     if (per_head > ctas_needed) per_head = ctas_needed;
     if (per_head < 1) per_head = 1;
     const dim3 grid(per_head, H);
-#define SQ_LR(BF, MM) quant_keys_lowrank_kernel<BITS, G, BF, MM><<<grid, LR_THREADS, 0, st>>>(p)
+#define SQ_LR(BF, MM) return squat_launch(quant_keys_lowrank_kernel<BITS, G, BF, MM>, grid, LR_THREADS, 0, st, p)
     if (dtype == SQUAT_BF16) { if (meta16) SQ_LR(true, true); else SQ_LR(true, false); }
     else { if (meta16) SQ_LR(false, true); else SQ_LR(false, false); }
 #undef SQ_LR
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
 }
 
 }  // namespace

@@ -130,7 +130,7 @@ __device__ __noinline__ unsigned patch_word(unsigned word, unsigned mask, const 
 // VAL_THREADS consecutive spans of one (batch, head) row -- grid (chunks of a row, heads, batch) -- so no index is divided
 // out of a flat CTA number; a span's token is a shift (d / 32 a power of two) or one 32-bit division.
 template <int G, int BITS, bool BF16, bool M16>
-__global__ void __launch_bounds__(VAL_THREADS) quant_values_kernel(const ValParams p)
+__global__ void __launch_bounds__(VAL_THREADS) quant_values_kernel(ValParams p)
 {
     constexpr float L = float((1 << BITS) - 1);
     constexpr int SPAN = 32;                        // channels per thread
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(VAL_THREADS) quant_values_kernel(const ValPara
     const unsigned q = sp / LPG;                                                 // its group
     const long long in_off = (long long)b * p.sb + (long long)h * p.sh + (long long)tok * p.st + (long long)sp * SPAN;
     const long long out_tok = (long long)b * p.osb + (long long)h * p.osh + tok;
+    grid_wait(p.v);
 
     uint4 raw[NV];
     {
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(
     const unsigned bh = blockIdx.z * gridDim.y + blockIdx.y;
     const int slot = (int)threadIdx.x >> per_tok_shift, c8 = (int)threadIdx.x - (slot << per_tok_shift);
     const int t0 = ((int)chunk * slots + slot) * TOK;
+    grid_wait(codes, scales, zeros);
     if (slot < slots && t0 < T) {
         const long long in_tok0 = b * isb + h * ish;
         u64 sc2[CH / 2], zr2[CH / 2];
@@ -437,10 +439,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(
 template <int G, int BITS, bool BF16, bool M16>
 int launch_values_inst(const ValParams &p, long long rows, cudaStream_t st)
 {
-    quant_values_kernel<G, BITS, BF16, M16><<<dim3(p.chunks_per_row, (unsigned)p.H, (unsigned)(rows / p.H)), VAL_THREADS, 0, st>>>(p);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
+    return squat_launch(quant_values_kernel<G, BITS, BF16, M16>, dim3(p.chunks_per_row, (unsigned)p.H, (unsigned)(rows / p.H)), VAL_THREADS, 0, st, p);
 }
 
 template <int G, int BITS>
@@ -513,7 +512,7 @@ int squat_launch_dequant(int kind, const unsigned char *codes, const void *scale
     const long long chunks = tok8 ? chunks8 : (T + slots * 4 - 1) / (slots * 4);
     if (chunks > 0x7fffffffLL || H > 65535 || batch > 65535) return SQUAT_ERR_UNSUPPORTED;
     const dim3 grid((unsigned)chunks, (unsigned)H, (unsigned)batch);
-#define SQ_D1(BB, KK, OO, MM, TT) dequant_kernel<BB, KK, OO, MM, TT><<<grid, 256, 0, st>>>(codes, scales, zeros, per_tok_shift, T, d, g_shift, isb, ish, isb / G, ish / G, out)
+#define SQ_D1(BB, KK, OO, MM, TT) return squat_launch(dequant_kernel<BB, KK, OO, MM, TT>, grid, 256, 0, st, codes, scales, zeros, per_tok_shift, T, d, g_shift, isb, ish, isb / G, ish / G, out)
 #define SQ_D(BB, KK, OO) do { if (meta16) { if (tok8) SQ_D1(BB, KK, OO, true, 8); else SQ_D1(BB, KK, OO, true, 4); } \
                               else { if (tok8) SQ_D1(BB, KK, OO, false, 8); else SQ_D1(BB, KK, OO, false, 4); } } while (0)
     const bool keys = kind == SQUAT_KEYS, obf = out_dtype == SQUAT_BF16;
@@ -528,7 +527,4 @@ int squat_launch_dequant(int kind, const unsigned char *codes, const void *scale
     }
 #undef SQ_D1
 #undef SQ_D
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
 }
