@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libsquat.so: argument marshalling only.
+"""Thin binding of libsquat.so: argument marshalling only, through ctypes, and for the calls that a serving loop makes per
+window and token through a small extension module (csrc/pycall.c: 8.9 -> 6.4 us a call, most of it the launch).
 
 Every function has the name of the C entry point it calls (include/squat.h) and takes
 torch tensors where the C function takes device pointers.  Nothing here computes: all
@@ -30,6 +31,7 @@ EXPORTED_SYMBOLS = (
 )
 
 _lib = None
+_call = None
 
 
 class SquatError(RuntimeError):
@@ -93,8 +95,21 @@ def _load():
         lib.squat_status_string.argtypes = [i]
         lib.squat_status_string.restype = c.c_char_p
         lib.squat_last_cuda_error.restype = c.c_char_p
+        from . import _squatcall                     # built beside the library; the calls below go through it
+        _squatcall.bind(*(c.cast(f, vp).value for f in (lib.squat_quantize_keys, lib.squat_quantize_keys_m16, lib.squat_quantize_values,
+                                                        lib.squat_quantize_values_m16, lib.squat_dequantize, lib.squat_dequantize_m16,
+                                                        lib.squat_decode_attention_ex)))
+        global _call
+        _call = _squatcall
         _lib = lib
     return _lib
+
+
+def _direct():
+    """The extension module with the library's hot entry points (loads both on first use)."""
+    if _call is None:
+        _load()
+    return _call
 
 
 def _check(status, where):
@@ -127,6 +142,10 @@ def _dev(t: torch.Tensor, name: str):
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     return t.data_ptr()
+
+
+def _opt(t, name: str):
+    return _dev(t, name) if t is not None and t.numel() else None
 
 
 class Subspace:
@@ -217,24 +236,24 @@ def squat_quantize_keys(s: Subspace, k: torch.Tensor, bits: int, group_size: int
     out strides are in tokens; by default the outputs are dense [B,H,T,...]."""
     _check_bhtd(k, "k")
     B, H, T, d = k.shape
+    sb, sh, st, _ = k.stride()
     osh = T if out_stride_h is None else out_stride_h
     osb = H * osh if out_stride_b is None else out_stride_b
-    fn = _load().squat_quantize_keys_m16 if _meta16(scales, zeros) else _load().squat_quantize_keys
-    _check(fn(s.handle, _dev(k, "k"), _dtype_code(k), B, H, T, d, k.stride(0), k.stride(1),
-                                       k.stride(2), bits, group_size, _dev(codes, "codes"), _dev(scales, "scales"),
-                                       _dev(zeros, "zeros"), osb, osh, _stream(stream)), "squat_quantize_keys")
+    _check(_direct().quantize_keys(_meta16(scales, zeros), s.handle.value, _dev(k, "k"), _dtype_code(k), B, H, T, d, sb, sh, st, bits,
+                                   group_size, _dev(codes, "codes"), _dev(scales, "scales"), _dev(zeros, "zeros"), osb, osh,
+                                   _stream(stream)), "squat_quantize_keys")
 
 
 def squat_quantize_values(v: torch.Tensor, bits: int, group_size: int, codes: torch.Tensor, scales: torch.Tensor,
                           zeros: torch.Tensor, out_stride_b: int = None, out_stride_h: int = None, stream=None):
     _check_bhtd(v, "v")
     B, H, T, d = v.shape
+    sb, sh, st, _ = v.stride()
     osh = T if out_stride_h is None else out_stride_h
     osb = H * osh if out_stride_b is None else out_stride_b
-    fn = _load().squat_quantize_values_m16 if _meta16(scales, zeros) else _load().squat_quantize_values
-    _check(fn(_dev(v, "v"), _dtype_code(v), B, H, T, d, v.stride(0), v.stride(1),
-                                         v.stride(2), bits, group_size, _dev(codes, "codes"), _dev(scales, "scales"),
-                                         _dev(zeros, "zeros"), osb, osh, _stream(stream)), "squat_quantize_values")
+    _check(_direct().quantize_values(_meta16(scales, zeros), _dev(v, "v"), _dtype_code(v), B, H, T, d, sb, sh, st, bits, group_size,
+                                     _dev(codes, "codes"), _dev(scales, "scales"), _dev(zeros, "zeros"), osb, osh, _stream(stream)),
+           "squat_quantize_values")
 
 
 def squat_dequantize(kind: int, codes: torch.Tensor, scales: torch.Tensor, zeros: torch.Tensor, batch: int,
@@ -244,10 +263,9 @@ def squat_dequantize(kind: int, codes: torch.Tensor, scales: torch.Tensor, zeros
     isb = n_kv_heads * ish if in_stride_b is None else in_stride_b
     if not out.is_contiguous():
         raise ValueError("out must be contiguous")
-    fn = _load().squat_dequantize_m16 if _meta16(scales, zeros) else _load().squat_dequantize
-    _check(fn(kind, _dev(codes, "codes"), _dev(scales, "scales"), _dev(zeros, "zeros"), batch,
-                                    n_kv_heads, n_tokens, head_dim, bits, group_size, isb, ish, _dev(out, "out"),
-                                    _dtype_code(out), _stream(stream)), "squat_dequantize")
+    _check(_direct().dequantize(_meta16(scales, zeros), kind, _dev(codes, "codes"), _dev(scales, "scales"), _dev(zeros, "zeros"), batch,
+                                n_kv_heads, n_tokens, head_dim, bits, group_size, isb, ish, _dev(out, "out"), _dtype_code(out),
+                                _stream(stream)), "squat_dequantize")
 
 
 def squat_write_path_workspace_bytes(dtype: torch.dtype, batch, n_q_heads, n_kv_heads, n_tokens, head_dim, bits,
@@ -467,26 +485,15 @@ def squat_decode_attention(q: torch.Tensor, k_codes, k_scales, k_zeros, v_codes,
     n_res = 0 if k_res is None else k_res.shape[2]
     if n_res and (not k_res.is_contiguous() or not v_res.is_contiguous() or k_res.dtype != v_res.dtype):
         raise ValueError("k_res and v_res must be contiguous [batch, n_kv_heads, n_res, d] of one dtype")
-    opt = lambda t, n: _dev(t, n) if t is not None and t.numel() else None
-    if k_scales is not None and k_scales.dtype == torch.float16:         # a cache with 16-bit scales and zero-points
-        for t in (k_zeros, v_scales, v_zeros):
-            if t.dtype != torch.float16:
-                raise ValueError("scales and zero-points must all be float16 or all float32")
-        _check(_load().squat_decode_attention_ex(
-            _dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, opt(k_codes, "k_codes"), opt(k_scales, "k_scales"),
-            opt(k_zeros, "k_zeros"), opt(v_codes, "v_codes"), opt(v_scales, "v_scales"), opt(v_zeros, "v_zeros"), 1, n_tokens,
-            csb, csh, bits, group_size, opt(k_res, "k_res"), opt(v_res, "v_res"), _dtype_code(k_res) if n_res else SQUAT_F32,
-            n_res, float(softmax_scale), None, 0, 0, _dev(out, "out"), _dev(workspace, "workspace"),
-            workspace.numel() * workspace.element_size(), _stream(stream)), "squat_decode_attention_ex")
-        return
-    _check(_load().squat_decode_attention(_dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, opt(k_codes, "k_codes"),
-                                          opt(k_scales, "k_scales"), opt(k_zeros, "k_zeros"), opt(v_codes, "v_codes"),
-                                          opt(v_scales, "v_scales"), opt(v_zeros, "v_zeros"), n_tokens, csb, csh, bits,
-                                          group_size, opt(k_res, "k_res"), opt(v_res, "v_res"),
-                                          _dtype_code(k_res) if n_res else SQUAT_F32, n_res, float(softmax_scale),
-                                          _dev(out, "out"), _dev(workspace, "workspace"),
-                                          workspace.numel() * workspace.element_size(), _stream(stream)),
-           "squat_decode_attention")
+    meta16 = k_scales is not None and k_scales.dtype == torch.float16         # a cache with 16-bit scales and zero-points
+    if meta16 and not (k_zeros.dtype == v_scales.dtype == v_zeros.dtype == torch.float16):
+        raise ValueError("scales and zero-points must all be float16 or all float32")
+    _check(_direct().decode_attention(
+        softmax_scale, _dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, _opt(k_codes, "k_codes"), _opt(k_scales, "k_scales"),
+        _opt(k_zeros, "k_zeros"), _opt(v_codes, "v_codes"), _opt(v_scales, "v_scales"), _opt(v_zeros, "v_zeros"), meta16, n_tokens,
+        csb, csh, bits, group_size, _opt(k_res, "k_res"), _opt(v_res, "v_res"), _dtype_code(k_res) if n_res else SQUAT_F32,
+        n_res, None, 0, 0, _dev(out, "out"), _dev(workspace, "workspace"),
+        workspace.numel() * workspace.element_size(), _stream(stream)), "squat_decode_attention")
 
 
 def squat_rope_table(n_positions: int, base: float = 10000.0, head_dim: int = 128) -> torch.Tensor:
@@ -520,23 +527,13 @@ def squat_decode_attention_pre_rope(q: torch.Tensor, k_codes, k_scales, k_zeros,
     n_res = 0 if k_res is None else k_res.shape[2]
     if n_res and (not k_res.is_contiguous() or not v_res.is_contiguous() or k_res.dtype != v_res.dtype):
         raise ValueError("k_res and v_res must be contiguous [batch, n_kv_heads, n_res, d] of one dtype")
-    opt = lambda t, n: _dev(t, n) if t is not None and t.numel() else None
-    if k_scales is not None and k_scales.dtype == torch.float16:         # a cache with 16-bit scales and zero-points
-        _check(_load().squat_decode_attention_ex(
-            _dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, opt(k_codes, "k_codes"), opt(k_scales, "k_scales"),
-            opt(k_zeros, "k_zeros"), opt(v_codes, "v_codes"), opt(v_scales, "v_scales"), opt(v_zeros, "v_zeros"), 1, n_tokens,
-            csb, csh, bits, group_size, opt(k_res, "k_res"), opt(v_res, "v_res"), _dtype_code(k_res) if n_res else SQUAT_F32,
-            n_res, float(softmax_scale), _dev(rope_table, "rope_table"), int(table_positions), int(first_pos),
-            _dev(out, "out"), _dev(workspace, "workspace"), workspace.numel() * workspace.element_size(), _stream(stream)),
-            "squat_decode_attention_ex")
-        return
-    _check(_load().squat_decode_attention_pre_rope(
-        _dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, opt(k_codes, "k_codes"), opt(k_scales, "k_scales"),
-        opt(k_zeros, "k_zeros"), opt(v_codes, "v_codes"), opt(v_scales, "v_scales"), opt(v_zeros, "v_zeros"), n_tokens,
-        ctypes.c_longlong(csb), ctypes.c_longlong(csh), bits, group_size, opt(k_res, "k_res"), opt(v_res, "v_res"),
-        _dtype_code(k_res) if n_res else SQUAT_F32, n_res, ctypes.c_float(softmax_scale), _dev(rope_table, "rope_table"),
-        int(table_positions), ctypes.c_longlong(first_pos), _dev(out, "out"), _dev(workspace, "workspace"),
-        ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)), "squat_decode_attention_pre_rope")
+    meta16 = k_scales is not None and k_scales.dtype == torch.float16         # a cache with 16-bit scales and zero-points
+    _check(_direct().decode_attention(
+        softmax_scale, _dev(q, "q"), _dtype_code(q), B, Hq, n_kv_heads, d, _opt(k_codes, "k_codes"), _opt(k_scales, "k_scales"),
+        _opt(k_zeros, "k_zeros"), _opt(v_codes, "v_codes"), _opt(v_scales, "v_scales"), _opt(v_zeros, "v_zeros"), meta16, n_tokens,
+        csb, csh, bits, group_size, _opt(k_res, "k_res"), _opt(v_res, "v_res"), _dtype_code(k_res) if n_res else SQUAT_F32,
+        n_res, _dev(rope_table, "rope_table"), int(table_positions), int(first_pos), _dev(out, "out"), _dev(workspace, "workspace"),
+        workspace.numel() * workspace.element_size(), _stream(stream)), "squat_decode_attention_pre_rope")
 
 
 def squat_get_device_status(clear: bool = True, stream=None) -> int:

@@ -6,6 +6,7 @@ buffer or on-chip region it belongs to and report through SQUAT_FLAG_BOUNDS inst
 environment variable SQUAT_LIBRARY=<path> before the package is first used."""
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -48,10 +49,19 @@ def _compile(src, verbose, obj_dir=OBJ_DIR, extra=()):
     return obj
 
 
+def build_pycall(force: bool = False) -> str:
+    """The extension module through which the binding makes its per-token and per-window calls (gcc, the CPython C API)."""
+    src, out = os.path.join(CSRC, "pycall.c"), os.path.join(_HERE, "_squatcall.so")
+    if force or not os.path.exists(out) or os.path.getmtime(out) < max(os.path.getmtime(src), os.path.getmtime(os.path.join(INCLUDE, "squat.h"))):
+        subprocess.run(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", out], check=True)
+    return out
+
+
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> str:
     obj_dir, lib = (OBJ_DIR_CHECKED, LIB_CHECKED) if checked else (OBJ_DIR, LIB)
     extra = ("-DSQUAT_CHECKED",) if checked else ()
     os.makedirs(obj_dir, exist_ok=True)
+    build_pycall(force)
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= _deps_mtime():
         return lib
     if force:
