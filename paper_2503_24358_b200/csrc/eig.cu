@@ -6,7 +6,7 @@
 //
 // Both are bound by latency: the first by 126 dependent steps (a column norm, a matrix-vector product and two barriers
 // each), the second by six dependent merges (a few secular-equation iterations each).  The flops of neither would fill a
-// tenth of the time.  Measured on the 32 heads of a 4096-token prompt: 98 + 83 us.  What was here before, one-sided Jacobi
+// tenth of the time.  Measured on the 32 heads of a 4096-token prompt: 97 + 72 us.  What was here before, one-sided Jacobi
 // on a Cholesky factor, needed 10 sweeps of 127 dependent rounds: 677 us.
 #include <cooperative_groups.h>
 #include <type_traits>
