@@ -7,14 +7,18 @@
 // holds exactly for every element down to 2^-21 of the channel's largest, and M is a sum of ten integer products of digit
 // planes, D_a^T D_b for a <= b (the ones with a > b are their transposes), accumulated in 32 bits in tensor memory without
 // any rounding.  Elements below that (about one in a million of normally distributed ones) leave a remainder r; they are
-// listed, and the reduction adds r x_i to row and column c in fp64.  A head whose list overflows, or that holds a non-finite
-// number, is summed by plain fp64 loops instead.  The only roundings are those of the fp64 sums of the parts.
+// listed, and the reduction adds r x_i to row and column c in fp64.  A head whose list overflows (one token 40 times the rest is
+// enough), or that holds a non-finite number, is left to the fp64 kernel of subspace.cu, which is launched in any case and
+// returns at once for every other head.  A whole build of 8 heads x 32768 rows takes 318 us, with one token 1000 times the rest
+// 495 us (378 in float32; with plain loops in the reduction instead of that kernel 7700).  The only roundings are those of the
+// fp64 sums of the parts.
 //
 //   gram_max_kernel     largest |x| per channel and chunk of rows
 //   gram_i8_kernel      one of three kinds of digit products (A = plane 0 with B = planes 0-3; 1 with 1-3; 2 with 2-3 and 3
 //                       with 3: 4 + 3 + 3 products, all that the 512 tensor-memory columns hold at a time) on a chunk of
 //                       rows.  Warps 0-15 turn rows into digit planes ([row][128 bytes], 128-byte swizzle, which the
 //                       descriptors read as M-major A and N-major B), warp 16 issues the products; four stages of 64 rows.
+//   (gram_kernel)       heads without the digits' help
 //   gram_i8_reduce_kernel   M = sum of the parts S + S^T, remainders
 //
 // Bound: the instructions that make the digits (100 per eight elements and kind, 16 warps: 0.85 us for 64 rows; the products
@@ -35,6 +39,7 @@ struct GramArgs {
     long long stride_h, stride_t;
     int n_rows;                                // n_tokens * q_per_kv
     int parts[3], total_parts;                 // row chunks per kind of product
+    int fp64_parts;                            // row chunks of the fp64 kernel, for the heads that it takes
     int max_chunks;                            // row chunks of the maximum kernel
     unsigned *maxima;                          // [H, max_chunks, D / 2] largest |x| bits, two channels a word
     int *rem_count;                            // [H] remainders listed (may exceed the capacity)
@@ -186,21 +191,25 @@ __device__ __forceinline__ void store_planes(unsigned char *dst, const u64 (&b)[
     *reinterpret_cast<uint2 *>(dst + PLANE) = make_uint2(__byte_perm(w[0], w[1], 0x5410) ^ 0x80808080u, __byte_perm(w[2], w[3], 0x5410) ^ 0x80808080u);
 }
 
-// what the digits of eight channels of a row leave over, for the reduction (rare)
-__device__ __noinline__ void list_remainders(SquatGramRem *rem, int *rem_count, int row, int c16, uint4 raw, const double *unit)
+// what the digits of eight channels of a row leave over, for the reduction (rare; with a full list nothing more is listed)
+__device__ __noinline__ void list_remainders(SquatGramRem *rem, int *rem_count, int row, int c16, uint4 raw, const double *unit, volatile unsigned *list_full)
 {
     const unsigned w[4] = {raw.x, raw.y, raw.z, raw.w};
     for (int e = 0; e < 8; ++e) {
         const int c = 8 * c16 + e;
-        const double x = (double)((e & 1) ? bf16hi_to_f32(w[e >> 1]) : bf16lo_to_f32(w[e >> 1])) / unit[c];
+        const double u = unit[c], per_unit = __longlong_as_double((2046ll << 52) - __double_as_longlong(u));      // 1 / u: a power of two
+        const double x = (double)((e & 1) ? bf16hi_to_f32(w[e >> 1]) : bf16lo_to_f32(w[e >> 1])) * per_unit;
         const double r = x * 32768.0 - rint(x * 32768.0);             // the digits hold the nearest multiple of 2^-15 units
         if (r == 0.0) continue;
         const int at = atomicAdd(rem_count, 1);
-        if (at >= SQUAT_GRAM_REM_CAP) continue;
+        if (at >= SQUAT_GRAM_REM_CAP) {
+            *list_full = 1;
+            return;
+        }
         SquatGramRem &o = rem[at];
         o.row = row;
         o.channel = c;
-        o.r = r * (1.0 / 32768.0) * unit[c];
+        o.r = r * (1.0 / 32768.0) * u;
     }
 }
 
@@ -211,6 +220,7 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
     __shared__ __align__(8) u64 full[STAGES], empty[STAGES];
     __shared__ double unit[D];                 // 2^(exponent) of a channel's digit unit
     __shared__ unsigned tmem_sm, timeout;
+    __shared__ volatile unsigned list_full;    // the head's list has overflowed: its remainders need not be listed any more
     const int h = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int part = blockIdx.y, kind = part < p.parts[0] ? 0 : part < p.parts[0] + p.parts[1] ? 1 : 2;
     const int chunk = part - (kind > 0 ? p.parts[0] : 0) - (kind > 1 ? p.parts[1] : 0);
@@ -222,7 +232,7 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        timeout = 0;
+        timeout = list_full = 0;
         for (int i = 0; i < STAGES; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[i])), "r"(CONV_WARPS) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[i])) : "memory");
@@ -231,7 +241,7 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
     }
     if (tid < D) {
         const int be = channel_exponent(p, h, tid);
-        if (be == 255 && kind == 0 && chunk == 0) atomicAdd(&p.rem_count[h], SQUAT_GRAM_REM_CAP + 1);   // not finite: plain loops
+        if (be == 255 && kind == 0 && chunk == 0) atomicAdd(&p.rem_count[h], SQUAT_GRAM_REM_CAP + 1);   // not finite
         unit[tid] = __longlong_as_double((long long)(max(min(be, 254), 13) - 140 + 1023) << 52);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -299,7 +309,8 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
                         unsigned char *dst = st + r * D + (((c16 >> 1) ^ (r & 7)) << 4);
                         if (kind < 2) store_planes<kind == 0>(dst, hb);
                         store_planes<true>(dst + 2 * PLANE, lb);
-                        if (kind == 0 && (any & 0x7fffffffu)) list_remainders(p.rem + (long long)h * SQUAT_GRAM_REM_CAP, p.rem_count + h, lo + s * ROWS + r, c16, raw[u][i], unit);
+                        if (kind == 0 && (any & 0x7fffffffu) && !list_full)
+                            list_remainders(p.rem + (long long)h * SQUAT_GRAM_REM_CAP, p.rem_count + h, lo + s * ROWS + r, c16, raw[u][i], unit, &list_full);
                     }
                     fetch(raw[u]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -380,47 +391,51 @@ constexpr int RED_UNITS = 136 * 16, RED_THREADS = 128;    // tiles on or above t
 
 __global__ void __launch_bounds__(RED_THREADS) gram_i8_reduce_kernel(const GramArgs p)
 {
-    const int h = blockIdx.y, H = gridDim.y, unit_id = blockIdx.x * RED_THREADS + threadIdx.x;
+    __shared__ long long key_sm[SQUAT_GRAM_REM_CAP], sorted_sm[SQUAT_GRAM_REM_CAP];
+    __shared__ double r_sm[SQUAT_GRAM_REM_CAP];
+    const int h = blockIdx.y, H = gridDim.y, tid = threadIdx.x, unit_id = blockIdx.x * RED_THREADS + tid;
+    grid_wait();
     int u = unit_id >> 4, ti = 0, len = 16;    // u-th tile of the upper triangle, row by row
     while (u >= len) { u -= len; --len; ++ti; }
     const int tj = ti + u, a = 8 * ti + ((unit_id >> 1) & 7), b = 8 * tj + 4 * (unit_id & 1);
     double m[4] = {0.0, 0.0, 0.0, 0.0};
-    const int n_rem = p.rem_count[h];
-    if (n_rem <= SQUAT_GRAM_REM_CAP) {
-        const double *src = p.partial + (long long)h * D * D;
+    const bool digits = p.rem_count[h] <= SQUAT_GRAM_REM_CAP;             // or the fp64 kernel's parts, tiles of the upper triangle
+    const int n_rem = digits ? p.rem_count[h] : 0, n_parts = digits ? p.total_parts : p.fp64_parts;
+    const double *src = p.partial + (long long)h * D * D;
 #pragma unroll 4
-        for (int c = 0; c < p.total_parts; ++c, src += (long long)H * D * D) {
-            const double2 x = *reinterpret_cast<const double2 *>(src + a * D + b), y = *reinterpret_cast<const double2 *>(src + a * D + b + 2);
-            m[0] += x.x + src[b * D + a];
-            m[1] += x.y + src[(b + 1) * D + a];
-            m[2] += y.x + src[(b + 2) * D + a];
-            m[3] += y.y + src[(b + 3) * D + a];
-        }
-        // remainders, in the order of (row, channel) whatever order they were listed in
-        const SquatGramRem *rem = p.rem + (long long)h * SQUAT_GRAM_REM_CAP;
-        long long done = -1;
-        for (int k = 0; k < n_rem; ++k) {
-            long long best = 0x7fffffffffffffffLL;
-            double r = 0.0;
-            for (int z = 0; z < n_rem; ++z) {
-                const long long key = (long long)rem[z].row * D + rem[z].channel;
-                if (key > done && key < best) { best = key; r = rem[z].r; }
-            }
-            done = best;
-            const int c = (int)(best % D);
-            const __nv_bfloat16 *row = row_ptr(p, h, (int)(best / D));
+    for (int c = 0; c < n_parts; ++c, src += (long long)H * D * D) {
+        const double2 x = *reinterpret_cast<const double2 *>(src + a * D + b), y = *reinterpret_cast<const double2 *>(src + a * D + b + 2);
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        if (digits) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (c == a) m[e] = fma(r, (double)__bfloat162float(row[b + e]), m[e]);
-                if (c == b + e) m[e] = fma(r, (double)__bfloat162float(row[a]), m[e]);
-            }
+            for (int e = 0; e < 4; ++e) t[e] = src[(b + e) * D + a];
         }
-    } else {
-        for (int n = 0; n < p.n_rows; ++n) {
-            const __nv_bfloat16 *row = row_ptr(p, h, n);
-            const double x = (double)__bfloat162float(row[a]);
+        m[0] += x.x + t[0];
+        m[1] += x.y + t[1];
+        m[2] += y.x + t[2];
+        m[3] += y.y + t[3];
+    }
+    // remainders, in the order of (row, channel) whatever order they were listed in
+    const SquatGramRem *rem = p.rem + (long long)h * SQUAT_GRAM_REM_CAP;
+    for (int k = tid; k < n_rem; k += RED_THREADS) key_sm[k] = (long long)rem[k].row * D + rem[k].channel;
+    __syncthreads();
+    for (int k = tid; k < n_rem; k += RED_THREADS) {
+        const long long key = key_sm[k];
+        int place = 0;
+        for (int z = 0; z < n_rem; ++z) place += key_sm[z] < key;            // an element is listed once: all keys differ
+        sorted_sm[place] = key;
+        r_sm[place] = rem[k].r;
+    }
+    __syncthreads();
+    for (int k = 0; k < n_rem; ++k) {
+        const int c = (int)(sorted_sm[k] % D);
+        if (c != a && (unsigned)(c - b) >= 4u) continue;
+        const double r = r_sm[k];
+        const __nv_bfloat16 *row = row_ptr(p, h, (int)(sorted_sm[k] / D));
 #pragma unroll
-            for (int e = 0; e < 4; ++e) m[e] = fma(x, (double)__bfloat162float(row[b + e]), m[e]);
+        for (int e = 0; e < 4; ++e) {
+            if (c == a) m[e] = fma(r, (double)__bfloat162float(row[b + e]), m[e]);
+            if (c == b + e) m[e] = fma(r, (double)__bfloat162float(row[a]), m[e]);
         }
     }
     double *g = p.gram + (long long)h * D * D;
@@ -483,8 +498,6 @@ int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_
     gram_i8_kernel<<<dim3(H, p.total_parts), THREADS, SMEM, st>>>(p);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
-    gram_i8_reduce_kernel<<<dim3(RED_UNITS / RED_THREADS, H), RED_THREADS, 0, st>>>(p);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
-    return SQUAT_OK;
+    if (const int rc = squat_launch_gram_parts(q, SQUAT_BF16, H, p.n_tokens, p.q_per_kv, stride_h, stride_t, s->gram_chunks_cap, s->gram_rem_count, s->gram_partial, &p.fp64_parts, st)) return rc;
+    return squat_launch(gram_i8_reduce_kernel, dim3(RED_UNITS / RED_THREADS, H), RED_THREADS, 0, st, p);
 }

@@ -59,9 +59,11 @@ int squat_allow_smem(const void *kernel, size_t bytes, std::atomic<unsigned long
 
 // Launches a kernel as a programmatic dependent of the one before it on the stream: its blocks are put in place while that
 // one's last blocks run and wait in grid_wait(), which takes about 1.5 us of launch gap out of every hand-over.  The quantizers,
-// the dequantizer and the readers are launched this way (a window's pair 20.5 -> 16.7 us); for the kernels of step 1 it gained
-// nothing, or lost, and so it did for grids of hundreds of blocks per SM, whose launch is a small part.  Every kernel launched this way calls grid_wait() before it touches global or tensor memory (a block that held tensor memory while it
-// waited could keep the kernel before it from getting its own).
+// the dequantizer and the readers are launched this way (a window's pair 20.5 -> 16.7 us); for the long kernels of step 1 it
+// gained nothing, or lost, and so it did for grids of hundreds of blocks per SM, whose launch is a small part; the two short ones
+// behind the integer Gram kernel use it (5 to 6 us together).  Every kernel launched this way calls grid_wait() before it
+// touches global or tensor memory (a block that held tensor memory while it waited could keep the kernel before it from
+// getting its own).
 template <class... Params, class... Args>
 int squat_launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
 {
@@ -92,6 +94,9 @@ __device__ __forceinline__ void grid_wait(Pointers &...pointers)
 // ---- kernel launchers (one per .cu) ---------------------------------------------------
 int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
                       long long stride_h, long long stride_t, cudaStream_t st);
+// Partial sums of the fp64 kernel, [*chunks <= chunks_cap, H, D, D]; with list_counts only of the heads whose list is overfull.
+int squat_launch_gram_parts(const void *q, int dtype, int H, int n_tokens, int q_per_kv, long long stride_h, long long stride_t,
+                            int chunks_cap, const int *list_counts, double *partial, int *chunks, cudaStream_t st);
 int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st);
 bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens);
 int squat_launch_eig(squat_subspace *s, cudaStream_t st);

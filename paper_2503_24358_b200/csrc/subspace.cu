@@ -86,11 +86,15 @@ __device__ __forceinline__ void gram_warp_body(const double *rows, double (&acc)
 
 template <bool BF16>
 __global__ void __launch_bounds__(GRAM_THREADS, GRAM_CTAS_PER_SM) gram_kernel(
-    const void *__restrict__ q, int n_tokens, int q_per_kv, long long stride_h, long long stride_t,
-    int rows_per_chunk, double *__restrict__ partial /* [chunks, H, D, D] */)
+    const void *q, int n_tokens, int q_per_kv, long long stride_h, long long stride_t,
+    int rows_per_chunk, const int *list_counts, double *__restrict__ partial /* [chunks, H, D, D] */)
 {
     __shared__ __align__(16) double rows[GRAM_ROWS * GRAM_LDR];
     const int h = blockIdx.y, chunk = blockIdx.x, H = gridDim.y;
+    if (list_counts) {
+        grid_wait(q);
+        if (list_counts[h] <= SQUAT_GRAM_REM_CAP) return;                 // gram_i8.cu has this head's sums
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long N = (long long)n_tokens * q_per_kv;
     const long long row_lo = (long long)chunk * rows_per_chunk;
@@ -415,25 +419,33 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
 
 }  // namespace
 
+int squat_launch_gram_parts(const void *q, int dtype, int H, int n_tokens, int q_per_kv, long long stride_h, long long stride_t,
+                            int chunks_cap, const int *list_counts, double *partial, int *chunks, cudaStream_t st)
+{
+    const long long N = (long long)n_tokens * q_per_kv;
+    long long rows_per_chunk = (N + chunks_cap - 1) / chunks_cap;
+    rows_per_chunk = (rows_per_chunk + GRAM_ROWS - 1) / GRAM_ROWS * GRAM_ROWS;
+    if (rows_per_chunk < 2 * GRAM_ROWS) rows_per_chunk = 2 * GRAM_ROWS;
+    *chunks = (int)((N + rows_per_chunk - 1) / rows_per_chunk);
+    if (*chunks < 1) *chunks = 1;
+    const dim3 grid(*chunks, H);
+    if (list_counts) return squat_launch(gram_kernel<true>, grid, GRAM_THREADS, 0, st, q, n_tokens, q_per_kv, stride_h, stride_t, (int)rows_per_chunk, list_counts, partial);
+    if (dtype == SQUAT_BF16)
+        gram_kernel<true><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, q_per_kv, stride_h, stride_t, (int)rows_per_chunk, list_counts, partial);
+    else
+        gram_kernel<false><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, q_per_kv, stride_h, stride_t, (int)rows_per_chunk, list_counts, partial);
+    squat_count_launch();
+    SQUAT_LAUNCH_CHECK();
+    return SQUAT_OK;
+}
+
 int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
                       long long stride_h, long long stride_t, cudaStream_t st)
 {
     if (squat_gram_i8_fits(s, dtype, n_q_heads, n_tokens)) return squat_launch_gram_i8(s, q, n_q_heads, n_tokens, stride_h, stride_t, st);
-    const int H = s->n_kv_heads, qpk = n_q_heads / H;
-    const long long N = (long long)n_tokens * qpk;
-    int chunks = s->gram_chunks_cap;
-    long long rows_per_chunk = (N + chunks - 1) / chunks;
-    rows_per_chunk = (rows_per_chunk + GRAM_ROWS - 1) / GRAM_ROWS * GRAM_ROWS;
-    if (rows_per_chunk < 2 * GRAM_ROWS) rows_per_chunk = 2 * GRAM_ROWS;
-    chunks = (int)((N + rows_per_chunk - 1) / rows_per_chunk);
-    if (chunks < 1) chunks = 1;
-    dim3 grid(chunks, H);
-    if (dtype == SQUAT_BF16)
-        gram_kernel<true><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, qpk, stride_h, stride_t, (int)rows_per_chunk, s->gram_partial);
-    else
-        gram_kernel<false><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, qpk, stride_h, stride_t, (int)rows_per_chunk, s->gram_partial);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
+    const int H = s->n_kv_heads;
+    int chunks = 0;
+    if (const int rc = squat_launch_gram_parts(q, dtype, H, n_tokens, n_q_heads / H, stride_h, stride_t, s->gram_chunks_cap, nullptr, s->gram_partial, &chunks, st)) return rc;
     gram_reduce_kernel<<<dim3(GRED_UNITS / GRED_THREADS, H), GRED_THREADS, 0, st>>>(s->gram_partial, chunks, H, s->gram);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
@@ -487,23 +499,11 @@ extern "C" int squat_gram_static(const void *q, int dtype, int n_q_heads, int n_
     double *partial = g_gram_static_ptr[dev];
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int H = n_kv_heads, qpk = n_q_heads / H;
-    const long long N = (long long)n_tokens * qpk;
-    int chunks = GRAM_STATIC_MAX_UNITS / H;                                   // >= 1
-    long long rows_per_chunk = (N + chunks - 1) / chunks;
-    rows_per_chunk = (rows_per_chunk + GRAM_ROWS - 1) / GRAM_ROWS * GRAM_ROWS;
-    if (rows_per_chunk < 2 * GRAM_ROWS) rows_per_chunk = 2 * GRAM_ROWS;
-    chunks = (int)((N + rows_per_chunk - 1) / rows_per_chunk);
-    if (chunks < 1) chunks = 1;
+    const int H = n_kv_heads;
     // every element the reduction reads is written by this call's first kernel, so nothing left in the
     // array by an earlier call is ever seen and nothing needs clearing
-    dim3 grid(chunks, H);
-    if (dtype == SQUAT_BF16)
-        gram_kernel<true><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, qpk, stride_h, stride_t, (int)rows_per_chunk, partial);
-    else
-        gram_kernel<false><<<grid, GRAM_THREADS, 0, st>>>(q, n_tokens, qpk, stride_h, stride_t, (int)rows_per_chunk, partial);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
+    int chunks = 0;
+    if (const int rc = squat_launch_gram_parts(q, dtype, H, n_tokens, n_q_heads / H, stride_h, stride_t, GRAM_STATIC_MAX_UNITS / H, nullptr, partial, &chunks, st)) return rc;
     gram_reduce_kernel<<<dim3(GRED_UNITS / GRED_THREADS, H), GRED_THREADS, 0, st>>>(partial, chunks, H, gram_out);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();

@@ -10,9 +10,19 @@ pytestmark = pytest.mark.gpu
 D = 128
 
 
+def _tiny(q, H, n, g):
+    """n elements of each KV head's queries far below their channel's largest (none of the others is); 1.5 and 1.25 alternate"""
+    q.copy_(q.sign() * q.abs().clamp(0.01, 4.0))
+    rows = q.view(H, -1, D)
+    for h in range(H):
+        at = torch.randperm(rows[h].numel(), generator=g)[:n]
+        rows[h].view(-1)[at] = 2.0 ** -26 * (1.25 + 0.25 * (torch.arange(n) % 2))
+
+
 @pytest.mark.parametrize("H,qpk,T,data", [
     (32, 1, 1024, "normal"), (8, 4, 300, "normal"), (1, 1, 4097, "normal"), (2, 2, 2049, "zeros"), (40, 1, 1100, "normal"),
-    (8, 1, 1500, "outliers"), (2, 1, 1024, "wide"), (4, 2, 5000, "normal")])
+    (8, 1, 1500, "outliers"), (2, 1, 1024, "wide"), (4, 2, 5000, "normal"), (2, 1, 1024, "listed"), (3, 2, 1000, "full list"),
+    (3, 2, 1000, "one head"), (1, 4, 1031, "wide")])
 def test_gram_is_exact(H, qpk, T, data):
     g = torch.Generator().manual_seed(7)
     q = torch.randn((H * qpk, T, D), generator=g)
@@ -25,6 +35,10 @@ def test_gram_is_exact(H, qpk, T, data):
         q[:, 17, :4] = 1e-6
     elif data == "wide":                                 # every exponent of a wide range: the list of remainders overflows
         q *= torch.exp2(torch.randint(-40, 8, q.shape, generator=g).float())
+    elif data in ("listed", "full list"):                # many remainders, then exactly as many as the list holds
+        _tiny(q, H, 200 if data == "listed" else 256, g)
+    elif data == "one head":                             # one more than it holds, in one head
+        _tiny(q[2:4], 1, 257, g)
     q = q.to(torch.bfloat16)
     s = sq.Subspace(H, D)
     sq.squat_build_subspace(s, q.cuda(), 8, 1e-3)
@@ -38,4 +52,35 @@ def test_gram_is_exact(H, qpk, T, data):
         err = np.abs((a[h] - ref).astype(np.float64))
         assert np.all(err <= 4e-15 * size + 0.0), (err / np.maximum(size, 1e-300)).max()
     assert sq.squat_get_device_status(clear=True) & ~sq.FLAG_ZERO_RANGE == 0
+    s.close()
+
+
+def _us(s, q, passes=5):
+    """Median time of a build from q, GPU events."""
+    ev = [[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(passes)]
+    for a, b in [ev[0]] + ev:
+        a.record()
+        sq.squat_build_subspace(s, q, 32, 1e-3)
+        b.record()
+    torch.cuda.synchronize()
+    return 1e3 * sorted(a.elapsed_time(b) for a, b in ev)[passes // 2]
+
+
+@pytest.mark.parametrize("H,T,data", [(8, 32768, "one token"), (32, 16384, "one token"), (8, 32768, "listed"), (32, 16384, "one head")])
+def test_time_does_not_hang_on_the_data(H, T, data):
+    # The digits can be no help with such queries: a build may then cost the integer kernel's pass and the fp64 kernel's, which
+    # is what the same queries in float32 take, and no more (half as much again for clocks and noise).
+    g = torch.Generator().manual_seed(3)
+    q = torch.randn((H, T, D), generator=g)
+    s = sq.Subspace(H, D)
+    usual, fp64 = _us(s, q.to(torch.bfloat16).cuda()), _us(s, q.cuda())
+    if data == "one token":
+        q[:, T // 3] *= 1000.0
+    elif data == "one head":
+        q[0, T // 3] *= 1000.0
+    else:
+        _tiny(q, H, 250, g)
+    took = _us(s, q.to(torch.bfloat16).cuda())
+    print(f"usual {usual:.0f} us, float32 {fp64:.0f} us, these {took:.0f} us")
+    assert took <= 1.5 * (usual + fp64)
     s.close()
