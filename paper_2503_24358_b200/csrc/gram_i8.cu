@@ -463,12 +463,15 @@ bool plan(const squat_subspace *s, int n_rows, int (&parts)[3])
 }  // namespace
 
 // bf16 queries and at least three CTAs per head; below 1024 rows the fp64 kernel's fewer launches win.  The loads step 32 tokens
-// at a time and cross one query head at most.
-bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens)
+// at a time and cross one query head at most.  Their offsets, in 16-byte units from a KV head's first row, are 32-bit and run on
+// for up to 320 rows (that are not loaded) behind the last one, so views that spread a KV head over 32 GB go to the fp64 kernel.
+bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens, long long stride_h, long long stride_t)
 {
     int parts[3];
-    const long long rows = (long long)n_tokens * (n_q_heads / s->n_kv_heads);
-    return dtype == SQUAT_BF16 && n_tokens >= 32 && rows >= 1024 && rows < (1 << 30) && plan(s, (int)rows, parts);
+    const int q_per_kv = n_q_heads / s->n_kv_heads;
+    const long long rows = (long long)n_tokens * q_per_kv;
+    const double reach = ((double)(q_per_kv + 11) * stride_h + (double)(n_tokens + 320) * stride_t) / 8;
+    return dtype == SQUAT_BF16 && n_tokens >= 32 && rows >= 1024 && rows < (1 << 30) && reach < 2147483648.0 && plan(s, (int)rows, parts);
 }
 
 int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st)

@@ -98,7 +98,7 @@ int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads
 int squat_launch_gram_parts(const void *q, int dtype, int H, int n_tokens, int q_per_kv, long long stride_h, long long stride_t,
                             int chunks_cap, const int *list_counts, double *partial, int *chunks, cudaStream_t st);
 int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st);
-bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens);
+bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens, long long stride_h, long long stride_t);
 int squat_launch_eig(squat_subspace *s, cudaStream_t st);
 int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_blocks, cudaStream_t st);
 int squat_launch_power(squat_subspace *s, const double *start, long long start_stride_h, int rank_r, int iters,

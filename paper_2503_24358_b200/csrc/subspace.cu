@@ -442,7 +442,7 @@ int squat_launch_gram_parts(const void *q, int dtype, int H, int n_tokens, int q
 int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
                       long long stride_h, long long stride_t, cudaStream_t st)
 {
-    if (squat_gram_i8_fits(s, dtype, n_q_heads, n_tokens)) return squat_launch_gram_i8(s, q, n_q_heads, n_tokens, stride_h, stride_t, st);
+    if (squat_gram_i8_fits(s, dtype, n_q_heads, n_tokens, stride_h, stride_t)) return squat_launch_gram_i8(s, q, n_q_heads, n_tokens, stride_h, stride_t, st);
     const int H = s->n_kv_heads;
     int chunks = 0;
     if (const int rc = squat_launch_gram_parts(q, dtype, H, n_tokens, n_q_heads / H, stride_h, stride_t, s->gram_chunks_cap, nullptr, s->gram_partial, &chunks, st)) return rc;

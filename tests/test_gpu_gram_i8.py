@@ -55,6 +55,28 @@ def test_gram_is_exact(H, qpk, T, data):
     s.close()
 
 
+@pytest.mark.parametrize("H,qpk,T,stride_h,stride_t", [
+    (1, 1, 1100, 0, 1 << 24), (1, 2, 600, 600 << 24, 1 << 24), (1, 3, 400, 1 << 33, 128), (2, 1, 1100, 1 << 33, 128)])
+def test_views_spread_over_more_than_32_gigabytes(H, qpk, T, stride_h, stride_t):
+    size = (H * qpk - 1) * stride_h + (T - 1) * stride_t + D
+    if torch.cuda.mem_get_info()[0] < 2 * size + (4 << 30):
+        pytest.skip("not enough free device memory")
+    x = torch.randn((H * qpk, T, D), generator=torch.Generator().manual_seed(5)).to(torch.bfloat16)
+    q = torch.empty(size, dtype=torch.bfloat16, device="cuda").as_strided((H * qpk, T, D), (stride_h, stride_t, 1))
+    q.copy_(x)
+    s = sq.Subspace(H, D)
+    sq.squat_build_subspace(s, q, 8, 1e-3)
+    a = sq.squat_subspace_export(s, ("gram",))["gram"]
+    for h in range(H):
+        y = x[h * qpk:(h + 1) * qpk].double().numpy().reshape(-1, D)
+        ref = y.astype(np.longdouble).T @ y.astype(np.longdouble)
+        size = np.sqrt(np.outer(np.diag(ref), np.diag(ref))).astype(np.float64)
+        assert np.all(np.abs((a[h] - ref).astype(np.float64)) <= 4e-15 * size)
+    s.close()
+    del q
+    torch.cuda.empty_cache()
+
+
 def _us(s, q, passes=5):
     """Median time of a build from q, GPU events."""
     ev = [[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(passes)]
