@@ -447,31 +447,44 @@ __global__ void __launch_bounds__(RED_THREADS) gram_i8_reduce_kernel(const GramA
     }
 }
 
-// Row chunks per kind of product: one wave of CTAs (one per SM), or, with few CTAs per head and many rows (a CTA costs 6 us
-// beside its rows), two waves, whose parts can be sized more evenly.  The kinds get equal shares: turning rows into digits
-// takes them equally long, and longer than the products.
+// Row chunks per kind of product: one wave of CTAs (one per SM) or two.  The kinds get equal shares (turning rows into digits
+// takes them equally long, and longer than the products), so a wave lasts as long as the kind with the fewest CTAs per head needs
+// for its share.  Two waves pay where one cannot be dealt out evenly -- four CTAs per head are 2 + 1 + 1 and last for all rows,
+// nine in two waves for 2/3 of them -- and the rows saved are more than the 2048 that the second wave's beginnings, ends and parts
+// cost.  Measured, one wave against two (whole power build): 32 heads x 4096 rows 163, 165 us; 5120 177, 177; 8192 218, 210; 32768
+// 548, 450.  18 heads (4 + 2 + 2 or 6 + 5 + 5) x 16384 222, 226; 24576 280, 271.  24 heads (2 + 2 + 2 or 4 + 4 + 4) x 32768 364, 370.
 bool plan(const squat_subspace *s, int n_rows, int (&parts)[3])
 {
-    const int wave = squat_sm_count() / s->n_kv_heads;
-    const int total = wave >= 10 || n_rows < 16384 ? wave : s->gram_chunks_cap;
-    if (total < 3 || total > s->gram_chunks_cap) return false;
-    parts[1] = parts[2] = total / 3;
-    parts[0] = total - 2 * parts[1];
-    return parts[0] >= 1 && n_rows / parts[1] < MAX_ROWS_PER_PART && n_rows / parts[0] < MAX_ROWS_PER_PART;
+    long long best = -1;
+    for (int waves = 1; waves <= 2; ++waves) {
+        const int total = waves == 1 ? squat_sm_count() / s->n_kv_heads : s->gram_chunks_cap, fewest = total / 3;
+        if (fewest < 1 || total > s->gram_chunks_cap || n_rows / fewest >= MAX_ROWS_PER_PART) continue;
+        const long long cost = (long long)waves * (n_rows / fewest) + 2048 * (waves - 1);
+        if (best >= 0 && cost >= best) continue;
+        best = cost;
+        parts[1] = parts[2] = fewest;
+        parts[0] = total - 2 * fewest;
+    }
+    return best >= 0;
 }
 
 }  // namespace
 
-// bf16 queries and at least three CTAs per head; below 1024 rows the fp64 kernel's fewer launches win.  The loads step 32 tokens
-// at a time and cross one query head at most.  Their offsets, in 16-byte units from a KV head's first row, are 32-bit and run on
-// for up to 320 rows (that are not loaded) behind the last one, so views that spread a KV head over 32 GB go to the fp64 kernel.
+// bf16 queries, and enough rows: the fp64 kernel's time grows with rows x heads, the integer kernels' beginnings, ends and parts
+// cost about 25 us more than its own.  Both sides (whole power build, fp64 and integer): 8 heads x 4096 rows 124, 128 us; 6144 134,
+// 132; 16 x 2560 124, 124; 4096 140, 130; 32 x 1536 126, 130; 2048 136, 135; 1 x 8192 136, 204; 1 x 65536 230, 230.  Above 49 heads there
+// are two waves at any rate: 64 x 1280 146, 150; 1536 159, 155; 96 x 1024 153, 157.
+// The loads step 32 tokens at a time and cross one query head at most.  Their offsets, in 16-byte units from a KV head's first row,
+// are 32-bit and run on for up to 320 rows (that are not loaded) behind the last one, so views that spread a KV head over 32 GB
+// go to the fp64 kernel.
 bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens, long long stride_h, long long stride_t)
 {
     int parts[3];
     const int q_per_kv = n_q_heads / s->n_kv_heads;
     const long long rows = (long long)n_tokens * q_per_kv;
     const double reach = ((double)(q_per_kv + 11) * stride_h + (double)(n_tokens + 320) * stride_t) / 8;
-    return dtype == SQUAT_BF16 && n_tokens >= 32 && rows >= 1024 && rows < (1 << 30) && reach < 2147483648.0 && plan(s, (int)rows, parts);
+    const long long enough = squat_sm_count() / s->n_kv_heads >= 3 ? 3 << 14 : 3 << 15;
+    return dtype == SQUAT_BF16 && n_tokens >= 32 && rows * s->n_kv_heads >= enough && rows < (1 << 30) && reach < 2147483648.0 && plan(s, (int)rows, parts);
 }
 
 int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st)

@@ -1,5 +1,6 @@
-"""GPU: the integer Gram kernel (bf16 queries, 1024 stacked rows or more) against exact sums, where it can go wrong: ragged
-rows, stacked heads, channels of zeros, elements far below their channel's largest (listed remainders, then a full list)."""
+"""GPU: the integer Gram kernel (bf16 queries, 49152 stacked rows or more over all heads, twice that above 49 heads) against exact
+sums, where it can go wrong: ragged rows, stacked heads, one wave of parts and two, channels of zeros, elements far below their
+channel's largest (listed remainders, a full list, an overfull one)."""
 import numpy as np
 import pytest
 import torch
@@ -8,6 +9,17 @@ import paper_2503_24358_b200 as sq
 
 pytestmark = pytest.mark.gpu
 D = 128
+
+
+def _gram(x):
+    """x^T x of bf16 numbers [rows, D]: sums over 16 rows in float64 (products of bf16 numbers are exact, so these are within
+    16 x 2^-53 of sum |x_i x_j|), added up in extended precision."""
+    ref = np.zeros((D, D), np.longdouble)
+    for n in range(0, len(x), 4096):
+        y = x[n:n + 4096]
+        y = np.concatenate([y, np.zeros((-len(y) % 16, D))]).reshape(-1, 16, D)
+        ref += (y.transpose(0, 2, 1) @ y).sum(0, dtype=np.longdouble)
+    return ref
 
 
 def _tiny(q, H, n, g):
@@ -20,9 +32,9 @@ def _tiny(q, H, n, g):
 
 
 @pytest.mark.parametrize("H,qpk,T,data", [
-    (32, 1, 1024, "normal"), (8, 4, 300, "normal"), (1, 1, 4097, "normal"), (2, 2, 2049, "zeros"), (40, 1, 1100, "normal"),
-    (8, 1, 1500, "outliers"), (2, 1, 1024, "wide"), (4, 2, 5000, "normal"), (2, 1, 1024, "listed"), (3, 2, 1000, "full list"),
-    (3, 2, 1000, "one head"), (1, 4, 1031, "wide")])
+    (32, 1, 1600, "normal"), (32, 1, 7001, "normal"), (8, 4, 1600, "normal"), (1, 1, 49153, "normal"), (2, 2, 12289, "zeros"),
+    (40, 1, 1300, "normal"), (18, 1, 21001, "normal"), (64, 1, 1601, "normal"), (8, 1, 6200, "outliers"), (2, 1, 24600, "wide"),
+    (4, 2, 6200, "normal"), (2, 1, 24600, "listed"), (3, 2, 8200, "full list"), (3, 2, 8200, "one head"), (1, 4, 12301, "wide")])
 def test_gram_is_exact(H, qpk, T, data):
     g = torch.Generator().manual_seed(7)
     q = torch.randn((H * qpk, T, D), generator=g)
@@ -47,7 +59,7 @@ def test_gram_is_exact(H, qpk, T, data):
     assert np.array_equal(a, sq.squat_subspace_export(s, ("gram",))["gram"])           # the same bits every time
     for h in {0, H // 2, H - 1}:
         x = q[h * qpk:(h + 1) * qpk].double().numpy().reshape(-1, D)
-        ref = x.astype(np.longdouble).T @ x.astype(np.longdouble)
+        ref = _gram(x)
         size = np.sqrt(np.outer(np.diag(ref), np.diag(ref))).astype(np.float64)
         err = np.abs((a[h] - ref).astype(np.float64))
         assert np.all(err <= 4e-15 * size + 0.0), (err / np.maximum(size, 1e-300)).max()
@@ -56,7 +68,7 @@ def test_gram_is_exact(H, qpk, T, data):
 
 
 @pytest.mark.parametrize("H,qpk,T,stride_h,stride_t", [
-    (1, 1, 1100, 0, 1 << 24), (1, 2, 600, 600 << 24, 1 << 24), (1, 3, 400, 1 << 33, 128), (2, 1, 1100, 1 << 33, 128)])
+    (1, 1, 49200, 0, 1 << 19), (1, 2, 24700, 24700 << 19, 1 << 19), (1, 3, 16500, 1 << 33, 128), (2, 1, 24700, 1 << 34, 128)])
 def test_views_spread_over_more_than_32_gigabytes(H, qpk, T, stride_h, stride_t):
     size = (H * qpk - 1) * stride_h + (T - 1) * stride_t + D
     if torch.cuda.mem_get_info()[0] < 2 * size + (4 << 30):
@@ -69,7 +81,7 @@ def test_views_spread_over_more_than_32_gigabytes(H, qpk, T, stride_h, stride_t)
     a = sq.squat_subspace_export(s, ("gram",))["gram"]
     for h in range(H):
         y = x[h * qpk:(h + 1) * qpk].double().numpy().reshape(-1, D)
-        ref = y.astype(np.longdouble).T @ y.astype(np.longdouble)
+        ref = _gram(y)
         size = np.sqrt(np.outer(np.diag(ref), np.diag(ref))).astype(np.float64)
         assert np.all(np.abs((a[h] - ref).astype(np.float64)) <= 4e-15 * size)
     s.close()
