@@ -10,7 +10,8 @@
 //            head, which are put together in float32.  31 bits of the largest term are more than a float32 sum keeps.
 //   values   sum_t (w_t scale_tg) code_tc + sum_t w_t zero_tg.  The same with the roles turned: A = the codes transposed (the
 //            same bytes in shared memory, described as M-major), B = the digits of w_t scale_tg, one column per channel
-//            group, head and digit.  Accumulated over the chunk's tiles in tensor memory.
+//            group, head and digit.  Accumulated over the chunk's tiles in tensor memory.  31 bits (28 at least) of the
+//            largest product of the channel group and head in the chunk, however far the scales lie apart.
 // A lane owns a token (its row of key codes, its weight, its value metadata); a warp makes the digits of the query for one
 // token group.  Key codes are A in tensor memory (row = lane), so they never cross shared memory, whose wavefronts were the
 // tightest pipe with both operands there (78 % busy); value codes, which must be read transposed, go through it.  The digits
@@ -19,8 +20,9 @@
 // (8 / BITS) i + j of the word); the same order is used for the other operand.
 //
 // Bound: HBM (bits / 8 + metadata bytes per cached element) for long caches.  The CUDA-core form that this replaces spent
-// two instructions per code and head and was bound by them.  64 x 32 heads x 4096 tokens (1.07 GB): 341 -> 216 us, 63 % of
-// DRAM throughput; 16 x 8 KV heads x 8160 tokens with four query heads each: 142 -> 61 us.
+// two instructions per code and head and was bound by them.  Whole call, 64 x 32 heads x 4096 tokens (1.07 GB): 374 -> 257 to 274
+// us by box, 58 % of DRAM throughput in a capture of this kernel; 16 x 8 KV heads x 8160 tokens with four query heads each: 149 -> 60
+// us.
 #pragma once
 #include <type_traits>
 #include "attention.cuh"
@@ -131,6 +133,45 @@ struct Meta {
         }
     }
 };
+
+__device__ __forceinline__ u64 pack2f(float lo, float hi)
+{
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2f(u64 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
+{
+    u64 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ u64 fmul2(u64 a, u64 b)
+{
+    u64 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// element by element, two at a time (N is 1 or even)
+template <int N>
+__device__ __forceinline__ void fma_n(float (&d)[N], const float (&a)[N], const float (&b)[N], const float (&c)[N])
+{
+    if constexpr (N == 1) d[0] = fmaf(a[0], b[0], c[0]);
+    else {
+#pragma unroll
+        for (int i = 0; i < N; i += 2) unpack2f(ffma2(pack2f(a[i], a[i + 1]), pack2f(b[i], b[i + 1]), pack2f(c[i], c[i + 1])), d[i], d[i + 1]);
+    }
+}
+template <int N>
+__device__ __forceinline__ void mul_n(float (&d)[N], const float (&a)[N], const float (&b)[N])
+{
+    if constexpr (N == 1) d[0] = a[0] * b[0];
+    else {
+#pragma unroll
+        for (int i = 0; i < N; i += 2) unpack2f(fmul2(pack2f(a[i], a[i + 1]), pack2f(b[i], b[i + 1])), d[i], d[i + 1]);
+    }
+}
 
 // Power of two that takes values up to mx (>= 0) to at most 2^30, and its inverse (NaN for a non-finite mx)
 __device__ __forceinline__ float fixed_scale(float mx, float &inv)
@@ -356,7 +397,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     __shared__ __align__(8) u64 mbar;
     __shared__ unsigned tmem_sm;
     __shared__ float2 qz_sm[MAX_TILES][NG][NQ];                 // inverse of the fixed point, sum of query x zero-point
-    __shared__ float red_sm[WARPS][NG * NQ + NQ + 1];
+    __shared__ float red_sm[WARPS][NG * NQ + NQ + 2], top_sm[WARPS][NG * NQ];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int parts = p.nchunk + (p.R > 0), chunk = blockIdx.x % parts, qpass = blockIdx.x / parts;
     const int h = blockIdx.y, b = blockIdx.z;
@@ -491,9 +532,19 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     };
 
     // ---------------------------------------------------------------- scores
-    float mx[NQ], vmax = 0.0f;
+    constexpr int P = NG * NQ;                                  // (channel group, head) pairs, g NQ + j
+    float mx[NQ], vmax = 0.0f, vmin = INFINITY;                 // largest score of a head; largest and smallest |value scale|
 #pragma unroll
     for (int j = 0; j < NQ; ++j) mx[j] = -INFINITY;
+    auto widen = [&]() {                                        // by the token in vs_next
+        float vs[NG];
+        vs_next.get(vs);
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            vmax = max_nan(vmax, fabsf(vs[g]));
+            vmin = fminf(vmin, fabsf(vs[g]));
+        }
+    };
     auto read_scores = [&](int tile) {
         wait_product();
         int d[NQ][4];
@@ -589,10 +640,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
                 sc_sm[(tile * NQ + j) * TILE] = s;
                 mx[j] = max_nan(mx[j], s);
             }
-            float vs[NG];
-            vs_next.get(vs);
-#pragma unroll
-            for (int g = 0; g < NG; ++g) vmax = max_nan(vmax, fabsf(vs[g]));
+            widen();
         }
     } else {
 #pragma unroll 1
@@ -634,10 +682,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
             tc_fence_before();
             __syncthreads();
             issue(buf, false, false);
-            float vs[NG];
-            vs_next.get(vs);
-#pragma unroll
-            for (int g = 0; g < NG; ++g) vmax = max_nan(vmax, fabsf(vs[g]));
+            widen();
         }
         read_scores(tiles - 1);
     }
@@ -651,23 +696,68 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
         if (lane == 0) red_sm[warp][j] = mx[j];
     }
     vmax = warp_max(vmax);
-    if (lane == 0) red_sm[warp][NQ] = vmax;
+    vmin = warp_max(-vmin);
+    if (lane == 0) {
+        red_sm[warp][NQ] = vmax;
+        red_sm[warp][NQ + 1] = vmin;
+    }
     tc_fence_before();                                          // the score columns have been read; the values' product reuses them
     __syncthreads();
+    auto over_warps = [](const auto &part, int i) { return max_nan(max_nan(part[0][i], part[1][i]), max_nan(part[2][i], part[3][i])); };
 #pragma unroll
-    for (int j = 0; j < NQ; ++j) mx[j] = max_nan(max_nan(red_sm[0][j], red_sm[1][j]), max_nan(red_sm[2][j], red_sm[3][j]));
-    vmax = max_nan(max_nan(red_sm[0][NQ], red_sm[1][NQ]), max_nan(red_sm[2][NQ], red_sm[3][NQ]));
-    float inv_v;
-    const float up_v = fixed_scale(vmax, inv_v);
+    for (int j = 0; j < NQ; ++j) mx[j] = over_warps(red_sm, j);
+    vmax = over_warps(red_sm, NQ);
+    // The digits of weight x value scale are to hold about 31 bits of the largest product of each channel group and head.  Where
+    // all scales of the chunk lie within a factor of 8 the largest stands for the products (the largest weight is 1, so 28 bits are
+    // the least).  Otherwise the products are looked at: channel groups may lie far apart, and a token far above the others may
+    // carry no weight.  That takes another pass over the scores and a barrier, with one token of 256 30 times the rest 271 -> 282 us
+    // on 64 x 32 heads x 4096 and 69 -> 73 on 16 x 8 KV heads x 8160 (cold caches); for every chunk it cost 4 to 6 %, the same maxima
+    // taken as logarithms beside the scores 1 to 5 %, this test 0 to 2 %.
+    float inv_v[NQ], up_v[P];                                   // inv_v: of the channel group that the warp reads at the end
+    if (__builtin_expect(vmax <= -8.0f * over_warps(red_sm, NQ + 1), 1)) {
+        float inv;
+        const float up = fixed_scale(vmax, inv);
+#pragma unroll
+        for (int i = 0; i < P; ++i) up_v[i] = up;
+#pragma unroll
+        for (int j = 0; j < NQ; ++j) inv_v[j] = inv;
+    } else {
+        float top[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) top[i] = 0.0f;
+#pragma unroll 2
+        for (int tile = 0; tile < tiles; ++tile) {
+            Meta<NG, M16> m;
+            m.load(p.vs, ctok0 + min(tile * TILE + tid, last_tok));
+            float vs[NG];
+            m.get(vs);
+#pragma unroll
+            for (int j = 0; j < NQ; ++j) {
+                const float w = expf(sc_sm[(tile * NQ + j) * TILE] - mx[j]);
+#pragma unroll
+                for (int g = 0; g < NG; ++g) top[g * NQ + j] = max_nan(top[g * NQ + j], fabsf(w * vs[g]));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            top[i] = warp_max(top[i]);
+            if (lane == 0) top_sm[warp][i] = top[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            float inv;
+            up_v[i] = fixed_scale(over_warps(top_sm, i), inv);
+            if (i / NQ == my_group) inv_v[i % NQ] = inv;
+        }
+    }
 
     // ---------------------------------------------------------------- weights, weighted values
-    float zacc[NG][NQ], den[NQ];
+    float zacc[P], den[NQ];
 #pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-        den[j] = 0.0f;
+    for (int j = 0; j < NQ; ++j) den[j] = 0.0f;
 #pragma unroll
-        for (int g = 0; g < NG; ++g) zacc[g][j] = 0.0f;
-    }
+    for (int i = 0; i < P; ++i) zacc[i] = 0.0f;
     unsigned char *const my_dig = digits_sm + tid / 8 * DIG_PIECE + tid % 8 * 16;
 #pragma unroll 1
     for (int tile = 0; tile < tiles; ++tile) {
@@ -686,17 +776,16 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
             load_vz(tile + 1);
         }
         uint32_t dig[S::N / 4];
+        float ww[P], ss[P], zz[P], x[P];
 #pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            const float vu = vs[g] * up_v;
+        for (int i = 0; i < P; ++i) { ww[i] = w[i % NQ]; ss[i] = vs[i / NQ]; zz[i] = vz[i / NQ]; }
+        fma_n(zacc, ww, zz, zacc);
+        mul_n(x, ww, ss);
+        mul_n(x, x, up_v);                                      // (exact: a power of two)
 #pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                zacc[g][j] = fmaf(w[j], vz[g], zacc[g][j]);
-                dig[g * NQ + j] = digits_of(w[j] * vu);
-            }
-        }
+        for (int i = 0; i < P; ++i) dig[i] = digits_of(x[i]);
 #pragma unroll
-        for (int i = NG * NQ; i < S::N / 4; ++i) dig[i] = 0;
+        for (int i = P; i < S::N / 4; ++i) dig[i] = 0;
 #pragma unroll
         for (int c = 0; c < S::N / 16; ++c)
             *reinterpret_cast<uint4 *>(my_dig + buf * S::DIG_BYTES + c * DIG_CHUNK) = make_uint4(dig[4 * c], dig[4 * c + 1], dig[4 * c + 2], dig[4 * c + 3]);
@@ -713,12 +802,12 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
         den[j] = attn_warp_sum(den[j]);
-        if (lane == 0) red_sm[warp][NG * NQ + j] = den[j];
+        if (lane == 0) red_sm[warp][P + j] = den[j];
+    }
 #pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            zacc[g][j] = attn_warp_sum(zacc[g][j]);
-            if (lane == 0) red_sm[warp][g * NQ + j] = zacc[g][j];
-        }
+    for (int i = 0; i < P; ++i) {
+        zacc[i] = attn_warp_sum(zacc[i]);
+        if (lane == 0) red_sm[warp][i] = zacc[i];
     }
     wait_product();
     int d[NQ][4];
@@ -730,16 +819,16 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((unsigned)S::TMEM_COLS) : "memory");
     const int c = channel_at<BITS>(tid);
-    inv_v *= 1.0f / (float)(1 << BITS * piece_at<BITS>(tid));
+    const float per_piece = 1.0f / (float)(1 << BITS * piece_at<BITS>(tid));
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
         if (j >= nq_here) break;
         const int zi = my_group * NQ + j;
         const float z = (red_sm[0][zi] + red_sm[1][zi]) + (red_sm[2][zi] + red_sm[3][zi]);
         const long long row = ((long long)b * p.Hq + hq0 + j) * parts + chunk;
-        p.part[row * D + c] = from_long_digits(d[j], inv_v) + z;
+        p.part[row * D + c] = from_long_digits(d[j], inv_v[j] * per_piece) + z;
         if (tid == 0) {
-            const int di = NG * NQ + j;
+            const int di = P + j;
             *reinterpret_cast<float2 *>(p.ml + row * 2) = make_float2(mx[j], (red_sm[0][di] + red_sm[1][di]) + (red_sm[2][di] + red_sm[3][di]));
         }
     }
