@@ -1,5 +1,6 @@
 """Thin binding of libsquat.so: argument marshalling only, through ctypes, and for the calls that a serving loop makes per
-window and token through a small extension module (csrc/pycall.c: 8.9 -> 6.4 us a call, most of it the launch).
+window and token through a small extension module where it could be built (csrc/pycall.c: 8.9 -> 6.4 us of host time a call,
+most of it the launch; a window's pair 16.8 -> 16.5 us, a decode step of one sequence 12.4 -> 12.2).
 
 Every function has the name of the C entry point it calls (include/squat.h) and takes
 torch tensors where the C function takes device pointers.  Nothing here computes: all
@@ -8,10 +9,12 @@ missing or does not load, every call raises -- there is no fallback.
 """
 import ctypes
 import os
+from importlib.machinery import EXTENSION_SUFFIXES
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
+PYCALL = os.path.join(_HERE, "_squatcall" + EXTENSION_SUFFIXES[0])       # the extension module, for this interpreter
 # SQUAT_LIBRARY selects another build of the same library (the bounds-checked one, libsquat_checked.so)
 LIB_PATH = os.environ.get("SQUAT_LIBRARY") or os.path.join(_HERE, "libsquat.so")
 
@@ -95,18 +98,44 @@ def _load():
         lib.squat_status_string.argtypes = [i]
         lib.squat_status_string.restype = c.c_char_p
         lib.squat_last_cuda_error.restype = c.c_char_p
-        from . import _squatcall                     # built beside the library; the calls below go through it
-        _squatcall.bind(*(c.cast(f, vp).value for f in (lib.squat_quantize_keys, lib.squat_quantize_keys_m16, lib.squat_quantize_values,
-                                                        lib.squat_quantize_values_m16, lib.squat_dequantize, lib.squat_dequantize_m16,
-                                                        lib.squat_decode_attention_ex)))
         global _call
-        _call = _squatcall
+        _call = _entry_points(lib)
         _lib = lib
     return _lib
 
 
+class _CtypesCalls:
+    """What the extension module does, through ctypes: for an installation without it."""
+
+    def __init__(self, lib):
+        self._lib = lib
+
+    def quantize_keys(self, meta16, *args):
+        return (self._lib.squat_quantize_keys_m16 if meta16 else self._lib.squat_quantize_keys)(*args)
+
+    def quantize_values(self, meta16, *args):
+        return (self._lib.squat_quantize_values_m16 if meta16 else self._lib.squat_quantize_values)(*args)
+
+    def dequantize(self, meta16, *args):
+        return (self._lib.squat_dequantize_m16 if meta16 else self._lib.squat_dequantize)(*args)
+
+    def decode_attention(self, softmax_scale, *args):
+        return self._lib.squat_decode_attention_ex(*args[:22], softmax_scale, *args[22:])
+
+
+def _entry_points(lib):
+    """The calls of a serving loop: the extension module built beside the library for this interpreter, else ctypes."""
+    if not os.path.exists(PYCALL):
+        return _CtypesCalls(lib)
+    from . import _squatcall
+    _squatcall.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+        lib.squat_quantize_keys, lib.squat_quantize_keys_m16, lib.squat_quantize_values, lib.squat_quantize_values_m16,
+        lib.squat_dequantize, lib.squat_dequantize_m16, lib.squat_decode_attention_ex)))
+    return _squatcall
+
+
 def _direct():
-    """The extension module with the library's hot entry points (loads both on first use)."""
+    """The library's hot entry points (loads the library on first use)."""
     if _call is None:
         _load()
     return _call

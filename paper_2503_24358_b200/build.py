@@ -5,8 +5,10 @@ sources with -DSQUAT_CHECKED: the key and value kernels then test every address 
 buffer or on-chip region it belongs to and report through SQUAT_FLAG_BOUNDS instead of accessing.  Select it with the
 environment variable SQUAT_LIBRARY=<path> before the package is first used."""
 import os
+import shutil
 import subprocess
 import sysconfig
+from importlib.machinery import EXTENSION_SUFFIXES
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -16,6 +18,7 @@ OBJ_DIR = os.path.join(_HERE, "build")
 LIB = os.path.join(_HERE, "libsquat.so")
 OBJ_DIR_CHECKED = os.path.join(_HERE, "build_checked")
 LIB_CHECKED = os.path.join(_HERE, "libsquat_checked.so")
+PYCALL = os.path.join(_HERE, "_squatcall" + EXTENSION_SUFFIXES[0])
 SOURCES = ["api.cu", "values.cu", "keys.cu", "subspace.cu", "gram_i8.cu", "eig.cu", "power.cu", "attention.cu", "attention_mma.cu", "attention_rope.cu", "peak.cu", "keys_lowrank.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE]
@@ -49,11 +52,16 @@ def _compile(src, verbose, obj_dir=OBJ_DIR, extra=()):
     return obj
 
 
-def build_pycall(force: bool = False) -> str:
-    """The extension module through which the binding makes its per-token and per-window calls (gcc, the CPython C API)."""
-    src, out = os.path.join(CSRC, "pycall.c"), os.path.join(_HERE, "_squatcall.so")
+def build_pycall(force: bool = False):
+    """The extension module through which the binding makes its per-token and per-window calls (gcc, the CPython C API).  Its
+    file name carries the interpreter's ABI tag.  Without a C compiler or the CPython headers there is none (None is returned)
+    and the binding calls through ctypes."""
+    src, out = os.path.join(CSRC, "pycall.c"), PYCALL
+    include, cc = sysconfig.get_paths()["include"], shutil.which(os.environ.get("CC") or "gcc")
+    if cc is None or not os.path.exists(os.path.join(include, "Python.h")):
+        return None
     if force or not os.path.exists(out) or os.path.getmtime(out) < max(os.path.getmtime(src), os.path.getmtime(os.path.join(INCLUDE, "squat.h"))):
-        subprocess.run(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", out], check=True)
+        subprocess.run([cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", include, src, "-o", out], check=True)
     return out
 
 
