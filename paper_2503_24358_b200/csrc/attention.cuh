@@ -38,27 +38,6 @@ __device__ __forceinline__ float attn_load_elem(const void *p, long long idx, in
     return reinterpret_cast<const float *>(p)[idx];
 }
 
-// scale / zero-point element i of a metadata array stored as float32 or binary16
-template <bool M16>
-__device__ __forceinline__ float attn_meta(const void *p, long long i)
-{
-    if (M16) return __half2float(__ldg(reinterpret_cast<const __half *>(p) + i));
-    return __ldg(reinterpret_cast<const float *>(p) + i);
-}
-
-// four consecutive elements starting at i (a multiple of 4)
-template <bool M16>
-__device__ __forceinline__ float4 attn_meta4(const void *p, long long i)
-{
-    if (M16) {
-        const uint2 r = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p) + i));
-        const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&r.x));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&r.y));
-        return make_float4(a.x, a.y, b.x, b.y);
-    }
-    return __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(p) + i));
-}
-
 constexpr int ATTN_MMA_TILE = 128;            // tokens per product
 constexpr int ATTN_MMA_MAX_TILES = 8;         // tiles per CTA: chunks of at most 1024 tokens
 // resident CTAs per SM the kernel is built for, by query heads per pass (96 or 128 registers: six CTAs of 80 were slower)

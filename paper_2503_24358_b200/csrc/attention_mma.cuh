@@ -26,17 +26,14 @@
 #pragma once
 #include <type_traits>
 #include "attention.cuh"
+#include "device_helpers.cuh"
 
 namespace {
 
 constexpr int D = SQUAT_D;
 constexpr int THREADS = 128, WARPS = 4;
 constexpr int TILE = ATTN_MMA_TILE, MAX_TILES = ATTN_MMA_MAX_TILES;
-typedef unsigned long long u64;
 
-__device__ __forceinline__ unsigned smem_u32(const void *ptr) { return (unsigned)__cvta_generic_to_shared(ptr); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // Shared-memory matrix descriptors.  Codes: 128-byte rows (token), 128-byte swizzle, groups of 8 rows 1024 bytes apart;
 // K-major for the scores (K = channel), M-major for the values (K = token).  Digits: no swizzle, N-major: 16 bytes of
@@ -56,12 +53,6 @@ __host__ __device__ constexpr unsigned idesc_i8(int n, bool a_m_major)
 {
     return (2u << 4) | (1u << 10) | ((a_m_major ? 1u : 0u) << 15) | (1u << 16) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24);
 }
-__device__ __forceinline__ void mma_i8(unsigned d_taddr, u64 a_desc, u64 b_desc, unsigned idesc, unsigned accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_taddr), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
 // the same with A in tensor memory (row = lane, four bytes a column)
 __device__ __forceinline__ void mma_i8_ta(unsigned d_taddr, unsigned a_taddr, u64 b_desc, unsigned idesc, unsigned accumulate)
 {
@@ -75,39 +66,12 @@ __device__ __forceinline__ void tmem_st16(unsigned taddr, const uint32_t (&r)[16
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
                    "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
-__device__ __forceinline__ void tc_commit(unsigned mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-// Bounded wait for a phase of an mbarrier: false when the limit ran out (the caller records it and moves on).
-__device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
-{
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 __device__ __forceinline__ void tmem_ld4(unsigned taddr, int (&r)[4])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ float warp_max(float x)
-{
-    float r;
-    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
 
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 // N scales or zero-points as they were loaded (float32 or binary16); they become floats where they are used, so that nothing
 // waits for a load where it is issued
 template <int N, bool M16>
@@ -134,25 +98,6 @@ struct Meta {
     }
 };
 
-__device__ __forceinline__ u64 pack2f(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2f(u64 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
-{
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ u64 fmul2(u64 a, u64 b)
-{
-    u64 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 // element by element, two at a time (N is 1 or even)
 template <int N>
 __device__ __forceinline__ void fma_n(float (&d)[N], const float (&a)[N], const float (&b)[N], const float (&c)[N])
@@ -160,7 +105,7 @@ __device__ __forceinline__ void fma_n(float (&d)[N], const float (&a)[N], const 
     if constexpr (N == 1) d[0] = fmaf(a[0], b[0], c[0]);
     else {
 #pragma unroll
-        for (int i = 0; i < N; i += 2) unpack2f(ffma2(pack2f(a[i], a[i + 1]), pack2f(b[i], b[i + 1]), pack2f(c[i], c[i + 1])), d[i], d[i + 1]);
+        for (int i = 0; i < N; i += 2) unpack2(ffma2(pack2(a[i], a[i + 1]), pack2(b[i], b[i + 1]), pack2(c[i], c[i + 1])), d[i], d[i + 1]);
     }
 }
 template <int N>
@@ -169,7 +114,7 @@ __device__ __forceinline__ void mul_n(float (&d)[N], const float (&a)[N], const 
     if constexpr (N == 1) d[0] = a[0] * b[0];
     else {
 #pragma unroll
-        for (int i = 0; i < N; i += 2) unpack2f(fmul2(pack2f(a[i], a[i + 1]), pack2f(b[i], b[i + 1])), d[i], d[i + 1]);
+        for (int i = 0; i < N; i += 2) unpack2(fmul2(pack2(a[i], a[i + 1]), pack2(b[i], b[i + 1])), d[i], d[i + 1]);
     }
 }
 

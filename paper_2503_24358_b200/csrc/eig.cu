@@ -10,31 +10,14 @@
 // on a Cholesky factor, needed 10 sweeps of 127 dependent rounds: 677 us.
 #include <cooperative_groups.h>
 #include <type_traits>
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 
 namespace {
 
 namespace cg = cooperative_groups;
 constexpr int D = SQUAT_D;
 
-// 1/sqrt(x) for a normal positive double: hardware seed y (relative error 2^-22), residual r = 1 - x y^2, and one
-// third-order correction y (1 + r/2 + 3 r^2/8); what is left, about r^3/3, is far below a double's rounding.
-__device__ __forceinline__ double rsqrt_nr(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double r = fma(-(x * y), y, 1.0);
-    return fma(y * r, fma(0.375, r, 0.5), y);
-}
 
-// 1/x for a normal double: hardware seed (about 20 bits), two Newton steps y <- y + y (1 - x y)
-__device__ __forceinline__ double rcp_nr(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
 
 __device__ __forceinline__ double sqrt_nr(double x) { return x > 1e-290 ? x * rsqrt_nr(x) : 0.0; }
 
@@ -45,11 +28,6 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-__device__ __forceinline__ void dmma(double &c0, double &c1, double a, double b)
-{
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                 : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
-}
 
 // ------------------------------------------------------------------------------------------------ tridiagonalisation
 // Step k zeroes column k below the subdiagonal with the reflector I - u u^T / h (u_i = 0 for i <= k):

@@ -25,13 +25,12 @@
 // of a stage take 0.25).  32 heads x 32768 rows: 642 -> 367 us for the three kernels; 8 heads x 32640: 182 -> 121; 32 heads x
 // 4096: 96 -> 81.
 #include <type_traits>
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 
 namespace {
 
 constexpr int D = SQUAT_D;
 constexpr int MAX_ROWS_PER_PART = 1 << 16;     // products up to 2^14: the sum stays within 32 bits
-typedef unsigned long long u64;
 
 struct GramArgs {
     const __nv_bfloat16 *q;
@@ -129,29 +128,6 @@ constexpr int ROWS = 64, STAGES = 4, CONV_WARPS = 16, CONV = 32 * CONV_WARPS, TH
 constexpr int PLANE = ROWS * D, STAGE = 4 * PLANE;
 constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE;
 
-__device__ __forceinline__ unsigned smem_u32(const void *ptr) { return (unsigned)__cvta_generic_to_shared(ptr); }
-__device__ __forceinline__ u64 pack2f(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
-{
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
-{
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 // planes: 128-byte rows (K), 128-byte swizzle, groups of 8 rows 1024 bytes apart; the next 128 columns of B are the next plane
 __device__ __forceinline__ u64 plane_desc(unsigned addr)
 {
@@ -161,16 +137,6 @@ __device__ __forceinline__ u64 plane_desc(unsigned addr)
 __host__ __device__ constexpr unsigned idesc(int n)
 {
     return (2u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-__device__ __forceinline__ void mma_i8(unsigned d_taddr, u64 a, u64 b, unsigned id, bool accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_taddr), "l"(a), "l"(b), "r"(id), "r"((unsigned)accumulate) : "memory");
-}
-__device__ __forceinline__ void commit(unsigned mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(unsigned taddr, int (&r)[16])
 {
@@ -254,9 +220,9 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
         const int c16 = tid & 15, r0 = tid >> 4;                      // channels 8 c16 .. 8 c16 + 7 of rows r0 + STEP i
         u64 s2[4];                                                    // 1 / unit, as the packed multiplicand of a channel pair
 #pragma unroll
-        for (int i = 0; i < 4; ++i) s2[i] = pack2f((float)(1.0 / unit[8 * c16 + 2 * i]), (float)(1.0 / unit[8 * c16 + 2 * i + 1]));
+        for (int i = 0; i < 4; ++i) s2[i] = pack2((float)(1.0 / unit[8 * c16 + 2 * i]), (float)(1.0 / unit[8 * c16 + 2 * i + 1]));
         // 1.5 2^23: the integer in the low bits; + 128: the low digit's carry
-        const u64 magic2 = pack2f(12582912.0f + 128.0f, 12582912.0f + 128.0f), minus2 = pack2f(-1.0f, -1.0f), frac2 = pack2f(32768.0f, 32768.0f);
+        const u64 magic2 = pack2(12582912.0f + 128.0f, 12582912.0f + 128.0f), minus2 = pack2(-1.0f, -1.0f), frac2 = pack2(32768.0f, 32768.0f);
         // rows are addressed in 16-byte units from the head's first, with 32-bit steps; rows past the end are not loaded
         const uint4 *base = reinterpret_cast<const uint4 *>(p.q + (long long)h * p.q_per_kv * p.stride_h) + c16;
         int t = (lo + r0) % p.n_tokens, left = hi - lo - r0;
@@ -295,7 +261,7 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
                         unsigned any = 0;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const u64 x = pack2f(bf16lo_to_f32(w[e]), bf16hi_to_f32(w[e]));
+                            const u64 x = pack2(bf16lo_to_f32(w[e]), bf16hi_to_f32(w[e]));
                             const u64 hm = ffma2(x, s2[e], magic2);
                             const u64 rr = ffma2(x, s2[e], ffma2(hm, minus2, magic2));
                             const u64 lm = ffma2(rr, frac2, magic2);
@@ -343,7 +309,7 @@ __global__ void __launch_bounds__(THREADS, 1) gram_i8_kernel(const GramArgs p)
                     mma_i8(tmem + 256, p3, p3, idesc(128), acc);
                 }
             }
-            commit(smem_u32(&empty[buf]));
+            tc_commit(smem_u32(&empty[buf]));
         }
     }
     __syncwarp();

@@ -35,7 +35,7 @@
 //
 // Work per key vector: 8128 fp32 multiply-adds (dense triangle, g = 1): 1984 on the CUDA cores
 // (sweeps: four triangles of 32 * 31 / 2), 6144 x 3 tf32 products on the tensor cores.
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 #include <cuda_fp16.h>
 
 namespace {
@@ -62,54 +62,7 @@ __host__ __device__ constexpr int tc_panel_off(int b) { return b == 0 ? 0 : (b =
 // instruction descriptor: fp32 accumulator, tf32 A and B, both K-major, N = n, M = 128
 __host__ __device__ constexpr unsigned tc_idesc(int n) { return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24); }
 
-typedef unsigned long long u64;
 
-__device__ __forceinline__ u64 pack2(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float lo_of(u64 v)
-{
-    return __uint_as_float((unsigned)(v & 0xffffffffull));
-}
-__device__ __forceinline__ float hi_of(u64 v)
-{
-    return __uint_as_float((unsigned)(v >> 32));
-}
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
-{
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-// Warp-wide min / max.  The NaN-propagating forms: a NaN key makes the group's grid NaN, which the check of the stored
-// scale reports (SQUAT_FLAG_NONFINITE), instead of vanishing in the reduction and corrupting the codes unnoticed.
-__device__ __forceinline__ float warp_min(float x)
-{
-    float r;
-    asm volatile("redux.sync.min.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float warp_max(float x)
-{
-    float r;
-    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float min_nan(float a, float b)
-{
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 __device__ __forceinline__ float min3_nan(float a, float b, float c)
 {
     float r;
@@ -140,7 +93,6 @@ __device__ __forceinline__ float div_by_levels(float rng)
 }
 
 // ---- tcgen05 / tensor-memory helpers (5th-generation tensor cores) -------------------------------------------
-__device__ __forceinline__ unsigned smem_u32(const void *ptr) { return (unsigned)__cvta_generic_to_shared(ptr); }
 __device__ __forceinline__ unsigned tf32_of(float x)             // round to nearest tf32 (10 mantissa bits)
 {
     unsigned r;
@@ -159,8 +111,6 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32])
                  : "r"(taddr) : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // shared-memory matrix descriptor, no swizzle, K-major: 8 x 16-byte core matrices, lbo bytes between the two
 // halves of a K step, sbo bytes between groups of 8 rows
 __device__ __forceinline__ u64 umma_desc(unsigned addr, unsigned lbo, unsigned sbo)
@@ -186,21 +136,6 @@ __device__ __forceinline__ void tmem_st4(unsigned taddr, float a, float b, float
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
                  ::"r"(taddr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)) : "memory");
-}
-__device__ __forceinline__ void umma_commit(unsigned mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-// Bounded wait for a phase of an mbarrier: false when the limit ran out (the caller records it and moves on).
-__device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
-{
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
 }
 
 // Starts the copy of one head's 64 KB image into shared memory on the bulk-copy engine (one CTA, one destination); the bytes are
@@ -655,7 +590,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_kernel(const KeyPara
 #ifdef SQUAT_CHECKED
                         }
 #endif
-                        umma_commit(my_mbar);
+                        tc_commit(my_mbar);
                     }
                     __syncwarp();
                 }
@@ -690,7 +625,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_kernel(const KeyPara
     // Every committed batch has been waited for unless a wait ran out; then commit once more per slot and give the
     // tensor core a bounded time to drain before the columns are handed back.
     if (shared_words[1] && wq == 0 && lane == 0) {
-        umma_commit(my_mbar);
+        tc_commit(my_mbar);
         mbar_wait(my_mbar, phase);
     }
     tc_fence_before();

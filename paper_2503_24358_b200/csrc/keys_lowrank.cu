@@ -17,7 +17,7 @@
 // and a named barrier).  The per-head table (d rows of [v_j | c_j], 8 KB) sits in shared memory and is read with
 // broadcast 16-byte loads, each serving both tokens of every lane.  The rounding arithmetic is the dense kernel's
 // (keys.cu), operation for operation.
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 #include <cuda_fp16.h>
 
 namespace {
@@ -32,47 +32,7 @@ constexpr int LR_THREADS = LR_WARPS * 32;
 constexpr int LR_CTAS_PER_SM = 3;          // 80 registers per thread: 24 warps per SM
 constexpr float kMagic = 12582912.0f;      // 1.5 * 2^23
 
-typedef unsigned long long u64;
 
-__device__ __forceinline__ u64 pack2(float lo, float hi)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float lo_of(u64 v) { return __uint_as_float((unsigned)(v & 0xffffffffull)); }
-__device__ __forceinline__ float hi_of(u64 v) { return __uint_as_float((unsigned)(v >> 32)); }
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c)
-{
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-// NaN-propagating reductions: a NaN key shows up in the stored scale and raises SQUAT_FLAG_NONFINITE
-__device__ __forceinline__ float warp_min(float x)
-{
-    float r;
-    asm volatile("redux.sync.min.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float warp_max(float x)
-{
-    float r;
-    asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float min_nan(float a, float b)
-{
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 // correctly rounded rng / L for L = 3 or 15 (as in keys.cu)
 template <int BITS>
 __device__ __forceinline__ float div_by_levels(float rng)

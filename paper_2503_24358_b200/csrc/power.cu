@@ -21,7 +21,7 @@
 // doubles, M (for r <= 32, where it fits beside them) row by row with the same stride: the 8 x 4 operand fragments
 // then fall on distinct banks, and the per-row triangular solves (lanes = consecutive rows) are conflict-free with any
 // stride.  No waiting on anything but __syncthreads.
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 
 namespace {
 
@@ -39,13 +39,6 @@ struct PowerLayout {
     static constexpr size_t doubles = small + (M_SHARED ? (size_t)D * LDM : 0);
 };
 
-// D += A B on the FP64 tensor path: A 8 x 4 (lane holds A[lane / 4][lane % 4]), B 4 x 8 (lane holds B[lane % 4][lane / 4]),
-// D 8 x 8 (lane holds D[lane / 4][2 (lane % 4)] and the element to its right)
-__device__ __forceinline__ void pw_dmma(double &c0, double &c1, double a, double b)
-{
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                 : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
-}
 
 // Y = M X: a warp owns 16 rows (two 8-row tiles) x all RP columns; per 4 values of k it loads two fragments of M and
 // RP / 8 of X and issues RP / 4 tensor operations.  M is symmetric; MS: M is the padded shared-memory copy (row stride
@@ -70,8 +63,8 @@ __device__ __forceinline__ void pw_mult(const double *__restrict__ M, const doub
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const double b = xb[8 * c * LDC + k0];
-            pw_dmma(acc[0][c][0], acc[0][c][1], a0, b);
-            pw_dmma(acc[1][c][0], acc[1][c][1], a1, b);
+            dmma(acc[0][c][0], acc[0][c][1], a0, b);
+            dmma(acc[1][c][0], acc[1][c][1], a1, b);
         }
     }
 #pragma unroll
@@ -103,7 +96,7 @@ __device__ __forceinline__ void pw_gram(const double *At, const double *Bt, doub
     for (int k0 = 0; k0 < D; k0 += 4) {
         const double a = pa[k0];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) pw_dmma(acc[c][0], acc[c][1], a, pb[8 * c * LDC + k0]);
+        for (int c = 0; c < NC; ++c) dmma(acc[c][0], acc[c][1], a, pb[8 * c * LDC + k0]);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {

@@ -18,7 +18,7 @@
 // rounded to float32 at the very end.
 #include <type_traits>
 #include <utility>
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 
 namespace {
 
@@ -49,17 +49,12 @@ struct GramTile {
     static constexpr int tj = ti + (U - (ti * 16 - ti * (ti - 1) / 2));
 };
 
-__device__ __forceinline__ void dmma_m8n8k4(double &c0, double &c1, double a, double b)
-{
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                 : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
-}
 
 template <int W, int... N>
 __device__ __forceinline__ void gram_warp_step(double (&acc)[GRAM_TILES_PER_WARP][2], const double (&F)[16],
                                                std::integer_sequence<int, N...>)
 {
-    (dmma_m8n8k4(acc[N][0], acc[N][1], F[GramTile<GRAM_TILES_PER_WARP * W + N>::ti], F[GramTile<GRAM_TILES_PER_WARP * W + N>::tj]), ...);
+    (dmma(acc[N][0], acc[N][1], F[GramTile<GRAM_TILES_PER_WARP * W + N>::ti], F[GramTile<GRAM_TILES_PER_WARP * W + N>::tj]), ...);
 }
 
 template <int W, int... N>
@@ -213,14 +208,6 @@ __global__ void __launch_bounds__(GRED_THREADS) gram_reduce_kernel(const double 
 
 static_assert(GRAM_TILES_PER_WARP * (GRAM_THREADS / 32) == 136, "the warps share the upper triangle evenly");
 
-// 1/x for a normal double: hardware seed (about 20 bits), two Newton steps y <- y + y (1 - x y)
-__device__ __forceinline__ double rcp_nr(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
 
 // ------------------------------------------------------------------------------------- assemble
 // P_inv and its LDL^T factorisation, one CTA per head.  The 136 tiles of 8 x 8 on or below the diagonal live in registers
@@ -327,7 +314,7 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
 #pragma unroll
             for (int n = 0; n < ASM_TILES; ++n) {
                 if (ti[n] == 16) continue;      // warp-uniform
-                dmma_m8n8k4(c[n][0], c[n][1], UL[(e + fk) * ASM_LDU + 8 * ti[n] + fr], U[(e + fk) * ASM_LDU + 8 * tj[n] + fr]);
+                dmma(c[n][0], c[n][1], UL[(e + fk) * ASM_LDU + 8 * ti[n] + fr], U[(e + fk) * ASM_LDU + 8 * tj[n] + fr]);
             }
         }
     }
@@ -384,8 +371,8 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
         for (int n = 0; n < ASM_TILES; ++n) {
             if (tj[n] == 16 || tj[n] <= p) continue;
             const double *lp = Lp + (8 * ti[n] + fr) * ASM_LDP + fk, *vp = Vp + (8 * tj[n] + fr) * ASM_LDP + fk;
-            dmma_m8n8k4(c[n][0], c[n][1], lp[0], vp[0]);
-            dmma_m8n8k4(c[n][0], c[n][1], lp[4], vp[4]);
+            dmma(c[n][0], c[n][1], lp[0], vp[0]);
+            dmma(c[n][0], c[n][1], lp[4], vp[4]);
         }
         if (p < 15) publish(p + 1);
         __syncthreads();

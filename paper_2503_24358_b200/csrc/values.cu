@@ -18,7 +18,7 @@
 // M16 instances store scale and zero-point as IEEE binary16 (the 18.75 % cache of the paper's "KV size" columns):
 // Delta = half(Delta32), z = half(m), and the decision t = (x - z) / Delta is taken against those stored values,
 // so codes are clamped (a rounded zero-point can lie above the minimum).
-#include "squat_internal.cuh"
+#include "device_helpers.cuh"
 #include <cuda_fp16.h>
 
 namespace {
@@ -26,16 +26,7 @@ namespace {
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer (ties to even)
 constexpr unsigned kMagicBits = 0x4B400000u;
 
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 pk2(float lo, float hi) { u64 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
-__device__ __forceinline__ void unpk2(u64 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ u64 sub2(u64 a, u64 b) { u64 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) { u64 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
 
-// NaN-propagating min / max: a NaN input makes the group's scale NaN, which is reported (SQUAT_FLAG_NONFINITE) and gives
-// codes 0, instead of being dropped by the reduction.
-__device__ __forceinline__ float min_nan(float a, float b) { float r; asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
-__device__ __forceinline__ float max_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
 __device__ __forceinline__ unsigned hmin2_nan_bits(unsigned a, unsigned b)
 {
     const __nv_bfloat162 r = __hmin2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
@@ -224,7 +215,7 @@ __global__ void __launch_bounds__(VAL_THREADS) quant_values_kernel(ValParams p)
     float rcp;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(delta));
     const float ra = __fmul_rn(rcp, 1.0f + 0x1p-20f), rb = __fmul_rn(rcp, 1.0f - 0x1p-20f);
-    const u64 m2 = pk2(m, m), ra2 = pk2(ra, ra), rb2 = pk2(rb, rb), magic2 = pk2(kMagic, kMagic);
+    const u64 m2 = pack2(m, m), ra2 = pack2(ra, ra), rb2 = pack2(rb, rb), magic2 = pack2(kMagic, kMagic);
 
     // ---- codes: two channels per instruction (packed f32x2).  Both ends of the bracket are rounded and packed (added
     // up shifted into place); the ends differ by at most one level, upwards, so the difference of the two packed words
@@ -238,9 +229,9 @@ __global__ void __launch_bounds__(VAL_THREADS) quant_values_kernel(ValParams p)
         for (int k = 0; k < PER_WORD; k += 2) {
             float x0, x1, ya0, ya1, yb0, yb1;
             pair_of((wd * PER_WORD + k) / 2, x0, x1);
-            const u64 dlt2 = sub2(pk2(x0, x1), m2);
-            unpk2(fma2(dlt2, ra2, magic2), ya0, ya1);
-            unpk2(fma2(dlt2, rb2, magic2), yb0, yb1);
+            const u64 dlt2 = fsub2(pack2(x0, x1), m2);
+            unpack2(ffma2(dlt2, ra2, magic2), ya0, ya1);
+            unpack2(ffma2(dlt2, rb2, magic2), yb0, yb1);
             if (M16) {                                  // rounded metadata: t may leave [0, L]
                 ya0 = fminf(fmaxf(ya0, kMagic), kMagic + L); yb0 = fminf(fmaxf(yb0, kMagic), kMagic + L);
                 ya1 = fminf(fmaxf(ya1, kMagic), kMagic + L); yb1 = fminf(fmaxf(yb1, kMagic), kMagic + L);
@@ -306,10 +297,10 @@ __device__ __forceinline__ u64 codes_pair(uint32_t lo, uint32_t hi, u64 bias)
     constexpr uint32_t FIELD = (1u << BITS) - 1u;
     const uint32_t word = (BITS == 4 && I >= 2) ? hi : lo;
     float b0, b1;
-    unpk2(bias, b0, b1);
+    unpack2(bias, b0, b1);
     const float f0 = __uint_as_float(and_or<(FIELD << S0)>(word, __float_as_uint(b0)));
     const float f1 = __uint_as_float(and_or<(FIELD << S1)>(word, __float_as_uint(b1)));
-    return sub2(pk2(f0, f1), bias);
+    return fsub2(pack2(f0, f1), bias);
 }
 
 // Dequantizer.  One thread owns 8 consecutive channels (16 bytes of bf16 output, 32 of float32) of TOK = 4 or 8
@@ -335,7 +326,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(
 #pragma unroll
     for (int i = 0; i < CH / 2; ++i) {
         const int s0 = (BITS * 2 * i) % 16, s1 = (BITS * (2 * i + 1)) % 16;
-        bias2[i] = pk2(__uint_as_float((unsigned)(150 - s0) << 23), __uint_as_float((unsigned)(150 - s1) << 23));
+        bias2[i] = pack2(__uint_as_float((unsigned)(150 - s0) << 23), __uint_as_float((unsigned)(150 - s1) << 23));
         asm volatile("" : "+l"(bias2[i]));              // held in registers: the logic instruction below takes them from there
     }
     // one CTA = one chunk of slots * TOK tokens of one (batch, head) row; no division anywhere
@@ -359,16 +350,16 @@ __global__ void __launch_bounds__(256) dequant_kernel(
                 for (int k = 0; k < 4; ++k) {
                     const float2 sf = __half22float2(*reinterpret_cast<const __half2 *>(&sw[k]));
                     const float2 zf = __half22float2(*reinterpret_cast<const __half2 *>(&zw[k]));
-                    sc2[k] = pk2(sf.x, sf.y);
-                    zr2[k] = pk2(zf.x, zf.y);
+                    sc2[k] = pack2(sf.x, sf.y);
+                    zr2[k] = pack2(zf.x, zf.y);
                 }
             } else {
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     const float4 s4 = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(scales) + base) + i);
                     const float4 z4 = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(zeros) + base) + i);
-                    sc2[2 * i] = pk2(s4.x, s4.y); sc2[2 * i + 1] = pk2(s4.z, s4.w);
-                    zr2[2 * i] = pk2(z4.x, z4.y); zr2[2 * i + 1] = pk2(z4.z, z4.w);
+                    sc2[2 * i] = pack2(s4.x, s4.y); sc2[2 * i + 1] = pack2(s4.z, s4.w);
+                    zr2[2 * i] = pack2(z4.x, z4.y); zr2[2 * i + 1] = pack2(z4.z, z4.w);
                 }
             }
         }
@@ -400,8 +391,8 @@ __global__ void __launch_bounds__(256) dequant_kernel(
                     s1 = __ldg(reinterpret_cast<const float *>(scales) + mi);
                     z1 = __ldg(reinterpret_cast<const float *>(zeros) + mi);
                 }
-                s2 = pk2(s1, s1);
-                z2 = pk2(z1, z1);
+                s2 = pack2(s1, s1);
+                z2 = pack2(z1, z1);
             }
             const uint32_t lo = cw[tt], hi = cw[tt] >> 16;        // 4-bit codes: channels 4..7 sit in the upper half
             u64 c2[CH / 2], y2[CH / 2];
@@ -410,14 +401,14 @@ __global__ void __launch_bounds__(256) dequant_kernel(
             c2[2] = codes_pair<BITS, 2>(lo, hi, bias2[2]);
             c2[3] = codes_pair<BITS, 3>(lo, hi, bias2[3]);
 #pragma unroll
-            for (int i = 0; i < CH / 2; ++i) y2[i] = KEYS ? fma2(c2[i], sc2[i], zr2[i]) : fma2(c2[i], s2, z2);
+            for (int i = 0; i < CH / 2; ++i) y2[i] = KEYS ? ffma2(c2[i], sc2[i], zr2[i]) : ffma2(c2[i], s2, z2);
             char *op_t = op0 + tt * ostep;
             if (OUT_BF16) {
                 uint32_t pk[CH / 2];
 #pragma unroll
                 for (int i = 0; i < CH / 2; ++i) {
                     float a, b_;
-                    unpk2(y2[i], a, b_);
+                    unpack2(y2[i], a, b_);
                     __nv_bfloat162 p2 = __floats2bfloat162_rn(a, b_);
                     pk[i] = *reinterpret_cast<uint32_t *>(&p2);
                 }
@@ -427,8 +418,8 @@ __global__ void __launch_bounds__(256) dequant_kernel(
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
                     float a, b_, c, e;
-                    unpk2(y2[2 * i], a, b_);
-                    unpk2(y2[2 * i + 1], c, e);
+                    unpack2(y2[2 * i], a, b_);
+                    unpack2(y2[2 * i + 1], c, e);
                     op[i] = make_float4(a, b_, c, e);
                 }
             }
