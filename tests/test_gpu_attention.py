@@ -313,3 +313,30 @@ def test_readers_over_a_cache_with_16_bit_metadata(bits, G, qpk, T, R):
     print("max err", _check(out, qn, units, H, G, kr, vr))
     out = _run_pre(q, cache, H, T, bits, G, 64, 64 + T + R, k_res, v_res)      # keys stored before it
     print("max err (pre)", _check_pre(out, qn, units, H, G, 64, kr, vr))
+
+
+# ---------------------------------------------------------------------------------------------------------
+# The C entry points for float32 metadata, which the binding reaches through the general one: the same bytes.
+
+def test_c_entry_points_of_the_readers():
+    lib = sq.binding._load()
+    B, H, T, bits, G, R, Hq = 2, 2, 320, 2, 32, 7, 4
+    cache, _ = _oracle_cache(21, B, H, T, bits, G)
+    g = torch.Generator().manual_seed(4)
+    q = torch.randn(B, Hq, D, generator=g).cuda()
+    k_res, v_res = (torch.randn(B, H, R, D, generator=g).to(torch.bfloat16).cuda() for _ in range(2))
+    out = torch.empty((B, Hq, D), dtype=torch.float32, device="cuda")
+    ws = torch.empty(lib.squat_decode_attention_workspace_bytes(B, Hq, T), dtype=torch.uint8, device="cuda")
+    table = sq.squat_rope_table(512).cuda()
+    first = [q.data_ptr(), sq.SQUAT_F32, B, Hq, H, D, *(x.data_ptr() for x in cache), T, H * T, T, bits, G,
+             k_res.data_ptr(), v_res.data_ptr(), sq.SQUAT_BF16, R, 0.05]
+    last = [out.data_ptr(), ws.data_ptr(), ws.numel(), sq.binding._stream()]
+    assert lib.squat_decode_attention(*first, *last) == 0
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy().astype(np.float64), _run(q, cache, H, T, bits, G, k_res, v_res, scale=0.05))
+    first[-1] = 0.0
+    assert lib.squat_decode_attention_pre_rope(*first, table.data_ptr(), 512, 64, *last) == 0
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy().astype(np.float64), _run_pre(q, cache, H, T, bits, G, 64, 512, k_res, v_res))
+    assert lib.squat_decode_attention(*first[:4], 0, *first[5:], *last) != 0
+    assert lib.squat_decode_attention_pre_rope(*first, table.data_ptr(), 512, 8, *last) != 0         # not a multiple of 32
