@@ -287,8 +287,9 @@ __global__ void __launch_bounds__(TRI_THREADS, 1) tridiag_kernel(
 // mu_i keeps its relative accuracy; the weights z are then recomputed from the roots (Gu and Eisenstat), for which the
 // computed roots are exact, and the vectors z_j / (d_j - lambda_i) come out orthogonal to working precision.
 // Nothing is deflated: neighbouring d are pushed at least DC_SEP apart (a few units in the last place of ||T||) and |z| is
-// kept above DC_ZMIN instead.  Both are backward errors of the size that any eigensolver commits, and the work does not
-// depend on the data.
+// kept above DC_ZMIN instead, so the work does not depend on the data.  The pushes are backward errors; they add up over the
+// copies of a multiple eigenvalue and over the merges, to at most (1 + 3 + 7 + .. + 127) DC_SEP = 2.2e-13 of ||T|| (measured on
+// a multiple of the identity: 1.5e-13; on simple spectra eigenvalues and residuals are within 2.4e-15).
 //
 // Four CTAs work on a head.  Each solves a 32 x 32 diagonal block alone (rotations to 2, merges to 4, 8, .. 32), two share a merge to 64
 // and four the one to 128; a CTA always owns 32 roots, eight lanes each, and the 32 eigenvectors that belong to them.
@@ -332,7 +333,8 @@ static_assert(sizeof(DcShared) <= 227 * 1024, "one CTA's shared memory");
 __device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // One root of 1/rho + sum_j z_j^2 / (d_j - lambda) in (d_i, d_{i+1}) (beyond d_{n-1}: up to rho |z|^2), by eight lanes.
-// Start: the two nearest poles kept exactly, the rest frozen at the middle of the interval.  Then the "middle way": both
+// Start: the two nearest poles kept exactly, the rest frozen at the middle of the interval.  Then the "middle way" of
+// R.-C. Li ("Solving secular equations stably and efficiently", 1993), from which this start is taken too: both
 // sums replaced by one pole each that matches value and slope, whose root is a quadratic's; a step that leaves the bracket
 // or (every fifth) one that has not paid is replaced by a bisection, geometric where the bracket spans orders of magnitude.
 template <int N>

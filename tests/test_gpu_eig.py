@@ -50,8 +50,11 @@ def test_eigen_pairs(kind):
         mu, V = out["eigval"][h], out["eigvec"][h]                    # rows of V
         ref = np.linalg.eigvalsh(both[h])[::-1]
         top = ref[0]
-        assert np.all(np.diff(mu) <= 0.0) and np.abs(mu - np.maximum(ref, 0.0)).max() <= 2e-12 * top
-        assert np.abs(V @ V.T - np.eye(D)).max() <= 1e-13
-        assert np.abs((both[h] / top) @ V.T - V.T * (mu / top)).max() <= 2e-12
+        # Simple spectra: four times the 2.4e-15 that is observed.  Multiple or clustered eigenvalues are pushed 2^-50 of the norm
+        # apart, copy by copy and in each of the seven merges: (1 + 3 + 7 + .. + 127) 2^-50 = 2.2e-13 at most, and their rounding.
+        tol = 1e-14 if kind in ("diagonal", "tridiagonal", "1e-70", "1e80") else 2.2e-13 + 3e-14
+        assert np.all(np.diff(mu) <= 0.0) and np.abs(mu - np.maximum(ref, 0.0)).max() <= tol * top
+        assert np.abs(V @ V.T - np.eye(D)).max() <= 1e-14                            # observed: 2.5e-15
+        assert np.abs((both[h] / top) @ V.T - V.T * (mu / top)).max() <= tol
     assert sq.squat_get_device_status(clear=True) & sq.FLAG_NO_CONVERGE == 0
     s.close()
