@@ -67,6 +67,27 @@ def test_gram_is_exact(H, qpk, T, data):
     s.close()
 
 
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+def test_elements_that_are_not_finite_stay_in_their_head_and_channel(bad):
+    H, T = 2, 24600
+    q = torch.randn((H, T, D), generator=torch.Generator().manual_seed(9)).to(torch.bfloat16)
+    q[0, 777, 5] = bad
+    s = sq.Subspace(H, D)
+    sq.squat_build_subspace(s, q.cuda(), 8, 1e-3)
+    a = sq.squat_subspace_export(s, ("gram",))["gram"]
+    x = q.double().numpy()
+    x[0, 777, 5] = 0.0
+    ok = np.ones((H, D, D), bool)
+    ok[0, 5] = ok[0, :, 5] = False
+    assert not np.isfinite(a[~ok]).any()
+    for h in range(H):
+        ref = _gram(x[h])
+        size = np.sqrt(np.outer(np.diag(ref), np.diag(ref))).astype(np.float64)
+        assert np.all((np.abs((a[h] - ref).astype(np.float64)) <= 4e-15 * size)[ok[h]])
+    sq.squat_get_device_status(clear=True)
+    s.close()
+
+
 @pytest.mark.parametrize("H,qpk,T,stride_h,stride_t", [
     (1, 1, 49200, 0, 1 << 19), (1, 2, 24700, 24700 << 19, 1 << 19), (1, 3, 16500, 1 << 33, 128), (2, 1, 24700, 1 << 34, 128)])
 def test_views_spread_over_more_than_32_gigabytes(H, qpk, T, stride_h, stride_t):
