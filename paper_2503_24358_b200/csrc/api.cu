@@ -47,8 +47,15 @@ int check_quant_args(const void *x, int dtype, int batch, int H, int T, int d, l
     return SQUAT_OK;
 }
 
+// The form for block updates (keys_block.cu) reads the same image of W as the dense kernel and relies on its zero diagonal
+// blocks of g channels.  W = 0 (no subspace) stays on the dense kernel: every block of it takes the exact rounding decision.
+int block_form(int rank_r, double lambda, int block_g)
+{
+    return (block_g == 32 || block_g == 64) && rank_r > 0 && lambda != 0.0 ? block_g : 0;
+}
+
 // The rank-r form of the update (keys_lowrank.cu) exists for element-wise updates with a small rank: its tables are
-// made from the eigen-pairs right after the eigensolver.  Every other build leaves the handle on the dense kernel.
+// made from the eigen-pairs right after the eigensolver.
 int lowrank_tables_if_small(squat_subspace *s, int rank_r, double lambda, int block_g, cudaStream_t st)
 {
     s->lowrank_r = 0;
@@ -215,6 +222,7 @@ int squat_build_subspace(squat_subspace *s, const void *q, int dtype, int n_q_he
     if (rc != SQUAT_OK) return rc;
     rc = lowrank_tables_if_small(s, rank_r, lambda, block_g, st);
     if (rc != SQUAT_OK) return rc;
+    s->block_g = block_form(rank_r, lambda, block_g);
     // channels of the first g-block are never corrected; with r = 0 or lambda = 0, W = 0 and none is
     const int exact = (rank_r == 0 || lambda == 0.0) ? D / 32 : (block_g + 31) / 32;
     return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
@@ -235,6 +243,7 @@ int squat_build_subspace_from_gram(squat_subspace *s, const double *gram, int ra
     if (rc != SQUAT_OK) return rc;
     rc = lowrank_tables_if_small(s, rank_r, lambda, block_g, st);
     if (rc != SQUAT_OK) return rc;
+    s->block_g = block_form(rank_r, lambda, block_g);
     const int exact = (rank_r == 0 || lambda == 0.0) ? D / 32 : (block_g + 31) / 32;
     return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
 }
@@ -261,7 +270,8 @@ int squat_build_subspace_power(squat_subspace *s, const void *q, int dtype, int 
     int rc = squat_launch_gram(s, q, dtype, n_q_heads, n_tokens, stride_h, stride_t, st);
     if (rc != SQUAT_OK) return rc;
     const bool no_update = rank_r == 0 || lambda == 0.0;
-    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis: dense kernel
+    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
+    s->block_g = block_form(rank_r, lambda, block_g);
     const int exact = no_update ? D / 32 : (block_g + 31) / 32;
     if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);      // W = 0: nothing to iterate
     rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
@@ -285,7 +295,8 @@ int squat_build_subspace_power_from_gram(squat_subspace *s, const double *gram, 
     if (gram != s->gram)
         SQUAT_CUDA(cudaMemcpyAsync(s->gram, gram, (size_t)s->n_kv_heads * D * D * sizeof(double), cudaMemcpyDeviceToDevice, st));
     const bool no_update = rank_r == 0 || lambda == 0.0;
-    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis: dense kernel
+    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
+    s->block_g = block_form(rank_r, lambda, block_g);
     const int exact = no_update ? D / 32 : (block_g + 31) / 32;
     if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);
     int rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
@@ -354,7 +365,7 @@ int squat_subspace_import(squat_subspace *s, const float *W_host, void *stream)
             for (int j = 0; j < D; ++j)
                 if (W_host[((size_t)h * D + jp) * D + j] != 0.0f) { uncorrected = jp; break; }
     const int exact = (uncorrected + 31) / 32;
-    s->lowrank_r = 0;                      // an imported W comes without its factors: dense kernel
+    s->lowrank_r = s->block_g = 0;         // an imported W comes without its factors or block size: dense kernel
     SQUAT_CUDA(cudaMemcpyAsync(s->Wt, wt.data(), hdd * sizeof(float), cudaMemcpyHostToDevice, st));
     int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, s->exact_blocks, st);
     if (rc != SQUAT_OK) return rc;
@@ -383,6 +394,10 @@ int quantize_keys_impl(const squat_subspace *s, const void *k, int dtype, int ba
         return squat_launch_quant_keys_lowrank(s->lr_table, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t,
                                                bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
                                                meta16, static_cast<cudaStream_t>(stream));
+    if (s->block_g > 0 && !s->prefer_dense)
+        return squat_launch_quant_keys_block(s->block_g, s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t,
+                                             bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
+                                             meta16, static_cast<cudaStream_t>(stream));
     return squat_launch_quant_keys(s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t, bits,
                                    group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status, s->exact_blocks,
                                    meta16, static_cast<cudaStream_t>(stream));

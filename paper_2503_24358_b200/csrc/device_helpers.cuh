@@ -26,6 +26,12 @@ __device__ __forceinline__ u64 fmul2(u64 a, u64 b)
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ u64 fadd2(u64 a, u64 b)
+{
+    u64 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ u64 fsub2(u64 a, u64 b)
 {
     u64 d;
@@ -58,6 +64,18 @@ __device__ __forceinline__ float max_nan(float a, float b)
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
+}
+
+// packed bf16 pairs
+__device__ __forceinline__ unsigned hmin2_nan_bits(unsigned a, unsigned b)
+{
+    const __nv_bfloat162 r = __hmin2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
+    return *reinterpret_cast<const unsigned *>(&r);
+}
+__device__ __forceinline__ unsigned hmax2_nan_bits(unsigned a, unsigned b)
+{
+    const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
+    return *reinterpret_cast<const unsigned *>(&r);
 }
 
 // ---- tensor cores and mbarriers

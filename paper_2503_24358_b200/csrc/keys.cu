@@ -35,15 +35,9 @@
 //
 // Work per key vector: 8128 fp32 multiply-adds (dense triangle, g = 1): 1984 on the CUDA cores
 // (sweeps: four triangles of 32 * 31 / 2), 6144 x 3 tf32 products on the tensor cores.
-#include "device_helpers.cuh"
-#include <cuda_fp16.h>
+#include "keys_common.cuh"
 
 namespace {
-
-constexpr int D = SQUAT_D;
-constexpr int BLK = 32;                   // channels per block
-constexpr int NBLK = D / BLK;             // 4
-constexpr float kMagic = 12582912.0f;     // 1.5 * 2^23
 
 constexpr int TC_SLOTS = 4;                          // 128-token tiles in flight per CTA
 constexpr int TC_WARPS = TC_SLOTS * 4;
@@ -53,44 +47,8 @@ constexpr int TC_EHI_COL = 96;
 constexpr int TC_TMEM_COLS = 512;
 static_assert(TC_SLOTS * TC_COLS_PER_TILE <= TC_TMEM_COLS, "tensor memory has 512 columns");
 constexpr int TC_E_FLOATS = 128 * BLK;               // one tile's E_hi (or E_lo): 128 rows x 32 channels
-constexpr int TC_DIAG_FLOATS = NBLK * BLK * BLK;     // four 32 x 32 diagonal blocks of W^T
-constexpr int TC_PANEL_FLOATS = BLK * (3 * BLK + 2 * BLK + BLK);     // panels of source blocks 0..2: (96 - 32 b) x 32
-constexpr int TC_IMG_FLOATS = TC_DIAG_FLOATS + 2 * TC_PANEL_FLOATS;  // = d * d: diag | hi panels | lo panels
-static_assert(TC_IMG_FLOATS == D * D, "the staged image of W has the size of W");
 constexpr unsigned TC_A_LBO = 128 * 16, TC_SBO = 128;                 // bytes
-__host__ __device__ constexpr int tc_panel_off(int b) { return b == 0 ? 0 : (b == 1 ? 3 * BLK * BLK : 5 * BLK * BLK); }
-// instruction descriptor: fp32 accumulator, tf32 A and B, both K-major, N = n, M = 128
-__host__ __device__ constexpr unsigned tc_idesc(int n) { return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24); }
 
-
-__device__ __forceinline__ float min3_nan(float a, float b, float c)
-{
-    float r;
-    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-__device__ __forceinline__ float max3_nan(float a, float b, float c)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-__device__ __forceinline__ void team_barrier(int id, int nthreads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-// Correctly rounded  rng / L  for L = 3 or 15 (q' = q + (rng - L q) * RN(1/L); checked against
-// true division over full mantissa ranges on the host).
-template <int BITS>
-__device__ __forceinline__ float div_by_levels(float rng)
-{
-    constexpr float L = float((1 << BITS) - 1);
-    constexpr float invL = 1.0f / L;
-    const float q = __fmul_rn(rng, invL);
-    const float r = __fmaf_rn(-L, q, rng);
-    return __fmaf_rn(r, invL, q);
-}
 
 // ---- tcgen05 / tensor-memory helpers (5th-generation tensor cores) -------------------------------------------
 __device__ __forceinline__ unsigned tf32_of(float x)             // round to nearest tf32 (10 mantissa bits)
@@ -99,32 +57,7 @@ __device__ __forceinline__ unsigned tf32_of(float x)             // round to nea
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return r;
 }
-// 32 consecutive columns of the warp's lanes into registers (lane l gets row l)
-__device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-// shared-memory matrix descriptor, no swizzle, K-major: 8 x 16-byte core matrices, lbo bytes between the two
-// halves of a K step, sbo bytes between groups of 8 rows
-__device__ __forceinline__ u64 umma_desc(unsigned addr, unsigned lbo, unsigned sbo)
-{
-    return (u64)((addr & 0x3FFFF) >> 4) | ((u64)(lbo >> 4) << 16) | ((u64)(sbo >> 4) << 32) | (1ull << 46);
-}
-// D[128 x N] (+)= A[128 x 8] * B[N x 8]^T, tf32 operands from shared memory, fp32 accumulation in tensor memory
-__device__ __forceinline__ void umma_tf32_ss(unsigned d_taddr, u64 a_desc, u64 b_desc, unsigned idesc, unsigned accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_taddr), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// the same with A from tensor memory (rows = lanes, 8 consecutive 32-bit columns)
+// umma_tf32_ss with A from tensor memory (rows = lanes, 8 consecutive 32-bit columns)
 __device__ __forceinline__ void umma_tf32_ts(unsigned d_taddr, unsigned a_taddr, u64 b_desc, unsigned idesc, unsigned accumulate)
 {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"

@@ -28,7 +28,9 @@ struct squat_subspace {
     float *lr_table;       // [H, d, 2 * SQUAT_LOWRANK_MAX_R] rows [v_j | c_j] of the rank-r form of W (keys_lowrank.cu)
     int lowrank_r;         // > 0: lr_table describes the same update as Wt (set by the SVD builds with g = 1 and a small rank);
                            // host-side, read when a key call is enqueued: calls on one handle are issued in execution order
-    int prefer_dense;      // 1: squat_quantize_keys uses the dense kernel even when lr_table is valid
+    int block_g;           // 32 or 64: W comes from block updates of that many channels, so its diagonal blocks are zero and the
+                           // kernel of keys_block.cu applies; 0 otherwise (host-side, like lowrank_r)
+    int prefer_dense;      // 1: squat_quantize_keys uses the dense kernel even when one of the other two forms applies
     double *gram;          // [H, d, d] Gram matrices
     double *gram_partial;  // [chunks, H, d, d] per-chunk partial Gram matrices (deterministic reduction)
     unsigned *gram_max;    // [H, gram_chunks_cap, d / 2], rem_count [H], rem [H, SQUAT_GRAM_REM_CAP]: see gram_i8.cu
@@ -114,6 +116,10 @@ int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int bat
                             long long sb, long long sh, long long st_, int bits, int G,
                             unsigned char *codes, void *scales, void *zeros,
                             long long osb, long long osh, unsigned *status, const int *exact_blocks_dev, int meta16, cudaStream_t st);
+int squat_launch_quant_keys_block(int block_g, const float *Wimg, const void *k, int dtype, int batch, int H, int T,
+                                  long long sb, long long sh, long long st_, int bits, int G,
+                                  unsigned char *codes, void *scales, void *zeros,
+                                  long long osb, long long osh, unsigned *status, int meta16, cudaStream_t st);
 int squat_launch_quant_values(const void *v, int dtype, int batch, int H, int T, int d,
                               long long sb, long long sh, long long st_, int bits, int G,
                               unsigned char *codes, void *scales, void *zeros,

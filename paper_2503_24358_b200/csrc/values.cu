@@ -26,18 +26,6 @@ namespace {
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer (ties to even)
 constexpr unsigned kMagicBits = 0x4B400000u;
 
-
-__device__ __forceinline__ unsigned hmin2_nan_bits(unsigned a, unsigned b)
-{
-    const __nv_bfloat162 r = __hmin2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
-    return *reinterpret_cast<const unsigned *>(&r);
-}
-__device__ __forceinline__ unsigned hmax2_nan_bits(unsigned a, unsigned b)
-{
-    const __nv_bfloat162 r = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
-    return *reinterpret_cast<const unsigned *>(&r);
-}
-
 // Correctly rounded  rng / L  for L = 3 or 15 and rng, rng / L in the normal range (q' = q + (rng - L q) * RN(1/L)).
 template <int BITS>
 __device__ __forceinline__ float div_by_levels(float rng)
