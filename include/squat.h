@@ -171,8 +171,9 @@ int squat_quantize_keys(const squat_subspace *s, const void *k, int dtype, int b
  * trailing blocks of P): a token then carries a state of r numbers and the update costs 2 r d multiply-adds per key
  * vector instead of d (d - 1) / 2.  squat_build_subspace and squat_build_subspace_from_gram prepare that form when
  * block_g = 1, lambda > 0 and 1 <= rank_r <= 8, and squat_quantize_keys / _m16 then use it (FP32 pipes only, no
- * tensor-core hand-over); every other build, and an imported W, runs the dense kernel.  Both compute the same
- * function Quant; results agree up to rounding ties.
+ * tensor-core hand-over).  Block updates of 32 or 64 channels (block_g, rank_r > 0, lambda > 0) have zero diagonal blocks in W
+ * and run a kernel that quantizes a block at a time.  Every other build, and an imported W, runs the dense kernel.  All
+ * compute the same function Quant; results agree up to rounding ties.
  *   prefer_dense   1: always run the dense kernel;  0: the default choice above.
  *   lowrank_rank   host, may be NULL: receives the rank the rank-r form is prepared for (0: not prepared).
  * Host-side state of the handle: like every call that takes the handle, issue it from one thread at a time, in the

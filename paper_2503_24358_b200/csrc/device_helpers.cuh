@@ -93,16 +93,21 @@ __device__ __forceinline__ void mma_i8(unsigned d_taddr, u64 a_desc, u64 b_desc,
                  " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
                  ::"r"(d_taddr), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// Bounded wait for a phase of an mbarrier: false when the limit ran out (the caller records it and moves on).
+// Bounded wait for a phase of an mbarrier: false when the limit ran out (the caller records it and moves on).  The polls branch on
+// the instruction's own predicate, four to a count: waiting warps poll often enough to take issue slots from working ones.
 __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
 {
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-        if (done) return true;
-    }
-    return false;
+    unsigned done;
+    asm volatile("{\n .reg .pred p;\n .reg .u32 n;\n mov.u32 n, 0x100000;\n"
+                 "POLL:\n"
+                 " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n @p bra DONE;\n"
+                 " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n @p bra DONE;\n"
+                 " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n @p bra DONE;\n"
+                 " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n @p bra DONE;\n"
+                 " sub.u32 n, n, 1;\n setp.ne.u32 p, n, 0;\n @p bra POLL;\n"
+                 "DONE:\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
+    return done;
 }
 
 // ---- fp64

@@ -23,8 +23,10 @@
 //
 // Bound: bytes first (304 per key vector with bf16 keys, 2 bits, G = 32, 16-bit scales), then the errors' trip through shared
 // memory (8 B written, 12 B read by the tensor core per element).  Measured against the kernel of keys.cu, which walks the chain
-// of the element-wise form whatever g is: 16 x 8 heads x 8160 tokens, 2 bits, G = 32, 16-bit scales 365 -> 139 us at g = 64 and
-// 357 -> 175 at g = 32; 4 bits, G = 128, g = 64 462 -> 150; 32 heads x 4096 48 -> 23; one window of 32 heads x 128 15.2 -> 6.6.
+// of the element-wise form whatever g is: 16 x 8 heads x 8160 tokens, 2 bits, G = 32, 16-bit scales 365 -> 130 us at g = 64 and
+// 357 -> 159 at g = 32; 4 bits, G = 128, g = 64 462 -> 142; 32 heads x 4096 48 -> 23; one window of 32 heads x 128 15.2 -> 6.6.
+// What is left (ablations, g = 64): the wait for the products 27 us, the errors' stores 17, exact decisions 5; asking L2 for the
+// next unit's keys ahead changed nothing, so it is the latency of a unit's steps at 16 warps per SM, not the loads.
 // No size was found where the other kernel is faster, so every handle built with such a g comes here.
 #include "keys_common.cuh"
 
@@ -99,11 +101,6 @@ struct QuadRows {
     }
 };
 
-// Grids of a thread's 4 channels
-struct Grid4 {
-    float m[4], scale[4], inv[4];
-};
-
 // Per-lane selectors of the transpositions below, fixed for the thread
 struct CodeLanes {
     bool up4;                       // lane holds the upper four tokens after the first exchange
@@ -166,70 +163,81 @@ __device__ __forceinline__ uint4 transpose_codes4(const unsigned (&w)[4], const 
                       __byte_perm(k1, r1, c.out & 0xffffu), __byte_perm(k1, r1, c.out >> 16));
 }
 
-// The exact decision of one element of an uncorrected block (see sweep_block in keys.cu): y is replaced, and the error with it.
-template <int BITS, bool M16>
-__device__ __forceinline__ void decide_exactly(float nd, float scale, float inv, float &y, float &e)
+// The exact decision of one element of an uncorrected block whose remainder e is close to half a step (see sweep_block in
+// keys.cu): y, the rounded float, moves by one where the remainder says so, and the error with it.
+template <int BITS, bool CLAMP>
+__device__ __forceinline__ void decide_exactly(float nd, float scale, float neg_inv, float &y, float &e)
 {
     constexpr float L = float((1 << BITS) - 1);
-    const float y0 = __fmaf_rn(nd, -inv, kMagic);
-    float c = __fsub_rn(y0, kMagic);
-    const float e0 = __fmaf_rn(c, scale, nd);
-    const float thr = __uint_as_float(__float_as_uint(0.5f * scale) - (__float_as_uint(y0) & 1u));
-    c = __fadd_rn(c, e0 > thr ? -1.0f : (e0 < -thr ? 1.0f : 0.0f));
-    if (M16) c = fminf(fmaxf(c, 0.0f), L);
-    y = __fadd_rn(c, kMagic);
-    e = __fmaf_rn(c, scale, nd);
+    if (CLAMP) {                                            // from the unclamped value
+        y = __fmaf_rn(nd, neg_inv, kMagic);
+        e = __fmaf_rn(__fsub_rn(y, kMagic), scale, nd);
+    }
+    const float thr = __uint_as_float(__float_as_uint(0.5f * scale) - (__float_as_uint(y) & 1u));
+    const float adj = e > thr ? -1.0f : (e < -thr ? 1.0f : 0.0f);
+    y = __fadd_rn(y, adj);
+    e = __fmaf_rn(adj, scale, e);
+    if (CLAMP) {
+        const float c = fminf(fmaxf(y, kMagic), kMagic + L);
+        e = c == y ? e : __fmaf_rn(__fsub_rn(c, kMagic), scale, nd);
+        y = c;
+    }
 }
+
+// Grids of a thread's 4 channels, as pairs
+struct Grid4 {
+    u64 m[2], scale[2], neg_inv[2];
+};
 
 // Codes of the thread's 4 channels x 8 tokens, and (STORE_E) the errors to the tile's E operands, a 16-byte row per token.
 // EXACT: uncorrected inputs, where exact ties are structural: an element whose remainder is within 1e-4 of half a step is
 // decided through that remainder as real arithmetic on the stored scale would; a row with such an element is looked at again.
-template <int BITS, bool M16, bool EXACT, bool STORE_E>
+// CLAMP: grids whose 16-bit zero-point or scale leaves an extreme half a step or more outside [0, L].
+template <int BITS, bool CLAMP, bool EXACT, bool STORE_E>
 __device__ __forceinline__ void quantize_quads(const u64 (&x)[KB_ROWS][2], const Grid4 &g, float *e_hi, float *e_lo, unsigned (&cw)[BITS])
 {
     constexpr float L = float((1 << BITS) - 1);
-    const u64 m01 = pack2(g.m[0], g.m[1]), m23 = pack2(g.m[2], g.m[3]);
-    const u64 s01 = pack2(g.scale[0], g.scale[1]), s23 = pack2(g.scale[2], g.scale[3]);
-    const u64 i01 = pack2(-g.inv[0], -g.inv[1]), i23 = pack2(-g.inv[2], -g.inv[3]);
     const u64 magic2 = pack2(kMagic, kMagic);
     float thr[4];
     if (EXACT) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) thr[j] = 0.4999f * g.scale[j];
+        for (int j = 0; j < 2; ++j) unpack2(fmul2(g.scale[j], pack2(0.4999f, 0.4999f)), thr[2 * j], thr[2 * j + 1]);
     }
 #pragma unroll
     for (int i = 0; i < KB_ROWS; ++i) {
-        const u64 n01 = fsub2(m01, x[i][0]), n23 = fsub2(m23, x[i][1]);        // -(x - m)
-        float y[4];
-        unpack2(ffma2(n01, i01, magic2), y[0], y[1]);
-        unpack2(ffma2(n23, i23, magic2), y[2], y[3]);
-        if (M16) {                                          // rounded metadata: t may leave [0, L]
+        u64 n[2], y[2], e[2];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) y[j] = fminf(fmaxf(y[j], kMagic), kMagic + L);
+        for (int j = 0; j < 2; ++j) {
+            n[j] = fsub2(g.m[j], x[i][j]);                  // -(x - m)
+            y[j] = ffma2(n[j], g.neg_inv[j], magic2);
+            if (CLAMP) y[j] = pack2(fminf(fmaxf(lo_of(y[j]), kMagic), kMagic + L), fminf(fmaxf(hi_of(y[j]), kMagic), kMagic + L));
+            if (EXACT || STORE_E) e[j] = ffma2(fsub2(y[j], magic2), g.scale[j], n[j]);
         }
-        if (EXACT || STORE_E) {
-            float e[4];
-            unpack2(ffma2(fsub2(pack2(y[0], y[1]), magic2), s01, n01), e[0], e[1]);
-            unpack2(ffma2(fsub2(pack2(y[2], y[3]), magic2), s23, n23), e[2], e[3]);
-            if (EXACT && (fabsf(e[0]) > thr[0] || fabsf(e[1]) > thr[1] || fabsf(e[2]) > thr[2] || fabsf(e[3]) > thr[3])) {
-                float nd[4];
-                unpack2(n01, nd[0], nd[1]);
-                unpack2(n23, nd[2], nd[3]);
+        if (EXACT && ((fabsf(lo_of(e[0])) > thr[0]) | (fabsf(hi_of(e[0])) > thr[1]) | (fabsf(lo_of(e[1])) > thr[2]) | (fabsf(hi_of(e[1])) > thr[3]))) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) decide_exactly<BITS, M16>(nd[j], g.scale[j], g.inv[j], y[j], e[j]);
+            for (int j = 0; j < 2; ++j) {
+                float y0, y1, e0, e1;
+                unpack2(y[j], y0, y1);
+                unpack2(e[j], e0, e1);
+                decide_exactly<BITS, CLAMP>(lo_of(n[j]), lo_of(g.scale[j]), lo_of(g.neg_inv[j]), y0, e0);
+                decide_exactly<BITS, CLAMP>(hi_of(n[j]), hi_of(g.scale[j]), hi_of(g.neg_inv[j]), y1, e1);
+                y[j] = pack2(y0, y1);
+                e[j] = pack2(e0, e1);
             }
-            if (STORE_E) {
-                // tf32 split by truncation: the tensor core reads the top 19 bits of a word, so e itself serves as E_hi
-                float l[4];
-                unpack2(fsub2(pack2(e[0], e[1]), pack2(__uint_as_float(__float_as_uint(e[0]) & 0xffffe000u), __uint_as_float(__float_as_uint(e[1]) & 0xffffe000u))), l[0], l[1]);
-                unpack2(fsub2(pack2(e[2], e[3]), pack2(__uint_as_float(__float_as_uint(e[2]) & 0xffffe000u), __uint_as_float(__float_as_uint(e[3]) & 0xffffe000u))), l[2], l[3]);
-                *reinterpret_cast<float4 *>(e_hi + i * 16) = make_float4(e[0], e[1], e[2], e[3]);
-                *reinterpret_cast<float4 *>(e_lo + i * 16) = make_float4(l[0], l[1], l[2], l[3]);
-            }
+        }
+        if (STORE_E) {
+            // tf32 split by truncation: the tensor core reads the top 19 bits of a word, so e itself serves as E_hi
+            ulonglong2 hi, lo;
+            hi.x = e[0];
+            hi.y = e[1];
+            lo.x = fsub2(e[0], e[0] & 0xffffe000ffffe000ull);
+            lo.y = fsub2(e[1], e[1] & 0xffffe000ffffe000ull);
+            *reinterpret_cast<ulonglong2 *>(e_hi + i * 16) = hi;
+            *reinterpret_cast<ulonglong2 *>(e_lo + i * 16) = lo;
         }
         // the low bits of a rounded float are its code; what is shifted in from above stays out of the 4 * BITS bits used
-        const unsigned a = (__float_as_uint(y[1]) << BITS) + __float_as_uint(y[0]);
-        const unsigned b = (__float_as_uint(y[3]) << BITS) + __float_as_uint(y[2]);
+        const unsigned a = ((unsigned)(y[0] >> 32) << BITS) + (unsigned)y[0];
+        const unsigned b = ((unsigned)(y[1] >> 32) << BITS) + (unsigned)y[1];
         const unsigned c4 = (b << (2 * BITS)) + a;
         if (BITS == 2) {                                    // byte i
             unsigned &d = cw[i >> 2];
@@ -241,27 +249,25 @@ __device__ __forceinline__ void quantize_quads(const u64 (&x)[KB_ROWS][2], const
     }
 }
 
+// The grid of one channel: m becomes the stored zero-point; returns whether a code could leave [0, L].
 template <int BITS, bool M16, bool EXACT>
-__device__ __forceinline__ void make_grid4(float (&mn)[4], const float (&mx)[4], Grid4 &g)
+__device__ __forceinline__ bool make_grid(float &m, float mx, float &scale, float &inv)
 {
     constexpr float L = float((1 << BITS) - 1);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float rng = __fsub_rn(mx[j], mn[j]);
-        float scale = EXACT ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);      // as in keys.cu
-        float rcp;
-        if (M16) {
-            scale = __half2float(__float2half_rn(scale));
-            g.m[j] = __half2float(__float2half_rn(mn[j]));
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(scale));
-            g.inv[j] = scale > 0.0f ? rcp : 0.0f;                                       // scale 0 (no range, or underflow): codes 0
-        } else {
-            g.m[j] = mn[j];
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(fmaxf(rng, 1e-30f)));    // constant group: x - m = 0 -> code 0
-            g.inv[j] = __fmul_rn(rcp, L);
-        }
-        g.scale[j] = scale;
+    const float rng = __fsub_rn(mx, m);
+    scale = EXACT ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);                // as in keys.cu
+    float rcp;
+    if (!M16) {
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(fmaxf(rng, 1e-30f)));        // constant group: x - m = 0 -> code 0
+        inv = __fmul_rn(rcp, L);
+        return false;
     }
+    const float lo = m;
+    scale = __half2float(__float2half_rn(scale));
+    m = __half2float(__float2half_rn(m));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(scale));
+    inv = scale > 0.0f ? rcp : 0.0f;                                                    // scale 0 (no range, or underflow): codes 0
+    return !(__fsub_rn(lo, m) >= -0.49f * scale && __fsub_rn(mx, m) <= (L + 0.49f) * scale);
 }
 
 template <int BITS, int NW, bool BF16, bool M16, int GB>
@@ -348,7 +354,7 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                                   // group and store nothing)
         const char *row;          // the thread's first token at its quad of block 0
         unsigned char *codes;     // code row of the token the thread stores (4 q + s)
-        long long meta;           // offset of the group's scales / zeros at the quad of block 0
+        long long meta;           // offset of the group's scales / zeros at the lane's own channel of block 0
     };
     auto locate = [&](int unit, Place &t) {
         const int h = unit / p.units_per_head;
@@ -361,7 +367,7 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
         const int tok0 = grp * G + wteam * 32;
         const long long out_tok0 = (long long)b * p.osb + (long long)h * p.osh;
         t.codes = p.codes + (out_tok0 + tok0 + 4 * q + s) * (D * BITS / 8) + half * (BLK * BITS / 8);
-        t.meta = (out_tok0 / G + grp) * D + half * BLK + 4 * q;
+        t.meta = (out_tok0 / G + grp) * D + half * BLK + 4 * q + s;
         const long long off = (long long)b * p.sb + (long long)h * p.sh + (long long)(tok0 + s) * p.st + half * BLK + 4 * q;
         t.row = static_cast<const char *>(p.k) + off * ES;
     };
@@ -403,7 +409,8 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
         for (int step = 0; step < Lay::STEPS; ++step) {
             const bool last = step + 1 == Lay::STEPS;
             u64 x[KB_ROWS][2];
-            float mn[4], mx[4];
+            float m, mx;                                 // extremes of the lane's own channel, 4 q + s: the quad's 4 lanes share out
+                                                         // their channels in two halving exchanges
             if (step == 0) {
                 if (BF16) {
                     unsigned a[2], b[2];
@@ -414,18 +421,13 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                         a[0] = hmin2_nan_bits(a[0], w.x); b[0] = hmax2_nan_bits(b[0], w.x);
                         a[1] = hmin2_nan_bits(a[1], w.y); b[1] = hmax2_nan_bits(b[1], w.y);
                     }
-#pragma unroll
-                    for (int o = 8; o < 32; o <<= 1)
-#pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            a[j] = hmin2_nan_bits(a[j], __shfl_xor_sync(0xffffffffu, a[j], o));
-                            b[j] = hmax2_nan_bits(b[j], __shfl_xor_sync(0xffffffffu, b[j], o));
-                        }
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        mn[2 * j] = bf16lo_to_f32(a[j]); mn[2 * j + 1] = bf16hi_to_f32(a[j]);
-                        mx[2 * j] = bf16lo_to_f32(b[j]); mx[2 * j + 1] = bf16hi_to_f32(b[j]);
-                    }
+                    const bool u = s & 2;
+                    unsigned ka = hmin2_nan_bits(u ? a[1] : a[0], __shfl_xor_sync(0xffffffffu, u ? a[0] : a[1], 16));
+                    unsigned kb = hmax2_nan_bits(u ? b[1] : b[0], __shfl_xor_sync(0xffffffffu, u ? b[0] : b[1], 16));
+                    ka = hmin2_nan_bits(ka, __shfl_xor_sync(0xffffffffu, ka, 8));
+                    kb = hmax2_nan_bits(kb, __shfl_xor_sync(0xffffffffu, kb, 8));
+                    m = (s & 1) ? bf16hi_to_f32(ka) : bf16lo_to_f32(ka);
+                    mx = (s & 1) ? bf16hi_to_f32(kb) : bf16lo_to_f32(kb);
                 }
 #pragma unroll
                 for (int i = 0; i < KB_ROWS; ++i) raw.get(i, x[i][0], x[i][1]);
@@ -462,66 +464,87 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                 }
             }
             // the keys of the next block, or of the next unit's first, are on their way from here on
-            if (!last) load_rows(cur.row + (step + 1) * (GB * ES));
-            else if (unit + 1 < u_hi) load_rows(nxt.row);
+            auto load_next = [&] {
+                if (!last) load_rows(cur.row + (step + 1) * (GB * ES));
+                else if (unit + 1 < u_hi) load_rows(nxt.row);
+            };
+            if (BF16) load_next();                       // float32 rows take the registers that x still needs: later (32-channel
+                                                         // blocks, 16-bit scales 111 -> 98 us for 8 x 8 heads x 8160)
             if (step != 0 || !BF16) {
-                float v[4];
-                unpack2(x[0][0], mn[0], mn[1]);
-                unpack2(x[0][1], mn[2], mn[3]);
+                float a[4], b[4], v[4];
+                unpack2(x[0][0], a[0], a[1]);
+                unpack2(x[0][1], a[2], a[3]);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mx[j] = mn[j];
+                for (int j = 0; j < 4; ++j) b[j] = a[j];
 #pragma unroll
                 for (int i = 1; i + 1 < KB_ROWS; i += 2) {
                     float w[4];
                     unpack2(x[i][0], v[0], v[1]); unpack2(x[i][1], v[2], v[3]);
                     unpack2(x[i + 1][0], w[0], w[1]); unpack2(x[i + 1][1], w[2], w[3]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) { mn[j] = min3_nan(mn[j], v[j], w[j]); mx[j] = max3_nan(mx[j], v[j], w[j]); }
+                    for (int j = 0; j < 4; ++j) { a[j] = min3_nan(a[j], v[j], w[j]); b[j] = max3_nan(b[j], v[j], w[j]); }
                 }
                 unpack2(x[KB_ROWS - 1][0], v[0], v[1]);
                 unpack2(x[KB_ROWS - 1][1], v[2], v[3]);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { mn[j] = min_nan(mn[j], v[j]); mx[j] = max_nan(mx[j], v[j]); }
+                for (int j = 0; j < 4; ++j) { a[j] = min_nan(a[j], v[j]); b[j] = max_nan(b[j], v[j]); }
+                const bool u = s & 2, w = s & 1;
 #pragma unroll
-                for (int o = 8; o < 32; o <<= 1)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        mn[j] = min_nan(mn[j], __shfl_xor_sync(0xffffffffu, mn[j], o));
-                        mx[j] = max_nan(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], o));
-                    }
-            }
-            if (NW > 1) {
-                // the team's warps trade their extremes through the first two rows of each chunk of their own E_hi rows (no
-                // product reads them now)
-                if (s == 0) {
-                    *reinterpret_cast<float4 *>(E_hi + e_mine) = make_float4(mn[0], mn[1], mn[2], mn[3]);
-                    *reinterpret_cast<float4 *>(E_hi + e_mine + 4) = make_float4(mx[0], mx[1], mx[2], mx[3]);
+                for (int j = 0; j < 2; ++j) {
+                    a[j] = min_nan(u ? a[j + 2] : a[j], __shfl_xor_sync(0xffffffffu, u ? a[j] : a[j + 2], 16));
+                    b[j] = max_nan(u ? b[j + 2] : b[j], __shfl_xor_sync(0xffffffffu, u ? b[j] : b[j + 2], 16));
                 }
+                m = min_nan(w ? a[1] : a[0], __shfl_xor_sync(0xffffffffu, w ? a[0] : a[1], 8));
+                mx = max_nan(w ? b[1] : b[0], __shfl_xor_sync(0xffffffffu, w ? b[0] : b[1], 8));
+            }
+            // What the lanes and the team's warps tell each other goes through the first rows of each chunk of the warp's own
+            // E_hi rows, which no product reads now: 0, 1, 2 zero-point, scale, reciprocal; 3, 4 extremes.
+            float *own = E_hi + e_warp + q * KB_CHUNK_FLOATS + s;
+            if (NW > 1) {
+                own[12] = m;
+                own[16] = mx;
                 team_barrier(team_id, 32 * NW);
 #pragma unroll
                 for (int o = 1; o < NW; ++o) {
-                    const float *peer = E_hi + half * 8 * KB_CHUNK_FLOATS + ((wq - wteam) + (wteam ^ o)) * 128 + q * KB_CHUNK_FLOATS;
-                    const float4 a = *reinterpret_cast<const float4 *>(peer), b = *reinterpret_cast<const float4 *>(peer + 4);
-                    mn[0] = min_nan(mn[0], a.x); mn[1] = min_nan(mn[1], a.y); mn[2] = min_nan(mn[2], a.z); mn[3] = min_nan(mn[3], a.w);
-                    mx[0] = max_nan(mx[0], b.x); mx[1] = max_nan(mx[1], b.y); mx[2] = max_nan(mx[2], b.z); mx[3] = max_nan(mx[3], b.w);
+                    const float *peer = own + ((wteam ^ o) - wteam) * 128;
+                    m = min_nan(m, peer[12]);
+                    mx = max_nan(mx, peer[16]);
                 }
-                team_barrier(team_id, 32 * NW);          // all have read; the rows may be overwritten
             }
+            float scale, inv;
+            const bool outside = step == 0 ? make_grid<BITS, M16, true>(m, mx, scale, inv) : make_grid<BITS, M16, false>(m, mx, scale, inv);
+            own[0] = m;
+            own[4] = scale;
+            own[8] = -inv;
+            __syncwarp();
             Grid4 g;
+            {
+                const ulonglong2 *quad = reinterpret_cast<const ulonglong2 *>(E_hi + e_warp + q * KB_CHUNK_FLOATS);
+                const ulonglong2 a = quad[0], b = quad[1], c = quad[2];
+                g.m[0] = a.x; g.m[1] = a.y; g.scale[0] = b.x; g.scale[1] = b.y; g.neg_inv[0] = c.x; g.neg_inv[1] = c.y;
+            }
+            // all have read; the rows may be overwritten
+            if (NW > 1) team_barrier(team_id, 32 * NW);
+            else __syncwarp();
+            const bool clamp = M16 && __any_sync(0xffffffffu, outside);
+
             unsigned cw[BITS];                           // 8 tokens x 4 channels x BITS bits
-            if (step == 0) make_grid4<BITS, M16, true>(mn, mx, g);
-            else make_grid4<BITS, M16, false>(mn, mx, g);
-            if (!SQ_CHK_R(p.status, E_hi + e_mine, (16 * (KB_ROWS - 1) + 4) * 4, E_hi, Lay::E_FLOATS * 4) ||
-                !SQ_CHK_R(p.status, E_lo + e_mine, (16 * (KB_ROWS - 1) + 4) * 4, E_lo, Lay::E_FLOATS * 4)) {
-                quantize_quads<BITS, M16, true, false>(x, g, nullptr, nullptr, cw);
+            float *eh = E_hi + e_mine, *el = E_lo + e_mine;
+            if (!SQ_CHK_R(p.status, eh, (16 * (KB_ROWS - 1) + 4) * 4, E_hi, Lay::E_FLOATS * 4) ||
+                !SQ_CHK_R(p.status, el, (16 * (KB_ROWS - 1) + 4) * 4, E_lo, Lay::E_FLOATS * 4)) {
+                quantize_quads<BITS, false, true, false>(x, g, nullptr, nullptr, cw);
             } else if (step == 0) {
-                quantize_quads<BITS, M16, true, true>(x, g, E_hi + e_mine, E_lo + e_mine, cw);
+                if (clamp) quantize_quads<BITS, M16, true, true>(x, g, eh, el, cw);
+                else quantize_quads<BITS, false, true, true>(x, g, eh, el, cw);
             } else if (!last) {
-                quantize_quads<BITS, M16, false, true>(x, g, E_hi + e_mine, E_lo + e_mine, cw);
+                if (clamp) quantize_quads<BITS, M16, false, true>(x, g, eh, el, cw);
+                else quantize_quads<BITS, false, false, true>(x, g, eh, el, cw);
             } else {
-                quantize_quads<BITS, M16, false, false>(x, g, nullptr, nullptr, cw);
+                if (clamp) quantize_quads<BITS, M16, false, false>(x, g, nullptr, nullptr, cw);
+                else quantize_quads<BITS, false, false, false>(x, g, nullptr, nullptr, cw);
             }
 
+            if (!BF16) load_next();
             if (!last) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the E rows, for the tensor core
                 tc_fence_before();
@@ -569,25 +592,18 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                 const uint4 c = transpose_codes4(reinterpret_cast<const unsigned(&)[4]>(cw), cl);
                 if (cur.active && SQ_CHK_G(p.status, cp, 16, p.x_codes)) *reinterpret_cast<uint4 *>(cp) = c;
             }
-            if (cur.active && wteam == 0 && s == 0 &&
-                SQ_CHK_G(p.status, static_cast<char *>(p.scales) + meta * (M16 ? 2 : 4), M16 ? 8 : 16, p.x_scales) &&
-                SQ_CHK_G(p.status, static_cast<char *>(p.zeros) + meta * (M16 ? 2 : 4), M16 ? 8 : 16, p.x_zeros)) {
-                if (M16) {                               // exact: the values are binary16 numbers already
-                    __half2 *sc = reinterpret_cast<__half2 *>(static_cast<__half *>(p.scales) + meta), *ze = reinterpret_cast<__half2 *>(static_cast<__half *>(p.zeros) + meta);
-                    const __half2 a0 = __floats2half2_rn(g.scale[0], g.scale[1]), a1 = __floats2half2_rn(g.scale[2], g.scale[3]);
-                    const __half2 b0 = __floats2half2_rn(g.m[0], g.m[1]), b1 = __floats2half2_rn(g.m[2], g.m[3]);
-                    *reinterpret_cast<uint2 *>(sc) = make_uint2(*reinterpret_cast<const unsigned *>(&a0), *reinterpret_cast<const unsigned *>(&a1));
-                    *reinterpret_cast<uint2 *>(ze) = make_uint2(*reinterpret_cast<const unsigned *>(&b0), *reinterpret_cast<const unsigned *>(&b1));
+            if (cur.active && wteam == 0 &&
+                SQ_CHK_G(p.status, static_cast<char *>(p.scales) + meta * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_scales) &&
+                SQ_CHK_G(p.status, static_cast<char *>(p.zeros) + meta * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_zeros)) {
+                if (M16) {
+                    static_cast<__half *>(p.scales)[meta] = __float2half_rn(scale);     // exact
+                    static_cast<__half *>(p.zeros)[meta] = __float2half_rn(m);
                 } else {
-                    *reinterpret_cast<float4 *>(static_cast<float *>(p.scales) + meta) = make_float4(g.scale[0], g.scale[1], g.scale[2], g.scale[3]);
-                    *reinterpret_cast<float4 *>(static_cast<float *>(p.zeros) + meta) = make_float4(g.m[0], g.m[1], g.m[2], g.m[3]);
+                    static_cast<float *>(p.scales)[meta] = scale;
+                    static_cast<float *>(p.zeros)[meta] = m;
                 }
-                unsigned flags = 0;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (!(g.scale[j] > 0.0f && g.scale[j] < __int_as_float(0x7f800000)))
-                        flags |= g.scale[j] == 0.0f ? SQUAT_FLAG_ZERO_RANGE : SQUAT_FLAG_NONFINITE;
-                if (flags) atomicOr(p.status, flags);
+                if (!(scale > 0.0f && scale < __int_as_float(0x7f800000)))
+                    atomicOr(p.status, scale == 0.0f ? SQUAT_FLAG_ZERO_RANGE : SQUAT_FLAG_NONFINITE);
             }
         }
         cur = nxt;
