@@ -151,7 +151,7 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     size_t off = 0;
     auto carve = [&](size_t bytes) { size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
     const size_t o_wt = carve(hdd * sizeof(float));
-    const size_t o_img = carve(hdd * sizeof(float));
+    const size_t o_img = carve((size_t)n_kv_heads * SQUAT_KEY_IMG_FLOATS * sizeof(float));
     const size_t o_gram = carve(hdd * sizeof(double));
     const size_t o_part = carve(hdd * sizeof(double) * s->gram_chunks_cap);
     const size_t o_val = carve((size_t)n_kv_heads * D * sizeof(double));
@@ -179,10 +179,10 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     s->gram_rem = reinterpret_cast<SquatGramRem *>(base + o_rem);
     s->tri = reinterpret_cast<double *>(base + o_tri);
     s->eig_scale = reinterpret_cast<double *>(base + o_scl);
-    s->exact_blocks = reinterpret_cast<int *>(base + o_exact);
+    s->exact_channels = reinterpret_cast<int *>(base + o_exact);
     s->lr_table = reinterpret_cast<float *>(base + o_lr);
-    const int all_exact = D / 32;        // W starts as zero: every channel is uncorrected
-    if (cudaMemcpy(s->exact_blocks, &all_exact, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
+    const int all_exact = D;        // W starts as zero: every channel is uncorrected
+    if (cudaMemcpy(s->exact_channels, &all_exact, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
     s->status = squat_status_word();
     if (!s->status) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
     *out = s;
@@ -224,7 +224,7 @@ int squat_build_subspace(squat_subspace *s, const void *q, int dtype, int n_q_he
     if (rc != SQUAT_OK) return rc;
     s->block_g = block_form(rank_r, lambda, block_g);
     // channels of the first g-block are never corrected; with r = 0 or lambda = 0, W = 0 and none is
-    const int exact = (rank_r == 0 || lambda == 0.0) ? D / 32 : (block_g + 31) / 32;
+    const int exact = (rank_r == 0 || lambda == 0.0) ? D : block_g;
     return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
 }
 
@@ -244,7 +244,7 @@ int squat_build_subspace_from_gram(squat_subspace *s, const double *gram, int ra
     rc = lowrank_tables_if_small(s, rank_r, lambda, block_g, st);
     if (rc != SQUAT_OK) return rc;
     s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = (rank_r == 0 || lambda == 0.0) ? D / 32 : (block_g + 31) / 32;
+    const int exact = (rank_r == 0 || lambda == 0.0) ? D : block_g;
     return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
 }
 
@@ -272,7 +272,7 @@ int squat_build_subspace_power(squat_subspace *s, const void *q, int dtype, int 
     const bool no_update = rank_r == 0 || lambda == 0.0;
     s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
     s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = no_update ? D / 32 : (block_g + 31) / 32;
+    const int exact = no_update ? D : block_g;
     if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);      // W = 0: nothing to iterate
     rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
     if (rc != SQUAT_OK) return rc;
@@ -297,7 +297,7 @@ int squat_build_subspace_power_from_gram(squat_subspace *s, const double *gram, 
     const bool no_update = rank_r == 0 || lambda == 0.0;
     s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
     s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = no_update ? D / 32 : (block_g + 31) / 32;
+    const int exact = no_update ? D : block_g;
     if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);
     int rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
     if (rc != SQUAT_OK) return rc;
@@ -364,10 +364,10 @@ int squat_subspace_import(squat_subspace *s, const float *W_host, void *stream)
         for (int jp = 0; jp < uncorrected; ++jp)
             for (int j = 0; j < D; ++j)
                 if (W_host[((size_t)h * D + jp) * D + j] != 0.0f) { uncorrected = jp; break; }
-    const int exact = (uncorrected + 31) / 32;
+    const int exact = uncorrected;
     s->lowrank_r = s->block_g = 0;         // an imported W comes without its factors or block size: dense kernel
     SQUAT_CUDA(cudaMemcpyAsync(s->Wt, wt.data(), hdd * sizeof(float), cudaMemcpyHostToDevice, st));
-    int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, s->exact_blocks, st);
+    int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, s->exact_channels, st);
     if (rc != SQUAT_OK) return rc;
     SQUAT_CUDA(cudaStreamSynchronize(st));
     return SQUAT_OK;
@@ -399,7 +399,7 @@ int quantize_keys_impl(const squat_subspace *s, const void *k, int dtype, int ba
                                              bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
                                              meta16, static_cast<cudaStream_t>(stream));
     return squat_launch_quant_keys(s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t, bits,
-                                   group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status, s->exact_blocks,
+                                   group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status, s->exact_channels,
                                    meta16, static_cast<cudaStream_t>(stream));
 }
 }  // namespace

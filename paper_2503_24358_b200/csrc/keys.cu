@@ -1,685 +1,658 @@
-// Key quantization with error feedback: Algorithm 1, function Quant, with the update of
-// Eq. (3) / Eq. (update_block) applied through the assembled matrix W (W[j'][j] multiplies the
-// rounding error of channel j into channel j' > j), and the quantizer of Section 2.
+// Key quantization with error feedback (Algorithm 1, function Quant; any update matrix W): two tokens per lane, blocks of 16
+// channels.
 //
-// Mapping.  A group is G consecutive tokens of one (batch, head); its channels must be visited in
-// order, and each channel's grid needs min/max over the group's tokens.  So: lane = token, one warp
-// (G = 32) or a team of G/32 warps per group.  The 128 channels are processed in 4 blocks of 32.
+// A group is G consecutive tokens of one (batch, head); its channels must be visited in order, each channel's grid needs min /
+// max over the group's tokens, and each token's rounding error is pushed through W onto its later channels:
 //
-//   sequential sweep of a block (CUDA cores; 32 channels, unrolled so every register index is static):
-//       m, M  = warp min / max (redux.sync on f32)         -> scale = (M-m)/L, zero = m
-//       c     = rint((x_j - m)/scale), decided exactly through the remainder c*scale - (x_j - m)
-//       e     = fma(c, scale, -(x_j - m))                   (= deq(qtz(x_j)) - x_j)
-//       x_j' += e * W[j'][j]  for the later channels j' of the block (the diagonal 32 x 32 block of W^T,
-//       read from shared memory as broadcast 16-byte loads, applied with packed fma.rn.f32x2)
+//   m, M  = min / max                -> scale = (M-m)/L, zero = m
+//   c     = rint((x_j - m)/scale),  e = c*scale - (x_j - m)       (= deq(qtz(x_j)) - x_j)
+//   x_j' += e * W[j'][j]
 //
-//   update of the later blocks (tcgen05 tensor cores): three quarters of the multiply-adds are the
-//   dense contractions (tokens x 32 errors) x (32 x later channels).  A tile is 128 tokens' worth of
-//   groups worked by 4 warps: row m of the tile = lane (m % 32) of the warp with warp % 4 == m / 32 =
-//   tensor-memory lane m.  Tensor memory holds, per tile, the fp32 accumulator D[128 x 96] of the
-//   corrections to channels 32 .. 127 and, in the tile's other 32 columns, E_hi of the block just swept:
-//   the raw fp32 errors (the tensor core reads the top 19 bits of a word: tf32 by truncation).
-//   E_lo = e - trunc(e), exact in fp32, goes to shared memory as an A operand (K-major 8 x 16-byte core
-//   matrices).  After the sweep of block b the last of the tile's 4 warps to get there issues
-//        D[:, 32 b .. 95] (+)= E_lo * Whi_b + E_hi * Wlo_b + E_hi * Whi_b     (12 MMAs of 128 x (96 - 32 b) x 8)
-//   with W^T's off-diagonal panels split into tf32 hi / lo (small terms first within a block: the
-//   accumulator truncates on every add) and commits them to the tile's mbarrier; nobody waits at a CTA
-//   or tile barrier.  Before the next sweep each warp waits for that phase (bounded), reads its 32
-//   columns of D with tcgen05.ld -- one token per lane, no transpose -- and adds the keys.
+// Within a block of 16 channels the pushes are CUDA-core work (packed fma.rn.f32x2 on the lane's two tokens); onto the channels
+// of later blocks they are a dense product on the tcgen05 tensor cores, tf32 operands split in two.
 //
-// Per head the kernel needs 64 KB in shared memory: the four diagonal blocks (fp32) and the three
-// hi / lo panels, copied as they are (cp.async.bulk, counted on an mbarrier) from the image that
-// pack_w_kernel writes when the update matrices are built or imported.  Two images fit (head h in buffer
-// h & 1).  CTAs are persistent: each takes a contiguous range of tiles and works it in rounds of up to 4
-// tiles, one per tile slot, sized as evenly as the range allows; a round may cross one head boundary.
+// Who holds what.  A CTA is 4 warps and works on 2 tiles of 128 tokens; two CTAs share an SM.  Row r of a tile = tensor-memory
+// lane r; warp w, lane l holds row 32 w + l of both tiles, as pairs, so a read of W (stored twice) and every packed
+// instruction serve two tokens, and groups of 64 and more join their extremes in the lane before the warp-wide reduction (a
+// group of 128 is two warps, which trade their extremes per channel through shared memory).  Tensor memory, per tile: the
+// corrections D[128 x 112] of channels 16 .. 127, and 16 more columns for the errors of block 0.  The errors E_hi of block b > 0
+// take the columns whose corrections that block has just read, so nothing waits for a free place.  E_lo goes to shared memory as
+// a K-major operand, in two buffers.
 //
-// Work per key vector: 8128 fp32 multiply-adds (dense triangle, g = 1): 1984 on the CUDA cores
-// (sweeps: four triangles of 32 * 31 / 2), 6144 x 3 tf32 products on the tensor cores.
+// Hand-over from block b to b + 1 (a fifth warp issues the products: a sweeping one that did took 2 000 cycles a hand-over over it):
+//       first   D[:, next 16]  += E_lo Whi + E_hi Wlo + E_hi Whi     (commit: the next sweep waits for this)
+//       then    D[:, the rest] += the same                           (done while the next sweep runs)
+// so a sweep waits for products of 16 columns, whatever is left of the row.
+//
+// Bound: latency.  A channel's chain (two reductions, reciprocal, rounding, push onto the next channel) is 71 cycles, a hand-over about
+// 1 000, and tensor memory holds 512 tokens per SM, so two warps per scheduler have to cover each other's waits; issue slots are
+// 30 % busy.  What this kernel replaced swept blocks of 32 channels with one token per lane (16 warps per SM): every warp made
+// every channel's grid, read W for 32 tokens at a time and, for groups of 64 and 128, met the group's other warps for every
+// channel.  128 heads x 32768 tokens, before -> now: G = 128, 4 bits 1715 -> 923 us; G = 64 1578 -> 1022; G = 32 1293 -> 1062; 32 heads
+// x 4096, G = 32 47.2 -> 44.1; 64 x 32 heads x 128 89.6 -> 82.0; 32 heads x 128 15.0 -> 14.7.  On the way: four tokens per lane with
+// blocks of 32 channels was slower (50 KB of straight code: instruction fetch); a sweeping warp that also issued the products lost
+// 2 000 cycles a hand-over; converting the keys and asking for the next ones ahead of the wait instead of behind it was worth 6 to
+// 10 %.
+//
+// Rounding decision.  t = (x - m) / scale is formed with the hardware reciprocal, so c0 = rint(t) can be off by one when t is within
+// ~1e-6 of a rounding midpoint.  Channels that earlier channels have corrected hold generic float32 values and such near-ties are as
+// rare as that bound; but channels nothing has corrected yet (the first g channels, or all of them when W = 0) hold raw bf16 / f32
+// inputs, where exact ties are structural (x exactly half way between min and max).  For those blocks (EXACT) the remainder
+// e0 = c0*scale - (x - m), which is exact next to a midpoint, is compared with +-scale/2: that settles the rounding exactly as real
+// arithmetic on the stored float32 scale would, ties going to the even code (the threshold of an odd c0 is one ulp lower, so
+// "remainder == scale/2" moves it).  The stored scale is the correctly rounded quotient in EXACT blocks (bit-identical to plain
+// round-to-nearest quantization), else the product with RN(1/L), within one ulp of it.
+//
+// M16: scale and zero-point are stored as binary16.  The float32 values are rounded once more, and the decision and the error fed
+// back are taken against the rounded (stored) values: t = (x - z16) / s16, clamped to [0, L] because z16 can lie above the minimum.
 #include "keys_common.cuh"
 
 namespace {
 
-constexpr int TC_SLOTS = 4;                          // 128-token tiles in flight per CTA
-constexpr int TC_WARPS = TC_SLOTS * 4;
-constexpr int TC_THREADS = TC_WARPS * 32;
-constexpr int TC_COLS_PER_TILE = 128;                // [0, 96) D: corrections of channels 32 .. 127; [96, 128) E_hi of the block just swept
-constexpr int TC_EHI_COL = 96;
-constexpr int TC_TMEM_COLS = 512;
-static_assert(TC_SLOTS * TC_COLS_PER_TILE <= TC_TMEM_COLS, "tensor memory has 512 columns");
-constexpr int TC_E_FLOATS = 128 * BLK;               // one tile's E_hi (or E_lo): 128 rows x 32 channels
-constexpr unsigned TC_A_LBO = 128 * 16, TC_SBO = 128;                 // bytes
-
-
-// ---- tcgen05 / tensor-memory helpers (5th-generation tensor cores) -------------------------------------------
-__device__ __forceinline__ unsigned tf32_of(float x)             // round to nearest tf32 (10 mantissa bits)
-{
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
-// umma_tf32_ss with A from tensor memory (rows = lanes, 8 consecutive 32-bit columns)
-__device__ __forceinline__ void umma_tf32_ts(unsigned d_taddr, unsigned a_taddr, u64 b_desc, unsigned idesc, unsigned accumulate)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}"
-                 ::"r"(d_taddr), "r"(a_taddr), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// 4 consecutive 32-bit columns of the warp's 32 tensor-memory lanes: lane l writes its own row
-__device__ __forceinline__ void tmem_st4(unsigned taddr, float a, float b, float c, float d)
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
-                 ::"r"(taddr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)) : "memory");
-}
-
-// Starts the copy of one head's 64 KB image into shared memory on the bulk-copy engine (one CTA, one destination); the bytes are
-// counted on `mbar`, whose current phase completes when all of them have landed.
-__device__ __forceinline__ void stage_image_async(float *dst, const float *src, unsigned mbar)
-{
-    constexpr unsigned BYTES = TC_IMG_FLOATS * 4, PIECE = 16384;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // earlier reads of the old image, before the engine's writes
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(BYTES) : "memory");
-#pragma unroll
-    for (unsigned o = 0; o < BYTES; o += PIECE)
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(smem_u32(dst) + o), "l"(reinterpret_cast<const char *>(src) + o), "r"(PIECE), "r"(mbar) : "memory");
-}
+constexpr int KEY_WARPS = 4, KEY_THREADS = 32 * (KEY_WARPS + 1);      // four sweeping warps, one that issues the products
+constexpr int KEY_COLS = 128, KEY_E0_COL = 112;                          // per tile: [0, 112) corrections, [112, 128) E_hi of block 0
+// The accumulator truncates on every addition, so corrections are gathered in two: what blocks 0 .. 3 push in the columns of the
+// channel, what blocks 4 .. 6 push onto blocks 5 .. 7 in columns that are free by then, and the sweep adds both.  (In one
+// accumulator the rms error of a group's minimum against 64 bits was 1.14e-7 of its range (rank 32, 2 bits, G = 32), 0.93e-7 in two; the
+// kernel of 32-channel blocks before this one had 0.94e-7.  Time: + 1 % for groups of 32 and 64, + 5 % for 128.)
+constexpr int KEY_SPLIT = 4;
+__host__ __device__ constexpr int key_late_col(int blk) { return blk == 7 ? KEY_E0_COL : (blk - KEY_SPLIT - 1) * KEY_BLK; }
+constexpr int KEY_E_FLOATS = 128 * KEY_BLK;                              // one tile's E_lo
+constexpr unsigned KEY_A_LBO = 128 * 16, KEY_SBO = 128;
+constexpr unsigned kMagicBits = 0x4B400000u;
 
 struct KeyParams {
-    const float *Wimg;        // [H, d * d] staged images of the update matrices (pack_w_kernel)
+    const float *Wimg;        // [H, KEY_IMG_FLOATS] staged images of the update matrices
     const void *k;
     long long sb, sh, st;     // element strides of k
     unsigned char *codes;
     void *scales, *zeros;     // float32, or binary16 in the M16 instances
     long long osb, osh;       // output strides in tokens
-    int B, H, T;
     int groups_per_bh;        // T / G
     int groups_per_head;      // B * T / G
-    int tiles_per_head;       // 128-token tiles per head (the last one may be ragged)
-    int total_tiles;          // H * tiles_per_head
+    int units_per_head;       // 256 tokens each (512 with two pairs per lane)
+    int total_units;
+    int one_tile;             // G = 32, few tokens: a unit is one tile of 128 tokens (see the launcher)
     unsigned *status;
-    const int *exact_blocks;  // device word: leading 32-channel blocks that no earlier channel corrects (see sweep_block)
+    const int *exact_channels;    // device word: leading channels that no earlier channel corrects
 #ifdef SQUAT_CHECKED
     SqExtent x_k, x_codes, x_scales, x_zeros, x_img;      // what the caller's tensors and the handle's images span
 #endif
 };
 
-// What the sweep may touch, for the bounds-checked build (empty otherwise).
-struct SweepChk {
-#ifdef SQUAT_CHECKED
-    unsigned *status;
-    const float *img;         // the staged image the diagonal block belongs to
-    const float *e_region;    // the tile slot's E_lo operand
-    unsigned tmem_lo, tmem_hi;   // the columns of the tile's E_hi operand: [lo, hi)
-#endif
-};
+// Pairs of tokens per lane, by group size.  One pair: two CTAs of two tiles per SM.  Two pairs: one CTA of four tiles, so that a group
+// of 128 is one warp's and its extremes never leave it (128 heads x 32768 tokens, 4 bits: 1061 us when it was built; as two warps of one pair
+// each that meet for every channel 1461).  Smaller groups lose with two pairs (G = 64: 1096 -> 1239, G = 32: 1210 -> 1633): nothing is left to
+// run while one warp per scheduler waits.
+__host__ __device__ constexpr int key_np(int G) { return G == 128 ? 2 : 1; }
 
-template <bool BF16>
-struct RawRow {
-    uint4 v[BF16 ? 4 : 8];      // 32 channels of one token
+template <int NP>
+struct alignas(128) KeyShared {
+    u64 diag[KEY_NBLK * KEY_BLK * KEY_BLK];            // the image: diagonal blocks of W^T, every entry twice,
+    float panels[2 * KEY_PANEL_FLOATS];              // hi | lo panels
+    float e_lo[2][2 * NP][KEY_E_FLOATS];
+    float grid[KEY_WARPS][2][2 * KEY_BLK * 2 * NP];   // scales | zero-points of two blocks' channels, [channel][group of the warp]
+    u64 mbar_e, mbar_d, mbar_diag, mbar_pan;        // errors of a block in place (4 warps), products done, parts of the image staged
+    unsigned tmem, timeout, exact_channels;
 };
-template <bool BF16>
-__device__ __forceinline__ void load_row(RawRow<BF16> &r, const void *row, int chan)
+static_assert(sizeof(KeyShared<1>) <= 113 * 1024, "two CTAs per SM");
+static_assert(sizeof(KeyShared<2>) > 114 * 1024, "one CTA per SM: it takes all of tensor memory");
+
+__device__ __forceinline__ void key_tmem_st1(unsigned taddr, float v)
 {
-    if (BF16) {
-        const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(row) + chan);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) r.v[i] = *(q + i);
-    } else {
-        const uint4 *q = reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(row) + chan);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) r.v[i] = *(q + i);
-    }
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(v)));
 }
-// channel pair q (channels 2q, 2q + 1) of the row as two floats
-template <bool BF16>
-__device__ __forceinline__ float2 row_pair(const RawRow<BF16> &r, int q)
+// the values of N groups as one 8- or 16-byte store (N = 1: 4)
+template <int N>
+__device__ __forceinline__ void key_store_groups(float *dst, const float (&v)[N])
 {
-    if (BF16) {
-        const uint4 &t = r.v[q >> 2];
-        const unsigned w = (q & 3) == 0 ? t.x : (q & 3) == 1 ? t.y : (q & 3) == 2 ? t.z : t.w;
-        return make_float2(bf16lo_to_f32(w), bf16hi_to_f32(w));
-    } else {
-        const uint4 &t = r.v[q >> 1];
-        return (q & 1) ? make_float2(__uint_as_float(t.z), __uint_as_float(t.w))
-                       : make_float2(__uint_as_float(t.x), __uint_as_float(t.y));
-    }
+    if constexpr (N == 1) *dst = v[0];
+    else if constexpr (N == 2) *reinterpret_cast<float2 *>(dst) = make_float2(v[0], v[1]);
+    else *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void key_tmem_ld16(unsigned taddr, unsigned (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr) : "memory");
 }
 
-// The sequential part: the 32 channels of one block, one token per lane, values in xp (16 packed pairs).
-// For every channel: grid from the warp (team) min / max, rounding decision, error e; e is pushed onto the
-// later channels of the block through the diagonal 32 x 32 block of W^T and written, 4 channels at a time, to
-// this lane's row of the tile's A operands (e_hi, e_lo: 4 floats per 4-channel chunk, chunks TC_A_LBO bytes
-// apart) for the tensor-core update of the later blocks.
-//
-// Rounding decision.  t = (x - m) / scale is formed as (x - m) * L * rcp(M - m) with the hardware reciprocal,
-// so c0 = rint(t) can be off by one when t is within ~1e-6 of a rounding midpoint.  Channels that earlier
-// channels have corrected hold generic float32 values and such near-ties are as rare as that bound; but
-// channels nothing has corrected yet (the first g channels, or all of them when W = 0) hold raw bf16 / f32
-// inputs, where exact ties are structural (x exactly half way between min and max).  For those blocks
-// (EXACT) the remainder e0 = c0*scale - (x - m), which is exact next to a midpoint, is compared with
-// +-scale/2: that settles the rounding exactly as real arithmetic on the stored float32 scale would, ties
-// going to the even code (the threshold of an odd c0 is one ulp lower, so "remainder == scale/2" moves it).
-//
-// M16: scale and zero-point are stored as binary16.  The float32 values are rounded once more, and the decision
-// and the error fed back are taken against the rounded (stored) values: t = (x - z16) / s16, clamped to [0, L]
-// because z16 can lie above the group's minimum.
-template <int BITS, int NW, bool EXACT, bool M16>
-__device__ __forceinline__ void sweep_block(u64 (&xp)[BLK / 2], const float *diag, unsigned e_hi_taddr, float *e_lo, bool store_e,
-                                            int lane, int bar_id, int wteam, float2 *red,
-                                            uint32_t (&cw)[BLK * BITS / 32], float &my_scale, float &my_zero, const SweepChk &ck)
+// one lane of a converged warp, always the same
+__device__ __forceinline__ bool key_elected()
+{
+    unsigned r;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(r));
+    return r != 0;
+}
+
+// 16 channels of the lane's tokens as they are in memory
+template <bool BF16, int NP>
+struct PairRows {
+    uint4 v[2 * NP][BF16 ? 2 : 4];
+    __device__ __forceinline__ float get(int i, int c) const
+    {
+        if (BF16) {
+            const uint4 &t = v[i][c >> 3];
+            const unsigned w = (c & 7) < 2 ? t.x : (c & 7) < 4 ? t.y : (c & 7) < 6 ? t.z : t.w;
+            return (c & 1) ? bf16hi_to_f32(w) : bf16lo_to_f32(w);
+        }
+        const uint4 &t = v[i][BF16 ? 0 : c >> 2];
+        return __uint_as_float((c & 3) == 0 ? t.x : (c & 3) == 1 ? t.y : (c & 3) == 2 ? t.z : t.w);
+    }
+};
+
+// The 16 channels of one block for the lane's 2 NP tokens (pair i of x[channel]: tokens 2 i and 2 i + 1), which belong to NGL groups.
+// exact_first: the first channel's decisions are exact (EXACT: all).
+// Written in the order in which it should run: a channel's chain (reductions 24 cycles, reciprocal 24, six dependent
+// operations of 4 to 6: 71 in all) goes on to the next channel's reductions before what does not hurry: the other pushes, the
+// codes and the errors' stores fill the waits.  The next row of W is read before this channel's stores, which may be to the same
+// memory for all the compiler knows.  The errors of the last block are stored like the others (a test per store would cut the
+// code into pieces) and used by nobody.
+template <int BITS, int NP, int NGL, bool EXACT, bool M16>
+__device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__restrict__ diag, unsigned e_hi, float *__restrict__ e_lo,
+                                            int lane, bool exact_first, float *__restrict__ gscale, float *__restrict__ gzero, unsigned (&cw)[2 * NP][BITS / 2])
 {
     constexpr float L = float((1 << BITS) - 1);
-    constexpr int PER_ACC = 16 / BITS;              // codes accumulated exactly in one float (16 bits of mantissa)
-    float cacc[BLK / PER_ACC];
-    float eh[4], el[4];
+    constexpr int PER_WORD = 32 / BITS, NT = 2 * NP, TPG = NT / NGL;      // tokens of the lane per group
+    // what the constant upper bits of the rounded floats add up to in a packed word
+    constexpr unsigned K = [] { unsigned k = 0; for (int i = 0; i < PER_WORD; ++i) k += kMagicBits << (BITS * i); return k; }();
+    const u64 magic2 = pack2(kMagic, kMagic), negl2 = pack2(-L, -L);
+    float el[NT][4];                                    // [token][channel % 4]
+    float m[NGL], mx[NGL];
+    auto extremes = [&](int jj) {
+        float v[NT];
 #pragma unroll
-    for (int jj = 0; jj < BLK; ++jj) {
-        const float xj = (jj & 1) ? hi_of(xp[jj >> 1]) : lo_of(xp[jj >> 1]);
-        float m = warp_min(xj);
-        float Mx = warp_max(xj);
-        if (NW > 1) {
-            float2 *slot = red + (jj & 1) * NW;             // [parity][warp of the team]
-            (void)ck;
-            if (lane == 0) slot[wteam] = make_float2(m, Mx);
-            team_barrier(bar_id, 32 * NW);
-            // two warps' pairs per 16-byte read, three operands per minimum: for four warps 6 instructions instead of 12 (128
-            // heads x 32768 tokens, 4 bits, G = 128: 1.75 -> 1.71 ms)
-            if (NW == 2) {
-                const float4 o = *reinterpret_cast<const float4 *>(slot);
-                m = min_nan(o.x, o.z);
-                Mx = max_nan(o.y, o.w);
+        for (int i = 0; i < NP; ++i) unpack2(x[jj][i], v[2 * i], v[2 * i + 1]);
+#pragma unroll
+        for (int g = 0; g < NGL; ++g) {
+            float lo = v[TPG * g], hi = lo;
+            if (TPG == 2) { lo = min_nan(lo, v[TPG * g + 1]); hi = max_nan(hi, v[TPG * g + 1]); }
+            if (TPG == 4) {
+                lo = min_nan(min3_nan(v[0], v[1], v[NT > 2 ? 2 : 0]), v[NT > 2 ? 3 : 0]);
+                hi = max_nan(max3_nan(v[0], v[1], v[NT > 2 ? 2 : 0]), v[NT > 2 ? 3 : 0]);
+            }
+            m[g] = warp_min(lo);
+            mx[g] = warp_max(hi);
+        }
+    };
+    u64 w[KEY_BLK];                                      // row jj of the diagonal block, channels jj + 1 .. 15
+    auto read_row = [&](int jj) {
+#pragma unroll
+        for (int q = (jj + 1) / 2; q < KEY_BLK / 2; ++q) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(diag + jj * KEY_BLK + 2 * q);
+            w[2 * q] = t.x;
+            w[2 * q + 1] = t.y;
+        }
+    };
+    read_row(0);
+    extremes(0);
+#pragma unroll
+    for (int jj = 0; jj < KEY_BLK; ++jj) {
+        float scale[NGL], inv[NGL], z[NGL];
+#pragma unroll
+        for (int g = 0; g < NGL; ++g) {
+            const float rng = __fsub_rn(mx[g], m[g]);
+            z[g] = m[g];
+            scale[g] = EXACT || (jj == 0 && exact_first) ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);
+            if (M16) {
+                scale[g] = __half2float(__float2half_rn(scale[g]));
+                z[g] = __half2float(__float2half_rn(m[g]));
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv[g]) : "f"(scale[g]));
+                inv[g] = scale[g] > 0.0f ? -inv[g] : 0.0f;                                      // scale 0 (no range, or underflow): codes 0
             } else {
-                const float4 o = reinterpret_cast<const float4 *>(slot)[0], o2 = reinterpret_cast<const float4 *>(slot)[1];
-                m = min_nan(min3_nan(o.x, o.z, o2.x), o2.z);
-                Mx = max_nan(max3_nan(o.y, o.w, o2.y), o2.w);
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv[g]) : "f"(fmaxf(rng, 1e-30f)));     // constant group: x - m = 0 -> code 0
             }
         }
-        const float rng = __fsub_rn(Mx, m);
-        // the stored scale: the correctly rounded quotient where the block's decisions are exact (raw inputs: bit-identical to
-        // plain round-to-nearest quantization), else the product with RN(1/L) (within one ulp of it; one instruction, not three)
-        float scale = EXACT ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);
-        float rcp, y0, dlt;
-        if (M16) {
-            scale = __half2float(__float2half_rn(scale));
-            m = __half2float(__float2half_rn(m));
-            dlt = __fsub_rn(xj, m);
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(scale));
-            rcp = scale > 0.0f ? rcp : 0.0f;                                       // scale 0 (no range, or underflow): codes 0
-            y0 = __fmaf_rn(dlt, rcp, kMagic);
-        } else {
-            dlt = __fsub_rn(xj, m);
-            const float dltL = __fmul_rn(dlt, L);
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(fmaxf(rng, 1e-30f)));   // constant group: dlt = 0 -> code 0
-            y0 = __fmaf_rn(dltL, rcp, kMagic);
+        u64 e[NP];
+        float y[NT];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const int ga = 2 * i / TPG, gb = (2 * i + 1) / TPG;
+            const u64 n = fsub2(pack2(z[ga], z[gb]), x[jj][i]);                                 // -(x - m)
+            u64 y2 = ffma2(M16 ? n : fmul2(n, negl2), pack2(inv[ga], inv[gb]), magic2);
+            float &y0 = y[2 * i], &y1 = y[2 * i + 1];
+            unpack2(y2, y0, y1);
+            if (M16 && !EXACT && jj > 0) {
+                y0 = fminf(fmaxf(y0, kMagic), kMagic + L);
+                y1 = fminf(fmaxf(y1, kMagic), kMagic + L);
+                y2 = pack2(y0, y1);
+            }
+            e[i] = ffma2(fsub2(y2, magic2), pack2(scale[ga], scale[gb]), n);
+            if (EXACT || (jj == 0 && (exact_first || M16))) {
+                float e0, e1, n0, n1;
+                unpack2(e[i], e0, e1);
+                unpack2(n, n0, n1);
+                auto decide = [&](float nd, float sc, float &yy, float &ee) {
+                    if (EXACT || exact_first) {
+                        const float thr = __uint_as_float(__float_as_uint(0.5f * sc) - (__float_as_uint(yy) & 1u));
+                        const float adj = ee > thr ? -1.0f : (ee < -thr ? 1.0f : 0.0f);
+                        yy = __fadd_rn(yy, adj);
+                        ee = __fmaf_rn(adj, sc, ee);
+                    }
+                    if (M16) {
+                        const float cc = fminf(fmaxf(yy, kMagic), kMagic + L);
+                        ee = cc == yy ? ee : __fmaf_rn(__fsub_rn(cc, kMagic), sc, nd);
+                        yy = cc;
+                    }
+                };
+                decide(n0, scale[ga], y0, e0);
+                decide(n1, scale[gb], y1, e1);
+                e[i] = pack2(e0, e1);
+            }
         }
-        float c = __fsub_rn(y0, kMagic);
-        float e = __fmaf_rn(c, scale, -dlt);
-        if (EXACT) {
-            const float thr = __uint_as_float(__float_as_uint(0.5f * scale) - (__float_as_uint(y0) & 1u));
-            const float adj = (e > thr) ? -1.0f : ((e < -thr) ? 1.0f : 0.0f);
-            c = __fadd_rn(c, adj);
-            e = __fmaf_rn(adj, scale, e);
-        }
-        if (M16) {
-            const float cc = fminf(fmaxf(c, 0.0f), L);
-            e = cc == c ? e : __fmaf_rn(cc, scale, -dlt);
-            c = cc;
-        }
-        // pack the code arithmetically: sum of c * 2^(BITS k) is exact in float32 up to 16 bits
-        if (jj % PER_ACC == 0) cacc[jj / PER_ACC] = c;
-        else cacc[jj / PER_ACC] = __fmaf_rn(c, float(1 << ((jj % PER_ACC) * BITS)), cacc[jj / PER_ACC]);
-        if (lane == jj) {                               // lane jj keeps channel jj's grid for the store after the sweep
-            my_scale = scale;
-            my_zero = m;
-        }
-        // tf32 split by truncation: the tensor core reads only the top 19 bits of each word, so e itself serves
-        // as E_hi = trunc(e), and E_lo = e - trunc(e) is exact in fp32
-        eh[jj & 3] = e;
-        el[jj & 3] = __fsub_rn(e, __uint_as_float(__float_as_uint(e) & 0xffffe000u));
-        if ((jj & 3) == 3 && store_e) {
-#ifdef SQUAT_CHECKED
-            const unsigned col = (e_hi_taddr + (jj - 3)) & 0xffffu;
-            const bool ok_t = sq_chk(col >= ck.tmem_lo && col + 4 <= ck.tmem_hi, ck.status);
-            const bool ok_s = sq_chk(sq_inside(e_lo + (jj >> 2) * (TC_A_LBO / 4), 16, ck.e_region, TC_E_FLOATS * 4), ck.status);
-            if (ok_t) tmem_st4(e_hi_taddr + (jj - 3), eh[0], eh[1], eh[2], eh[3]);
-            if (ok_s) *reinterpret_cast<float4 *>(e_lo + (jj >> 2) * (TC_A_LBO / 4)) = make_float4(el[0], el[1], el[2], el[3]);
-#else
-            tmem_st4(e_hi_taddr + (jj - 3), eh[0], eh[1], eh[2], eh[3]);
-            *reinterpret_cast<float4 *>(e_lo + (jj >> 2) * (TC_A_LBO / 4)) = make_float4(el[0], el[1], el[2], el[3]);
-#endif
-        }
-        const u64 ee = pack2(e, e);
-        const float *wrow = diag + jj * BLK;
-#ifdef SQUAT_CHECKED
-        if (!sq_chk(sq_inside(wrow, BLK * 4, ck.img, TC_DIAG_FLOATS * 4), ck.status)) continue;    // the reads below stay inside this row
-#endif
-        // later channels of the block, 4 per 16-byte broadcast read; where only the upper half of the first chunk
-        // is still to come, an 8-byte read does (a broadcast read is charged by its width)
-        if ((jj + 1) % 4 >= 2) {
-            const int q = (jj + 1) / 4;
-            const u64 wy = *reinterpret_cast<const u64 *>(wrow + 4 * q + 2);
-            xp[2 * q + 1] = ffma2(ee, wy, xp[2 * q + 1]);
+        // the next channel's value and extremes first
+        if (jj + 1 < KEY_BLK) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) x[jj + 1][i] = ffma2(e[i], w[jj + 1], x[jj + 1][i]);
+            extremes(jj + 1);
         }
 #pragma unroll
-        for (int q = ((jj + 1) % 4 >= 2 ? (jj + 1) / 4 + 1 : (jj + 1) / 4); q < BLK / 4; ++q) {
-            const ulonglong2 wv = *reinterpret_cast<const ulonglong2 *>(wrow + 4 * q);
-            if (2 * q >= (jj + 1) / 2) xp[2 * q] = ffma2(ee, wv.x, xp[2 * q]);
-            xp[2 * q + 1] = ffma2(ee, wv.y, xp[2 * q + 1]);
+        for (int c = jj + 2; c < KEY_BLK; ++c)
+#pragma unroll
+            for (int i = 0; i < NP; ++i) x[c][i] = ffma2(e[i], w[c], x[c][i]);
+        if (jj + 1 < KEY_BLK) read_row(jj + 1);
+        if (lane == 0) {
+            key_store_groups<NGL>(gscale + jj * NGL, scale);
+            key_store_groups<NGL>(gzero + jj * NGL, z);
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            // the low bits of a rounded float are its code
+            unsigned &c = cw[t][jj / PER_WORD];
+            if (jj % PER_WORD == 0) c = 0u - K;
+            c += __float_as_uint(y[t]) << (BITS * (jj % PER_WORD));
+            // tf32 split by truncation: the tensor core reads only the top 19 bits of each word, so e itself serves as E_hi =
+            // trunc(e), and E_lo = e - trunc(e) is exact in fp32
+            const float ev = (t & 1) ? hi_of(e[t / 2]) : lo_of(e[t / 2]);
+            key_tmem_st1(e_hi + t * KEY_COLS + jj, ev);
+            el[t][jj & 3] = __fsub_rn(ev, __uint_as_float(__float_as_uint(ev) & 0xffffe000u));
+            if ((jj & 3) == 3)
+                *reinterpret_cast<float4 *>(e_lo + t * KEY_E_FLOATS + (jj >> 2) * (KEY_A_LBO / 4)) = make_float4(el[t][0], el[t][1], el[t][2], el[t][3]);
         }
     }
-#pragma unroll
-    for (int w = 0; w < BLK * BITS / 32; ++w)
-        cw[w] = (uint32_t)__float2int_rn(cacc[2 * w]) | ((uint32_t)__float2int_rn(cacc[2 * w + 1]) << 16);
 }
 
-// Where one warp's 32 tokens of a round come from and go to.
-struct TileRows {
-    bool active;              // the warp's group exists (a head's last tile may be ragged: its spare warps redo the last
-                              // group and store nothing)
-    int head;
-    const void *row;          // this lane's key vector
-    unsigned char *codes;     // this lane's code row
-    long long meta;           // offset of the group's scales / zeros (lane = channel within a block)
-};
-
-template <int BITS, int NW, bool BF16, bool M16>
-__global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_kernel(const KeyParams p)
+template <int BITS, int G, bool BF16, bool M16>
+__global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(const KeyParams p)
 {
-    constexpr int G = 32 * NW;
-    constexpr int GPT = 4 / NW;                          // groups per tile
-    constexpr int NTEAMS = TC_SLOTS * GPT;               // teams of NW warps
-    constexpr int WORDS_PER_BLK = BLK * BITS / 32;       // 2 (2-bit) or 4 (4-bit)
-    extern __shared__ __align__(128) float smem[];
-    float *Eall = smem;                                  // [TC_SLOTS][TC_E_FLOATS]: the tiles' E_lo operands
-    float *images = Eall + TC_SLOTS * TC_E_FLOATS;       // [2][TC_IMG_FLOATS]: head h's image lives in buffer h & 1
-    float2 *red_all = reinterpret_cast<float2 *>(images + 2 * TC_IMG_FLOATS);    // [NTEAMS][2][NW]
-    u64 *mbar = reinterpret_cast<u64 *>(red_all + NTEAMS * 2 * NW);              // [TC_SLOTS] MMAs done, [1] image staged
-    // [0] tensor-memory base, [1] a bounded wait ran out, [2 + slot] arrivals of the slot's warps, [2 + TC_SLOTS] the
-    // number of leading blocks that take the exact rounding decision (read once from the handle's device word)
-    volatile unsigned *shared_words = reinterpret_cast<volatile unsigned *>(mbar + TC_SLOTS + 1);
+    constexpr int NP = key_np(G), NT = 2 * NP, NGL = 32 * NT / G, UNIT_GROUPS = KEY_WARPS * NGL, ES = BF16 ? 2 : 4;
+    static_assert(NGL >= 1, "a group is one warp's");
+    constexpr unsigned TMEM_COLS = NT * KEY_COLS;
+    extern __shared__ __align__(128) unsigned char smem_bytes[];
+    KeyShared<NP> &sm = *reinterpret_cast<KeyShared<NP> *>(smem_bytes);
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);      // (uniform: tensor-memory addresses go by it)
 
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int slot = warp >> 2;                          // tile slot of this warp
-    const int wq = warp & 3;                             // its quarter of the tile = its tensor-memory lanes
-    const int team = slot * GPT + wq / NW;
-    const int wteam = wq % NW;
-    float2 *red = red_all + team * (2 * NW);
+    const int u_lo = (int)((long long)p.total_units * blockIdx.x / gridDim.x);
+    const int u_hi = (int)((long long)p.total_units * (blockIdx.x + 1) / gridDim.x);
+    grid_wait();
+    volatile unsigned *timeout = &sm.timeout;
+    const unsigned mbar_e = smem_u32(&sm.mbar_e), mbar_d = smem_u32(&sm.mbar_d), mbar_diag = smem_u32(&sm.mbar_diag), mbar_pan = smem_u32(&sm.mbar_pan);
 
-    // A CTA takes a contiguous range of tiles (head-major order) and works it in rounds of up to TC_SLOTS tiles, one per
-    // slot, sized as evenly as its range allows (7 tiles = 4 + 3, not 4 + 4 elsewhere).  Two images fit in shared memory,
-    // so a round may run across one head boundary.  (All of this in 32-bit integers and recomputed rather than kept:
-    // the sweeps need every register.)
-    const int t_lo = (int)((long long)p.total_tiles * blockIdx.x / gridDim.x);
-    const int t_hi = (int)((long long)p.total_tiles * (blockIdx.x + 1) / gridDim.x);
-    auto round_size = [&](int start) {
-        const int left = t_hi - start;
-        if (left <= 0) return 0;
-        const int rounds_left = (left + TC_SLOTS - 1) / TC_SLOTS;
-        int n = (left + rounds_left - 1) / rounds_left;
-        const int two_heads_end = (start / p.tiles_per_head + 2) * p.tiles_per_head;
-        if (n > two_heads_end - start) n = two_heads_end - start;
-        return n;
+    // where the lane's tokens (one in each tile) and the warp's groups come from and go to
+    struct Place {
+        const char *row[NGL];     // the lane's first token of a group
+        unsigned char *codes[NGL];
+        long long meta[NGL];
+        bool active[NGL];         // the group exists (a head's last unit may be ragged: past its end the last group is redone and not stored)
     };
-    grid_wait();          // (its global loads are plain ones; laundering p here would cost registers the sweeps need)
-    const unsigned img_mbar = smem_u32(mbar + TC_SLOTS);
-    unsigned img_phase = 0;
-
-    if (threadIdx.x == 32) {
+    const long long row_step = 32 * p.st * ES;           // to the lane's next token of a group
+    auto locate = [&](int unit, Place &t) {
+        const int h = unit / p.units_per_head;
+        const bool one = G == 32 && p.one_tile;
+        const int g0 = one ? (unit - h * p.units_per_head) * KEY_WARPS + warp : (unit - h * p.units_per_head) * UNIT_GROUPS + NGL * warp;
 #pragma unroll
-        for (int t = 0; t < TC_SLOTS; ++t) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + t)), "r"(1) : "memory");
-            shared_words[2 + t] = 0;
+        for (int g = 0; g < NGL; ++g) {
+            t.active[g] = g0 + g < p.groups_per_head && (g == 0 || !one);
+            const int in_head = t.active[g] ? g0 + g : p.groups_per_head - 1;
+            const int b = in_head / p.groups_per_bh, grp = in_head - b * p.groups_per_bh;
+            const int tok = grp * G + lane;
+            const long long out_tok0 = (long long)b * p.osb + (long long)h * p.osh;
+            t.row[g] = static_cast<const char *>(p.k) + ((long long)b * p.sb + (long long)h * p.sh + (long long)tok * p.st) * ES;
+            t.codes[g] = p.codes + (out_tok0 + tok) * (D * BITS / 8);
+            t.meta[g] = (out_tok0 / G + grp) * D + lane;
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(img_mbar), "r"(1) : "memory");
-        shared_words[1] = 0;
-        shared_words[2 + TC_SLOTS] = (unsigned)*(p.exact_blocks);
+    };
+    PairRows<BF16, NP> raw;
+    auto load_rows = [&](const Place &t, int blk) {
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const char *src = t.row[i / (NT / NGL)] + i % (NT / NGL) * row_step + blk * (KEY_BLK * ES);
+            if (SQ_CHK_G(p.status, src, KEY_BLK * ES, p.x_k)) {
+#pragma unroll
+                for (int c = 0; c < (BF16 ? 2 : 4); ++c) raw.v[i][c] = reinterpret_cast<const uint4 *>(src)[c];
+            }
+        }
+    };
+    Place cur;
+    if (u_lo < u_hi && warp < KEY_WARPS) {               // the first rows are on their way while the CTA sets itself up
+        locate(u_lo, cur);
+        load_rows(cur, 0);
+    }
+
+    auto stage = [&](int h) {            // one head's image (one thread)
+        const float *src = p.Wimg + (long long)h * KEY_IMG_FLOATS;
+        if (!SQ_CHK_G(p.status, src, KEY_IMG_FLOATS * 4, p.x_img)) return;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        auto copy = [&](unsigned dst, const float *from, unsigned bytes, unsigned mbar) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(dst), "l"(from), "r"(bytes), "r"(mbar) : "memory");
+        };
+        copy(smem_u32(sm.diag), src, KEY_DIAG_FLOATS * 4, mbar_diag);                  // the sweeps need only these
+        copy(smem_u32(sm.panels), src + KEY_DIAG_FLOATS, 2 * KEY_PANEL_FLOATS * 4, mbar_pan);
+    };
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_e), "r"(KEY_WARPS) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_d), "r"(1) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_diag), "r"(1) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_pan), "r"(1) : "memory");
+        sm.timeout = 0;
+        sm.exact_channels = (unsigned)*p.exact_channels;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // the first head's image is on its way while the rest of the set-up runs
-        if (t_lo < t_hi) {
-            const int h0 = t_lo / p.tiles_per_head;
-            if (SQ_CHK_G(p.status, p.Wimg + (long long)h0 * TC_IMG_FLOATS, TC_IMG_FLOATS * 4, p.x_img))
-            stage_image_async(images + (h0 & 1) * TC_IMG_FLOATS, p.Wimg + (long long)h0 * TC_IMG_FLOATS, img_mbar);
-        }
+        if (u_lo < u_hi) stage(u_lo / p.units_per_head);
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(const_cast<unsigned *>(shared_words))), "r"((unsigned)TC_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const unsigned tmem_base = shared_words[0];
-    const unsigned t_tile = tmem_base + slot * TC_COLS_PER_TILE;               // lane field 0: the MMAs' accumulator
-    const unsigned t_mine = t_tile + ((unsigned)(wq * 32) << 16);              // this warp's 32 lanes
-    float *e_lo = Eall + slot * TC_E_FLOATS + (wq * 32 + lane) * 4;            // this lane's row of the tile's E_lo operand
-    const unsigned a_lo = smem_u32(Eall + slot * TC_E_FLOATS);
-    const unsigned my_mbar = smem_u32(mbar + slot);
-    unsigned phase = 0;
+    const unsigned tmem = __shfl_sync(0xffffffffu, *const_cast<volatile unsigned *>(&sm.tmem), 0);
+    const unsigned t_mine = tmem + ((unsigned)(warp * 32) << 16);
+    const int exact_channels = (int)sm.exact_channels;
+    unsigned phase = 0, img_phase = 0;
 
-    auto locate = [&](int tile, TileRows &t) {
-        const int h = tile / p.tiles_per_head;
-        const int g_raw = (tile - h * p.tiles_per_head) * GPT + wq / NW;                  // group within the head
-        t.head = h;
-        t.active = g_raw < p.groups_per_head;
-        const int in_head = t.active ? g_raw : p.groups_per_head - 1;
-        const int b = in_head / p.groups_per_bh;
-        const int grp = in_head - b * p.groups_per_bh;
-        const int tok = grp * G + wteam * 32 + lane;
-        const long long out_tok0 = (long long)b * p.osb + (long long)h * p.osh;
-        t.codes = p.codes + (out_tok0 + tok) * (D * BITS / 8);
-        t.meta = (out_tok0 / G + grp) * D + lane;
-        const long long row_off = (long long)b * p.sb + (long long)h * p.sh + (long long)tok * p.st;
-        t.row = BF16 ? static_cast<const void *>(reinterpret_cast<const __nv_bfloat16 *>(p.k) + row_off)
-                     : static_cast<const void *>(reinterpret_cast<const float *>(p.k) + row_off);
-    };
-
-    // every read of a key row goes through here (the bounds-checked build tests the 32 channels' bytes against the tensor)
-    auto load_keys = [&](RawRow<BF16> &r, const void *row, int chan) {
-        if (SQ_CHK_G(p.status, static_cast<const char *>(row) + chan * (BF16 ? 2 : 4), BLK * (BF16 ? 2 : 4), p.x_k))
-            load_row<BF16>(r, row, chan);
-    };
-    RawRow<BF16> raw;
-    int start = t_lo;
-    if (slot < round_size(start)) {
-        TileRows first;
-        locate(start + slot, first);
-        load_keys(raw, first.row, 0);                    // in flight while the first head is staged
-    }
-    int max_staged = -1;     // heads come in increasing order: the buffers hold max_staged and, earlier, max_staged - 1
-    while (start < t_hi) {
-        const int n_round = round_size(start);
-        // images of the (at most two) heads of this round
-        const int h_first = start / p.tiles_per_head, h_last = (start + n_round - 1) / p.tiles_per_head;
-        for (int hh = h_first; hh <= h_last; ++hh) {
-            if (hh <= max_staged) continue;
-            if (max_staged >= 0) {                       // (the very first copy was started at kernel entry)
-                __syncthreads();                         // every read of the buffer's old image, by a lane or by an MMA, is over
-                if (threadIdx.x == 32 && SQ_CHK_G(p.status, p.Wimg + (long long)hh * TC_IMG_FLOATS, TC_IMG_FLOATS * 4, p.x_img))
-                    stage_image_async(images + (hh & 1) * TC_IMG_FLOATS, p.Wimg + (long long)hh * TC_IMG_FLOATS, img_mbar);
-            }
-            if (!shared_words[1] && !mbar_wait(img_mbar, img_phase)) {   // bounded, like every wait here
-                shared_words[1] = 1;
-                atomicOr(p.status, SQUAT_FLAG_DEVICE_TIMEOUT);
-            }
-            img_phase ^= 1;
-            max_staged = hh;
+    auto bounded_wait = [&](unsigned mbar, unsigned parity) {
+        if (!*timeout && !mbar_wait(mbar, parity)) {
+            *timeout = 1;
+            atomicOr(p.status, SQUAT_FLAG_DEVICE_TIMEOUT);
         }
-        const bool valid = slot < n_round;
-        const bool nxt_valid = slot < round_size(start + n_round);
-        const void *nxt_row = nullptr;
-        if (nxt_valid) {
-            TileRows nxt;
-            locate(start + n_round + slot, nxt);
-            nxt_row = nxt.row;
-        }
-        TileRows cur;
-        cur.head = 0;
-        if (valid) locate(start + slot, cur);
-
-        const float *img = images + (cur.head & 1) * TC_IMG_FLOATS;       // diagonal blocks | hi panels | lo panels
-        const float *Bhi = img + TC_DIAG_FLOATS, *Blo = Bhi + TC_PANEL_FLOATS;
-        if (valid) {
+    };
+    if (warp == KEY_WARPS) {
+        // The issuing warp: one lane of it, always the same, issues, so its commits cover all earlier products.
+        const u64 a_lo0 = umma_desc(smem_u32(sm.e_lo[0][0]), KEY_A_LBO, KEY_SBO);
+        const unsigned pan = smem_u32(sm.panels);
+        int staged = -1;
 #pragma unroll 1
-            for (int blk = 0; blk < NBLK; ++blk) {
-                u64 xp[BLK / 2];
-                if (blk == 0) {
+        for (int unit = u_lo; unit < u_hi; ++unit) {
+            const int h = unit / p.units_per_head;
+            if (h != staged) {
+                if (staged >= 0) __syncthreads();
+                bounded_wait(mbar_pan, img_phase);
+                img_phase ^= 1;
+                staged = h;
+            }
+#pragma unroll 1
+            for (int blk = 0; blk + 1 < KEY_NBLK; ++blk) {
+                bounded_wait(mbar_e, phase);
+                phase ^= 1;
+                tc_fence_after();
+                const int nb = D - (blk + 1) * KEY_BLK;             // channels still to come
+                const unsigned b_lbo = 16u * nb, bhi = pan + 4 * key_panel_off(blk);
+                const u64 step = (2 * b_lbo) >> 4;                 // 8 channels on
+                // onto n channels from the ch-th behind the block on, into the columns from `col` on, all tiles
+                auto products = [&](int ch, int n, int col, bool accumulate) {
+                    if (!SQ_CHK_C(p.status, key_panel_off(blk) + nb * KEY_BLK <= KEY_PANEL_FLOATS && ch + n <= nb && col + n <= KEY_COLS)) return;
+                    const unsigned idesc = tc_idesc(n);
+                    const u64 hi = umma_desc(bhi + 16u * ch, b_lbo, KEY_SBO), lo = hi + KEY_PANEL_FLOATS * 4 / 16;
 #pragma unroll
-                    for (int q = 0; q < BLK / 2; ++q) {
-                        const float2 kv = row_pair<BF16>(raw, q);
-                        xp[q] = pack2(kv.x, kv.y);
+                    for (int i = 0; i < NT; ++i) {
+                        if (G == 32 && i > 0 && p.one_tile) break;
+                        const unsigned d = tmem + i * KEY_COLS + col, a_hi = tmem + i * KEY_COLS + (blk == 0 ? KEY_E0_COL : (blk - 1) * KEY_BLK);
+                        const u64 a_lo = a_lo0 + ((blk & 1) * NT + i) * (KEY_E_FLOATS * 4 / 16);
+                        umma_tf32_ss(d, a_lo, hi, idesc, accumulate);                                           // E_lo (shared memory) x Whi
+                        umma_tf32_ss(d, a_lo + 2 * KEY_A_LBO / 16, hi + step, idesc, 1u);
+                        umma_tf32_ts(d, a_hi, lo, idesc, 1u);                                                   // E_hi (tensor memory) x Wlo
+                        umma_tf32_ts(d, a_hi + 8, lo + step, idesc, 1u);
+                        umma_tf32_ts(d, a_hi, hi, idesc, 1u);                                                   // E_hi x Whi
+                        umma_tf32_ts(d, a_hi + 8, hi + step, idesc, 1u);
                     }
-                } else {
-                    // the MMAs that complete this block's corrections were committed after the previous sweep
-                    if (!shared_words[1] && !mbar_wait(my_mbar, phase)) {
-                        shared_words[1] = 1;
-                        atomicOr(p.status, SQUAT_FLAG_DEVICE_TIMEOUT);
-                    }
-                    phase ^= 1;
-                    tc_fence_after();
-                    unsigned dv[32];
-#ifdef SQUAT_CHECKED
-                    {
-                        const unsigned col = (t_mine + (blk - 1) * BLK) & 0xffffu, lo = t_tile & 0xffffu;
-                        if (!sq_chk(col >= lo && col + 32 <= lo + TC_EHI_COL && ((t_mine >> 16) & 0x7f) == (unsigned)(wq * 32) &&
-                                    lo + TC_COLS_PER_TILE <= (tmem_base & 0xffffu) + TC_TMEM_COLS, p.status)) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) dv[i] = 0;
-                        } else
-                            tmem_ld32(t_mine + (blk - 1) * BLK, dv);
-                    }
-#else
-                    tmem_ld32(t_mine + (blk - 1) * BLK, dv);
-#endif
-#pragma unroll
-                    for (int q = 0; q < BLK / 2; ++q) {
-                        const float2 kv = row_pair<BF16>(raw, q);
-                        xp[q] = pack2(__fadd_rn(kv.x, __uint_as_float(dv[2 * q])), __fadd_rn(kv.y, __uint_as_float(dv[2 * q + 1])));
+                };
+                if (key_elected()) {
+                    if (blk < KEY_SPLIT) {
+                        products(0, KEY_BLK, blk * KEY_BLK, blk != 0);
+                        tc_commit(mbar_d);
+                        products(KEY_BLK, nb - KEY_BLK, (blk + 1) * KEY_BLK, blk != 0);
+                    } else {
+                        products(0, KEY_BLK, key_late_col(blk + 1), blk != KEY_SPLIT);
+                        tc_commit(mbar_d);
+#pragma unroll 1
+                        for (int t = blk + 2; t < KEY_NBLK; ++t) products((t - blk - 1) * KEY_BLK, KEY_BLK, key_late_col(t), blk != KEY_SPLIT);
                     }
                 }
-                const bool more = blk + 1 < NBLK;
-                // prefetch: the next block of this tile, or the first block of the next round's tile
-                if (more) load_keys(raw, cur.row, (blk + 1) * BLK);
-                else if (nxt_valid) load_keys(raw, nxt_row, 0);
+                __syncwarp();
+            }
+        }
+        // Every batch of products has been waited for by the sweeping warps unless a wait ran out; then commit once more and
+        // give the tensor core a bounded time to drain before the columns are handed back.
+        if (*timeout) {
+            if (key_elected()) tc_commit(mbar_pan);
+            mbar_wait(mbar_pan, img_phase);
+        }
+        tc_fence_before();
+        __syncthreads();
+        return;
+    }
 
-                const float *diag = img + blk * BLK * BLK;
-                uint32_t cw[WORDS_PER_BLK];
-                float my_scale = 0.0f, my_zero = 0.0f;
-                SweepChk ck;
-#ifdef SQUAT_CHECKED
-                ck.status = p.status;
-                ck.img = img;
-                ck.e_region = Eall + slot * TC_E_FLOATS;
-                ck.tmem_lo = (t_tile & 0xffffu) + TC_EHI_COL;
-                ck.tmem_hi = (t_tile & 0xffffu) + TC_COLS_PER_TILE;
-#endif
-                if (blk < (int)shared_words[2 + TC_SLOTS])
-                    sweep_block<BITS, NW, true, M16>(xp, diag, t_mine + TC_EHI_COL, e_lo, more, lane, 1 + team, wteam, red, cw, my_scale, my_zero, ck);
-                else
-                    sweep_block<BITS, NW, false, M16>(xp, diag, t_mine + TC_EHI_COL, e_lo, more, lane, 1 + team, wteam, red, cw, my_scale, my_zero, ck);
-
-                if (more) {
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // E_hi is in tensor memory
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // E_lo rows, for the tensor core
-                    tc_fence_before();
-                    __threadfence_block();
-                    __syncwarp();
-                    // the last of the slot's four warps to get here issues the MMAs; nobody waits at a barrier
-                    bool last = false;
-                    if (lane == 0) last = (atomicAdd(const_cast<unsigned *>(shared_words) + 2 + slot, 1u) & 3u) == 3u;
-                    if (last) {
-                        __threadfence_block();
-                        tc_fence_after();
-                        const int nb = 3 * BLK - blk * BLK;        // channels still to come: 96, 64, 32
-                        const unsigned idesc = tc_idesc(nb);
-                        const unsigned b_lbo = 16u * nb;
-                        const unsigned bhi = smem_u32(Bhi + tc_panel_off(blk)), blo = smem_u32(Blo + tc_panel_off(blk));
-                        const unsigned d = t_tile + blk * BLK;
-#ifdef SQUAT_CHECKED
-                        // the windows the descriptors open: A = this slot's E_lo operand, B = the panels of source block blk
-                        // inside the staged image, D / A-from-tensor-memory = columns of this tile
-                        const unsigned img_lo = smem_u32(img), e_lo_lo = smem_u32(Eall + slot * TC_E_FLOATS);
-                        const unsigned panel_bytes = (unsigned)nb * BLK * 4;
-                        const bool desc_ok =
-                            a_lo == e_lo_lo && a_lo + (BLK / 8 - 1) * 2 * TC_A_LBO + 2 * TC_A_LBO <= e_lo_lo + TC_E_FLOATS * 4 &&
-                            bhi >= img_lo + TC_DIAG_FLOATS * 4 && bhi + panel_bytes <= img_lo + (TC_DIAG_FLOATS + TC_PANEL_FLOATS) * 4 &&
-                            blo >= img_lo + (TC_DIAG_FLOATS + TC_PANEL_FLOATS) * 4 && blo + panel_bytes <= img_lo + TC_IMG_FLOATS * 4 &&
-                            (a_lo & 15u) == 0 && (bhi & 15u) == 0 && (blo & 15u) == 0 &&
-                            (d & 0xffffu) + nb <= (t_tile & 0xffffu) + TC_EHI_COL &&
-                            (t_tile & 0xffffu) + TC_COLS_PER_TILE <= (tmem_base & 0xffffu) + TC_TMEM_COLS;
-                        if (sq_chk(desc_ok, p.status)) {
-#endif
+    int staged = -1;
+#pragma unroll 1
+    for (int unit = u_lo; unit < u_hi; ++unit) {
+        const int h = unit / p.units_per_head;
+        if (h != staged) {
+            if (staged >= 0) {                           // (the first copy was started at kernel entry)
+                // every read of the old image is over: by the lanes, and by the products, the last of which were waited for
+                __syncthreads();
+                if (threadIdx.x == 0) stage(h);
+            }
+            bounded_wait(mbar_diag, img_phase);
+            img_phase ^= 1;
+            staged = h;
+        }
+        Place nxt = cur;
+        if (unit + 1 < u_hi) locate(unit + 1, nxt);
+        unsigned cw[NT][BITS / 2], cw_even[NT][BITS / 2];
+#pragma unroll 1
+        for (int blk = 0; blk < KEY_NBLK; ++blk) {
+            const bool more = blk + 1 < KEY_NBLK;
+            u64 x[KEY_BLK][NP];
 #pragma unroll
-                        for (int ks = 0; ks < BLK / 8; ++ks)         // E_lo (shared memory) x Whi
-                            umma_tf32_ss(d, umma_desc(a_lo + ks * 2 * TC_A_LBO, TC_A_LBO, TC_SBO),
-                                         umma_desc(bhi + ks * 2 * b_lbo, b_lbo, TC_SBO), idesc, (blk | ks) != 0);
+            for (int c = 0; c < KEY_BLK; ++c)
 #pragma unroll
-                        for (int ks = 0; ks < BLK / 8; ++ks)         // E_hi (tensor memory) x Wlo
-                            umma_tf32_ts(d, t_tile + TC_EHI_COL + 8 * ks, umma_desc(blo + ks * 2 * b_lbo, b_lbo, TC_SBO), idesc, 1u);
+                for (int i = 0; i < NP; ++i) x[c][i] = pack2(raw.get(2 * i, c), raw.get(2 * i + 1, c));
+            if (more) load_rows(cur, blk + 1);           // (before the wait: what can be done ahead of it is)
+            else if (unit + 1 < u_hi) load_rows(nxt, 0);
+            if (blk > 0) {
+                bounded_wait(mbar_d, phase);             // the products that complete this block's corrections
+                phase ^= 1;
+                tc_fence_after();
+                unsigned d[NT][16];
 #pragma unroll
-                        for (int ks = 0; ks < BLK / 8; ++ks)         // E_hi x Whi
-                            umma_tf32_ts(d, t_tile + TC_EHI_COL + 8 * ks, umma_desc(bhi + ks * 2 * b_lbo, b_lbo, TC_SBO), idesc, 1u);
-#ifdef SQUAT_CHECKED
-                        }
-#endif
-                        tc_commit(my_mbar);
-                    }
-                    __syncwarp();
-                }
-
-                if (cur.active) {
-                    unsigned char *cp = cur.codes + blk * (BLK * BITS / 8);
-                    if (!SQ_CHK_G(p.status, cp, BLK * BITS / 8, p.x_codes)) {
-                    } else if (WORDS_PER_BLK == 2)
-                        *reinterpret_cast<uint2 *>(cp) = make_uint2(cw[0], cw[1]);
-                    else
-                        *reinterpret_cast<uint4 *>(cp) = make_uint4(cw[0], cw[1], cw[WORDS_PER_BLK > 2 ? 2 : 0], cw[WORDS_PER_BLK > 2 ? 3 : 0]);
-                    if (wteam == 0 && SQ_CHK_G(p.status, static_cast<char *>(p.scales) + (cur.meta + blk * BLK) * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_scales) &&
-                        SQ_CHK_G(p.status, static_cast<char *>(p.zeros) + (cur.meta + blk * BLK) * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_zeros)) {
-                        if (M16) {
-                            reinterpret_cast<__half *>(p.scales)[cur.meta + blk * BLK] = __float2half_rn(my_scale);   // exact
-                            reinterpret_cast<__half *>(p.zeros)[cur.meta + blk * BLK] = __float2half_rn(my_zero);
-                        } else {
-                            reinterpret_cast<float *>(p.scales)[cur.meta + blk * BLK] = my_scale;
-                            reinterpret_cast<float *>(p.zeros)[cur.meta + blk * BLK] = my_zero;
-                        }
-                        if (!(my_scale > 0.0f && my_scale < __int_as_float(0x7f800000)))
-                            atomicOr(p.status, my_scale == 0.0f ? SQUAT_FLAG_ZERO_RANGE : SQUAT_FLAG_NONFINITE);
-                    }
+                for (int t = 0; t < NT; ++t) key_tmem_ld16(t_mine + t * KEY_COLS + (blk - 1) * KEY_BLK, d[t]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int c = 0; c < KEY_BLK; ++c)
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) x[c][i] = fadd2(x[c][i], pack2(__uint_as_float(d[2 * i][c]), __uint_as_float(d[2 * i + 1][c])));
+                if (blk > KEY_SPLIT) {
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) key_tmem_ld16(t_mine + t * KEY_COLS + key_late_col(blk), d[t]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int c = 0; c < KEY_BLK; ++c)
+#pragma unroll
+                        for (int i = 0; i < NP; ++i) x[c][i] = fadd2(x[c][i], pack2(__uint_as_float(d[2 * i][c]), __uint_as_float(d[2 * i + 1][c])));
                 }
             }
-        } else if (nxt_valid) {
-            load_keys(raw, nxt_row, 0);
+
+            const u64 *diag = sm.diag + blk * KEY_BLK * KEY_BLK;
+            const unsigned e_hi = t_mine + (blk == 0 ? KEY_E0_COL : (blk - 1) * KEY_BLK);
+            float *e_lo = &sm.e_lo[blk & 1][0][(warp * 32 + lane) * 4];
+            float *gscale = &sm.grid[warp][0][(blk & 1) * KEY_BLK * NGL], *gzero = &sm.grid[warp][1][(blk & 1) * KEY_BLK * NGL];
+            // element-wise updates leave channel 0 alone uncorrected: then the usual code decides that one exactly (a block's worth of
+            // the exact code is longer by a third, and has to be fetched)
+            if (exact_channels > max(1, blk * KEY_BLK)) sweep_pairs<BITS, NP, NGL, true, M16>(x, diag, e_hi, e_lo, lane, true, gscale, gzero, cw);
+            else sweep_pairs<BITS, NP, NGL, false, M16>(x, diag, e_hi, e_lo, lane, blk == 0, gscale, gzero, cw);
+
+            if (more) {
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // E_hi is in tensor memory
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // E_lo rows, for the tensor core
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar_e) : "memory");
+            }
+            if (blk & 1) {                               // 32 channels are complete
+                __syncwarp();                            // (the grids lane 0 wrote)
+                const int at = (blk >> 1) * 32;
+#pragma unroll
+                for (int i = 0; i < NT; ++i) {
+                    unsigned char *cp = cur.codes[i / (NT / NGL)] + i % (NT / NGL) * (32 * D * BITS / 8) + at * BITS / 8;
+                    if (cur.active[i / (NT / NGL)] && SQ_CHK_G(p.status, cp, 32 * BITS / 8, p.x_codes)) {
+                        if (BITS == 2) *reinterpret_cast<uint2 *>(cp) = make_uint2(cw_even[i][0], cw[i][0]);
+                        else *reinterpret_cast<uint4 *>(cp) = make_uint4(cw_even[i][0], cw_even[i][BITS / 2 - 1], cw[i][0], cw[i][BITS / 2 - 1]);
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < NGL; ++g) {
+                    const float2 sz = make_float2(sm.grid[warp][0][lane * NGL + g], sm.grid[warp][1][lane * NGL + g]);
+                    const long long meta = cur.meta[g] + at;
+                    if (cur.active[g] && SQ_CHK_G(p.status, static_cast<char *>(p.scales) + meta * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_scales) &&
+                        SQ_CHK_G(p.status, static_cast<char *>(p.zeros) + meta * (M16 ? 2 : 4), M16 ? 2 : 4, p.x_zeros)) {
+                        if (M16) {
+                            static_cast<__half *>(p.scales)[meta] = __float2half_rn(sz.x);      // exact
+                            static_cast<__half *>(p.zeros)[meta] = __float2half_rn(sz.y);
+                        } else {
+                            static_cast<float *>(p.scales)[meta] = sz.x;
+                            static_cast<float *>(p.zeros)[meta] = sz.y;
+                        }
+                        if (!(sz.x > 0.0f && sz.x < __int_as_float(0x7f800000)))
+                            atomicOr(p.status, sz.x == 0.0f ? SQUAT_FLAG_ZERO_RANGE : SQUAT_FLAG_NONFINITE);
+                    }
+                }
+                __syncwarp();                            // before the next sweep writes grids
+            } else {
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+#pragma unroll
+                    for (int w = 0; w < BITS / 2; ++w) cw_even[i][w] = cw[i][w];
+            }
         }
-        start += n_round;
+        cur = nxt;
     }
 
-    // Every committed batch has been waited for unless a wait ran out; then commit once more per slot and give the
-    // tensor core a bounded time to drain before the columns are handed back.
-    if (shared_words[1] && wq == 0 && lane == 0) {
-        tc_commit(my_mbar);
-        mbar_wait(my_mbar, phase);
-    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((unsigned)TC_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
-// Writes, per head, the 64 KB image of the update matrix that the key kernel stages in shared memory:
-//   [0, 4096)        the four diagonal 32 x 32 blocks of W^T, row-major: block b, row jj, column c = W^T[32 b + jj][32 b + c]
-//   [4096, 10240)    hi panels of source blocks b = 0, 1, 2: B_b(n, k) = W[32 (b + 1) + n][32 b + k] = W^T[32 b + k][32 (b + 1) + n],
-//                    n < 96 - 32 b, k < 32, rounded to tf32, K-major in 8 x 16-byte core matrices:
-//                    float index (k / 4) * 4 N + 4 n + k % 4 with N = 96 - 32 b
-//   [10240, 16384)   lo panels: tf32(W - hi), same layout
-// PACK_SLICES CTAs per head (grid (heads, slices): the kernel is a chain of two dependent global accesses, so more CTAs,
-// not more work per thread, shorten it); each thread takes (panel, 4-k chunk, channel n): four coalesced row reads, one
-// 16-byte store.
-__global__ void __launch_bounds__(256) pack_w_kernel(const float *__restrict__ Wt, float *__restrict__ Wimg, int exact_blocks,
-                                                     int *__restrict__ exact_blocks_dev)
+// Writes, per head, the image that quant_keys_kernel stages in shared memory:
+//   u64 [8][16][16]   diagonal 16 x 16 blocks of W^T, row-major, every entry as a pair of equal floats
+//   hi panels         of source blocks b = 0 .. 6: B_b(n, k) = W[16 (b + 1) + n][16 b + k] = W^T[16 b + k][16 (b + 1) + n],
+//                     n < 112 - 16 b, k < 16, rounded to tf32, K-major in 8 x 16-byte core matrices:
+//                     float index (k / 4) * 4 N + 4 n + k % 4 with N = 112 - 16 b
+//   lo panels         tf32(W - hi), same layout
+// Grid (heads, slices): the kernel is a chain of two dependent global accesses, so more CTAs, not more work per thread, shorten
+// it; each thread takes (panel, 4-k chunk, channel n): four coalesced row reads, one 16-byte store.
+__global__ void __launch_bounds__(256) pack_w_kernel(const float *__restrict__ Wt, float *__restrict__ Wimg, int exact_channels,
+                                                        int *__restrict__ exact_channels_dev)
 {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *exact_blocks_dev = exact_blocks;    // travels with the matrices it describes
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *exact_channels_dev = exact_channels;    // travels with the matrices it describes
     const float *src = Wt + (long long)blockIdx.x * D * D;
-    float *img = Wimg + (long long)blockIdx.x * TC_IMG_FLOATS;
+    float *img = Wimg + (long long)blockIdx.x * KEY_IMG_FLOATS;
     const int first = blockIdx.y * blockDim.x + threadIdx.x, stride = gridDim.y * blockDim.x;
-    for (int i = first; i < TC_DIAG_FLOATS / 4; i += stride) {
-        const int b = i / (BLK * BLK / 4), r = i % (BLK * BLK / 4), jj = r / (BLK / 4), c4 = r % (BLK / 4);
-        reinterpret_cast<float4 *>(img)[i] = __ldg(reinterpret_cast<const float4 *>(src + (b * BLK + jj) * D + b * BLK + 4 * c4));
+    for (int i = first; i < KEY_NBLK * KEY_BLK * KEY_BLK / 2; i += stride) {
+        const int b = i / (KEY_BLK * KEY_BLK / 2), r = i % (KEY_BLK * KEY_BLK / 2), jj = r / (KEY_BLK / 2), c2 = r % (KEY_BLK / 2);
+        const float2 v = __ldg(reinterpret_cast<const float2 *>(src + (b * KEY_BLK + jj) * D + b * KEY_BLK + 2 * c2));
+        reinterpret_cast<float4 *>(img)[i] = make_float4(v.x, v.x, v.y, v.y);
     }
-    float *Bhi = img + TC_DIAG_FLOATS, *Blo = Bhi + TC_PANEL_FLOATS;
-    for (int i = first; i < TC_PANEL_FLOATS / 4; i += stride) {
-        const int f = 4 * i;                                 // first float of the 16-byte unit
-        const int b = f < tc_panel_off(1) ? 0 : (f < tc_panel_off(2) ? 1 : 2);
-        const int nb = 3 * BLK - b * BLK;
-        const int r = (f - tc_panel_off(b)) / 4;             // unit within the panel: kc * nb + n
-        const int kc = r / nb, n = r % nb;
-        const float *g = src + (b * BLK + 4 * kc) * D + (b + 1) * BLK + n;
+    float *hi = img + KEY_DIAG_FLOATS, *lo = hi + KEY_PANEL_FLOATS;
+    for (int i = first; i < KEY_PANEL_FLOATS / 4; i += stride) {
+        int b = 0;
+#pragma unroll
+        for (int t = 1; t < KEY_NBLK - 1; ++t) b += 4 * i >= key_panel_off(t);
+        const int nb = D - (b + 1) * KEY_BLK, r = i - key_panel_off(b) / 4, kc = r / nb, n = r % nb;   // unit within the panel: kc * nb + n
+        const float *g = src + (b * KEY_BLK + 4 * kc) * D + (b + 1) * KEY_BLK + n;
         const float w0 = __ldg(g), w1 = __ldg(g + D), w2 = __ldg(g + 2 * D), w3 = __ldg(g + 3 * D);
         const float4 whi = make_float4(__uint_as_float(tf32_of(w0)), __uint_as_float(tf32_of(w1)),
                                        __uint_as_float(tf32_of(w2)), __uint_as_float(tf32_of(w3)));
-        reinterpret_cast<float4 *>(Bhi)[i] = whi;
-        reinterpret_cast<float4 *>(Blo)[i] =
+        reinterpret_cast<float4 *>(hi)[i] = whi;
+        reinterpret_cast<float4 *>(lo)[i] =
             make_float4(__uint_as_float(tf32_of(__fsub_rn(w0, whi.x))), __uint_as_float(tf32_of(__fsub_rn(w1, whi.y))),
                         __uint_as_float(tf32_of(__fsub_rn(w2, whi.z))), __uint_as_float(tf32_of(__fsub_rn(w3, whi.w))));
     }
 }
 
-template <int BITS, int NW, bool BF16, bool M16>
-int launch_keys_inst(const KeyParams &p, int grid, size_t smem, cudaStream_t st)
+template <int BITS, int G, bool BF16, bool M16>
+int launch_inst(const KeyParams &p, int grid, cudaStream_t st)
 {
     static std::atomic<unsigned long long> allowed{0};
-    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(quant_keys_kernel<BITS, NW, BF16, M16>), smem, allowed)) return rc;
-    return squat_launch(quant_keys_kernel<BITS, NW, BF16, M16>, grid, TC_THREADS, smem, st, p);
+    if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(quant_keys_kernel<BITS, G, BF16, M16>), sizeof(KeyShared<key_np(G)>), allowed)) return rc;
+    return squat_launch(quant_keys_kernel<BITS, G, BF16, M16>, grid, KEY_THREADS, sizeof(KeyShared<key_np(G)>), st, p);
 }
-
-template <int BITS, int NW>
-int launch_keys(KeyParams p, int dtype, int meta16, cudaStream_t st)
+template <int BITS, int G>
+int launch(const KeyParams &p, int grid, int dtype, int meta16, cudaStream_t st)
 {
-    const long long groups_per_head = (long long)p.B * p.groups_per_bh;
-    const long long tiles_per_head = (groups_per_head + 4 / NW - 1) / (4 / NW);
-    if (tiles_per_head * p.H > 0x7fffffffLL) return SQUAT_ERR_UNSUPPORTED;          // the kernel counts tiles in 32 bits
-    p.groups_per_head = (int)groups_per_head;
-    p.tiles_per_head = (int)tiles_per_head;
-    p.total_tiles = (int)(tiles_per_head * p.H);
-
-    const int sms = squat_sm_count();
-    constexpr int GPT = 4 / NW;
-    constexpr int NTEAMS = TC_SLOTS * GPT;
-    // 193 KB: well over half an SM's shared memory, so two CTAs (each asking for all 512 tensor-memory columns)
-    // never share an SM
-    const size_t smem = sizeof(float) * (TC_SLOTS * TC_E_FLOATS + 2 * TC_IMG_FLOATS) +
-                        sizeof(float2) * (NTEAMS * 2 * NW) + sizeof(u64) * (TC_SLOTS + 1) + 4 * (3 + TC_SLOTS) + 8;
-    const int grid = p.total_tiles < sms ? p.total_tiles : sms;                     // one tile per CTA at least
-    int rc;
-    if (dtype == SQUAT_BF16) rc = meta16 ? launch_keys_inst<BITS, NW, true, true>(p, grid, smem, st) : launch_keys_inst<BITS, NW, true, false>(p, grid, smem, st);
-    else rc = meta16 ? launch_keys_inst<BITS, NW, false, true>(p, grid, smem, st) : launch_keys_inst<BITS, NW, false, false>(p, grid, smem, st);
-    return rc;
+    if (dtype == SQUAT_BF16) return meta16 ? launch_inst<BITS, G, true, true>(p, grid, st) : launch_inst<BITS, G, true, false>(p, grid, st);
+    return meta16 ? launch_inst<BITS, G, false, true>(p, grid, st) : launch_inst<BITS, G, false, false>(p, grid, st);
 }
 
 }  // namespace
 
-int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_blocks, int *exact_blocks_dev, cudaStream_t st)
+int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_channels, int *exact_channels_dev, cudaStream_t st)
 {
     constexpr int PACK_SLICES = 8;
-    pack_w_kernel<<<dim3(H, PACK_SLICES), 256, 0, st>>>(Wt, Wimg, exact_blocks, exact_blocks_dev);
+    pack_w_kernel<<<dim3(H, PACK_SLICES), 256, 0, st>>>(Wt, Wimg, exact_channels, exact_channels_dev);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
     return SQUAT_OK;
 }
 
 int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
-                            long long sb, long long sh, long long st_, int bits, int G,
-                            unsigned char *codes, void *scales, void *zeros,
-                            long long osb, long long osh, unsigned *status, const int *exact_blocks, int meta16, cudaStream_t st)
+                                 long long sb, long long sh, long long st_, int bits, int G,
+                                 unsigned char *codes, void *scales, void *zeros,
+                                 long long osb, long long osh, unsigned *status, const int *exact_channels, int meta16, cudaStream_t st)
 {
     KeyParams p;
     p.Wimg = Wimg; p.k = k; p.sb = sb; p.sh = sh; p.st = st_;
     p.codes = codes; p.scales = scales; p.zeros = zeros; p.osb = osb; p.osh = osh;
-    p.B = batch; p.H = H; p.T = T; p.groups_per_bh = T / G;
+    p.groups_per_bh = T / G;
     p.status = status;
-    p.exact_blocks = exact_blocks;
+    p.exact_channels = exact_channels;
+    const long long groups_per_head = (long long)batch * p.groups_per_bh;
+    const int np = key_np(G), places = 2 / np * squat_sm_count();
+    // Where there is at most one tile of 128 tokens per SM (a window of a few sequences), a CTA takes one tile: a hand-over then
+    // waits for half the products (4 x 32 heads x 128 tokens, G = 32: 16.3 -> 16.0 us; with 256 tiles two CTAs per SM of one tile
+    // each take 22.4 us, one CTA of two 16.5).
+    p.one_tile = G == 32 && H * ((groups_per_head + 3) / 4) <= squat_sm_count();
+    const long long unit = p.one_tile ? 4 : 256 * np / G;
+    const long long units_per_head = (groups_per_head + unit - 1) / unit;
+    if (groups_per_head > 0x3fffffffLL || units_per_head * H > 0x7fffffffLL) return SQUAT_ERR_UNSUPPORTED;      // counted in 32 bits
+    if (units_per_head == 0) return SQUAT_OK;
+    p.groups_per_head = (int)groups_per_head;
+    p.units_per_head = (int)units_per_head;
+    p.total_units = (int)(units_per_head * H);
 #ifdef SQUAT_CHECKED
     {
         const unsigned long long es = dtype == SQUAT_BF16 ? 2 : 4, ms = meta16 ? 2 : 4;
-        const long long ng = T / G;
         p.x_k = {k, (unsigned long long)((batch - 1) * sb + (H - 1) * sh + (long long)(T - 1) * st_ + D) * es};
         p.x_codes = {codes, (unsigned long long)((batch - 1) * osb + (H - 1) * osh + T) * (D * bits / 8)};
-        const unsigned long long meta_elems = (unsigned long long)(((batch - 1) * osb + (H - 1) * osh) / G + ng) * D;
+        const unsigned long long meta_elems = (unsigned long long)(((batch - 1) * osb + (H - 1) * osh) / G + T / G) * D;
         p.x_scales = {scales, meta_elems * ms};
         p.x_zeros = {zeros, meta_elems * ms};
-        p.x_img = {Wimg, (unsigned long long)H * TC_IMG_FLOATS * 4};
+        p.x_img = {Wimg, (unsigned long long)H * KEY_IMG_FLOATS * 4};
     }
 #endif
-    if ((long long)H * batch * (T / G) == 0) return SQUAT_OK;
+    const int grid = p.total_units < places ? p.total_units : places;
     if (bits == 2) {
-        if (G == 32) return launch_keys<2, 1>(p, dtype, meta16, st);
-        if (G == 64) return launch_keys<2, 2>(p, dtype, meta16, st);
-        if (G == 128) return launch_keys<2, 4>(p, dtype, meta16, st);
+        if (G == 32) return launch<2, 32>(p, grid, dtype, meta16, st);
+        if (G == 64) return launch<2, 64>(p, grid, dtype, meta16, st);
+        if (G == 128) return launch<2, 128>(p, grid, dtype, meta16, st);
     } else if (bits == 4) {
-        if (G == 32) return launch_keys<4, 1>(p, dtype, meta16, st);
-        if (G == 64) return launch_keys<4, 2>(p, dtype, meta16, st);
-        if (G == 128) return launch_keys<4, 4>(p, dtype, meta16, st);
+        if (G == 32) return launch<4, 32>(p, grid, dtype, meta16, st);
+        if (G == 64) return launch<4, 64>(p, grid, dtype, meta16, st);
+        if (G == 128) return launch<4, 128>(p, grid, dtype, meta16, st);
     }
     return SQUAT_ERR_UNSUPPORTED;
 }

@@ -32,6 +32,12 @@
 
 namespace {
 
+__device__ __forceinline__ void team_barrier(int id, int nthreads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+constexpr int BLK = 32;                               // channels per warp and step
 constexpr int KB_THREADS = 256;
 constexpr int KB_ROWS = 8;                            // tokens per thread and block
 constexpr unsigned KB_LBO = 128 * 16 + 16, KB_SBO = 128;   // bytes between 4-channel chunks of an E operand (16 more than the 128
@@ -39,7 +45,7 @@ constexpr unsigned KB_LBO = 128 * 16 + 16, KB_SBO = 128;   // bytes between 4-ch
 constexpr int KB_CHUNK_FLOATS = KB_LBO / 4;
 
 struct KeyBlockParams {
-    const float *Wimg;        // [H, d * d] staged images of the update matrices (pack_w_kernel)
+    const float *Wimg;        // [H, KEY_IMG_FLOATS] staged images of the update matrices (pack_w_kernel)
     const void *k;
     long long sb, sh, st;     // element strides of k
     unsigned char *codes;
@@ -55,18 +61,34 @@ struct KeyBlockParams {
 #endif
 };
 
+// where the panel of step s starts (g = 32: 96, 64, 32 later channels)
+__host__ __device__ constexpr int kb_panel_off(int s) { return s == 0 ? 0 : s == 1 ? 32 * 96 : 32 * (96 + 64); }
+
 template <int GB>
 struct KbLayout {
     static constexpr int SLOTS = 64 / GB;                         // tiles of 128 tokens per CTA
     static constexpr int STEPS = D / GB;
     static constexpr int CHUNKS = GB / 4;                         // 4-channel chunks of an operand
     static constexpr int E_FLOATS = CHUNKS * KB_CHUNK_FLOATS;     // one tile's E_hi (or E_lo)
-    static constexpr int W_FLOATS = GB == 64 ? 64 * 64 : TC_PANEL_FLOATS;    // hi (or lo) panels
+    static constexpr int W_FLOATS = GB == 64 ? 64 * 64 : 32 * (96 + 64 + 32);    // hi (or lo) panels, K-major, GB source channels x the later ones
     static constexpr int SLOT_COLS = GB == 64 ? 64 : 128;
     static constexpr int TMEM_COLS = SLOTS * SLOT_COLS;
     static constexpr int WARPS_PER_TILE = 8 / SLOTS;
     static constexpr size_t SMEM = sizeof(float) * (2 * SLOTS * E_FLOATS + 2 * W_FLOATS) + sizeof(u64) * (SLOTS + 1) + 4 * (2 + SLOTS) + 8;
 };
+
+// 32 consecutive columns of the warp's lanes into registers (lane l gets row l)
+__device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
 
 // 4 channels of the thread's 8 tokens as they are in memory
 template <bool BF16>
@@ -297,26 +319,22 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
     grid_wait();
     const unsigned img_mbar = smem_u32(mbar + Lay::SLOTS);
 
-    // one head's panels into shared memory (one thread); g = 64 takes only the rows that lead to channels 64 .. 127
+    // One head's panels into shared memory (one thread).  The image has them by 16 source channels with all later channels; of those
+    // only the channels behind the block of g are taken, and the source blocks of a step put side by side along K.
     auto stage_panels = [&](int h) {
-        const float *src = p.Wimg + (long long)h * TC_IMG_FLOATS + TC_DIAG_FLOATS;
-        if (!SQ_CHK_G(p.status, p.Wimg + (long long)h * TC_IMG_FLOATS, TC_IMG_FLOATS * 4, p.x_img)) return;
+        const float *src = p.Wimg + (long long)h * KEY_IMG_FLOATS + KEY_DIAG_FLOATS;
+        if (!SQ_CHK_G(p.status, src, 2 * KEY_PANEL_FLOATS * 4, p.x_img)) return;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(img_mbar), "r"(2 * Lay::W_FLOATS * 4) : "memory");
-        auto copy = [&](float *dst, const float *from, unsigned bytes) {
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(smem_u32(dst)), "l"(from), "r"(bytes), "r"(img_mbar) : "memory");
-        };
-        for (int part = 0; part < 2; ++part) {
-            float *dst = part ? W_lo : W_hi;
-            const float *from = src + part * TC_PANEL_FLOATS;
-            if (GB == 64) {
-                for (int kc = 0; kc < 8; ++kc) copy(dst + kc * 256, from + kc * (4 * 96) + 4 * 32, 1024);     // source channels 0 .. 31
-                copy(dst + 8 * 256, from + tc_panel_off(1), 8192);                                             // 32 .. 63
-            } else {
-                copy(dst, from, Lay::W_FLOATS * 4);
+        for (int part = 0; part < 2; ++part)
+            for (int b = 0; b < (D - GB) / KEY_BLK; ++b) {                 // source blocks that lead anywhere
+                const int step = b * KEY_BLK / GB, n = D - (step + 1) * GB, nb = D - (b + 1) * KEY_BLK;        // taken, present
+                float *dst = (part ? W_lo : W_hi) + (GB == 64 ? 0 : kb_panel_off(step)) + (b * KEY_BLK - step * GB) * n;
+                const float *from = src + part * KEY_PANEL_FLOATS + key_panel_off(b) + 4 * (nb - n);
+                for (int kc = 0; kc < KEY_BLK / 4; ++kc)
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(smem_u32(dst + kc * 4 * n)), "l"(from + kc * 4 * nb), "r"(16u * n), "r"(img_mbar) : "memory");
             }
-        }
     };
 
     if (threadIdx.x == 0) {
@@ -560,7 +578,7 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                     const int nb = D - (step + 1) * GB;                 // channels still to come
                     const unsigned idesc = tc_idesc(nb), b_lbo = 16u * nb;
                     const unsigned a_hi = smem_u32(E_hi), a_lo = smem_u32(E_lo);
-                    const int off = GB == 64 ? 0 : tc_panel_off(step < 3 ? step : 0);
+                    const int off = GB == 64 ? 0 : kb_panel_off(step);
                     const unsigned b_hi = smem_u32(W_hi + off), b_lo = smem_u32(W_lo + off);
                     const unsigned d = t_tile + step * GB;
                     if (SQ_CHK_C(p.status, off + nb * GB <= Lay::W_FLOATS && step * GB + nb <= Lay::SLOT_COLS)) {
@@ -665,7 +683,7 @@ int squat_launch_quant_keys_block(int block_g, const float *Wimg, const void *k,
         const unsigned long long meta_elems = (unsigned long long)(((batch - 1) * osb + (H - 1) * osh) / G + T / G) * D;
         p.x_scales = {scales, meta_elems * ms};
         p.x_zeros = {zeros, meta_elems * ms};
-        p.x_img = {Wimg, (unsigned long long)H * TC_IMG_FLOATS * 4};
+        p.x_img = {Wimg, (unsigned long long)H * KEY_IMG_FLOATS * 4};
     }
 #endif
     if ((long long)H * batch * (T / G) == 0) return SQUAT_OK;
