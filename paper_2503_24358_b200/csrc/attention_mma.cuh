@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     __shared__ unsigned tmem_sm;
     __shared__ float2 qz_sm[MAX_TILES][NG][NQ];                 // inverse of the fixed point, sum of query x zero-point
     __shared__ float red_sm[WARPS][NG * NQ + NQ + 2], top_sm[WARPS][NG * NQ];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);       // (uniform)
     const int parts = p.nchunk + (p.R > 0), chunk = blockIdx.x % parts, qpass = blockIdx.x / parts;
     const int h = blockIdx.y, b = blockIdx.z;
     const int qpk = p.Hq / p.H, hq0 = h * qpk + qpass * NQ, nq_here = min(NQ, qpk - qpass * NQ);
@@ -388,6 +388,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     auto load_vs = [&](int tile) { vs_next.load(p.vs, ctok0 + min(tile * TILE + tid, last_tok)); };
     auto load_vz = [&](int tile) { vz_next.load(p.vz, ctok0 + min(tile * TILE + tid, last_tok)); };
     if (!ROPE) load_kmeta(0);
+    load_vs(0);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sm)), "r"((unsigned)S::TMEM_COLS) : "memory");
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const unsigned tmem = tmem_sm, t_lanes = tmem + ((unsigned)(warp * 32) << 16), t_mine = t_lanes + 32 + my_group * NQ * 4;
+    const unsigned tmem = __shfl_sync(0xffffffffu, tmem_sm, 0), t_lanes = tmem + ((unsigned)(warp * 32) << 16), t_mine = t_lanes + 32 + my_group * NQ * 4;
     bool ok = true;
 
     // a row of key codes as 128 bytes in tensor memory, this lane's
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
     // 32 rows.  One product is in flight at a time; the digits of the next one are made meanwhile in the other buffer.
     unsigned issued = 0;
     auto issue = [&](int buf, bool values, bool accumulate) {
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
             const u64 a = codes_desc(smem_u32(codes_sm)), dg = digits_desc(smem_u32(digits_sm + buf * S::DIG_BYTES));
 #pragma unroll
@@ -531,7 +532,6 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
 #pragma unroll 1
         for (int tile = 0; tile < tiles; ++tile) {
             const int tok = tile * TILE + 32 * warp;                   // the warp's first token; n_tok is a multiple of 32
-            load_vs(tile);
             if (tok < n_tok) {
                 __syncwarp();
 #pragma unroll
@@ -586,12 +586,13 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
                 mx[j] = max_nan(mx[j], s);
             }
             widen();
+            load_vs(tile + 1 < tiles ? tile + 1 : 0);               // (0: for the weighted values)
         }
+        load_vz(0);
     } else {
 #pragma unroll 1
         for (int tile = 0; tile < tiles; ++tile) {
             const int buf = tile & 1;
-            load_vs(tile);
             float ks[4], kz[4];
             ks_next.get(ks);
             kz_next.get(kz);
@@ -619,6 +620,8 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
                     else *reinterpret_cast<uint32_t *>(dst) = dig[i][0];
                 }
             }
+            widen();
+            load_vs(tile + 1 < tiles ? tile + 1 : 0);               // (0: for the weighted values)
             if (tile > 0) read_scores(tile - 1);                    // also frees the keys' columns and the accumulator
             unpack_keys();
             if (tile + 1 < tiles) load_keys(tile + 1);
@@ -627,12 +630,10 @@ __global__ void __launch_bounds__(THREADS, ATTN_CTAS_PER_SM(NQ, ROPE)) attn_mma_
             tc_fence_before();
             __syncthreads();
             issue(buf, false, false);
-            widen();
         }
+        load_vz(0);
         read_scores(tiles - 1);
     }
-    load_vs(0);
-    load_vz(0);
 
     // ---------------------------------------------------------------- maxima over the chunk
 #pragma unroll

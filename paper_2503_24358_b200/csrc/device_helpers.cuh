@@ -86,6 +86,13 @@ __device__ __forceinline__ void tc_commit(unsigned mbar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
+// one lane of a converged warp, always the same
+__device__ __forceinline__ bool elect_one()
+{
+    unsigned r;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(r));
+    return r != 0;
+}
 // 8-bit operands from shared memory, 32-bit integer accumulators in tensor memory
 __device__ __forceinline__ void mma_i8(unsigned d_taddr, u64 a_desc, u64 b_desc, unsigned idesc, unsigned accumulate)
 {

@@ -118,14 +118,6 @@ __device__ __forceinline__ void key_tmem_ld16(unsigned taddr, unsigned (&r)[16])
                  : "r"(taddr) : "memory");
 }
 
-// one lane of a converged warp, always the same
-__device__ __forceinline__ bool key_elected()
-{
-    unsigned r;
-    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(r));
-    return r != 0;
-}
-
 // 16 channels of the lane's tokens as they are in memory
 template <bool BF16, int NP>
 struct PairRows {
@@ -410,7 +402,7 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
                         umma_tf32_ts(d, a_hi + 8, hi + step, idesc, 1u);
                     }
                 };
-                if (key_elected()) {
+                if (elect_one()) {
                     if (blk < KEY_SPLIT) {
                         products(0, KEY_BLK, blk * KEY_BLK, blk != 0);
                         tc_commit(mbar_d);
@@ -428,7 +420,7 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
         // Every batch of products has been waited for by the sweeping warps unless a wait ran out; then commit once more and
         // give the tensor core a bounded time to drain before the columns are handed back.
         if (*timeout) {
-            if (key_elected()) tc_commit(mbar_pan);
+            if (elect_one()) tc_commit(mbar_pan);
             mbar_wait(mbar_pan, img_phase);
         }
         tc_fence_before();
