@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(D) lowrank_table_kernel(const double *__restri
                                                           int r, double lambda, float *__restrict__ table)
 {
     __shared__ double Vs[R][D];            // Vs[i][j] = v_j[i] = component j of eigenvector i
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the assembly of W may start beside this kernel (see there)
     const int h = blockIdx.x, j = threadIdx.x;
     const double *vec = eigvec + (long long)h * D * D;
     for (int i = 0; i < R; ++i) Vs[i][j] = i < r ? vec[(long long)i * D + j] : 0.0;

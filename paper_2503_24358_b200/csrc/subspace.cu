@@ -377,7 +377,10 @@ __global__ void __launch_bounds__(ASM_THREADS, 1) assemble_kernel(
         if (p < 15) publish(p + 1);
         __syncthreads();
     }
-    if (g == 1) return;
+    if (g == 1) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");      // (see the launcher) what follows this kernel follows the tables' too
+        return;
+    }
     // g > 1: block column t becomes L[rest, blk] * inverse(unit-lower diagonal block)
     if (g == 64) block_solve<64>(A, tid);
     else if (g == 32) block_solve<32>(A, tid);
@@ -444,9 +447,19 @@ int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int bloc
     constexpr size_t smem = ASM_SMEM;
     static std::atomic<unsigned long long> allowed{0};
     if (const int rc = squat_allow_smem(reinterpret_cast<const void *>(assemble_kernel), smem, allowed)) return rc;
-    assemble_kernel<<<s->n_kv_heads, ASM_THREADS, smem, st>>>(s->eigval, s->eigvec, rank_r, lambda, block_g, s->Wt, left_rows);
-    squat_count_launch();
-    SQUAT_LAUNCH_CHECK();
+    // Behind the tables of the rank-r form the assembly is a programmatic dependent that waits only at its end: the tables' kernel
+    // lets its dependents start at once, both read the eigen-pairs, which were complete before that kernel began, and neither
+    // reads what the other writes.  Two short kernels of few CTAs side by side: 8 heads x 256 tokens, r = 8,
+    // whole prompt pass 239.7 -> 229.0 us.
+    if (s->lowrank_r > 0) {
+        const double *vals = s->eigval, *vecs = s->eigvec;
+        const int rc = squat_launch(assemble_kernel, s->n_kv_heads, ASM_THREADS, smem, st, vals, vecs, rank_r, lambda, block_g, s->Wt, left_rows);
+        if (rc != SQUAT_OK) return rc;
+    } else {
+        assemble_kernel<<<s->n_kv_heads, ASM_THREADS, smem, st>>>(s->eigval, s->eigvec, rank_r, lambda, block_g, s->Wt, left_rows);
+        squat_count_launch();
+        SQUAT_LAUNCH_CHECK();
+    }
     return squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact_channels, s->exact_channels, st);
 }
 
