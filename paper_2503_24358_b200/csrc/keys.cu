@@ -28,8 +28,8 @@
 // 1 000, and tensor memory holds 512 tokens per SM, so two warps per scheduler have to cover each other's waits; issue slots are
 // 30 % busy.  What this kernel replaced swept blocks of 32 channels with one token per lane (16 warps per SM): every warp made
 // every channel's grid, read W for 32 tokens at a time and, for groups of 64 and 128, met the group's other warps for every
-// channel.  128 heads x 32768 tokens, before -> now: G = 128, 4 bits 1715 -> 923 us; G = 64 1578 -> 1022; G = 32 1293 -> 1062; 32 heads
-// x 4096, G = 32 47.2 -> 44.1; 64 x 32 heads x 128 89.6 -> 82.0; 32 heads x 128 15.0 -> 14.7.  On the way: four tokens per lane with
+// channel.  128 heads x 32768 tokens, before -> now: G = 128, 4 bits 1715 -> 919 us; G = 64 1578 -> 1023; G = 32 1293 -> 1059; 32 heads
+// x 4096, G = 32 47.2 -> 43.8; 64 x 32 heads x 128 89.6 -> 81.1; 32 heads x 128 15.0 -> 15.1.  On the way: four tokens per lane with
 // blocks of 32 channels was slower (50 KB of straight code: instruction fetch); a sweeping warp that also issued the products lost
 // 2 000 cycles a hand-over; converting the keys and asking for the next ones ahead of the wait instead of behind it was worth 6 to
 // 10 %.
@@ -52,11 +52,20 @@ namespace {
 constexpr int KEY_WARPS = 4, KEY_THREADS = 32 * (KEY_WARPS + 1);      // four sweeping warps, one that issues the products
 constexpr int KEY_COLS = 128, KEY_E0_COL = 112;                          // per tile: [0, 112) corrections, [112, 128) E_hi of block 0
 // The accumulator truncates on every addition, so corrections are gathered in two: what blocks 0 .. 3 push in the columns of the
-// channel, what blocks 4 .. 6 push onto blocks 5 .. 7 in columns that are free by then, and the sweep adds both.  (In one
-// accumulator the rms error of a group's minimum against 64 bits was 1.14e-7 of its range (rank 32, 2 bits, G = 32), 0.93e-7 in two; the
-// kernel of 32-channel blocks before this one had 0.94e-7.  Time: + 1 % for groups of 32 and 64, + 5 % for 128.)
-constexpr int KEY_SPLIT = 4;
-__host__ __device__ constexpr int key_late_col(int blk) { return blk == 7 ? KEY_E0_COL : (blk - KEY_SPLIT - 1) * KEY_BLK; }
+// channel, what blocks 4 .. 6 push onto blocks 5 .. 7 in columns that are free by then; the sweep adds both, each made larger by
+// what truncation has taken from it on average.  Rms error of a group's minimum against 64 bits, as a part of its range (rank 32, 2
+// bits, G = 32): one accumulator 1.14e-7, two 0.93e-7, corrected 0.67e-7; the kernel of 32-channel blocks before this one 0.94e-7.
+// Time: the second accumulator + 1 % for groups of 32 and 64, + 5 % for 128; the correction none.
+// Accuracy (rms error of a group's minimum against 64 bits, as a part of its range; rank 32, 2 bits, G = 32).  Corrections are gathered
+// apart from the keys and added once, when the channel's turn comes, so that a large key (an outlier channel) does not round every
+// push.  The tensor core's accumulator truncates on every addition; what that takes on average from a sum
+// that n source blocks have added to is 2, 4, 4, 6, 6, 6, 6 x 2^-24 of it (the regression of the corrected values' error on the
+// sum, on the part) and is given back: 1.14e-7 -> 0.71e-7 together.  The kernel of 32-channel blocks before this one: 0.94e-7.
+__device__ __forceinline__ u64 key_untruncate(int n)
+{
+    const float f = 1.0f + (float)min((n + 2) / 2, 3) * 0x1p-23f;
+    return pack2(f, f);
+}
 constexpr int KEY_E_FLOATS = 128 * KEY_BLK;                              // one tile's E_lo
 constexpr unsigned KEY_A_LBO = 128 * 16, KEY_SBO = 128;
 constexpr unsigned kMagicBits = 0x4B400000u;
@@ -142,7 +151,7 @@ struct PairRows {
 // memory for all the compiler knows.  The errors of the last block are stored like the others (a test per store would cut the
 // code into pieces) and used by nobody.
 template <int BITS, int NP, int NGL, bool EXACT, bool M16>
-__device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__restrict__ diag, unsigned e_hi, float *__restrict__ e_lo,
+__device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (&cor)[KEY_BLK][NP], const u64 *__restrict__ diag, unsigned e_hi, float *__restrict__ e_lo,
                                             int lane, bool exact_first, float *__restrict__ gscale, float *__restrict__ gzero, unsigned (&cw)[2 * NP][BITS / 2])
 {
     constexpr float L = float((1 << BITS) - 1);
@@ -152,10 +161,11 @@ __device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__
     const u64 magic2 = pack2(kMagic, kMagic), negl2 = pack2(-L, -L);
     float el[NT][4];                                    // [token][channel % 4]
     float m[NGL], mx[NGL];
-    auto extremes = [&](int jj) {
+    u64 x[NP];                                          // the channel's corrected values
+    auto extremes = [&]() {
         float v[NT];
 #pragma unroll
-        for (int i = 0; i < NP; ++i) unpack2(x[jj][i], v[2 * i], v[2 * i + 1]);
+        for (int i = 0; i < NP; ++i) unpack2(x[i], v[2 * i], v[2 * i + 1]);
 #pragma unroll
         for (int g = 0; g < NGL; ++g) {
             float lo = v[TPG * g], hi = lo;
@@ -178,7 +188,9 @@ __device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__
         }
     };
     read_row(0);
-    extremes(0);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) x[i] = fadd2(key[0][i], cor[0][i]);
+    extremes();
 #pragma unroll
     for (int jj = 0; jj < KEY_BLK; ++jj) {
         float scale[NGL], inv[NGL], z[NGL];
@@ -196,12 +208,17 @@ __device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__
                 asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv[g]) : "f"(fmaxf(rng, 1e-30f)));     // constant group: x - m = 0 -> code 0
             }
         }
+        u64 pre[NP];                                    // the next channel, but for this channel's push
+        if (jj + 1 < KEY_BLK) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) pre[i] = fadd2(key[jj + 1][i], cor[jj + 1][i]);
+        }
         u64 e[NP];
         float y[NT];
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             const int ga = 2 * i / TPG, gb = (2 * i + 1) / TPG;
-            const u64 n = fsub2(pack2(z[ga], z[gb]), x[jj][i]);                                 // -(x - m)
+            const u64 n = fsub2(pack2(z[ga], z[gb]), x[i]);                                 // -(x - m)
             u64 y2 = ffma2(M16 ? n : fmul2(n, negl2), pack2(inv[ga], inv[gb]), magic2);
             float &y0 = y[2 * i], &y1 = y[2 * i + 1];
             unpack2(y2, y0, y1);
@@ -236,13 +253,13 @@ __device__ __forceinline__ void sweep_pairs(u64 (&x)[KEY_BLK][NP], const u64 *__
         // the next channel's value and extremes first
         if (jj + 1 < KEY_BLK) {
 #pragma unroll
-            for (int i = 0; i < NP; ++i) x[jj + 1][i] = ffma2(e[i], w[jj + 1], x[jj + 1][i]);
-            extremes(jj + 1);
+            for (int i = 0; i < NP; ++i) x[i] = ffma2(e[i], w[jj + 1], pre[i]);
+            extremes();
         }
 #pragma unroll
         for (int c = jj + 2; c < KEY_BLK; ++c)
 #pragma unroll
-            for (int i = 0; i < NP; ++i) x[c][i] = ffma2(e[i], w[c], x[c][i]);
+            for (int i = 0; i < NP; ++i) cor[c][i] = ffma2(e[i], w[c], cor[c][i]);
         if (jj + 1 < KEY_BLK) read_row(jj + 1);
         if (lane == 0) {
             key_store_groups<NGL>(gscale + jj * NGL, scale);
@@ -384,17 +401,17 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
                 const int nb = D - (blk + 1) * KEY_BLK;             // channels still to come
                 const unsigned b_lbo = 16u * nb, bhi = pan + 4 * key_panel_off(blk);
                 const u64 step = (2 * b_lbo) >> 4;                 // 8 channels on
-                // onto n channels from the ch-th behind the block on, into the columns from `col` on, all tiles
-                auto products = [&](int ch, int n, int col, bool accumulate) {
-                    if (!SQ_CHK_C(p.status, key_panel_off(blk) + nb * KEY_BLK <= KEY_PANEL_FLOATS && ch + n <= nb && col + n <= KEY_COLS)) return;
+                // onto n channels from the ch-th behind the block on, all tiles
+                auto products = [&](int ch, int n) {
+                    if (!SQ_CHK_C(p.status, key_panel_off(blk) + nb * KEY_BLK <= KEY_PANEL_FLOATS && ch + n <= nb)) return;
                     const unsigned idesc = tc_idesc(n);
                     const u64 hi = umma_desc(bhi + 16u * ch, b_lbo, KEY_SBO), lo = hi + KEY_PANEL_FLOATS * 4 / 16;
 #pragma unroll
                     for (int i = 0; i < NT; ++i) {
                         if (G == 32 && i > 0 && p.one_tile) break;
-                        const unsigned d = tmem + i * KEY_COLS + col, a_hi = tmem + i * KEY_COLS + (blk == 0 ? KEY_E0_COL : (blk - 1) * KEY_BLK);
+                        const unsigned d = tmem + i * KEY_COLS + blk * KEY_BLK + ch, a_hi = tmem + i * KEY_COLS + (blk == 0 ? KEY_E0_COL : (blk - 1) * KEY_BLK);
                         const u64 a_lo = a_lo0 + ((blk & 1) * NT + i) * (KEY_E_FLOATS * 4 / 16);
-                        umma_tf32_ss(d, a_lo, hi, idesc, accumulate);                                           // E_lo (shared memory) x Whi
+                        umma_tf32_ss(d, a_lo, hi, idesc, blk != 0);                                            // E_lo (shared memory) x Whi
                         umma_tf32_ss(d, a_lo + 2 * KEY_A_LBO / 16, hi + step, idesc, 1u);
                         umma_tf32_ts(d, a_hi, lo, idesc, 1u);                                                   // E_hi (tensor memory) x Wlo
                         umma_tf32_ts(d, a_hi + 8, lo + step, idesc, 1u);
@@ -403,16 +420,9 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
                     }
                 };
                 if (elect_one()) {
-                    if (blk < KEY_SPLIT) {
-                        products(0, KEY_BLK, blk * KEY_BLK, blk != 0);
-                        tc_commit(mbar_d);
-                        products(KEY_BLK, nb - KEY_BLK, (blk + 1) * KEY_BLK, blk != 0);
-                    } else {
-                        products(0, KEY_BLK, key_late_col(blk + 1), blk != KEY_SPLIT);
-                        tc_commit(mbar_d);
-#pragma unroll 1
-                        for (int t = blk + 2; t < KEY_NBLK; ++t) products((t - blk - 1) * KEY_BLK, KEY_BLK, key_late_col(t), blk != KEY_SPLIT);
-                    }
+                    products(0, KEY_BLK);
+                    tc_commit(mbar_d);
+                    if (nb > KEY_BLK) products(KEY_BLK, nb - KEY_BLK);
                 }
                 __syncwarp();
             }
@@ -448,11 +458,14 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
 #pragma unroll 1
         for (int blk = 0; blk < KEY_NBLK; ++blk) {
             const bool more = blk + 1 < KEY_NBLK;
-            u64 x[KEY_BLK][NP];
+            u64 key[KEY_BLK][NP], cor[KEY_BLK][NP];      // keys, and what earlier channels have pushed onto them
 #pragma unroll
             for (int c = 0; c < KEY_BLK; ++c)
 #pragma unroll
-                for (int i = 0; i < NP; ++i) x[c][i] = pack2(raw.get(2 * i, c), raw.get(2 * i + 1, c));
+                for (int i = 0; i < NP; ++i) {
+                    key[c][i] = pack2(raw.get(2 * i, c), raw.get(2 * i + 1, c));
+                    cor[c][i] = 0;
+                }
             if (more) load_rows(cur, blk + 1);           // (before the wait: what can be done ahead of it is)
             else if (unit + 1 < u_hi) load_rows(nxt, 0);
             if (blk > 0) {
@@ -460,22 +473,14 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
                 phase ^= 1;
                 tc_fence_after();
                 unsigned d[NT][16];
+                const u64 up = key_untruncate(blk);
 #pragma unroll
                 for (int t = 0; t < NT; ++t) key_tmem_ld16(t_mine + t * KEY_COLS + (blk - 1) * KEY_BLK, d[t]);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int c = 0; c < KEY_BLK; ++c)
 #pragma unroll
-                    for (int i = 0; i < NP; ++i) x[c][i] = fadd2(x[c][i], pack2(__uint_as_float(d[2 * i][c]), __uint_as_float(d[2 * i + 1][c])));
-                if (blk > KEY_SPLIT) {
-#pragma unroll
-                    for (int t = 0; t < NT; ++t) key_tmem_ld16(t_mine + t * KEY_COLS + key_late_col(blk), d[t]);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                    for (int c = 0; c < KEY_BLK; ++c)
-#pragma unroll
-                        for (int i = 0; i < NP; ++i) x[c][i] = fadd2(x[c][i], pack2(__uint_as_float(d[2 * i][c]), __uint_as_float(d[2 * i + 1][c])));
-                }
+                    for (int i = 0; i < NP; ++i) cor[c][i] = fmul2(pack2(__uint_as_float(d[2 * i][c]), __uint_as_float(d[2 * i + 1][c])), up);
             }
 
             const u64 *diag = sm.diag + blk * KEY_BLK * KEY_BLK;
@@ -484,8 +489,8 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
             float *gscale = &sm.grid[warp][0][(blk & 1) * KEY_BLK * NGL], *gzero = &sm.grid[warp][1][(blk & 1) * KEY_BLK * NGL];
             // element-wise updates leave channel 0 alone uncorrected: then the usual code decides that one exactly (a block's worth of
             // the exact code is longer by a third, and has to be fetched)
-            if (exact_channels > max(1, blk * KEY_BLK)) sweep_pairs<BITS, NP, NGL, true, M16>(x, diag, e_hi, e_lo, lane, true, gscale, gzero, cw);
-            else sweep_pairs<BITS, NP, NGL, false, M16>(x, diag, e_hi, e_lo, lane, blk == 0, gscale, gzero, cw);
+            if (exact_channels > max(1, blk * KEY_BLK)) sweep_pairs<BITS, NP, NGL, true, M16>(key, cor, diag, e_hi, e_lo, lane, true, gscale, gzero, cw);
+            else sweep_pairs<BITS, NP, NGL, false, M16>(key, cor, diag, e_hi, e_lo, lane, blk == 0, gscale, gzero, cw);
 
             if (more) {
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // E_hi is in tensor memory
