@@ -11,10 +11,10 @@
 // Within a block of 16 channels the pushes are CUDA-core work (packed fma.rn.f32x2 on the lane's two tokens); onto the channels
 // of later blocks they are a dense product on the tcgen05 tensor cores, tf32 operands split in two.
 //
-// Who holds what.  A CTA is 4 warps and works on 2 tiles of 128 tokens; two CTAs share an SM.  Row r of a tile = tensor-memory
-// lane r; warp w, lane l holds row 32 w + l of both tiles, as pairs, so a read of W (stored twice) and every packed
-// instruction serve two tokens, and groups of 64 and more join their extremes in the lane before the warp-wide reduction (a
-// group of 128 is two warps, which trade their extremes per channel through shared memory).  Tensor memory, per tile: the
+// Who holds what.  A CTA is 4 sweeping warps on 2 tiles of 128 tokens, two CTAs per SM; for groups of 128 on 4 tiles, one CTA.  Row r of
+// a tile = tensor-memory lane r; warp w, lane l holds row 32 w + l of every tile, as pairs of tokens, so a read of W (stored
+// twice) and every packed instruction serve two tokens, and a warp's tokens are whole groups: groups of 64 and 128 join their
+// extremes in the lane before the warp-wide reduction and never meet another warp.  Tensor memory, per tile: the
 // corrections D[128 x 112] of channels 16 .. 127, and 16 more columns for the errors of block 0.  The errors E_hi of block b > 0
 // take the columns whose corrections that block has just read, so nothing waits for a free place.  E_lo goes to shared memory as
 // a K-major operand, in two buffers.
@@ -51,11 +51,6 @@ namespace {
 
 constexpr int KEY_WARPS = 4, KEY_THREADS = 32 * (KEY_WARPS + 1);      // four sweeping warps, one that issues the products
 constexpr int KEY_COLS = 128, KEY_E0_COL = 112;                          // per tile: [0, 112) corrections, [112, 128) E_hi of block 0
-// The accumulator truncates on every addition, so corrections are gathered in two: what blocks 0 .. 3 push in the columns of the
-// channel, what blocks 4 .. 6 push onto blocks 5 .. 7 in columns that are free by then; the sweep adds both, each made larger by
-// what truncation has taken from it on average.  Rms error of a group's minimum against 64 bits, as a part of its range (rank 32, 2
-// bits, G = 32): one accumulator 1.14e-7, two 0.93e-7, corrected 0.67e-7; the kernel of 32-channel blocks before this one 0.94e-7.
-// Time: the second accumulator + 1 % for groups of 32 and 64, + 5 % for 128; the correction none.
 // Accuracy (rms error of a group's minimum against 64 bits, as a part of its range; rank 32, 2 bits, G = 32).  Corrections are gathered
 // apart from the keys and added once, when the channel's turn comes, so that a large key (an outlier channel) does not round every
 // push.  The tensor core's accumulator truncates on every addition; what that takes on average from a sum
