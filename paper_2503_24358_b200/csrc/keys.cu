@@ -482,6 +482,10 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
             const unsigned e_hi = t_mine + (blk == 0 ? KEY_E0_COL : (blk - 1) * KEY_BLK);
             float *e_lo = &sm.e_lo[blk & 1][0][(warp * 32 + lane) * 4];
             float *gscale = &sm.grid[warp][0][(blk & 1) * KEY_BLK * NGL], *gzero = &sm.grid[warp][1][(blk & 1) * KEY_BLK * NGL];
+            // (recorded only: every address of a sweep is a constant away from these)
+            (void)SQ_CHK_R(p.status, e_lo, (KEY_E_FLOATS * (NT - 1) + (KEY_BLK / 4 - 1) * KEY_A_LBO / 4 + 4) * 4, sm.e_lo[blk & 1], sizeof(sm.e_lo[0]));
+            (void)SQ_CHK_R(p.status, diag, KEY_BLK * KEY_BLK * 8, sm.diag, sizeof(sm.diag));
+            (void)SQ_CHK_C(p.status, (e_hi & 0xffffu) >= (tmem & 0xffffu) && (e_hi & 0xffffu) + KEY_BLK <= (tmem & 0xffffu) + KEY_COLS);
             // element-wise updates leave channel 0 alone uncorrected: then the usual code decides that one exactly (a block's worth of
             // the exact code is longer by a third, and has to be fetched)
             if (exact_channels > max(1, blk * KEY_BLK)) sweep_pairs<BITS, NP, NGL, true, M16>(key, cor, diag, e_hi, e_lo, lane, true, gscale, gzero, cw);
