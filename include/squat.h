@@ -153,9 +153,14 @@ int squat_subspace_eig_sweeps(const squat_subspace *s, void *stream, int *sweeps
  * (corrected) values, round half to even, push each token's error on its later channels
  * through W.  Splitting n_tokens at multiples of G over several calls gives identical bytes.
  * bits in {2, 4}; group_size in {32, 64, 128}; d = 128; n_kv_heads must match the handle.
- * The updates that cross 32-channel blocks are computed on the tensor cores as three tf32
- * products per multiply-add (operands split hi + lo), accumulated in fp32; the result agrees
- * with fp32 arithmetic to a few 1e-7 of sum |e W|.  Every wait on the tensor core is bounded; if
+ * Rounding: a channel that nothing has corrected (channel 0; the first block_g channels; all of
+ * them when W = 0; in the dense kernel also those of a group whose errors so far are all 0, as
+ * behind constant channels) is decided as real arithmetic on the stored scale would, ties to
+ * even, and its scale is the correctly rounded quotient.  Any other channel may be decided the
+ * other way within 1e-6 * L of a tie, and its scale is within one ulp of the quotient.
+ * The updates that cross blocks of 16 channels (of block_g channels where block_g is 32 or 64) are
+ * computed on the tensor cores as three tf32 products per multiply-add (operands split hi + lo),
+ * accumulated in fp32; the result agrees with fp32 arithmetic to a few 1e-7 of sum |e W|.  Every wait on the tensor core is bounded; if
  * one runs out the kernel still ends, SQUAT_FLAG_DEVICE_TIMEOUT is set in the device status word
  * and the outputs of that call are invalid.
  */

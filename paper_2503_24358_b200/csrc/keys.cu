@@ -36,12 +36,18 @@
 //
 // Rounding decision.  t = (x - m) / scale is formed with the hardware reciprocal, so c0 = rint(t) can be off by one when t is within
 // ~1e-6 of a rounding midpoint.  Channels that earlier channels have corrected hold generic float32 values and such near-ties are as
-// rare as that bound; but channels nothing has corrected yet (the first g channels, or all of them when W = 0) hold raw bf16 / f32
-// inputs, where exact ties are structural (x exactly half way between min and max).  For those blocks (EXACT) the remainder
+// rare as that bound; but channels nothing has corrected yet hold raw bf16 / f32 inputs, where exact ties are structural (x exactly
+// half way between min and max).  These are channel 0; the channels that W leaves uncorrected (the first g, or all of them when W = 0);
+// and those of a group in which no error has been made so far, as behind constant channels.  There the remainder
 // e0 = c0*scale - (x - m), which is exact next to a midpoint, is compared with +-scale/2: that settles the rounding exactly as real
 // arithmetic on the stored float32 scale would, ties going to the even code (the threshold of an odd c0 is one ulp lower, so
-// "remainder == scale/2" moves it).  The stored scale is the correctly rounded quotient in EXACT blocks (bit-identical to plain
-// round-to-nearest quantization), else the product with RN(1/L), within one ulp of it.
+// "remainder == scale/2" moves it), and the stored scale is the correctly rounded quotient (bit-identical to plain round-to-nearest
+// quantization); elsewhere it is the product with RN(1/L), within one ulp of it.  Channel 0 is settled in the usual code; for the
+// others a block is swept by the EXACT instance: where W says so, or where the usual code, at the block's first channel, finds a group
+// whose errors in channel 0 (block 0) or corrections (later blocks) are all 0.  That test is free behind the next channel's
+// reductions; as a test of its own ahead of the block it cost 2 % at G = 32 (40.5 -> 41.3 us for 32 heads x 4096).  A block swept twice
+// costs its time: keys that are all constant take 1.2 (G = 32) to 1.45 times (G = 128) as long as others.  Exact decisions in all of
+// the first 32 channels, corrected or not, would cost 5 % (G = 32, 1062 -> 1115 us for 128 heads x 32768), 1 % (G = 64) and 12 % (G = 128).
 //
 // M16: scale and zero-point are stored as binary16.  The float32 values are rounded once more, and the decision and the error fed
 // back are taken against the rounded (stored) values: t = (x - z16) / s16, clamped to [0, L] because z16 can lie above the minimum.
@@ -122,6 +128,18 @@ __device__ __forceinline__ void key_tmem_ld16(unsigned taddr, unsigned (&r)[16])
                  : "r"(taddr) : "memory");
 }
 
+// which of the warp's groups have only zeros in v (warp-uniform)
+template <int NP, int NGL>
+__device__ __forceinline__ void key_raw_groups(const u64 (&v)[NP], bool (&raw)[NGL])
+{
+    constexpr int NT = 2 * NP, TPG = NT / NGL;
+    bool nz[NGL] = {};
+#pragma unroll
+    for (int t = 0; t < NT; ++t) nz[t / TPG] |= !(((t & 1) ? hi_of(v[t / 2]) : lo_of(v[t / 2])) == 0.0f);
+#pragma unroll
+    for (int g = 0; g < NGL; ++g) raw[g] = !__any_sync(0xffffffffu, nz[g]);
+}
+
 // 16 channels of the lane's tokens as they are in memory
 template <bool BF16, int NP>
 struct PairRows {
@@ -139,15 +157,17 @@ struct PairRows {
 };
 
 // The 16 channels of one block for the lane's 2 NP tokens (pair i of x[channel]: tokens 2 i and 2 i + 1), which belong to NGL groups.
-// exact_first: the first channel's decisions are exact (EXACT: all).
+// EXACT: decisions are exact in the groups of raw[], and in channel 0 (the first of block 0: `first`).  The usual code decides channel 0 alone
+// exactly; where it finds a group without errors or corrections so far it says so in raw[] and returns true, having changed nothing
+// that the EXACT instance, which then sweeps the block from its start, does not write again.
 // Written in the order in which it should run: a channel's chain (reductions 24 cycles, reciprocal 24, six dependent
 // operations of 4 to 6: 71 in all) goes on to the next channel's reductions before what does not hurry: the other pushes, the
 // codes and the errors' stores fill the waits.  The next row of W is read before this channel's stores, which may be to the same
 // memory for all the compiler knows.  The errors of the last block are stored like the others (a test per store would cut the
 // code into pieces) and used by nobody.
 template <int BITS, int NP, int NGL, bool EXACT, bool M16>
-__device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (&cor)[KEY_BLK][NP], const u64 *__restrict__ diag, unsigned e_hi, float *__restrict__ e_lo,
-                                            int lane, bool exact_first, float *__restrict__ gscale, float *__restrict__ gzero, unsigned (&cw)[2 * NP][BITS / 2])
+__device__ __forceinline__ bool sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (&cor)[KEY_BLK][NP], const u64 *__restrict__ diag, unsigned e_hi, float *__restrict__ e_lo,
+                                            int lane, bool first, bool (&raw)[NGL], float *__restrict__ gscale, float *__restrict__ gzero, unsigned (&cw)[2 * NP][BITS / 2])
 {
     constexpr float L = float((1 << BITS) - 1);
     constexpr int PER_WORD = 32 / BITS, NT = 2 * NP, TPG = NT / NGL;      // tokens of the lane per group
@@ -193,7 +213,7 @@ __device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (
         for (int g = 0; g < NGL; ++g) {
             const float rng = __fsub_rn(mx[g], m[g]);
             z[g] = m[g];
-            scale[g] = EXACT || (jj == 0 && exact_first) ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);
+            scale[g] = (EXACT && raw[g]) || (jj == 0 && first) ? div_by_levels<BITS>(rng) : __fmul_rn(rng, 1.0f / L);
             if (M16) {
                 scale[g] = __half2float(__float2half_rn(scale[g]));
                 z[g] = __half2float(__float2half_rn(m[g]));
@@ -223,25 +243,27 @@ __device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (
                 y2 = pack2(y0, y1);
             }
             e[i] = ffma2(fsub2(y2, magic2), pack2(scale[ga], scale[gb]), n);
-            if (EXACT || (jj == 0 && (exact_first || M16))) {
+            if (EXACT || (jj == 0 && (first || M16))) {
                 float e0, e1, n0, n1;
                 unpack2(e[i], e0, e1);
                 unpack2(n, n0, n1);
-                auto decide = [&](float nd, float sc, float &yy, float &ee) {
-                    if (EXACT || exact_first) {
-                        const float thr = __uint_as_float(__float_as_uint(0.5f * sc) - (__float_as_uint(yy) & 1u));
+                auto decide = [&](float nd, int g, float &yy, float &ee) {
+                    if (EXACT || first) {
+                        const bool settle = !EXACT || raw[g] || (jj == 0 && first);      // (else nothing lies beyond, and 0 x 0 is added)
+                        const float half = settle ? 0.5f * scale[g] : __int_as_float(0x7f800000), step = settle ? scale[g] : 0.0f;
+                        const float thr = __uint_as_float(__float_as_uint(half) - (__float_as_uint(yy) & 1u));
                         const float adj = ee > thr ? -1.0f : (ee < -thr ? 1.0f : 0.0f);
                         yy = __fadd_rn(yy, adj);
-                        ee = __fmaf_rn(adj, sc, ee);
+                        ee = __fmaf_rn(adj, step, ee);
                     }
                     if (M16) {
                         const float cc = fminf(fmaxf(yy, kMagic), kMagic + L);
-                        ee = cc == yy ? ee : __fmaf_rn(__fsub_rn(cc, kMagic), sc, nd);
+                        ee = cc == yy ? ee : __fmaf_rn(__fsub_rn(cc, kMagic), scale[g], nd);
                         yy = cc;
                     }
                 };
-                decide(n0, scale[ga], y0, e0);
-                decide(n1, scale[gb], y1, e1);
+                decide(n0, ga, y0, e0);
+                decide(n1, gb, y1, e1);
                 e[i] = pack2(e0, e1);
             }
         }
@@ -250,6 +272,16 @@ __device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (
 #pragma unroll
             for (int i = 0; i < NP; ++i) x[i] = ffma2(e[i], w[jj + 1], pre[i]);
             extremes();
+        }
+        if (!EXACT && jj == 0) {                        // (while those reductions run; no push has been made yet)
+            bool any = false;
+            u64 v[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) v[i] = first ? e[i] : cor[0][i];
+            key_raw_groups<NP, NGL>(v, raw);
+#pragma unroll
+            for (int g = 0; g < NGL; ++g) any |= raw[g];
+            if (any) return true;
         }
 #pragma unroll
         for (int c = jj + 2; c < KEY_BLK; ++c)
@@ -275,6 +307,7 @@ __device__ __forceinline__ void sweep_pairs(const u64 (&key)[KEY_BLK][NP], u64 (
                 *reinterpret_cast<float4 *>(e_lo + t * KEY_E_FLOATS + (jj >> 2) * (KEY_A_LBO / 4)) = make_float4(el[t][0], el[t][1], el[t][2], el[t][3]);
         }
     }
+    return false;
 }
 
 template <int BITS, int G, bool BF16, bool M16>
@@ -486,10 +519,12 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
             (void)SQ_CHK_R(p.status, e_lo, (KEY_E_FLOATS * (NT - 1) + (KEY_BLK / 4 - 1) * KEY_A_LBO / 4 + 4) * 4, sm.e_lo[blk & 1], sizeof(sm.e_lo[0]));
             (void)SQ_CHK_R(p.status, diag, KEY_BLK * KEY_BLK * 8, sm.diag, sizeof(sm.diag));
             (void)SQ_CHK_C(p.status, (e_hi & 0xffffu) >= (tmem & 0xffffu) && (e_hi & 0xffffu) + KEY_BLK <= (tmem & 0xffffu) + KEY_COLS);
-            // element-wise updates leave channel 0 alone uncorrected: then the usual code decides that one exactly (a block's worth of
-            // the exact code is longer by a third, and has to be fetched)
-            if (exact_channels > max(1, blk * KEY_BLK)) sweep_pairs<BITS, NP, NGL, true, M16>(key, cor, diag, e_hi, e_lo, lane, true, gscale, gzero, cw);
-            else sweep_pairs<BITS, NP, NGL, false, M16>(key, cor, diag, e_hi, e_lo, lane, blk == 0, gscale, gzero, cw);
+            // Where W leaves channels of the block uncorrected, every group is decided exactly; else the groups that the usual code finds raw.
+            bool raw[NGL], exact = exact_channels > max(1, blk * KEY_BLK);
+#pragma unroll
+            for (int g = 0; g < NGL; ++g) raw[g] = true;
+            if (!exact) exact = sweep_pairs<BITS, NP, NGL, false, M16>(key, cor, diag, e_hi, e_lo, lane, blk == 0, raw, gscale, gzero, cw);
+            if (exact) sweep_pairs<BITS, NP, NGL, true, M16>(key, cor, diag, e_hi, e_lo, lane, blk == 0, raw, gscale, gzero, cw);
 
             if (more) {
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // E_hi is in tensor memory

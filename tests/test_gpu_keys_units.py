@@ -81,6 +81,41 @@ def test_uncorrected_channels_are_decided_exactly(uncorrected, G):
     s.close()
 
 
+@pytest.mark.parametrize("constant", [1, 15, 16, 17, 32, 100])
+@pytest.mark.parametrize("G,bits,m16", [(32, 2, False), (64, 4, False), (128, 2, False), (128, 4, True), (32, 4, True)])
+def test_channel_behind_constant_ones_is_decided_exactly(constant, G, bits, m16):
+    """Constant leading channels leave no error, so under a full W the channel behind them holds raw values like an uncorrected one:
+    its codes and grid are those of plain rounding.  Every third group is such a one; the others are ordinary, and which groups
+    share a warp or a call changes no byte."""
+    H, T, L, n = 2, 9 * 128, 2 ** bits - 1, constant
+    gen = torch.Generator().manual_seed(100 * constant + G)
+    W = torch.tril(0.2 * torch.randn((H, D, D), generator=gen), -1)
+    k = torch.randint(-6, 7, (1, H, T // G, G, D), generator=gen).float()
+    k[:, :, ::3, :, :n] = 1.5
+    k = k.view(1, H, T, D).to(torch.bfloat16).cuda()
+    s = sq.Subspace(H, D)
+    sq.squat_subspace_import(s, W.numpy())
+    meta = torch.float16 if m16 else torch.float32
+    out = [t if t.dtype == torch.uint8 else t.to(meta) for t in alloc_key_outputs(1, H, T, D, bits, G)]
+    sq.squat_quantize_keys(s, k, bits, G, *out)
+    windows = [torch.zeros_like(t) for t in out]
+    for lo in range(0, T, G):
+        sq.squat_quantize_keys(s, k[:, :, lo:lo + G], bits, G, windows[0][:, :, lo:], windows[1][:, :, lo // G:], windows[2][:, :, lo // G:],
+                               out_stride_b=H * T, out_stride_h=T)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(out, windows))
+    assert sq.squat_get_device_status(clear=True) == sq.FLAG_ZERO_RANGE      # the constant groups are reported
+    x = k[0].double().cpu().numpy().reshape(H, T // G, G, D)[:, ::3, :, n]
+    scale, zero = (t[0].float().cpu().numpy()[:, ::3, n] for t in out[1:])
+    want = (x.max(2) - x.min(2)).astype(np.float32) / np.float32(L)
+    assert np.array_equal(zero, x.min(2).astype(np.float32))
+    assert np.array_equal(scale, want.astype(np.float16).astype(np.float32) if m16 else want)
+    code = np.clip(np.rint((x - zero[..., None]) / scale[..., None].astype(np.float64)), 0, L)
+    got = oracle.unpack(out[0][0].cpu().numpy().reshape(H * T, -1), D, bits).reshape(H, T // G, G, D)[:, ::3, :, n]
+    assert np.array_equal(got, code)
+    s.close()
+
+
 def test_units_match_the_oracle_for_two_pairs_per_lane():
     # 5 groups of 128 per head: a ragged second unit; element by element under the replay protocol
     cfg = si.get_config(1).with_(batch=1, n_kv_heads=2, n_q_heads=2, n_tokens=640)
