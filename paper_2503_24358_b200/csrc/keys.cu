@@ -59,9 +59,12 @@ constexpr int KEY_WARPS = 4, KEY_THREADS = 32 * (KEY_WARPS + 1);      // four sw
 constexpr int KEY_COLS = 128, KEY_E0_COL = 112;                          // per tile: [0, 112) corrections, [112, 128) E_hi of block 0
 // Accuracy (rms error of a group's minimum against 64 bits, as a part of its range; rank 32, 2 bits, G = 32).  Corrections are gathered
 // apart from the keys and added once, when the channel's turn comes, so that a large key (an outlier channel) does not round every
-// push.  The tensor core's accumulator truncates on every addition; what that takes on average from a sum
-// that n source blocks have added to is 2, 4, 4, 6, 6, 6, 6 x 2^-24 of it (the regression of the corrected values' error on the
-// sum, on the part) and is given back: 1.14e-7 -> 0.71e-7 together.  The kernel of 32-channel blocks before this one: 0.94e-7.
+// push.  The tensor core's accumulator truncates on every addition: without a remedy the error regressed on the sum that n = 1 .. 7
+// source blocks have added to has slopes of -1.8, -4.5, -5.2, -8.3, -7.4, -11.5, -8.4 x 2^-24 (r = 64, 4 bits, G = 128: -1.3, -6.9, -4.6, -9.9,
+// -7.4, -13.6, -7.3).  2, 4, 4, 6, 6, 6, 6 x 2^-24 of the sum are given back,
+// fitted on the first setting alone: slopes of 1.3 at most there and 2.2 in the second (a standard error of about 1).  Rms 1.08e-7
+// -> 0.70e-7, 0.56 -> 0.52, float32 keys with G = 64 1.04 -> 0.67, channels a factor of 1000 apart 4.4 -> 2.6.  The kernel of 32-channel
+// blocks before this one: 0.93, 0.77, 0.90, 3.3e-7.  tests/test_gpu_keys_accuracy.py holds these.
 __device__ __forceinline__ u64 key_untruncate(int n)
 {
     const float f = 1.0f + (float)min((n + 2) / 2, 3) * 0x1p-23f;

@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(LR_THREADS, LR_CTAS_PER_SM) quant_keys_lowrank
                     float e = __fmaf_rn(c, scale, -dlt);
                     if (jj == 0 && blk == 0) {
                         // channel 0 is a raw input, where exact ties are structural: settle the rounding through the exact
-                        // remainder, ties to the even code (see sweep_block in keys.cu)
+                        // remainder, ties to the even code (see the rounding decision in keys.cu)
                         const float thr = __uint_as_float(__float_as_uint(0.5f * scale) - (__float_as_uint(y0) & 1u));
                         const float adj = (e > thr) ? -1.0f : ((e < -thr) ? 1.0f : 0.0f);
                         c = __fadd_rn(c, adj);

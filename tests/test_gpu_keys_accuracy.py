@@ -14,9 +14,9 @@ pytestmark = pytest.mark.gpu
 D = 128
 
 
-def _replay(H, T, rank, bits, G, g, dtype, spread, dense=False, seed=5):
-    """(error of each group's zero-point, the group's range, what channels of earlier blocks of `unit` channels have pushed onto the
-    element that is the minimum), each [H, groups, D]; float64."""
+def _replay(H, T, rank, bits, G, g, dtype, spread, seed=5):
+    """(error of each group's zero-point, the group's range, what the channels of earlier blocks (16 channels, or g) have pushed onto
+    the element that is the minimum), each [H, groups, D]; float64."""
     gen = torch.Generator().manual_seed(seed)
     q = torch.randn((H, 1024, 16), generator=gen) @ torch.randn((H, 16, D), generator=gen) + 0.1 * torch.randn((H, 1024, D), generator=gen)
     k = torch.randn((1, H, T, D), generator=gen)
@@ -25,8 +25,6 @@ def _replay(H, T, rank, bits, G, g, dtype, spread, dense=False, seed=5):
     k = k.to(dtype)
     s = sq.Subspace(H, D)
     sq.squat_build_subspace(s, q.to(dtype).cuda(), rank, 1e-3, g)
-    if dense:
-        sq.squat_subspace_select_key_kernel(s, 1)
     W = torch.from_numpy(sq.squat_subspace_export(s)["W"]).double()
     kc, ks, kz = alloc_key_outputs(1, H, T, D, bits, G)
     sq.squat_quantize_keys(s, k.cuda(), bits, G, kc, ks, kz)
@@ -47,28 +45,33 @@ def _replay(H, T, rank, bits, G, g, dtype, spread, dense=False, seed=5):
     return zero - low, xg.amax(2) - low, far.view(H, T // G, G, D).gather(2, at.unsqueeze(2)).squeeze(2)
 
 
+# Bounds: what the kernel of 32-channel blocks, which every handle ran before, showed on the same inputs (0.929, 0.771, 0.896 and 3.34e-7
+# with element-wise updates; 0.321, 0.545, 0.296 and 1.84e-7 with blocks).  Seen here: 0.695, 0.524, 0.673, 2.56e-7; 0.204, 0.545, 0.296,
+# 1.84e-7.
 @pytest.mark.parametrize("rank,bits,G,dtype,spread,bound", [
-    (32, 2, 32, torch.bfloat16, 1.0, 1),
-    (64, 4, 128, torch.bfloat16, 1.0, 1),
-    (32, 2, 64, torch.float32, 1.0, 1),
-    (32, 2, 32, torch.float32, 1000.0, 1),
+    (32, 2, 32, torch.bfloat16, 1.0, 0.929e-7),
+    (64, 4, 128, torch.bfloat16, 1.0, 0.771e-7),
+    (32, 2, 64, torch.float32, 1.0, 0.896e-7),
+    (32, 2, 32, torch.float32, 1000.0, 3.34e-7),         # channels a factor of 1000 apart
 ])
 def test_corrected_values_of_the_dense_kernel(rank, bits, G, dtype, spread, bound):
+    """The tensor core's accumulator truncates; what a sum loses by that on average is given back.  Without, the error regressed
+    on the sum has slopes down to -10 to -14 x 2^-24 in the later blocks, and three of the four bounds are missed; with it none is seen
+    beyond 2.2 (a standard error of about 1).  4 lies between the two."""
     err, rng, far = _replay(4, 2048, rank, bits, G, 1, dtype, spread)
-    rms = (err / rng).square().mean().sqrt().item()
-    slope = [2 ** 24 * ((err * far)[..., c:c + 16].sum() / far.square()[..., c:c + 16].sum()).item() for c in range(16, D, 16)]
-    print(f"DENSE r{rank} b{bits} G{G} {dtype} spread {spread}: rms {rms * 1e7:.3f}e-7; slopes {[round(v, 2) for v in slope]}")
+    assert (err / rng).square().mean().sqrt() <= bound
+    if spread == 1.0:
+        for c in range(16, D, 16):
+            slope = (err * far)[..., c:c + 16].sum() / far.square()[..., c:c + 16].sum()
+            assert abs(slope) <= 4 * 2.0 ** -24, (c, slope * 2 ** 24)
 
 
 @pytest.mark.parametrize("rank,bits,G,g,dtype,spread,bound", [
-    (32, 2, 32, 64, torch.bfloat16, 1.0, 1),
-    (32, 2, 32, 32, torch.bfloat16, 1.0, 1),
-    (64, 4, 128, 32, torch.float32, 1.0, 1),
-    (32, 2, 32, 32, torch.float32, 1000.0, 1),
+    (32, 2, 32, 64, torch.bfloat16, 1.0, 0.321e-7),
+    (32, 2, 32, 32, torch.bfloat16, 1.0, 0.546e-7),
+    (64, 4, 128, 32, torch.float32, 1.0, 0.297e-7),
+    (32, 2, 32, 32, torch.float32, 1000.0, 1.85e-7),
 ])
 def test_corrected_values_of_the_block_kernel(rank, bits, G, g, dtype, spread, bound):
-    for dense in (False, True):
-        err, rng, far = _replay(4, 2048, rank, bits, G, g, dtype, spread, dense)
-        rms = (err / rng).square().mean().sqrt().item()
-        slope = [2 ** 24 * ((err * far)[..., c:c + g].sum() / far.square()[..., c:c + g].sum()).item() for c in range(g, D, g)]
-        print(f"BLOCK dense={dense} r{rank} b{bits} G{G} g{g} {dtype} spread {spread}: rms {rms * 1e7:.3f}e-7; slopes {[round(v, 2) for v in slope]}")
+    err, rng, _ = _replay(4, 2048, rank, bits, G, g, dtype, spread)
+    assert (err / rng).square().mean().sqrt() <= bound
