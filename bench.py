@@ -102,10 +102,11 @@ def key_flops_per_vector(d, g, r=None):
     return 2 * (tri if r is None else min(tri, 2 * r * d))
 
 
-def key_fma_split(d, g, blk=16):
-    """The same multiply-adds split into those inside blocks of blk channels, which the key kernel runs on the FP32 pipes, and those
-    across blocks, which it runs on the tensor cores.  W[j'][j] is non-zero iff j' lies in a later g-block than j.  The dense
-    kernel's blocks are of 16 channels; the kernel for block updates (g = 32, 64) has none inside a block."""
+def key_fma_split(d, g, blk=32):
+    """The same multiply-adds split into those inside blocks of blk channels, counted for the FP32 pipes, and those across blocks,
+    counted for the tensor cores.  W[j'][j] is non-zero iff j' lies in a later g-block than j.  The split at 32 channels is the
+    one all reported rooflines use; the key kernel itself splits at 16 (g = 1: 960 and 7 168 instead of 1 984 and 6 144), so
+    its own FP32 floor is lower."""
     alu = sum(1 for j in range(d) for jp in range(j + 1, d) if jp // g > j // g and jp // blk == j // blk)
     tensor = sum(1 for j in range(d) for jp in range(j + 1, d) if jp // g > j // g and jp // blk != j // blk)
     return alu, tensor

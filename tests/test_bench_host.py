@@ -44,7 +44,7 @@ def test_algorithmic_counts():
     assert bench.key_flops_per_vector(128, 64) == 2 * 4096
     assert bench.key_flops_per_vector(128, 1, 32) == 2 * 8128          # r = 32: the triangle (8128) beats 2 r d = 8192
     assert bench.key_flops_per_vector(128, 1, 8) == 2 * 2048           # r = 8: the rank-r form is the cheaper count
-    assert bench.key_fma_split(128, 1) == (8 * 120, 8128 - 8 * 120)      # eight 16 x 16 triangles stay on the FP32 pipes
+    assert bench.key_fma_split(128, 1) == (4 * 496, 8128 - 4 * 496)      # four 32 x 32 triangles stay on the FP32 pipes
     assert sum(bench.key_fma_split(128, 32)) == 6144 and bench.key_fma_split(128, 32)[0] == 0
     assert sum(bench.key_fma_split(128, 64)) == 4096
     assert bench.bytes_per_vector(128, 2, 32, 2) == 320
@@ -66,11 +66,10 @@ def test_key_roofline_is_the_slowest_of_the_three_floors():
     cfg = si.get_config(1)
     vec = cfg.batch * cfg.n_kv_heads * cfg.n_tokens
     r = bench.key_roofline(args, cfg, 0.053, vec, peaks, fp32)
-    # dense kernel on workload 1: 960 multiply-adds per vector inside blocks of 16 channels; the 7 168 others, three products each,
-    # set the floor
-    assert r["bound"] == "tensor" and r["peak"] == 0.5 * 1649.9
-    assert abs(r["pipes"]["fp32_floor_us"] - 2 * 960 * vec / 73.0e12 * 1e6) < 1e-9
-    assert abs(r["pipes"]["tensor_floor_us"] - 6 * 7168 * vec / (0.5 * 1649.9e12) * 1e6) < 1e-9
+    # dense kernel on workload 1: the in-block triangles (1 984 multiply-adds per vector on the FP32 pipes) set the floor
+    assert r["bound"] == "alu" and r["peak"] == 73.0
+    assert abs(r["pipes"]["fp32_floor_us"] - 2 * 1984 * vec / 73.0e12 * 1e6) < 1e-9
+    assert abs(r["pipes"]["tensor_floor_us"] - 6 * 6144 * vec / (0.5 * 1649.9e12) * 1e6) < 1e-9
     assert abs(r["pipes"]["hbm_floor_us"] - 320 * vec / 6549.8e9 * 1e6) < 1e-9
     assert r["pipes"]["floor_us"] == max(r["pipes"][k] for k in ("fp32_floor_us", "tensor_floor_us", "hbm_floor_us"))
     assert abs(r["frac"] - r["pipes"]["floor_us"] / 53.0) < 1e-9 and abs(r["frac"] - r["achieved"] / r["peak"]) < 1e-12
