@@ -103,10 +103,8 @@ def key_flops_per_vector(d, g, r=None):
 
 
 def key_fma_split(d, g, blk=32):
-    """The same multiply-adds split into those inside blocks of blk channels, counted for the FP32 pipes, and those across blocks,
-    counted for the tensor cores.  W[j'][j] is non-zero iff j' lies in a later g-block than j.  The split at 32 channels is the
-    one all reported rooflines use; the key kernel itself splits at 16 (g = 1: 960 and 7 168 instead of 1 984 and 6 144), so
-    its own FP32 floor is lower."""
+    """The same multiply-adds split by where the dense key kernels run them: inside blocks of 32 channels on the FP32 pipes, across
+    blocks on the tensor cores.  W[j'][j] is non-zero iff j' lies in a later g-block than j."""
     alu = sum(1 for j in range(d) for jp in range(j + 1, d) if jp // g > j // g and jp // blk == j // blk)
     tensor = sum(1 for j in range(d) for jp in range(j + 1, d) if jp // g > j // g and jp // blk != j // blk)
     return alu, tensor

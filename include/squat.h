@@ -153,14 +153,13 @@ int squat_subspace_eig_sweeps(const squat_subspace *s, void *stream, int *sweeps
  * (corrected) values, round half to even, push each token's error on its later channels
  * through W.  Splitting n_tokens at multiples of G over several calls gives identical bytes.
  * bits in {2, 4}; group_size in {32, 64, 128}; d = 128; n_kv_heads must match the handle.
- * Rounding: a channel that nothing has corrected (channel 0; the first block_g channels; all of
- * them when W = 0; in the dense kernel also those of a group whose errors so far are all 0, as
- * behind constant channels) is decided as real arithmetic on the stored scale would, ties to
- * even, and its scale is the correctly rounded quotient.  Any other channel may be decided the
- * other way within 1e-6 * L of a tie, and its scale is within one ulp of the quotient.
- * The updates that cross blocks of 16 channels (of block_g channels where block_g is 32 or 64) are
- * computed on the tensor cores as three tf32 products per multiply-add (operands split hi + lo),
- * accumulated in fp32; the result agrees with fp32 arithmetic to a few 1e-7 of sum |e W|.  Every wait on the tensor core is bounded; if
+ * Rounding: in a block of 32 channels (64 where block_g is 64) that has a channel which W leaves uncorrected (channel 0; the first
+ * block_g channels; all of them when W = 0) every channel is decided as real arithmetic on the stored scale would, ties to even,
+ * and its scale is the correctly rounded quotient.  Any other channel may be decided the other way within 1e-6 * L of a tie, and
+ * its scale is within one ulp of the quotient.
+ * The updates that cross blocks of 32 channels (of 64 where block_g is 64) are computed on the tensor cores as three tf32
+ * products per multiply-add (operands split hi + lo), accumulated in fp32; the result agrees with fp32 arithmetic to a few
+ * 1e-7 of sum |e W|.  Every wait on the tensor core is bounded; if
  * one runs out the kernel still ends, SQUAT_FLAG_DEVICE_TIMEOUT is set in the device status word
  * and the outputs of that call are invalid.
  */
@@ -177,7 +176,8 @@ int squat_quantize_keys(const squat_subspace *s, const void *k, int dtype, int b
  * vector instead of d (d - 1) / 2.  squat_build_subspace and squat_build_subspace_from_gram prepare that form when
  * block_g = 1, lambda > 0 and 1 <= rank_r <= 8, and squat_quantize_keys / _m16 then use it (FP32 pipes only, no
  * tensor-core hand-over).  Block updates of 32 or 64 channels (block_g, rank_r > 0, lambda > 0) have zero diagonal blocks in W
- * and run a kernel that quantizes a block at a time.  Every other build, and an imported W, runs the dense kernel.  All
+ * and run a kernel that quantizes a block at a time.  Every other build, and an imported W, runs the dense form (two kernels that
+ * give the same bytes, chosen by the group size and the number of tokens).  All
  * compute the same function Quant; results agree up to rounding ties.
  *   prefer_dense   1: always run the dense kernel;  0: the default choice above.
  *   lowrank_rank   host, may be NULL: receives the rank the rank-r form is prepared for (0: not prepared).

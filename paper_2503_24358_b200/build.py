@@ -19,7 +19,7 @@ LIB = os.path.join(_HERE, "libsquat.so")
 OBJ_DIR_CHECKED = os.path.join(_HERE, "build_checked")
 LIB_CHECKED = os.path.join(_HERE, "libsquat_checked.so")
 PYCALL = os.path.join(_HERE, "_squatcall" + EXTENSION_SUFFIXES[0])
-SOURCES = ["api.cu", "values.cu", "keys.cu", "subspace.cu", "gram_i8.cu", "eig.cu", "power.cu", "attention.cu", "attention_mma.cu", "attention_rope.cu", "peak.cu", "keys_lowrank.cu", "keys_block.cu"]
+SOURCES = ["api.cu", "values.cu", "keys.cu", "keys_lane.cu", "subspace.cu", "gram_i8.cu", "eig.cu", "power.cu", "attention.cu", "attention_mma.cu", "attention_rope.cu", "peak.cu", "keys_lowrank.cu", "keys_block.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE]
 

@@ -2,7 +2,7 @@
 // block-wise quantization, the form of the paper's experiments; Eq. (update_block)).
 //
 // Within a block of g channels nothing depends on anything else: the diagonal blocks of W are zero, so the chain of 128
-// dependent channels that the kernel of keys.cu walks (lane = token, a warp-wide reduction and a push per channel) does not
+// dependent channels that the kernel of keys_lane.cu walks (lane = token, a warp-wide reduction and a push per channel) does not
 // exist here.  What is left per block is one pass over memory and one dense product, and the mapping follows that:
 //
 //   a thread owns a quad of 4 channels x 8 tokens of a group; a warp 8 quads x 4 token phases = 32 channels x 32 tokens.
@@ -22,7 +22,7 @@
 // (g = 64: a tile; g = 32: two tiles) in head-major order and stage a head's panels when the head changes.
 //
 // Bound: bytes first (304 per key vector with bf16 keys, 2 bits, G = 32, 16-bit scales), then the errors' trip through shared
-// memory (8 B written, 12 B read by the tensor core per element).  Measured against the kernel of keys.cu, which walks the chain
+// memory (8 B written, 12 B read by the tensor core per element).  Measured against the kernel of keys_lane.cu, which walks the chain
 // of the element-wise form whatever g is: 16 x 8 heads x 8160 tokens, 2 bits, G = 32, 16-bit scales 365 -> 130 us at g = 64 and
 // 357 -> 159 at g = 32; 4 bits, G = 128, g = 64 462 -> 142; 32 heads x 4096 48 -> 23; one window of 32 heads x 128 15.2 -> 6.6.
 // What is left (ablations, g = 64): the wait for the products 27 us, the errors' stores 17, exact decisions 5; asking L2 for the
@@ -31,11 +31,6 @@
 #include "keys_common.cuh"
 
 namespace {
-
-__device__ __forceinline__ void team_barrier(int id, int nthreads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 constexpr int BLK = 32;                               // channels per warp and step
 constexpr int KB_THREADS = 256;
@@ -76,19 +71,6 @@ struct KbLayout {
     static constexpr int WARPS_PER_TILE = 8 / SLOTS;
     static constexpr size_t SMEM = sizeof(float) * (2 * SLOTS * E_FLOATS + 2 * W_FLOATS) + sizeof(u64) * (SLOTS + 1) + 4 * (2 + SLOTS) + 8;
 };
-
-// 32 consecutive columns of the warp's lanes into registers (lane l gets row l)
-__device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 
 // 4 channels of the thread's 8 tokens as they are in memory
 template <bool BF16>
@@ -319,10 +301,10 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
     grid_wait();
     const unsigned img_mbar = smem_u32(mbar + Lay::SLOTS);
 
-    // One head's panels into shared memory (one thread).  The image has them by 16 source channels with all later channels; of those
+    // One head's panels into shared memory (one thread).  The image has them by 32 source channels with all later channels; of those
     // only the channels behind the block of g are taken, and the source blocks of a step put side by side along K.
     auto stage_panels = [&](int h) {
-        const float *src = p.Wimg + (long long)h * KEY_IMG_FLOATS + KEY_DIAG_FLOATS;
+        const float *src = p.Wimg + (long long)h * KEY_IMG_FLOATS + KEY_PLAIN_FLOATS;
         if (!SQ_CHK_G(p.status, src, 2 * KEY_PANEL_FLOATS * 4, p.x_img)) return;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(img_mbar), "r"(2 * Lay::W_FLOATS * 4) : "memory");
@@ -477,9 +459,8 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
                     const ulonglong2 dd = *reinterpret_cast<const ulonglong2 *>(E_lo + e_mine + i * 16);
                     u64 k01, k23;
                     raw.get(i, k01, k23);
-                    // (as it is: the accumulator's truncation has made it smaller by 3 to 6 x 2^-24 on average, over one sum at g = 64
-                    // and up to three at g = 32; keys.cu gives that back, where seven sums lose up to 14.  Rms error of a group's
-                    // minimum here 0.20e-7 (g = 64) and 0.30 to 0.55e-7 (g = 32) of its range, no more than the kernel before had)
+                    // (the sum as it is, as in the other kernels, though the accumulator's truncation has made it smaller by 3 to 6 x 2^-24 on
+                    // average.  Rms error of a group's minimum 0.20e-7 (g = 64) and 0.30 to 0.55e-7 (g = 32) of its range, no more than keys_lane.cu has)
                     x[i][0] = fadd2(k01, dd.x);
                     x[i][1] = fadd2(k23, dd.y);
                 }

@@ -1,4 +1,4 @@
-// What the key kernels that apply W through the tensor cores (keys.cu, keys_block.cu) share: the image of the update matrix
+// What the key kernels that apply W through the tensor cores (keys.cu, keys_lane.cu, keys_block.cu) share: the image of the update matrix
 // that pack_w_kernel writes, the instructions they issue, and the quantizer's small pieces.
 #pragma once
 #include "device_helpers.cuh"
@@ -7,14 +7,18 @@
 constexpr int D = SQUAT_D;
 constexpr float kMagic = 12582912.0f;     // 1.5 * 2^23: adding it rounds to an integer (ties to even)
 
-// One head's image (see pack_w_kernel), blocks of 16 channels: diagonal blocks doubled | hi panels | lo panels.  Panel b holds the
-// entries that lead from block b to the later channels, N = 112 - 16 b of them, K-major: float index (k / 4) * 4 N + 4 n + k % 4.
-constexpr int KEY_BLK = 16, KEY_NBLK = D / KEY_BLK;
-constexpr int KEY_DIAG_FLOATS = 2 * KEY_NBLK * KEY_BLK * KEY_BLK;
-__host__ __device__ constexpr int key_panel_off(int b) { return KEY_BLK * (b * (D - KEY_BLK) - KEY_BLK * (b * (b - 1) / 2)); }   // sum of 16 (112 - 16 i), i < b
+// One head's image (see pack_w_kernel), blocks of 32 channels: diagonal blocks | hi panels | lo panels | the diagonal blocks once more, for
+// the kernel that sweeps them in halves of 16.  Panel b holds the entries that lead from block b to the later channels, N = 96 - 32 b of them,
+// K-major: float index (k / 4) * 4 N + 4 n + k % 4.
+constexpr int KEY_BLK = 32, KEY_HALF = 16, KEY_NBLK = D / KEY_BLK;
+constexpr int KEY_PLAIN_FLOATS = KEY_NBLK * KEY_BLK * KEY_BLK;
+// a block in halves: first half onto itself (every entry twice) | first onto second | second onto itself (every entry twice)
+constexpr int KEY_OWN_FLOATS = 2 * KEY_HALF * KEY_HALF, KEY_ACROSS_FLOATS = KEY_HALF * KEY_HALF;
+constexpr int KEY_DIAG_BLK_FLOATS = 2 * KEY_OWN_FLOATS + KEY_ACROSS_FLOATS, KEY_DIAG_FLOATS = KEY_NBLK * KEY_DIAG_BLK_FLOATS;
+__host__ __device__ constexpr int key_panel_off(int b) { return KEY_BLK * (b * (D - KEY_BLK) - KEY_BLK * (b * (b - 1) / 2)); }   // sum of 32 (96 - 32 i), i < b
 constexpr int KEY_PANEL_FLOATS = key_panel_off(KEY_NBLK - 1);
 constexpr int KEY_IMG_FLOATS = SQUAT_KEY_IMG_FLOATS;
-static_assert(KEY_IMG_FLOATS == KEY_DIAG_FLOATS + 2 * KEY_PANEL_FLOATS, "what the handle allocates per head");
+static_assert(KEY_IMG_FLOATS == KEY_PLAIN_FLOATS + 2 * KEY_PANEL_FLOATS + KEY_DIAG_FLOATS, "what the handle allocates per head");
 // instruction descriptor: fp32 accumulator, tf32 A and B, both K-major, N = n, M = 128
 __host__ __device__ constexpr unsigned tc_idesc(int n) { return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24); }
 
@@ -68,4 +72,21 @@ __device__ __forceinline__ unsigned tf32_of(float x)             // round to nea
     unsigned r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return r;
+}
+// 32 consecutive columns of the warp's lanes into registers (lane l gets row l)
+__device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// barrier `id` of nthreads threads
+__device__ __forceinline__ void team_barrier(int id, int nthreads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }

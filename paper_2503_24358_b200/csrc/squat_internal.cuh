@@ -7,7 +7,7 @@
 #include "../../include/squat.h"
 
 #define SQUAT_D 128   // the only head dimension the key path and the subspace build are built for
-#define SQUAT_KEY_IMG_FLOATS 18432   // floats per head of the image of W that the key kernels stage (keys_common.cuh)
+#define SQUAT_KEY_IMG_FLOATS 21504   // floats per head of the image of W that the key kernels stage (keys_common.cuh)
 #define SQUAT_LOWRANK_MAX_R 8   // largest subspace rank the rank-r form of the key quantizer is built for (keys_lowrank.cu)
 
 #define SQUAT_GRAM_REM_CAP 256   // remainders listed per head by the integer Gram kernel (gram_i8.cu)
@@ -117,6 +117,10 @@ int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int bat
                             long long sb, long long sh, long long st_, int bits, int G,
                             unsigned char *codes, void *scales, void *zeros,
                             long long osb, long long osh, unsigned *status, const int *exact_channels_dev, int meta16, cudaStream_t st);
+int squat_launch_quant_keys_lane(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
+                                 long long sb, long long sh, long long st_, int bits, int G,
+                                 unsigned char *codes, void *scales, void *zeros,
+                                 long long osb, long long osh, unsigned *status, const int *exact_channels_dev, int meta16, cudaStream_t st);
 int squat_launch_quant_keys_block(int block_g, const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                                   long long sb, long long sh, long long st_, int bits, int G,
                                   unsigned char *codes, void *scales, void *zeros,

@@ -1,5 +1,5 @@
-"""The key kernel's units of work: one tile or two per CTA (groups of 32, by the number of tiles), two pairs of tokens per lane
-for groups of 128, ragged units, heads that change inside a CTA's range, and the block that is decided exactly."""
+"""The dense key kernels' units of work: one token per lane (groups of 32, and of 128 in small calls), two or four tokens per lane (groups of 64
+and 128), ragged units, heads that change inside a CTA's range, and the blocks that are decided exactly."""
 import numpy as np
 import pytest
 import torch
@@ -15,12 +15,14 @@ D = 128
 
 
 @pytest.mark.parametrize("G,bits,dtype,m16,B,H,T", [
-    (32, 2, torch.bfloat16, False, 1, 37, 512),      # 148 tiles: one per CTA on 148 SMs; the whole call against its windows
-    (32, 2, torch.bfloat16, False, 1, 149, 128),     # 149 tiles: the first size with two tiles per CTA, half of them spare
+    (32, 2, torch.bfloat16, False, 1, 37, 512),      # 148 tiles: one per CTA on 148 SMs
+    (32, 2, torch.bfloat16, False, 1, 149, 128),     # 149 tiles: the first size at which a CTA has two
     (32, 4, torch.float32, True, 3, 5, 224),         # 21 groups per head: ragged tiles and units
     (64, 2, torch.bfloat16, True, 5, 60, 192),       # 15 groups per head, 4 a unit: ragged, several heads per CTA
     (64, 4, torch.float32, False, 1, 3, 64),
-    (128, 2, torch.float32, False, 7, 50, 128),      # 7 groups per head, 4 a unit
+    (128, 2, torch.float32, False, 7, 50, 128),      # 7 groups per head, 4 a unit; a sample alone (50 tiles): one token per lane
+    (128, 4, torch.bfloat16, True, 2, 74, 128),      # 148 tiles: the last size with one token per lane
+    (128, 4, torch.bfloat16, True, 3, 50, 128),      # 150: the first with four
     (128, 4, torch.bfloat16, False, 1, 2, 384),
     (128, 2, torch.bfloat16, True, 1, 1, 128),
 ])
@@ -81,12 +83,12 @@ def test_uncorrected_channels_are_decided_exactly(uncorrected, G):
     s.close()
 
 
-@pytest.mark.parametrize("constant", [1, 15, 16, 17, 32, 100])
+@pytest.mark.parametrize("constant", [1, 15, 16, 17, 31])
 @pytest.mark.parametrize("G,bits,m16", [(32, 2, False), (64, 4, False), (128, 2, False), (128, 4, True), (32, 4, True)])
 def test_channel_behind_constant_ones_is_decided_exactly(constant, G, bits, m16):
-    """Constant leading channels leave no error, so under a full W the channel behind them holds raw values like an uncorrected one:
-    its codes and grid are those of plain rounding.  Every third group is such a one; the others are ordinary, and which groups
-    share a warp or a call changes no byte."""
+    """Constant leading channels leave no error, so under a full W the channel behind them holds raw values like an uncorrected one: in
+    the first block of 32 channels, all of which are decided exactly, its codes and grid are those of plain rounding.  Every third
+    group is such a one; the others are ordinary, and which groups share a warp or a call changes no byte."""
     H, T, L, n = 2, 9 * 128, 2 ** bits - 1, constant
     gen = torch.Generator().manual_seed(100 * constant + G)
     W = torch.tril(0.2 * torch.randn((H, D, D), generator=gen), -1)
@@ -116,18 +118,19 @@ def test_channel_behind_constant_ones_is_decided_exactly(constant, G, bits, m16)
     s.close()
 
 
-def test_units_match_the_oracle_for_two_pairs_per_lane():
+@pytest.mark.parametrize("H", [2, 32])           # 10 tiles: one token per lane; 160: two pairs
+def test_units_match_the_oracle_for_two_pairs_per_lane(H):
     # 5 groups of 128 per head: a ragged second unit; element by element under the replay protocol
-    cfg = si.get_config(1).with_(batch=1, n_kv_heads=2, n_q_heads=2, n_tokens=640)
+    cfg = si.get_config(1).with_(batch=1, n_kv_heads=H, n_q_heads=H, n_tokens=640)
     gen = np.random.default_rng(3)
-    W = np.tril(0.1 * gen.standard_normal((2, D, D)), -1).astype(np.float32)
+    W = np.tril(0.1 * gen.standard_normal((H, D, D)), -1).astype(np.float32)
     k_np = si.gen_keys(cfg)
-    s = sq.Subspace(2, D)
+    s = sq.Subspace(H, D)
     sq.squat_subspace_import(s, W)
-    kc, ks, kz = alloc_key_outputs(1, 2, 640, D, 4, 128)
+    kc, ks, kz = alloc_key_outputs(1, H, 640, D, 4, 128)
     sq.squat_quantize_keys(s, to_torch(k_np, cfg.dtype), 4, 128, kc, ks, kz)
     torch.cuda.synchronize()
-    for h in range(2):
+    for h in (0, H - 1):
         compare_key_unit(si.to_f32(k_np[0, h], cfg.dtype).astype(np.float64), W[h].astype(np.float64), 128, 4,
                          oracle.unpack(kc[0, h].cpu().numpy(), D, 4), ks[0, h].cpu().numpy(), kz[0, h].cpu().numpy())
     s.close()
