@@ -58,10 +58,25 @@ int block_form(int rank_r, double lambda, int block_g)
 // made from the eigen-pairs right after the eigensolver.
 int lowrank_tables_if_small(squat_subspace *s, int rank_r, double lambda, int block_g, cudaStream_t st)
 {
-    s->lowrank_r = 0;
     if (block_g != 1 || rank_r < 1 || rank_r > SQUAT_LOWRANK_MAX_R || !(lambda > 0.0)) return SQUAT_OK;
     const int rc = squat_launch_lowrank_tables(s, rank_r, lambda, st);
     if (rc == SQUAT_OK) s->lowrank_r = rank_r;
+    return rc;
+}
+
+// A build that ends early leaves the previous W or parts of the next one; the dense kernels read whatever image there is.  So
+// the handle has no other form from a build's beginning to its end.
+void begin_build(squat_subspace *s) { s->lowrank_r = s->block_g = 0; }
+
+// The end of every build: update matrices from the eigen-pairs or the iterated basis, their image, and the form that it allows.
+int finish_build(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, cudaStream_t st)
+{
+    const bool no_update = rank_r == 0 || lambda == 0.0;
+    // channels of the first g-block are never corrected; with W = 0 none is
+    const int exact = no_update ? D : block_g;
+    const int rc = squat_launch_assemble(s, rank_r, lambda, block_g, left_rows, exact, st);
+    if (rc == SQUAT_OK) s->block_g = block_form(rank_r, lambda, block_g);
+    else s->lowrank_r = 0;
     return rc;
 }
 
@@ -216,16 +231,14 @@ int squat_build_subspace(squat_subspace *s, const void *q, int dtype, int n_q_he
     const long long vec = 16 / (long long)elem_size(dtype);
     if (stride_t < D || stride_h < 0 || stride_t % vec || stride_h % vec) return SQUAT_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    begin_build(s);
     int rc = squat_launch_gram(s, q, dtype, n_q_heads, n_tokens, stride_h, stride_t, st);
     if (rc != SQUAT_OK) return rc;
     rc = squat_launch_eig(s, st);
     if (rc != SQUAT_OK) return rc;
     rc = lowrank_tables_if_small(s, rank_r, lambda, block_g, st);
     if (rc != SQUAT_OK) return rc;
-    s->block_g = block_form(rank_r, lambda, block_g);
-    // channels of the first g-block are never corrected; with r = 0 or lambda = 0, W = 0 and none is
-    const int exact = (rank_r == 0 || lambda == 0.0) ? D : block_g;
-    return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
+    return finish_build(s, rank_r, lambda, block_g, 0, st);
 }
 
 int squat_build_subspace_from_gram(squat_subspace *s, const double *gram, int rank_r, double lambda, int block_g,
@@ -237,15 +250,14 @@ int squat_build_subspace_from_gram(squat_subspace *s, const double *gram, int ra
     if (!(lambda >= 0.0) || !std::isfinite(lambda)) return SQUAT_ERR_INVALID_ARG;
     if (block_g <= 0 || D % block_g != 0) return SQUAT_ERR_SHAPE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    begin_build(s);
     if (gram != s->gram)
         SQUAT_CUDA(cudaMemcpyAsync(s->gram, gram, (size_t)s->n_kv_heads * D * D * sizeof(double), cudaMemcpyDeviceToDevice, st));
     int rc = squat_launch_eig(s, st);
     if (rc != SQUAT_OK) return rc;
     rc = lowrank_tables_if_small(s, rank_r, lambda, block_g, st);
     if (rc != SQUAT_OK) return rc;
-    s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = (rank_r == 0 || lambda == 0.0) ? D : block_g;
-    return squat_launch_assemble(s, rank_r, lambda, block_g, 0, exact, st);
+    return finish_build(s, rank_r, lambda, block_g, 0, st);
 }
 
 int squat_build_subspace_power(squat_subspace *s, const void *q, int dtype, int n_q_heads, int n_tokens,
@@ -267,16 +279,13 @@ int squat_build_subspace_power(squat_subspace *s, const void *q, int dtype, int 
     const long long vec = 16 / (long long)elem_size(dtype);
     if (stride_t < D || stride_h < 0 || stride_t % vec || stride_h % vec) return SQUAT_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    begin_build(s);
     int rc = squat_launch_gram(s, q, dtype, n_q_heads, n_tokens, stride_h, stride_t, st);
     if (rc != SQUAT_OK) return rc;
-    const bool no_update = rank_r == 0 || lambda == 0.0;
-    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
-    s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = no_update ? D : block_g;
-    if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);      // W = 0: nothing to iterate
+    if (rank_r == 0 || lambda == 0.0) return finish_build(s, 0, lambda, block_g, 0, st);      // W = 0: nothing to iterate
     rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
     if (rc != SQUAT_OK) return rc;
-    return squat_launch_assemble(s, rank_r, lambda, block_g, 64, exact, st);
+    return finish_build(s, rank_r, lambda, block_g, 64, st);      // (the iterated basis is no eigenbasis: no rank-r form)
 }
 
 int squat_build_subspace_power_from_gram(squat_subspace *s, const double *gram, int rank_r, double lambda, int block_g,
@@ -292,16 +301,13 @@ int squat_build_subspace_power_from_gram(squat_subspace *s, const double *gram, 
     if (rank_r > 0 && (!start_block || ((uintptr_t)start_block & 7u))) return SQUAT_ERR_INVALID_ARG;
     if (start_stride_h != 0 && start_stride_h < (long long)D * rank_r) return SQUAT_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    begin_build(s);
     if (gram != s->gram)
         SQUAT_CUDA(cudaMemcpyAsync(s->gram, gram, (size_t)s->n_kv_heads * D * D * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    const bool no_update = rank_r == 0 || lambda == 0.0;
-    s->lowrank_r = 0;                      // the iterated basis is no eigenbasis
-    s->block_g = block_form(rank_r, lambda, block_g);
-    const int exact = no_update ? D : block_g;
-    if (no_update) return squat_launch_assemble(s, 0, lambda, block_g, 0, exact, st);
+    if (rank_r == 0 || lambda == 0.0) return finish_build(s, 0, lambda, block_g, 0, st);
     int rc = squat_launch_power(s, start_block, start_stride_h, rank_r, iters, lambda, st);
     if (rc != SQUAT_OK) return rc;
-    return squat_launch_assemble(s, rank_r, lambda, block_g, 64, exact, st);
+    return finish_build(s, rank_r, lambda, block_g, 64, st);      // (the iterated basis is no eigenbasis: no rank-r form)
 }
 
 int squat_subspace_export(const squat_subspace *s, void *stream, float *W_host, double *gram_host,
@@ -365,7 +371,7 @@ int squat_subspace_import(squat_subspace *s, const float *W_host, void *stream)
             for (int j = 0; j < D; ++j)
                 if (W_host[((size_t)h * D + jp) * D + j] != 0.0f) { uncorrected = jp; break; }
     const int exact = uncorrected;
-    s->lowrank_r = s->block_g = 0;         // an imported W comes without its factors or block size: dense kernel
+    begin_build(s);                        // an imported W comes without its factors or block size: dense kernels
     SQUAT_CUDA(cudaMemcpyAsync(s->Wt, wt.data(), hdd * sizeof(float), cudaMemcpyHostToDevice, st));
     int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, s->exact_channels, st);
     if (rc != SQUAT_OK) return rc;
