@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
         if (unit + 1 < u_hi) locate(unit + 1, nxt);
 #pragma unroll 1
         for (int blk = 0; blk < KEY_NBLK; ++blk) {
-            const bool more = blk + 1 < KEY_NBLK, first = blk == 0;
+            const bool more = blk + 1 < KEY_NBLK, first = blk == 0 && exact_channels > 0;
             bool exact = exact_channels > max(1, blk * KEY_BLK), open = false;
             const float *diag = sm.diag + blk * KEY_DIAG_BLK_FLOATS;
             const unsigned d_col = t_mine + (blk - 1) * KEY_BLK, e_hi = blk == 0 ? t_mine + KEY_E0_COL : d_col;

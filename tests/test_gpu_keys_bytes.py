@@ -29,6 +29,8 @@ CASES = [
     (128, 4, "bf16", False, 1, 2, 384, 1, "c62da23f20b06714"),         # 6 tiles: one token per lane
     (64, 2, "bf16", False, 1, 3, 256, 128, "7372d6c77882c383"),        # W = 0
     (128, 2, "bf16", False, 1, 150, 128, 128, "6b6e5b4df51c33e3"),
+    (64, 4, "bf16", True, 1, 3, 256, 0, "76478f6db04c3cdb"),           # entries that are never applied, but the first block is not decided exactly
+    (128, 2, "f32", False, 1, 150, 128, 0, "9ea59e97ea437615"),
     (64, 2, "ties", False, 1, 3, 640, 1, "6e4ce3bbc05e452f"),          # channels that hold raw values behind constant ones: exact ties where W corrects
     (64, 4, "ties", True, 1, 3, 640, 1, "9e1dd4054d8f4bc9"),
     (128, 2, "ties", False, 2, 75, 256, 1, "e6da49f205675825"),
@@ -39,6 +41,8 @@ def digest(G, bits, keys, m16, B, H, T, uncorrected):
     rng = np.random.default_rng([G, bits, B, H, T, uncorrected])
     W = np.tril(rng.integers(-60, 61, (H, D, D)), -1).astype(np.float32) / 256
     W[:, :uncorrected] = 0                              # row j' of W: what is pushed onto channel j'
+    if uncorrected == 0:
+        W[:, 0, 1] = 1
     if keys == "ties":
         k = rng.integers(-6, 7, (B, H, T // G, G, D))
         k[:, :, ::2, :, :1] = 2
