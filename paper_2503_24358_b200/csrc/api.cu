@@ -73,9 +73,9 @@ int finish_build(squat_subspace *s, int rank_r, double lambda, int block_g, int 
 {
     const bool no_update = rank_r == 0 || lambda == 0.0;
     // channels of the first g-block are never corrected; with W = 0 none is
-    const int exact = no_update ? D : block_g;
-    const int rc = squat_launch_assemble(s, rank_r, lambda, block_g, left_rows, exact, st);
-    if (rc == SQUAT_OK) s->block_g = block_form(rank_r, lambda, block_g);
+    const int exact = no_update ? D : block_g, form = block_form(rank_r, lambda, block_g);
+    const int rc = squat_launch_assemble(s, rank_r, lambda, block_g, left_rows, exact, form, st);
+    if (rc == SQUAT_OK) s->block_g = form;
     else s->lowrank_r = 0;
     return rc;
 }
@@ -177,7 +177,7 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     const size_t o_rem = carve((size_t)n_kv_heads * SQUAT_GRAM_REM_CAP * sizeof(SquatGramRem));
     const size_t o_tri = carve((size_t)n_kv_heads * 3 * D * sizeof(double));
     const size_t o_scl = carve((size_t)n_kv_heads * sizeof(double));
-    const size_t o_exact = carve(sizeof(int));
+    const size_t o_words = carve(2 * sizeof(int));
     const size_t o_lr = carve((size_t)n_kv_heads * D * 2 * SQUAT_LOWRANK_MAX_R * sizeof(float));
     char *base = nullptr;
     if (cudaMalloc(&base, off) != cudaSuccess) { cudaGetLastError(); delete s; return SQUAT_ERR_ALLOC; }
@@ -194,10 +194,10 @@ int squat_subspace_create(int n_kv_heads, int head_dim, squat_subspace **out)
     s->gram_rem = reinterpret_cast<SquatGramRem *>(base + o_rem);
     s->tri = reinterpret_cast<double *>(base + o_tri);
     s->eig_scale = reinterpret_cast<double *>(base + o_scl);
-    s->exact_channels = reinterpret_cast<int *>(base + o_exact);
+    s->words = reinterpret_cast<int *>(base + o_words);
     s->lr_table = reinterpret_cast<float *>(base + o_lr);
-    const int all_exact = D;        // W starts as zero: every channel is uncorrected
-    if (cudaMemcpy(s->exact_channels, &all_exact, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
+    const int zero_w[2] = {D, 0};   // W starts as zero: every channel is uncorrected
+    if (cudaMemcpy(s->words, zero_w, sizeof(zero_w), cudaMemcpyHostToDevice) != cudaSuccess) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
     s->status = squat_status_word();
     if (!s->status) { cudaFree(base); delete s; return SQUAT_ERR_CUDA; }
     *out = s;
@@ -373,7 +373,7 @@ int squat_subspace_import(squat_subspace *s, const float *W_host, void *stream)
     const int exact = uncorrected;
     begin_build(s);                        // an imported W comes without its factors or block size: dense kernels
     SQUAT_CUDA(cudaMemcpyAsync(s->Wt, wt.data(), hdd * sizeof(float), cudaMemcpyHostToDevice, st));
-    int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, s->exact_channels, st);
+    int rc = squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact, 0, s->words, st);
     if (rc != SQUAT_OK) return rc;
     SQUAT_CUDA(cudaStreamSynchronize(st));
     return SQUAT_OK;
@@ -400,12 +400,20 @@ int quantize_keys_impl(const squat_subspace *s, const void *k, int dtype, int ba
         return squat_launch_quant_keys_lowrank(s->lr_table, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t,
                                                bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
                                                meta16, static_cast<cudaStream_t>(stream));
-    if (s->block_g > 0 && !s->prefer_dense)
-        return squat_launch_quant_keys_block(s->block_g, s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t,
-                                             bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
-                                             meta16, static_cast<cudaStream_t>(stream));
+    // A captured call runs again whenever its graph is launched, perhaps after the handle has been built with another block size: then
+    // the graph holds both kernels, and each looks at the image's own word and leaves what is not its (a launch of 2 us).
+    int not_form = 0;
+    if (s->block_g > 0 && !s->prefer_dense) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) != cudaSuccess) cudaGetLastError();
+        if (capture == cudaStreamCaptureStatusActive) not_form = s->block_g;
+        rc = squat_launch_quant_keys_block(s->block_g, s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t,
+                                           bits, group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status,
+                                           not_form ? s->words + 1 : nullptr, meta16, static_cast<cudaStream_t>(stream));
+        if (rc != SQUAT_OK || !not_form) return rc;
+    }
     return squat_launch_quant_keys(s->Wimg, k, dtype, batch, n_kv_heads, n_tokens, stride_b, stride_h, stride_t, bits,
-                                   group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status, s->exact_channels,
+                                   group_size, codes, scales, zeros, out_stride_b, out_stride_h, s->status, s->words, not_form,
                                    meta16, static_cast<cudaStream_t>(stream));
 }
 }  // namespace

@@ -69,7 +69,8 @@ struct KeyParams {
     int units_per_head;       // 256 tokens each (512 with two pairs per lane)
     int total_units;
     unsigned *status;
-    const int *exact_channels;    // device word: leading channels that no earlier channel corrects
+    const int *words;         // device words: leading channels that no earlier channel corrects, and the image's block size;
+    int not_form;             // not 0: an image of that block size is not this kernel's (see quantize_keys_impl)
 #ifdef SQUAT_CHECKED
     SqExtent x_k, x_codes, x_scales, x_zeros, x_img;      // what the caller's tensors and the handle's images span
 #endif
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
     const int u_lo = (int)((long long)p.total_units * blockIdx.x / gridDim.x);
     const int u_hi = (int)((long long)p.total_units * (blockIdx.x + 1) / gridDim.x);
     grid_wait();
+    if (p.not_form && p.words[1] == p.not_form) return;
     volatile unsigned *timeout = &sm.timeout;
     const unsigned mbar_e = smem_u32(&sm.mbar_e), mbar_d = smem_u32(&sm.mbar_d), mbar_r = smem_u32(&sm.mbar_r), mbar_diag = smem_u32(&sm.mbar_diag), mbar_pan = smem_u32(&sm.mbar_pan);
 
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_diag), "r"(1) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar_pan), "r"(1) : "memory");
         sm.timeout = 0;
-        sm.exact_channels = (unsigned)*p.exact_channels;
+        sm.exact_channels = (unsigned)p.words[0];
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (u_lo < u_hi) stage(u_lo / p.units_per_head);
     }
@@ -606,9 +608,12 @@ __global__ void __launch_bounds__(KEY_THREADS, 2 / key_np(G)) quant_keys_kernel(
 // Grid (heads, slices): the kernel is a chain of two dependent global accesses, so more CTAs, not more work per thread, shorten
 // it; each thread takes (panel, 4-k chunk, channel n): four coalesced row reads, one 16-byte store.
 __global__ void __launch_bounds__(256) pack_w_kernel(const float *__restrict__ Wt, float *__restrict__ Wimg, int exact_channels,
-                                                        int *__restrict__ exact_channels_dev)
+                                                     int block_form, int *__restrict__ words_dev)
 {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *exact_channels_dev = exact_channels;    // travels with the matrices it describes
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {      // these travel with the matrices they describe
+        words_dev[0] = exact_channels;
+        words_dev[1] = block_form;
+    }
     const float *src = Wt + (long long)blockIdx.x * D * D;
     float *img = Wimg + (long long)blockIdx.x * KEY_IMG_FLOATS;
     const int first = blockIdx.y * blockDim.x + threadIdx.x, stride = gridDim.y * blockDim.x;
@@ -661,10 +666,10 @@ int launch(const KeyParams &p, int grid, int dtype, int meta16, cudaStream_t st)
 
 }  // namespace
 
-int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_channels, int *exact_channels_dev, cudaStream_t st)
+int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_channels, int block_form, int *words_dev, cudaStream_t st)
 {
     constexpr int PACK_SLICES = 8;
-    pack_w_kernel<<<dim3(H, PACK_SLICES), 256, 0, st>>>(Wt, Wimg, exact_channels, exact_channels_dev);
+    pack_w_kernel<<<dim3(H, PACK_SLICES), 256, 0, st>>>(Wt, Wimg, exact_channels, block_form, words_dev);
     squat_count_launch();
     SQUAT_LAUNCH_CHECK();
     return SQUAT_OK;
@@ -673,7 +678,7 @@ int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int e
 int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                                  long long sb, long long sh, long long st_, int bits, int G,
                                  unsigned char *codes, void *scales, void *zeros,
-                                 long long osb, long long osh, unsigned *status, const int *exact_channels, int meta16, cudaStream_t st)
+                                 long long osb, long long osh, unsigned *status, const int *words, int not_form, int meta16, cudaStream_t st)
 {
     // Which kernel: us of keys_lane.cu against this one, bf16 keys.  128 heads x 32768: G = 32 1298 / 1350, G = 64 1583 / 1198, G = 128 1719 / 1277.  32
     // heads x 4096: 45.0 / 49.8, 54.4 / 44.7, 59.0 / 46.4.  32 heads x 128 (one tile per CTA or less): 14.2 / 16.5, 18.2 / 16.0, 19.6 / 22.4.  So groups
@@ -681,13 +686,14 @@ int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int bat
     // chip idle, have one token per lane.
     const long long tiles = H * (((long long)batch * (T / G) * G + 127) / 128);
     if (G == 32 || (G == 128 && tiles <= squat_sm_count()))
-        return squat_launch_quant_keys_lane(Wimg, k, dtype, batch, H, T, sb, sh, st_, bits, G, codes, scales, zeros, osb, osh, status, exact_channels, meta16, st);
+        return squat_launch_quant_keys_lane(Wimg, k, dtype, batch, H, T, sb, sh, st_, bits, G, codes, scales, zeros, osb, osh, status, words, not_form, meta16, st);
     KeyParams p;
     p.Wimg = Wimg; p.k = k; p.sb = sb; p.sh = sh; p.st = st_;
     p.codes = codes; p.scales = scales; p.zeros = zeros; p.osb = osb; p.osh = osh;
     p.groups_per_bh = T / G;
     p.status = status;
-    p.exact_channels = exact_channels;
+    p.words = words;
+    p.not_form = not_form;
     const long long groups_per_head = (long long)batch * p.groups_per_bh;
     const int np = key_np(G), places = 2 / np * squat_sm_count();
     const long long unit = 256 * np / G;

@@ -51,6 +51,7 @@ struct KeyBlockParams {
     int units_per_head;
     int total_units;
     unsigned *status;
+    const int *form;          // not null: device word, the image's block size; one of another is not this kernel's (see quantize_keys_impl)
 #ifdef SQUAT_CHECKED
     SqExtent x_k, x_codes, x_scales, x_zeros, x_img;      // what the caller's tensors and the handle's images span
 #endif
@@ -299,6 +300,7 @@ __global__ void __launch_bounds__(KB_THREADS, 2) quant_keys_block_kernel(const K
     const int u_lo = (int)((long long)p.total_units * blockIdx.x / gridDim.x);
     const int u_hi = (int)((long long)p.total_units * (blockIdx.x + 1) / gridDim.x);
     grid_wait();
+    if (p.form && *p.form != GB) return;
     const unsigned img_mbar = smem_u32(mbar + Lay::SLOTS);
 
     // One head's panels into shared memory (one thread).  The image has them by 32 source channels with all later channels; of those
@@ -652,13 +654,14 @@ int launch(KeyBlockParams p, int H, int B, int dtype, int meta16, cudaStream_t s
 int squat_launch_quant_keys_block(int block_g, const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                                   long long sb, long long sh, long long st_, int bits, int G,
                                   unsigned char *codes, void *scales, void *zeros,
-                                  long long osb, long long osh, unsigned *status, int meta16, cudaStream_t st)
+                                  long long osb, long long osh, unsigned *status, const int *form, int meta16, cudaStream_t st)
 {
     KeyBlockParams p;
     p.Wimg = Wimg; p.k = k; p.sb = sb; p.sh = sh; p.st = st_;
     p.codes = codes; p.scales = scales; p.zeros = zeros; p.osb = osb; p.osh = osh;
     p.groups_per_bh = T / G;
     p.status = status;
+    p.form = form;
 #ifdef SQUAT_CHECKED
     {
         const unsigned long long es = dtype == SQUAT_BF16 ? 2 : 4, ms = meta16 ? 2 : 4;

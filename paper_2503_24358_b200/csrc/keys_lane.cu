@@ -84,7 +84,9 @@ struct KeyParams {
     int tiles_per_head;       // 128-token tiles per head (the last one may be ragged)
     int total_tiles;          // H * tiles_per_head
     unsigned *status;
-    const int *exact_channels;    // device word: leading channels that no earlier channel corrects; their blocks are decided exactly (see sweep_block)
+    const int *words;         // device words: leading channels that no earlier channel corrects, whose blocks are decided exactly (see
+                              // sweep_block), and the image's block size;
+    int not_form;             // not 0: an image of that block size is not this kernel's (see quantize_keys_impl)
 #ifdef SQUAT_CHECKED
     SqExtent x_k, x_codes, x_scales, x_zeros, x_img;      // what the caller's tensors and the handle's images span
 #endif
@@ -309,6 +311,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_lane_kernel(const Ke
         return n;
     };
     grid_wait();          // (its global loads are plain ones; laundering p here would cost registers the sweeps need)
+    if (p.not_form && p.words[1] == p.not_form) return;
     const unsigned img_mbar = smem_u32(mbar + TC_SLOTS);
     unsigned img_phase = 0;
 
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) quant_keys_lane_kernel(const Ke
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(img_mbar), "r"(1) : "memory");
         shared_words[1] = 0;
-        shared_words[2 + TC_SLOTS] = (unsigned)*(p.exact_channels);
+        shared_words[2 + TC_SLOTS] = (unsigned)p.words[0];
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // the first head's image is on its way while the rest of the set-up runs
         if (t_lo < t_hi) {
@@ -591,14 +594,15 @@ int launch_keys(KeyParams p, int dtype, int meta16, cudaStream_t st)
 int squat_launch_quant_keys_lane(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                             long long sb, long long sh, long long st_, int bits, int G,
                             unsigned char *codes, void *scales, void *zeros,
-                            long long osb, long long osh, unsigned *status, const int *exact_channels, int meta16, cudaStream_t st)
+                            long long osb, long long osh, unsigned *status, const int *words, int not_form, int meta16, cudaStream_t st)
 {
     KeyParams p;
     p.Wimg = Wimg; p.k = k; p.sb = sb; p.sh = sh; p.st = st_;
     p.codes = codes; p.scales = scales; p.zeros = zeros; p.osb = osb; p.osh = osh;
     p.B = batch; p.H = H; p.T = T; p.groups_per_bh = T / G;
     p.status = status;
-    p.exact_channels = exact_channels;
+    p.words = words;
+    p.not_form = not_form;
 #ifdef SQUAT_CHECKED
     {
         const unsigned long long es = dtype == SQUAT_BF16 ? 2 : 4, ms = meta16 ? 2 : 4;

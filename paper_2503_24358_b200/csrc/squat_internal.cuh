@@ -21,16 +21,18 @@ struct squat_subspace {
     int head_dim;
     int device;
     int gram_chunks_cap;   // capacity (in row chunks per head) of gram_partial
-    int *exact_channels;     // device word: leading channels that receive no correction (d when W = 0); written in
-                           // stream order by the kernel that packs W, read by the key kernel, so it always belongs to the W it is
-                           // launched with (a host-side copy could be overtaken by a build enqueued from another thread or stream)
+    int *words;            // two device words that belong to the image of W: leading channels that receive no correction (d when W = 0);
+                           // the block size that block_g below will be (0: none).  Written in stream order by the kernel that packs
+                           // W, read by the key kernels, so they always belong to the W those are launched with (a host-side
+                           // copy could be overtaken by a build enqueued from another thread or stream)
     float *Wt;             // [H, d, d] float32, Wt[h][j][j'] = W[j'][j]  (row j = update vector of channel j)
     float *Wimg;           // [H, SQUAT_KEY_IMG_FLOATS] the same matrices as the key kernels stage them in shared memory (pack_w_kernel)
     float *lr_table;       // [H, d, 2 * SQUAT_LOWRANK_MAX_R] rows [v_j | c_j] of the rank-r form of W (keys_lowrank.cu)
     int lowrank_r;         // > 0: lr_table describes the same update as Wt (set by the SVD builds with g = 1 and a small rank);
                            // host-side, read when a key call is enqueued: calls on one handle are issued in execution order
     int block_g;           // 32 or 64: W comes from block updates of that many channels, so its diagonal blocks are zero and the
-                           // kernel of keys_block.cu applies; 0 otherwise (host-side, like lowrank_r)
+                           // kernel of keys_block.cu applies; 0 otherwise, and from the beginning of a build until all of it has been
+                           // enqueued (host-side, like lowrank_r)
     int prefer_dense;      // 1: squat_quantize_keys uses the dense kernel even when one of the other two forms applies
     double *gram;          // [H, d, d] Gram matrices
     double *gram_partial;  // [chunks, H, d, d] per-chunk partial Gram matrices (deterministic reduction)
@@ -103,7 +105,7 @@ int squat_launch_gram_parts(const void *q, int dtype, int H, int n_tokens, int q
 int squat_launch_gram_i8(squat_subspace *s, const void *q, int n_q_heads, int n_tokens, long long stride_h, long long stride_t, cudaStream_t st);
 bool squat_gram_i8_fits(const squat_subspace *s, int dtype, int n_q_heads, int n_tokens, long long stride_h, long long stride_t);
 int squat_launch_eig(squat_subspace *s, cudaStream_t st);
-int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_channels, cudaStream_t st);
+int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_channels, int block_form, cudaStream_t st);
 int squat_launch_power(squat_subspace *s, const double *start, long long start_stride_h, int rank_r, int iters,
                        double lambda, cudaStream_t st);
 
@@ -112,19 +114,19 @@ int squat_launch_quant_keys_lowrank(const float *table, const void *k, int dtype
                                     long long sb, long long sh, long long st_, int bits, int G,
                                     unsigned char *codes, void *scales, void *zeros,
                                     long long osb, long long osh, unsigned *status, int meta16, cudaStream_t st);
-int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_channels, int *exact_channels_dev, cudaStream_t st);
+int squat_launch_pack_update_matrices(const float *Wt, float *Wimg, int H, int exact_channels, int block_form, int *words_dev, cudaStream_t st);
 int squat_launch_quant_keys(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                             long long sb, long long sh, long long st_, int bits, int G,
                             unsigned char *codes, void *scales, void *zeros,
-                            long long osb, long long osh, unsigned *status, const int *exact_channels_dev, int meta16, cudaStream_t st);
+                            long long osb, long long osh, unsigned *status, const int *words_dev, int not_form, int meta16, cudaStream_t st);
 int squat_launch_quant_keys_lane(const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                                  long long sb, long long sh, long long st_, int bits, int G,
                                  unsigned char *codes, void *scales, void *zeros,
-                                 long long osb, long long osh, unsigned *status, const int *exact_channels_dev, int meta16, cudaStream_t st);
+                                 long long osb, long long osh, unsigned *status, const int *words_dev, int not_form, int meta16, cudaStream_t st);
 int squat_launch_quant_keys_block(int block_g, const float *Wimg, const void *k, int dtype, int batch, int H, int T,
                                   long long sb, long long sh, long long st_, int bits, int G,
                                   unsigned char *codes, void *scales, void *zeros,
-                                  long long osb, long long osh, unsigned *status, int meta16, cudaStream_t st);
+                                  long long osb, long long osh, unsigned *status, const int *form_dev, int meta16, cudaStream_t st);
 int squat_launch_quant_values(const void *v, int dtype, int batch, int H, int T, int d,
                               long long sb, long long sh, long long st_, int bits, int G,
                               unsigned char *codes, void *scales, void *zeros,

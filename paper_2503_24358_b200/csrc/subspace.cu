@@ -442,7 +442,7 @@ int squat_launch_gram(squat_subspace *s, const void *q, int dtype, int n_q_heads
     return SQUAT_OK;
 }
 
-int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_channels, cudaStream_t st)
+int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int block_g, int left_rows, int exact_channels, int block_form, cudaStream_t st)
 {
     constexpr size_t smem = ASM_SMEM;
     static std::atomic<unsigned long long> allowed{0};
@@ -460,7 +460,7 @@ int squat_launch_assemble(squat_subspace *s, int rank_r, double lambda, int bloc
         squat_count_launch();
         SQUAT_LAUNCH_CHECK();
     }
-    return squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact_channels, s->exact_channels, st);
+    return squat_launch_pack_update_matrices(s->Wt, s->Wimg, s->n_kv_heads, exact_channels, block_form, s->words, st);
 }
 
 // ------------------------------------------------------------------------- allocation-free Gram entry

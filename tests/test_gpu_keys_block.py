@@ -104,6 +104,36 @@ def test_block_keys_ragged_tiles_strides_and_windows(g, G, B, H, T):
     s.close()
 
 
+@pytest.mark.parametrize("captured,rebuilt", [(64, 1), (64, 32), (32, 64), (32, 16), (1, 64)])
+def test_a_captured_key_call_follows_the_handle(captured, rebuilt):
+    """A graph that holds a key call quantizes by the matrices that its handle has when the graph is launched, whatever block size they were
+    built with: the dense kernel's bytes for matrices that are not the captured kernel's."""
+    cfg = si.get_config(1).with_(batch=2, n_kv_heads=3, n_q_heads=3, n_tokens=256)
+    q = to_torch(si.gen_queries(cfg, n_tokens=256), cfg.dtype)
+    k = to_torch(si.gen_keys(cfg), cfg.dtype)
+    s = _build(cfg, 32, captured)
+    want_first = _quantize(s, cfg, k, 2, 32)
+    out = [torch.zeros_like(t) for t in want_first]
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        sq.squat_quantize_keys(s, k, 2, 32, *out)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(out, want_first))
+    sq.squat_build_subspace(s, q, 32, cfg.lam, rebuilt)
+    sq.squat_subspace_select_key_kernel(s, True)
+    want = _quantize(s, cfg, k, 2, 32)
+    for t in out:
+        t.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(out, want))
+    assert not torch.equal(out[0], want_first[0])
+    s.close()
+
+
 @pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
 @pytest.mark.parametrize("g,channel", [(64, 5), (64, 70), (32, 40)])
 def test_block_keys_nonfinite_stays_in_its_group_and_later_blocks(g, channel, value):

@@ -24,11 +24,12 @@ static int launch(const char *name)
     return 0;
 }
 static unsigned word;
+int fake_capturing = 0;
 int cudaMalloc(void **p, size_t n) { *p = aligned_alloc(256, (n + 255) / 256 * 256); return *p ? 0 : 2; }
 int cudaFree(void *p) { free(p); return 0; }
 int cudaGetDevice(int *d) { *d = 0; return 0; }
 int cudaGetSymbolAddress(void **p, const void *s) { *p = &word; return 0; }
-int cudaStreamIsCapturing(void *st, int *status) { *status = 0; return 0; }
+int cudaStreamIsCapturing(void *st, int *status) { *status = fake_capturing; return 0; }
 const char *cudaGetErrorName(int e) { return "error"; }
 const char *cudaGetErrorString(int e) { return "error"; }
 void **__cudaRegisterFatBinary(void *p) { static void *h; return &h; }
@@ -121,4 +122,16 @@ def test_a_build_that_fails_half_way_leaves_the_dense_form(lib, how, fail, after
     assert h.build(how, *before) == 0
     assert h.build(how, *after, fail=fail.encode()) != 0
     assert h.key_kernel() == "quant_keys"
+    h.close()
+
+
+def test_a_captured_call_with_block_updates_holds_the_dense_form_too(lib):
+    h = Handle(lib)
+    capturing = ctypes.c_int.in_dll(lib, "fake_capturing")
+    for block, want in ((64, "quant_keys_block quant_keys"), (1, "quant_keys")):
+        assert h.build("svd", 32, block) == 0
+        capturing.value = 1
+        assert h.key_kernel() == want
+        capturing.value = 0
+        assert h.key_kernel() == want.split()[0]
     h.close()
