@@ -33,7 +33,7 @@ def run_cases():
         torch.cuda.synchronize()
         return [hashlib.sha256(t.contiguous().cpu().numpy().tobytes()).hexdigest() for t in ts]
 
-    cases = [  # (name, base config, batch, heads, tokens, bits, G, rank, meta16)
+    cases = [  # (name, base config, batch, heads, tokens, bits, G, rank, meta16[, block size])
         ("dense f32 config 0", 0, 1, 8, 256, 2, 32, 32, False),
         ("dense ragged tiles", 1, 3, 3, 96, 2, 32, 32, False),
         ("dense one group per head", 1, 1, 5, 32, 4, 32, 16, False),
@@ -43,12 +43,18 @@ def run_cases():
         ("rank-r form", 1, 3, 2, 160, 2, 32, 8, False),
         ("rank-r form G=128 m16", 1, 2, 2, 256, 4, 128, 5, True),
         ("rank-r form f32 G=64", 0, 1, 3, 192, 2, 64, 3, False),
+        ("dense two pairs per lane", 1, 1, 160, 128, 2, 128, 32, False),
+        ("dense one pair, several heads per CTA", 1, 3, 100, 64, 4, 64, 16, True),
+        ("block updates of 64", 1, 3, 170, 128, 4, 128, 32, True, 64),
+        ("block updates of 64 f32, ragged", 0, 3, 2, 96, 2, 32, 16, False, 64),
+        ("block updates of 32", 1, 5, 70, 192, 2, 64, 32, False, 32),
+        ("block updates of 32 f32 m16", 0, 1, 3, 128, 4, 128, 16, True, 32),
     ]
-    for name, ci, B, H, T, bits, G, r, m16 in cases:
+    for name, ci, B, H, T, bits, G, r, m16, *block in cases:
         cfg = si.get_config(ci).with_(batch=B, n_kv_heads=H, n_q_heads=H, n_tokens=T)
         s = sq.Subspace(H, D)
         sq.squat_get_device_status(clear=True)
-        sq.squat_build_subspace(s, to_torch(si.gen_queries(cfg, n_tokens=max(T, 256)), cfg.dtype), r, cfg.lam, 1)
+        sq.squat_build_subspace(s, to_torch(si.gen_queries(cfg, n_tokens=max(T, 256)), cfg.dtype), r, cfg.lam, block[0] if block else 1)
         k, v = to_torch(si.gen_keys(cfg), cfg.dtype), to_torch(si.gen_values(cfg), cfg.dtype)
         # outputs sit at a token offset of a longer cache: strided stores
         Tc, off = T + 2 * G, G

@@ -104,6 +104,72 @@ def test_block_keys_ragged_tiles_strides_and_windows(g, G, B, H, T):
     s.close()
 
 
+@pytest.mark.parametrize("g,G,bits", [(64, 32, 2), (64, 128, 4), (32, 64, 2), (32, 32, 4)])
+def test_block_keys_clamp_where_a_16_bit_grid_leaves_the_extremes_outside(g, G, bits):
+    """Channels far from 0 against their range: the binary16 zero-point lies up to an eighth above or below the minimum, more than half a
+    step of the grid.  In uncorrected channels (the exact decision), in the middle and in the last block; every third group is
+    ordinary, so that one call holds both instances.  Algorithm 1 is replayed in float64 with the kernel's own codes and grids: a code is the
+    clamped nearest one but for what float32 leaves open, half a unit in the last place of the key's and of the
+    correction's sum (2^-24 of the value each) and 1e-6 L for the reciprocal; in uncorrected channels it is the nearest one."""
+    cfg = si.get_config(0).with_(batch=1, n_kv_heads=2, n_q_heads=2, n_tokens=9 * 128)
+    gen = torch.Generator().manual_seed(g + G)
+    k = torch.randn((1, 2, cfg.n_tokens // 128, 128, D), generator=gen)
+    far = [3, 31, 40, 63, 64, 100, 127]
+    for grp in range(9):
+        if grp % 3:
+            k[:, :, grp, :, far] = 300 + 0.07 * grp + 0.3 * torch.rand((1, 2, 128, len(far)), generator=gen)
+    k = k.view(1, 2, -1, D)
+    sq.squat_get_device_status(clear=True)
+    s = _build(cfg, 16, g)
+    kc, ks, kz = _quantize(s, cfg, k.cuda(), bits, G, True)
+    torch.cuda.synchronize()
+    L, T = 2 ** bits - 1, cfg.n_tokens
+    codes = torch.from_numpy(oracle.unpack(kc.cpu().numpy().reshape(2 * T, -1), D, bits)).view(2, T // G, G, D).double()
+    scale, zero = ks[0].double().cpu().unsqueeze(2), kz[0].double().cpu().unsqueeze(2)
+    deq = (codes * scale + zero).view(2, T, D)
+    W = torch.from_numpy(sq.squat_subspace_export(s)["W"]).double()
+    x = k[0].double().clone()
+    for j in range(D - 1):
+        x[:, :, j + 1:] += (deq[:, :, j] - x[:, :, j]).unsqueeze(2) * W[:, None, j + 1:, j]
+    x = x.view(2, T // G, G, D)
+    t = (x - zero) / scale
+    outside = (t < -0.5) | (t > L + 0.5)                 # the case is met: on both sides in uncorrected channels, and in corrected ones, whose
+    assert all((t[..., n] < -0.5).any() and (t[..., n] > L + 0.5).any() for n in far if n < g)         # ranges are wider
+    assert outside[..., g:].any() and not outside[:, ::3 * 128 // G].any()
+    off = (codes - t.clamp(0, L)).abs() - 0.5
+    assert off[..., :g].max() <= 0
+    assert (off <= 2 ** -23 * x.abs() / scale + 1e-6 * L).all()
+    low, high = x.amin(2, keepdim=True), x.amax(2, keepdim=True)
+    noise = 2 ** -22 * torch.maximum(low.abs(), high.abs())
+    assert ((zero - low).abs() <= 2 ** -11 * low.abs() + noise).all()                      # one rounding to binary16
+    assert ((scale - (high - low) / L).abs() <= 2 ** -11 * scale + 2 * noise / L).all()
+    assert sq.squat_get_device_status(clear=True) == 0
+    s.close()
+
+
+@pytest.mark.parametrize("g,G,bits,dtype,m16,B,H,T", [
+    (64, 32, 4, "f32", True, 3, 2, 160), (32, 64, 4, "bf16", True, 5, 3, 64), (64, 128, 4, "f32", False, 1, 310, 128), (32, 128, 2, "f32", True, 3, 2, 384)])
+def test_block_keys_windows_of_other_forms(g, G, bits, dtype, m16, B, H, T):
+    """The ragged units and window calls of the test above for 4 bits, float32 keys and 16-bit grids: identical bytes however a call is cut;
+    grids of the uncorrected channels equal to the dense kernel's, and codes but for what ties move."""
+    cfg = si.get_config(1).with_(batch=B, n_kv_heads=H, n_q_heads=H, n_tokens=T)
+    k = torch.randn((B, H, T, D), generator=torch.Generator().manual_seed(g + T)).to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda()
+    s = _build(si.get_config(1).with_(n_kv_heads=H, n_q_heads=H, n_tokens=256), 16, g)
+    whole = _quantize(s, cfg, k, bits, G, m16)
+    parts = [torch.zeros_like(t) for t in whole]
+    for b in range(B):
+        for lo in range(0, T, G):
+            sq.squat_quantize_keys(s, k[b:b + 1, :, lo:lo + G], bits, G, parts[0][b:b + 1, :, lo:], parts[1][b:b + 1, :, lo // G:], parts[2][b:b + 1, :, lo // G:],
+                                   out_stride_b=H * T, out_stride_h=T)
+    sq.squat_subspace_select_key_kernel(s, True)
+    dense = _quantize(s, cfg, k, bits, G, m16)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(whole, parts))
+    assert all(torch.equal(a[..., :n], b[..., :n]) for a, b, n in zip(whole, dense, (g * bits // 8, g, g)))
+    assert (whole[0] == dense[0]).float().mean().item() >= 0.99
+    s.close()
+
+
 @pytest.mark.parametrize("captured,rebuilt", [(64, 1), (64, 32), (32, 64), (32, 16), (1, 64)])
 def test_a_captured_key_call_follows_the_handle(captured, rebuilt):
     """A graph that holds a key call quantizes by the matrices that its handle has when the graph is launched, whatever block size they were
