@@ -102,6 +102,12 @@ def key_flops_per_vector(d, g, r=None):
     return 2 * (tri if r is None else min(tri, 2 * r * d))
 
 
+def dense_key_kernel(G, vectors):
+    """The kernel of the dense form that a launch runs: one token per lane for groups of 32, and of 128 in calls of at most a tile of
+    128 tokens per SM (148)."""
+    return "quant_keys_lane_kernel" if G == 32 or (G == 128 and vectors <= 148 * 128) else "quant_keys_kernel"
+
+
 def key_fma_split(d, g, blk=32):
     """The same multiply-adds split by where the dense key kernels run them: inside blocks of 32 channels on the FP32 pipes, across
     blocks on the tensor cores.  W[j'][j] is non-zero iff j' lies in a later g-block than j."""
@@ -720,7 +726,7 @@ def key_roofline(args, cfg, key_ms, vec_per_launch, peaks, fp32_peak, lowrank_r=
             "frac_vs_fp32_target_definition": "all %d algorithmic flop per vector (2 x min(dense triangle, 2 r d)) at the nominal "
                                               "FP32 peak of %.2f TFLOP/s: the reading the 50 %% target was stated in"
                                               % (key_flops_per_vector(d, cfg.block_g, cfg.rank_r), ALU_PEAK_TFLOPS),
-            "traffic": None, "kernel": "quant_keys_lowrank_kernel (rank-r form of the update)" if lowrank_r > 0 else "quant_keys_kernel", "ms_per_launch": key_ms, "key_vectors_per_launch": vec_per_launch,
+            "traffic": None, "kernel": "quant_keys_lowrank_kernel (rank-r form of the update)" if lowrank_r > 0 else dense_key_kernel(G, vec_per_launch), "ms_per_launch": key_ms, "key_vectors_per_launch": vec_per_launch,
             "key_vectors_per_s": vec_per_launch / t_s, "kv_input_gbs": vec_per_launch * d * elem / t_s / 1e9,
             "hbm_frac_of_" + peaks["source"]: kbytes / t_s / 1e9 / peaks["hbm_gbs"]}
     tr = key_kernel_traffic(cfg, args)

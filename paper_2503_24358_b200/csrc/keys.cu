@@ -20,8 +20,7 @@
 // a block ahead.  E_lo goes to shared memory as a K-major operand.
 //
 // A block is swept in halves of 16 channels.  Between them the first half's errors, read back from tensor memory, are pushed onto the
-// second half's values.  Straight code for 32 channels (50 KB for four tokens per lane) was slower by a third: it does not stay in the
-// instruction cache.
+// second half's values.  Straight code for 32 channels was slower by a third (50 KB and more for four tokens per lane).
 //
 // Hand-over from block b to b + 1 (a fifth warp issues the products: a sweeping one that did took 2 000 cycles a hand-over over it), onto
 // slices of 32 channels so that all products into a column have the same shape and are ordered by that:
@@ -29,7 +28,7 @@
 //       the others     D += E_lo Whi                           (commit: with one buffer of E_lo the next sweep waits for this too)
 //                      D += E_hi Wlo + E_hi Whi                (done while the next sweep runs)
 //
-// Bound: latency and instruction fetch.  A channel's chain (two reductions, reciprocal, rounding, push onto the next channel) is 71
+// Bound: latency.  A channel's chain (two reductions, reciprocal, rounding, push onto the next channel) is 71
 // cycles; one or two warps per scheduler make 160 to 200 of it.  128 heads x 32768 tokens take, in cycles of a unit of 128 channels, 25 000 (four
 // tokens per lane) in sweeps, 8 000 in pushes onto second halves, 6 000 in waits for products.  keys_lane.cu -> here: 128 heads x 32768, G = 128, 4
 // bits 1719 -> 1277 us, G = 64 1583 -> 1198; 32 heads x 4096, G = 128 59.0 -> 46.4, G = 64 54.4 -> 44.7; 64 x 32 heads x 128, G = 128 116 -> 94.
@@ -134,8 +133,8 @@ struct PairRows {
 // code into pieces) and used by nobody.
 // EXACT: decisions through the remainder.  The usual instance decides so in channel 0 alone (raw values; `head`).  In the other
 // channels of block 0 (`first`) it stores the rounded quotient too and says in `open` whether a remainder reached half a step: one element in
-// a million, and the block is swept again by the EXACT instance, whose code is so not fetched for every unit (128 heads x 32768, G = 128: 1355
-// -> 1269 us).  Deciding again at once, behind a branch per channel, made the sweep 1.6 times as long, and settling every channel in one
+// a million, and the block is swept again by the EXACT instance, which so does not run in every unit (128 heads x 32768, G = 128: 1355 -> 1269
+// us).  Deciding again at once, behind a branch per channel, made the sweep 1.6 times as long, and settling every channel in one
 // code the call 1.3 times.
 // ahead(jj): what is to be asked for at channel jj.
 template <int BITS, int NP, bool EXACT, bool M16, class Ahead>
@@ -261,8 +260,8 @@ __device__ __forceinline__ void sweep_half(const Ahead &ahead, bool head, bool f
 
 // The errors of a block's first half, read back from tensor memory, pushed onto the second half's values one by one in the channels'
 // order.  x: pairs of channels (2 q, 2 q + 1) of the lane's tokens, so that an entry of W is read once and not twice: a broadcast read is
-// charged by its width, and reads of W are the most of what shared memory does.  A loop over quads of channels: straight code for
-// all 16 pushed the sweep out of the instruction cache.
+// charged by its width, and reads of W are the most of what shared memory does.  A loop over quads of channels:
+// against straight code for all 16 it is faster for groups of 128 (1376 -> 1269 us for 128 heads x 32768) and slower for 64 (1164 -> 1197).
 template <int NT>
 __device__ __forceinline__ void push_across(u64 (&x)[KEY_HALF / 2][NT], unsigned e_hi, const float *__restrict__ across)
 {
