@@ -182,7 +182,8 @@ int squat_quantize_keys(const squat_subspace *s, const void *k, int dtype, int b
  *   prefer_dense   1: always run the dense kernel;  0: the default choice above.
  *   lowrank_rank   host, may be NULL: receives the rank the rank-r form is prepared for (0: not prepared).
  * Host-side state of the handle: like every call that takes the handle, issue it from one thread at a time, in the
- * order the work is to execute.
+ * order the work is to execute.  A key call captured into a graph quantizes by the matrices that the handle has when the graph
+ * runs, whatever block size they were built with; a call captured in the rank-r form needs a handle that is in that form then.
  */
 int squat_subspace_select_key_kernel(squat_subspace *s, int prefer_dense, int *lowrank_rank);
 
